@@ -269,23 +269,20 @@ int iedg_trace_solve(iedg_mesh* mesh, const double* K, const double* R, double* 
  *   lu_persistent: 1 = the batched LU runs as a persistent grid (resident CTAs per
  *                  SM x SMs) that takes elements from an atomic queue; 0 = one CTA
  *                  per element.
- *   lu_panel:      FP64 LU panel width, 16 or 32 (32 falls back to 16 when the panel
- *                  does not fit in shared memory).
+ *   lu_panel:      panel width of the FP64 LU's DFMA form, 16 or 32 (32 falls back to 16
+ *                  when the panel does not fit in shared memory).
  *   asm_chunk:     assembly column chunk, 8, 16 or 32 (0 = default: 8 for FP64, 16
  *                  for FP32; too large a chunk for shared memory falls back).
- *   lu_tensor:     1 = the Schur complement K = D - W Z of the partial LU on the tensor
- *                  cores (tcgen05, accumulation in tensor memory).  FP64 path: the FP64
- *                  operands are split exactly into integer slices of 7 bits, the slice
- *                  products of equal weight accumulate exactly in FP32 over K chunks of
- *                  64 and are summed in FP64 (results agree with the DFMA form to
- *                  FP64 rounding); the panel factorisation stays on DFMA; persistent
- *                  grid, panel 16; its per-CTA slice buffers (16 (nt + 1) nu floats
- *                  per resident CTA) are allocated by this call when it selects the
- *                  form (IEDG_ERR_OOM if they do not fit), not by the compute calls.  Mixed path: TF32 operands split in high and low
- *                  parts, three products ("3xTF32").  2 (mixed FP32 form only) = every
- *                  trailing update of the FP32 LU on the tensor cores (3xTF32, 128 x 64
+ *   lu_tensor:     tensor cores (tcgen05, accumulation in tensor memory) in the partial LU.
+ *                  FP64 path: the trailing updates as integer products of 8-bit digits of
+ *                  the FP64 operands, summed exactly and joined to FP64 (the error of an
+ *                  update is below that of the DFMA form).  1 = always; 0 = on elements
+ *                  of at least 64 u-unknowns, where it is the faster form, DFMA updates
+ *                  below.  Mixed path: 1 = the Schur complement K = D - W Z, TF32 operands
+ *                  split in high and low parts, three products ("3xTF32"); 2 (mixed FP32
+ *                  form only) = every trailing update of the FP32 LU (3xTF32, 128 x 64
  *                  tiles accumulated in TMEM and subtracted from the trailing block by
- *                  reductions in L2).  0 = DFMA / FFMA updates.  Default 0, except 2
+ *                  reductions in L2); 0 = FFMA updates.  Default 0, except 2
  *                  for mixed FP32 handles of meshes with mixed orders.  Handles created with
  *                  IEDG_PRECISION_MIXED_TF32 or _MIXED_BF16 always take the tensor-core
  *                  form in their own operand precision (the schedule never changes

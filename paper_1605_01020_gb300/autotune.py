@@ -21,8 +21,8 @@ def mesh_key(mesh, precision, gpu_name):
 
 def candidates(precision, order):
     """Candidate schedules: persistent LU on/off x FP64 panel 16/32 x assembly chunk,
-    and the tensor-core forms (the FP64 Schur complement by exact operand splitting;
-    on the mixed path the FP32 LU with every trailing update in 3xTF32, or only its
+    and the tensor-core forms (FP64: the digit form, which 0 also takes on elements of
+    64 u-unknowns or more; on the mixed path the FP32 LU with every trailing update in 3xTF32, or only its
     deferred Schur complement; handles with TF32 or BF16 Schur operands always take
     the tensor-core form).
     order 0 (mixed orders): the FP64 panel stays 16 (the largest elements' panel of
@@ -30,7 +30,7 @@ def candidates(precision, order):
     panels = [16, 32] if (precision == 0 and 1 <= order <= 3) else [16]
     chunks = [8, 16] if precision == 0 else [16, 32]
     if precision == 0:
-        # DFMA forms, then the tensor-core Schur form (persistent, panel 16 only)
+        # the form chosen by size, then the tensor-core form (persistent, panel 16 only)
         out = [dict(lu_persistent=a, lu_panel=b, asm_chunk=c, lu_tensor=0)
                for a, b, c in itertools.product([1, 0], panels, chunks)]
         return out + [dict(lu_persistent=1, lu_panel=16, asm_chunk=c, lu_tensor=1) for c in chunks]

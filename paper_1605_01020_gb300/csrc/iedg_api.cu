@@ -562,8 +562,6 @@ static int check_desc(const iedg_mesh_desc* D, bool mixed) {
 static void destroy_impl(iedg_mesh* M) {
   for (iedg_mesh* C : M->groups) destroy_impl(C);
   M->groups.clear();
-  if (M->oz_scratch) cudaFree(M->oz_scratch);
-  M->oz_scratch = nullptr;
   free_all(M);
   delete M;
 }
@@ -1212,14 +1210,6 @@ extern "C" int iedg_set_schedule(iedg_mesh* M, const iedg_schedule* in) {
   for (int i = 0; i < 4; ++i) {
     const int c = in->asm_chunk_by_order[i];
     if (c != 0 && c != 8 && c != 16 && c != 32) return fail(M, IEDG_ERR_INVALID_ARG, "schedule values out of range");
-  }
-  if (M->precision == IEDG_PRECISION_FP64 && in->lu_tensor == 1) {
-    // the FP64 tensor-core Schur form needs per-CTA slice buffers: allocated here, so
-    // that compute calls allocate nothing
-    const cudaError_t err = prepare_lu64_oz(M);
-    if (err != cudaSuccess)
-      return fail(M, err == cudaErrorMemoryAllocation ? IEDG_ERR_OOM : IEDG_ERR_CUDA,
-                  std::string("FP64 tensor-core Schur buffers: ") + cudaGetErrorString(err));
   }
   M->sched.lu_persistent = in->lu_persistent;
   M->sched.lu_panel = in->lu_panel;

@@ -348,7 +348,7 @@ __device__ __forceinline__ long long inf_key() {
 
 template <class T, int NB>
 __device__ __forceinline__ void lu_element(const LuElem& el, T* __restrict__ S, int8_t* __restrict__ status,
-                                           int* __restrict__ pivots, const int64_t e, bool defer_schur = false) {
+                                           int* __restrict__ pivots, const int64_t e) {
   extern __shared__ __align__(16) unsigned char smraw[];
   T* sm = reinterpret_cast<T*>(smraw);
   __shared__ int piv[NB];
@@ -417,7 +417,7 @@ __device__ __forceinline__ void lu_element(const LuElem& el, T* __restrict__ S, 
       __syncthreads();
     }
     // U11 / L11 (and, when the factors are kept, L21) back to the element matrix
-    const int wrows = (pivots || defer_schur) ? rows : nb;   // L21 is the W of the deferred form
+    const int wrows = pivots ? rows : nb;
     for (int idx = tid; idx < wrows * nb; idx += LU_THREADS) {
       int r = idx / nb, j = idx % nb;
       A[(int64_t)(kb + r) * ld + kb + j] = P[r * NB + j];
@@ -456,24 +456,12 @@ __device__ __forceinline__ void lu_element(const LuElem& el, T* __restrict__ S, 
       }
     }
     __syncthreads();
-    const int r0 = kb + nb;
-    if (defer_schur) {
-      // the trace block of the trace rows gets all panels at once afterwards
-      lu64_update_rect<T, NB>(A, ld, P, Uc, kb, nb, r0, n, r0, nu);
-      lu64_update_rect<T, NB>(A, ld, P, Uc, kb, nb, r0, nu, nu, ncol);
-    } else {
-      // A22 -= L21 U12, rows [kb+nb, n), cols [kb+nb, n]
-      lu64_update_rect<T, NB>(A, ld, P, Uc, kb, nb, r0, n, r0, ncol);
-    }
+    // A22 -= L21 U12, rows [kb+nb, n), cols [kb+nb, n]
+    lu64_update_rect<T, NB>(A, ld, P, Uc, kb, nb, kb + nb, n, kb + nb, ncol);
   }
   // status: a non-finite pivot candidate, an exact zero pivot, or a non-finite Schur
-  // complement (deferred form: the caller checks the Schur complement after forming it)
+  // complement
   nonfin = __syncthreads_or(nonfin);
-  if (defer_schur) {
-    if (tid == 0) status[e] = nonfin ? IEDG_ELEM_NONFINITE : (sing ? IEDG_ELEM_SINGULAR : IEDG_ELEM_OK);
-    __syncthreads();
-    return;
-  }
   int bad = 0;
   for (int idx = tid; idx < (n - nu) * (ncol - nu); idx += LU_THREADS) {
     int r = nu + idx / (ncol - nu), c = nu + idx % (ncol - nu);
@@ -485,184 +473,496 @@ __device__ __forceinline__ void lu_element(const LuElem& el, T* __restrict__ S, 
                        : (sing ? IEDG_ELEM_SINGULAR : (bad ? IEDG_ELEM_NONFINITE : IEDG_ELEM_OK));
 }
 
-// ----------------------------------------------------------- FP64 Schur complement on tcgen05
-// [K | R] = [D | G] - W [Z | z] of the FP64 form with the products on the tensor cores,
-// by an exact splitting of the FP64 operands (the Ozaki scheme): each row i of W is
-// scaled by a power of two 2^e_i >= its largest entry, each column j of Z by 2^f_j,
-// and the scaled entries are written as sums of OZ_S integer slices of OZ_BETA bits,
-//   W_ik = 2^e_i sum_s v_s 2^(-s beta),  Z_kj = 2^f_j sum_t w_t 2^(-t beta)  (+ a rest
-// below 2^-(S beta)), v, w integers with |v|, |w| <= 2^beta, exact in TF32.  The slice
-// products of one level l = s + t (2 <= l <= S + 1) share the scale 2^(e_i + f_j - l beta)
-// and accumulate in one FP32 TMEM accumulator: with beta = 7 and K chunks of 64 every
-// partial sum is an integer below 2^23, so the tensor cores add exactly; each chunk's
-// levels are then scaled and summed in FP64.  Levels above S + 1 (below 2^-63 of the
-// product scale) are dropped.  The splitting and the level sums are FP64 work
-// (about a quarter of the FP64 multiply-adds the product itself would take).
-constexpr int OZ_S = 8, OZ_BETA = 7, OZ_L = 8;           // slices, bits per slice, levels 2..9
-constexpr int OZ_KC = 64, OZ_KS = 16;                    // exact-accumulation chunk, staging step
-constexpr int OZ_TM = 128, OZ_TN = 32;
-constexpr int OZ_TMEM_COLS = OZ_L * OZ_TN;              // 256
-constexpr int OZ_A_BYTES = OZ_TM * OZ_KS * 4, OZ_B_BYTES = OZ_TN * OZ_KS * 4;
-constexpr int OZ_STAGE_BYTES = OZ_S * (OZ_A_BYTES + OZ_B_BYTES);   // 80 KB
+// ------------------------------------------------------------------ FP64 partial LU, digit form
+// FP64 partial LU of the bordered element matrices with every trailing update on the
+// tensor cores, by splitting the FP64 operands into 8-bit digits.
+//
+// Same factorisation as lu_element<double>: right-looking, 32-column
+// panels, pivots among the u-rows only (largest |a|, lowest row on ties).  GB300 issues
+// two FP64 multiply-adds per SM and clock against 4096 BF16 ones on the tensor cores,
+// so the bulk of the arithmetic, A22 -= L21 U12 (rows x 32 times 32 x columns), goes
+// there in integers:
+//   * each row of L21 and each column of U12 is scaled by the power of two of its
+//     largest entry and rounded to a 63-bit integer X, |X| < 2^62, written in balanced
+//     base 256: X = sum_s d_s 256^(8-s), s = 1..8, |d_s| <= 128, exact in BF16;
+//   * digit products of equal weight, s + t = l, l = 2..9, share one FP32 accumulator in
+//     TMEM.  A level's sum is an integer of at most 8 32 2^14 = 2^22, so the tensor core
+//     adds exactly (the splitting of Ozaki, Ogita, Oishi and Rump, "Error-free
+//     transformations of matrix multiplication", 2012, with K short enough that no
+//     level has to be flushed).  Levels past 9 (below 2^-60 of the largest product)
+//     are dropped;
+//   * the levels are joined in a 64-bit integer, normalised to an FP64 number with
+//     integer instructions, and subtracted: one FP64 addition per entry and panel
+//     where the DFMA form spends 32 multiply-adds.
+// The error of an update is 2^-57 of the largest product of its row and column plus the
+// rounding of one FP64 subtraction; the DFMA form rounds 32 times.
+//
+// Roles: the 128 TMEM lanes are columns of A22 (the MMA's A operand is U12^T), so a
+// warp's accesses of A22 are rows of 32 consecutive columns; the B operand stacks the
+// digits t of 16 rows of L21, so that digit s of U12 meets all digits t <= 9 - s in one
+// instruction whose columns land on the levels s + 1 .. 9 in order.
+//
+// Panel factorisation, the trace rows of L21 and U12 = L11^-1 A12 stay on the FP64 pipe,
+// which bounds the kernel: per element of 320 + 280 unknowns 2.3 M multiply-adds there
+// and 2 M additions of the updates (65 M multiply-adds in the DFMA form).  Two CTAs per
+// SM, so that one element's panels overlap the other's updates.
+// Measured, all elements of a mesh, DFMA form -> this one: 3D p = 3, 4096 elements
+// 505.9 -> 100.5 ms; p = 2, 2002 elements 26.5 -> 8.3 ms; p = 4, 210 elements 238.6 -> 57.9 ms;
+// 2D p = 3 (64 + 48 unknowns), 851 elements 1.53 -> 0.82 ms.  Below 64 u-unknowns an
+// element is at most two panels, which leaves too little to the tensor cores, and the
+// DFMA form stays: 2D p = 2 (36 + 32), 1600 elements 0.78 ms DFMA, 0.95 ms digits; 3D p = 1
+// (40 + 40), 8000 elements 4.98 and 4.92 ms.  Counters at p = 3: FP64 pipe 43 % busy, issue
+// slots 32 %, tensor pipe 8 %, 42 MB of DRAM traffic per element: latency of the panel
+// steps and of the trailing block's loads, not a pipe, is what is left.
+constexpr int LT_NB = 32;                       // panel width
+constexpr int LT_S = 8;                         // digits per operand, and levels kept
+constexpr int LT_TC = 128, LT_TR = 16;          // columns and rows of one MMA group
+constexpr int LT_RB = 64;                       // rows of L21 staged at a time
+constexpr int LT_SLICE = LT_TC * LT_NB * 2;     // one digit of a column tile
+constexpr int LT_A_BYTES = LT_S * LT_SLICE;     // 64 KB
+constexpr int LT_GROUP = LT_S * LT_TR * LT_NB * 2;          // all digits of 16 rows
+constexpr int LT_B_BYTES = LT_RB / LT_TR * LT_GROUP;        // 32 KB
+constexpr int LT_LVL_COLS = LT_S * LT_TR;       // TMEM columns of one accumulator set
+constexpr int LT_TMEM_COLS = 2 * LT_LVL_COLS;   // two sets: epilogue of one, MMAs into the other
+constexpr int LT_BAD_EXP = 1 << 13;             // exponent of a row or column with a non-finite entry
 
-// Scratch of one CTA for the slices and scales of its current element.
-struct OzScratch {
-  float* ws;      // [S][nt][nu]      slices of W, K contiguous
-  float* zs;      // [S][nt + 1][nu]  slices of Z^T, K contiguous
-  double* rs;     // [nt]             2^e_i
-  double* cs;     // [nt + 1]         2^f_j
+__host__ __device__ inline int lt_stride(int nu) { return nu | 1; }   // odd: conflict-free columns
+
+__host__ inline size_t lt_smem(const Dims& dm) {
+  const size_t panel = sizeof(double) * (size_t)LT_NB * lt_stride(dm.nu), dig = LT_A_BYTES + LT_B_BYTES;
+  return (panel > dig ? panel : dig) + 128;      // operand tiles start on a 128-byte boundary
+}
+
+__device__ __forceinline__ int exponent_of(double x) { return (__double2hiint(x) >> 20) & 0x7ff; }
+// biased exponent of a row's (column's) largest entry as the epilogue adds it
+__device__ __forceinline__ int scale_of(int emax) { return emax == 0x7ff ? LT_BAD_EXP : emax; }
+
+// Digits of eight values with common exponent emax >= theirs: out(s, 8 packed BF16) for
+// s = 0 (most significant) .. 7.  Entries below 2^-62 of the scale and subnormals are 0.
+template <class Out>
+__device__ __forceinline__ void split8(const double (&x)[8], int emax, Out out) {
+  uint32_t lo[8], hi[8];
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    const long long b = __double_as_longlong(x[i]);
+    const int e = exponent_of(x[i]), sh = emax - e;
+    unsigned long long m = ((unsigned long long)b & 0xFFFFFFFFFFFFFull) | 0x10000000000000ull;
+    m = (e == 0 || sh > 62) ? 0ull : (m << 9) >> sh;
+    const unsigned long long v = (b < 0 ? 0ull - m : m) + 0x8080808080808080ull;   // digits + 128
+    lo[i] = (uint32_t)v;
+    hi[i] = (uint32_t)(v >> 32);
+  }
+#pragma unroll
+  for (int s = 0; s < LT_S; ++s) {
+    uint32_t w[4];
+#pragma unroll
+    for (int p = 0; p < 4; ++p) {
+      float f[2];
+#pragma unroll
+      for (int q = 0; q < 2; ++q) {
+        const uint32_t word = s < 4 ? hi[2 * p + q] : lo[2 * p + q];
+        // byte -> float 2^23 + byte, minus 2^23 + 128: at most 8 significant bits, so
+        // the upper half of the FP32 pattern is the BF16 value
+        f[q] = __uint_as_float(__byte_perm(word, 0x4B000000u, 0x7440u | (uint32_t)(3 - (s & 3)))) - 8388736.0f;
+      }
+      w[p] = __byte_perm(__float_as_uint(f[0]), __float_as_uint(f[1]), 0x7632);
+    }
+    out(s, make_uint4(w[0], w[1], w[2], w[3]));
+  }
+}
+
+// One thread: all digit products of one 16-row group into the accumulator set at d.
+__device__ __forceinline__ void lt_issue(uint32_t d, uint32_t a, uint32_t b, int ksteps) {
+  for (int ks = 0; ks < ksteps; ++ks)
+#pragma unroll
+    for (int s = 0; s < LT_S; ++s)
+      tc::mma_bf16(d + (uint32_t)(s * LT_TR), tc::desc_kmajor(a + s * LT_SLICE + ks * 256, 128, 512),
+                   tc::desc_kmajor(b + ks * 256, 128, 512), tc::idesc_bf16(LT_TC, LT_TR * (LT_S - s)),
+                   (ks == 0 && s == 0) ? 0u : 1u);
+}
+
+// minus the product sum whose level sums are t[0..7], scales ef = row + column exponent
+__device__ __forceinline__ double join_levels(const float (&t)[8], int ef) {
+  uint32_t p[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    // integer-valued |t| <= 2^22 -> bits 0x4B400000 + t; two neighbouring levels per word
+    const uint32_t a = __float_as_uint(t[2 * i] + 12582912.0f), b = __float_as_uint(t[2 * i + 1] + 12582912.0f);
+    p[i] = (a << 8) + b - 0x8B400000u;
+  }
+  long long v = (long long)(int)p[2] * 32 + (((int)p[3] + 1024) >> 11);
+  v += (long long)(int)p[1] * (1 << 21);
+  v += (long long)((unsigned long long)p[0] << 37);
+  if (v == 0) return 0.0;
+  const unsigned long long mag = v < 0 ? 0ull - (unsigned long long)v : (unsigned long long)v;
+  const int lz = __clzll((long long)mag);
+  const unsigned long long mn = mag << lz;
+  const int field = ef - 1015 - lz;
+  const unsigned long long sign = v > 0 ? 0x8000000000000000ull : 0ull;
+  if ((unsigned)(field - 1) < 2045u) {
+    const unsigned long long r = (mn >> 11) + ((mn >> 10) & 1ull) + ((unsigned long long)(unsigned)(field - 1) << 52);
+    return __longlong_as_double((long long)(r | sign));
+  }
+  if (ef >= LT_BAD_EXP) return __longlong_as_double(0x7FF8000000000000ll);
+  return __longlong_as_double((long long)(sign | (field <= 0 ? 0ull : 0x7FF0000000000000ull)));
+}
+
+// the eight levels of 8 rows (TMEM columns c .. c+7 of each level) of this thread's column
+__device__ __forceinline__ void load_levels(uint32_t taddr, float (&v)[8][8]) {
+  uint32_t r[8][8];
+#pragma unroll
+  for (int l = 0; l < 8; ++l)
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                 : "=r"(r[l][0]), "=r"(r[l][1]), "=r"(r[l][2]), "=r"(r[l][3]), "=r"(r[l][4]), "=r"(r[l][5]),
+                   "=r"(r[l][6]), "=r"(r[l][7])
+                 : "r"(taddr + (uint32_t)(l * LT_TR)));
+  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+  for (int l = 0; l < 8; ++l)
+#pragma unroll
+    for (int j = 0; j < 8; ++j) v[l][j] = __uint_as_float(r[l][j]);
+}
+
+// Tensor-core state of a CTA, the same in every thread: bit b of phase is the parity of
+// barrier b's next completion, bit b of pending says that a commit on it was not waited for.
+struct LtTc {
+  uint32_t tmem;
+  uint64_t* mbar;
+  uint32_t phase, pending;
+  int failed, limit;
 };
 
-__device__ __forceinline__ double pow2_at_least(double m) {
-  if (!(m > 0.0)) return 1.0;
-  int ex;
-  frexp(m, &ex);                  // m = f 2^ex, f in [0.5, 1): m < 2^ex
-  return ldexp(1.0, ex);
+// Order of |v| as a signed integer, -1 for NaN (never chosen), as in the DFMA form.
+__device__ __forceinline__ long long pivot_key(double v) {
+  const long long k = __double_as_longlong(v) & 0x7FFFFFFFFFFFFFFFLL;
+  return k > 0x7FF0000000000000LL ? -1LL : k;
 }
 
-__device__ void oz_split(const double* __restrict__ A, int ld, int n, int nu, const OzScratch& sc) {
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = LU_THREADS / 32;
-  const int nt = n - nu, nt1 = nt + 1;
-  // row scales of W (one warp per row) and column scales of Z (one thread per column)
-  for (int i = warp; i < nt; i += nw) {
-    const double* row = A + (int64_t)(nu + i) * ld;
-    double mx = 0.0;
-    for (int k = lane; k < nu; k += 32) mx = fmax(mx, fabs(row[k]));
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-    if (lane == 0) sc.rs[i] = pow2_at_least(mx);
-  }
-  for (int j = tid; j < nt1; j += LU_THREADS) {
-    double mx = 0.0;
-    for (int k = 0; k < nu; ++k) mx = fmax(mx, fabs(A[(int64_t)k * ld + nu + j]));
-    sc.cs[j] = pow2_at_least(mx);
-  }
-  __syncthreads();
-  const double up = ldexp(1.0, OZ_BETA);
-  for (int idx = tid; idx < nt * nu; idx += LU_THREADS) {
-    const int i = idx / nu, k = idx % nu;
-    double x = A[(int64_t)(nu + i) * ld + k] / sc.rs[i];          // exact: power of two
-#pragma unroll
-    for (int s = 0; s < OZ_S; ++s) {
-      const double t = x * up;
-      const double v = rint(t);
-      x = t - v;
-      sc.ws[((size_t)s * nt + i) * nu + k] = (float)v;
-    }
-  }
-  for (int idx = tid; idx < nt1 * nu; idx += LU_THREADS) {
-    const int k = idx / nt1, j = idx % nt1;
-    double x = A[(int64_t)k * ld + nu + j] / sc.cs[j];
-#pragma unroll
-    for (int s = 0; s < OZ_S; ++s) {
-      const double t = x * up;
-      const double v = rint(t);
-      x = t - v;
-      sc.zs[((size_t)s * nt1 + j) * nu + k] = (float)v;
-    }
-  }
-  __syncthreads();
-}
+struct LtShared {
+  int piv[LT_NB];
+  double inv[LT_NB];                 // reciprocal pivots of the panel
+  int perm[LU_MAX_NU];               // net row permutation of the panel's interchanges
+  long long rv[LU_THREADS / 32];
+  int ri[LU_THREADS / 32];
+  int sing;
+  int ce[2][LT_TC];                  // column exponents, two halves of the panel's rows
+  int re[LT_RB];                     // row exponents of the staged rows
+};
 
-// Stage K columns k0 .. k0+15 of every slice of the tile's W rows and Z columns.
-__device__ __forceinline__ void oz_stage(const OzScratch& sc, int nt, int nu, int rt, int ct, int k0, char* stage) {
-  const int tid = threadIdx.x, nt1 = nt + 1;
-  char* sa = stage;
-  char* sb = stage + OZ_S * OZ_A_BYTES;
-  for (int idx = tid; idx < OZ_S * OZ_TM * OZ_KS; idx += LU_THREADS) {
-    const int s = idx / (OZ_TM * OZ_KS), r = (idx / OZ_KS) % OZ_TM, k = idx % OZ_KS;
-    const int i = rt + r, kk = k0 + k;
-    const float v = (i < nt && kk < nu) ? sc.ws[((size_t)s * nt + i) * nu + kk] : 0.f;
-    const uint32_t off = (uint32_t)((r >> 3) * (OZ_KS / 4) * 128 + (k >> 2) * 128 + (r & 7) * 16 + (k & 3) * 4);
-    *reinterpret_cast<float*>(sa + s * OZ_A_BYTES + off) = v;
-  }
-  for (int idx = tid; idx < OZ_S * OZ_TN * OZ_KS; idx += LU_THREADS) {
-    const int s = idx / (OZ_TN * OZ_KS), r = (idx / OZ_KS) % OZ_TN, k = idx % OZ_KS;
-    const int j = ct + r, kk = k0 + k;
-    const float v = (j < nt1 && kk < nu) ? sc.zs[((size_t)s * nt1 + j) * nu + kk] : 0.f;
-    const uint32_t off = (uint32_t)((r >> 3) * (OZ_KS / 4) * 128 + (k >> 2) * 128 + (r & 7) * 16 + (k & 3) * 4);
-    *reinterpret_cast<float*>(sb + s * OZ_B_BYTES + off) = v;
-  }
-}
-
-// One thread: every slice pair of levels 2..S+1 for the staged K step; level l goes
-// to TMEM columns (l - 2) OZ_TN ..; `first` starts the chunk's accumulators.
-__device__ __forceinline__ void oz_issue(uint32_t tmem, const char* stage, bool first) {
-  const uint32_t a0 = tc::smem_u32(stage), b0 = a0 + OZ_S * OZ_A_BYTES;
-  constexpr uint32_t IDESC = tc::idesc_tf32(OZ_TM, OZ_TN);
-  constexpr uint32_t SBO = (OZ_KS / 4) * 128;
-  for (int s = 1; s <= OZ_S; ++s)
-    for (int t = 1; t <= OZ_S; ++t) {
-      const int l = s + t;
-      if (l > OZ_L + 1) continue;
-      const uint32_t d = tmem + (uint32_t)((l - 2) * OZ_TN);
-      // the first product of a level in the chunk is the one with s = 1
-#pragma unroll
-      for (int kst = 0; kst < OZ_KS / 8; ++kst) {
-        const uint32_t ko = kst * 256;
-        const bool acc = !(first && s == 1 && kst == 0);
-        tc::mma_tf32(d, tc::desc_kmajor(a0 + (s - 1) * OZ_A_BYTES + ko, 128, SBO),
-                     tc::desc_kmajor(b0 + (t - 1) * OZ_B_BYTES + ko, 128, SBO), IDESC, acc ? 1u : 0u);
+// Panel columns kb .. kb+nb-1 over the u-rows, P column-major (column j at P + j PR).
+// Two barriers per column: the pass that applies column j's multipliers also finds
+// column j+1's pivot candidates; one warp swaps the pivot rows, another forms the
+// reciprocal once (an FP64 division in every thread would load the FP64 pipe).
+__device__ __forceinline__ void lt_panel(LtShared& sh, double* P, int PR, int prow, int nb, int& nonfin) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  constexpr long long INF = 0x7FF0000000000000LL;
+  for (int j = 0; j < nb; ++j) {
+    long long best = -1;
+    int bi = j;
+    auto candidate = [&](double v, int r) {
+      const long long k = pivot_key(v);
+      nonfin |= k < 0 || k >= INF;
+      if (k > best) { best = k; bi = r; }
+    };
+    if (j == 0) {
+      for (int r = tid; r < prow; r += LU_THREADS) candidate(P[r], r);
+    } else {
+      const double inv = sh.inv[j - 1];
+      const double* piv_row = P + (j - 1);
+      for (int r = j + tid; r < prow; r += LU_THREADS) {
+        double* row = P + r;
+        const double l = row[(j - 1) * PR] * inv;
+        row[(j - 1) * PR] = l;
+        const double v = fma(-l, piv_row[j * PR], row[j * PR]);
+        row[j * PR] = v;
+        candidate(v, r);
+        for (int c = j + 1; c < nb; ++c) row[c * PR] = fma(-l, piv_row[c * PR], row[c * PR]);
       }
     }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      const long long ov = __shfl_xor_sync(0xffffffffu, best, o);
+      const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
+      if (ov > best || (ov == best && oi < bi)) { best = ov; bi = oi; }
+    }
+    if (lane == 0) { sh.rv[warp] = best; sh.ri[warp] = bi; }
+    __syncthreads();
+    if (warp < 2) {
+      long long bk = sh.rv[0];
+      int pr = sh.ri[0];
+      for (int w = 1; w < LU_THREADS / 32; ++w) {
+        const long long k = sh.rv[w];
+        if (k > bk || (k == bk && sh.ri[w] < pr)) { bk = k; pr = sh.ri[w]; }
+      }
+      if (bk <= 0) pr = j;                  // no nonzero candidate: singular
+      const double pv = P[pr + j * PR];
+      if (warp == 1) {
+        if (lane == 0) sh.inv[j] = pv != 0.0 ? 1.0 / pv : 0.0;
+      }
+      asm volatile("bar.sync 1, 64;" ::: "memory");   // pv read before the rows trade places
+      if (warp == 0) {
+        if (lane == 0) {
+          if (bk <= 0) sh.sing = 1;
+          sh.piv[j] = pr;
+          if (pr != j) { const int t = sh.perm[j]; sh.perm[j] = sh.perm[pr]; sh.perm[pr] = t; }
+        }
+        if (pr != j) {
+          const double t = P[j + lane * PR];
+          P[j + lane * PR] = P[pr + lane * PR];
+          P[pr + lane * PR] = t;
+        }
+      }
+    }
+    __syncthreads();
+  }
+  // the last column's multipliers
+  const double inv = sh.inv[nb - 1];
+  for (int r = nb + tid; r < prow; r += LU_THREADS) P[r + (nb - 1) * PR] *= inv;
+  __syncthreads();
 }
 
-__device__ void schur_ozaki(double* __restrict__ A, int ld, int n, int nu, const OzScratch& sc, char* smem,
-                            TcState* tcs) {
+// A22 -= L21 U12 over rows [r0, n), columns [c0, ncol).  Returns false when a completion
+// wait ran out.  `bad` collects non-finite results of the trace block (last panel).
+__device__ __forceinline__ bool lt_trailing(LtShared& sh, double* __restrict__ A, int ld, int kb, int nb, int r0, int n,
+                                            int nu, int c0, int ncol, unsigned char* dig, LtTc* tcs, int& bad) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int nt = n - nu, ncol = n + 1;
   const int q = warp & 3, h = warp >> 2;
-  oz_split(A, ld, n, nu, sc);
-  for (int rt = 0; rt < nt && !tcs->failed; rt += OZ_TM) {
-    for (int ct = 0; ct < ncol - nu && !tcs->failed; ct += OZ_TN) {
-      for (int kc = 0; kc < nu && !tcs->failed; kc += OZ_KC) {
-        for (int k0 = kc; k0 < min(kc + OZ_KC, nu); k0 += OZ_KS) {
-          oz_stage(sc, nt, nu, rt, ct, k0, smem);
-          tc::fence_proxy_async();
-          __syncthreads();
-          tc::fence_after_sync();
-          if (tid == 0) {
-            oz_issue(tcs->tmem, smem, k0 == kc);
-            tc::mma_commit(tcs->mbar);
-          }
-          tcs->pending[0] = 1;
-          const bool ok = __syncthreads_and(tc::mbar_wait(tcs->mbar, tcs->phase[0], tcs->limit));
-          if (!ok) { tcs->failed = 1; break; }
-          tcs->phase[0] ^= 1u;
-          tcs->pending[0] = 0;
-          tc::fence_after_sync();
+  unsigned char *da = dig, *db = dig + LT_A_BYTES;
+  const uint32_t ua = tc::smem_u32(da), ub = tc::smem_u32(db);
+  const int ksteps = nb > 16 ? 2 : 1;
+  for (int ct = c0; ct < ncol; ct += LT_TC) {
+    {
+      // U12 columns ct .. ct+127: thread = column (and half of the panel's rows)
+      const int c = tid & (LT_TC - 1), kh = tid >> 7, col = ct + c;
+      double x[2][8];
+      int em = 0;
+#pragma unroll
+      for (int u = 0; u < 2; ++u)
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          const int k = 16 * kh + 8 * u + i;
+          x[u][i] = (k < nb && col < ncol) ? A[(int64_t)(kb + k) * ld + col] : 0.0;
+          em = max(em, exponent_of(x[u][i]));
         }
-        if (tcs->failed) break;
-        // epilogue: warp (q, h) owns rows 32 q .. 32 q + 31 and columns 16 h .. 16 h + 15
-        const int i = rt + 32 * q + lane;
-        const double rsc = i < nt ? sc.rs[i] : 0.0;
-#pragma unroll 1
-        for (int c8 = 0; c8 < 2; ++c8) {
-          const int c0 = 16 * h + 8 * c8;
-          double sum[8];
+      sh.ce[kh][c] = em;
+      __syncthreads();
+      em = max(em, sh.ce[kh ^ 1][c]);
 #pragma unroll
-          for (int j = 0; j < 8; ++j) sum[j] = 0.0;
-#pragma unroll 1
-          for (int l = 0; l < OZ_L; ++l) {
-            float v8[8];
-            tc::tmem_ld8(tcs->tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(l * OZ_TN + c0), v8);
-            const double w = ldexp(1.0, -(l + 2) * OZ_BETA);
+      for (int u = 0; u < 2; ++u)
+        split8(x[u], em, [&](int s, uint4 v) {
+          *reinterpret_cast<uint4*>(da + s * LT_SLICE + tc::core_off16(c, 16 * kh + 8 * u)) = v;
+        });
+    }
+    const int c = 32 * q + lane, col = ct + c;
+    int ecol = 0;                                    // set after the first barrier below
+    for (int rb = r0; rb < n; rb += LT_RB) {
+      {
+        // L21 rows rb .. rb+63: lane = row and eight of the panel's columns
+        const int rr = 8 * warp + (lane & 7), k8 = lane >> 3, row = rb + rr;
+        double x[8];
+        int em = 0;
 #pragma unroll
-            for (int j = 0; j < 8; ++j) sum[j] = fma((double)v8[j], w, sum[j]);
+        for (int i = 0; i < 8; i += 2) {
+          const int k = 8 * k8 + i;
+          double2 t = make_double2(0.0, 0.0);
+          if (row < n && k + 1 < nb) t = *reinterpret_cast<const double2*>(A + (int64_t)row * ld + kb + k);
+          else if (row < n && k < nb) t.x = A[(int64_t)row * ld + kb + k];
+          x[i] = t.x;
+          x[i + 1] = t.y;
+          em = max(em, max(exponent_of(t.x), exponent_of(t.y)));
+        }
+        em = max(em, __shfl_xor_sync(0xffffffffu, em, 8));
+        em = max(em, __shfl_xor_sync(0xffffffffu, em, 16));
+        if (k8 == 0) sh.re[rr] = scale_of(em);
+        split8(x, em, [&](int s, uint4 v) {
+          *reinterpret_cast<uint4*>(db + (rr >> 4) * LT_GROUP + s * (LT_TR * LT_NB * 2) +
+                                    tc::core_off16(rr & 15, 8 * k8)) = v;
+        });
+      }
+      tc::fence_proxy_async();
+      __syncthreads();
+      tc::fence_after_sync();
+      if (rb == r0) ecol = scale_of(max(sh.ce[0][c], sh.ce[1][c]));
+      const int ng = (min(LT_RB, n - rb) + LT_TR - 1) / LT_TR;
+      if (tid == 0) {
+        lt_issue(tcs->tmem, ua, ub, ksteps);
+        tc::mma_commit(tcs->mbar);
+      }
+      tcs->pending |= 1u;
+      for (int g = 0; g < ng; ++g) {
+        const int b = g & 1;
+        if (g + 1 < ng) {        // the other accumulator set was read before the last barrier
+          if (tid == 0) {
+            lt_issue(tcs->tmem + (uint32_t)((b ^ 1) * LT_LVL_COLS), ua, ub + (g + 1) * LT_GROUP, ksteps);
+            tc::mma_commit(tcs->mbar + (b ^ 1));
           }
-          if (i >= nt) continue;
-          double* dst = A + (int64_t)(nu + i) * ld + nu + ct + c0;
+          tcs->pending |= 1u << (b ^ 1);
+        }
+        // this thread's column, rows 8h .. 8h+7 of the group
+        const int row0 = rb + LT_TR * g + 8 * h;
+        double* dst = A + (int64_t)row0 * ld + col;
+        double a[8];
 #pragma unroll
-          for (int j = 0; j < 8; ++j) {
-            const int jj = ct + c0 + j;
-            if (jj < ncol - nu) dst[j] -= (rsc * sc.cs[jj]) * sum[j];
+        for (int i = 0; i < 8; ++i) a[i] = (col < ncol && row0 + i < n) ? dst[(int64_t)i * ld] : 0.0;
+        const bool ok = tc::mbar_wait(tcs->mbar + b, (tcs->phase >> b) & 1u, tcs->limit);
+        if (ok) {
+          tc::fence_after_sync();
+          float t[8][8];
+          load_levels(tcs->tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(b * LT_LVL_COLS + 8 * h), t);
+#pragma unroll
+          for (int i = 0; i < 8; ++i) {
+            const float lv[8] = {t[0][i], t[1][i], t[2][i], t[3][i], t[4][i], t[5][i], t[6][i], t[7][i]};
+            a[i] += join_levels(lv, ecol + sh.re[LT_TR * g + 8 * h + i]);
+            if (col < ncol && row0 + i < n) {
+              dst[(int64_t)i * ld] = a[i];
+              bad |= row0 + i >= nu && col >= nu && exponent_of(a[i]) == 0x7ff;
+            }
           }
         }
         tc::fence_before_sync();
-        __syncthreads();
+        if (__syncthreads_or(!ok)) { tcs->failed = 1; return false; }
+        tc::fence_after_sync();
+        tcs->phase ^= 1u << b;
+        tcs->pending &= ~(1u << b);
       }
     }
   }
+  return true;
+}
+
+__device__ __forceinline__ bool lt_element(LtShared& sh, const LuElem& el, double* __restrict__ S,
+                                           int8_t* __restrict__ status, int64_t e, unsigned char* smem, LtTc* tcs) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int n = el.n, nu = el.nu, ld = el.ld, ncol = n + 1;
+  double* A = S + el.off;
+  double* P = reinterpret_cast<double*>(smem);
+  const int PR = lt_stride(nu);
+  int nonfin = 0, bad = 0;
+  if (tid == 0) sh.sing = 0;
+  for (int kb = 0; kb < nu; kb += LT_NB) {
+    const int nb = min(LT_NB, nu - kb), prow = nu - kb;
+    for (int r = warp; r < prow; r += LU_THREADS / 32)
+      P[r + lane * PR] = lane < nb ? A[(int64_t)(kb + r) * ld + kb + lane] : 0.0;
+    for (int r = tid; r < prow; r += LU_THREADS) sh.perm[r] = r;
+    __syncthreads();
+    lt_panel(sh, P, PR, prow, nb, nonfin);
+    // [L11 \ U11], L21 of the u-rows back
+    for (int r = warp; r < prow; r += LU_THREADS / 32)
+      if (lane < nb) A[(int64_t)(kb + r) * ld + kb + lane] = P[r + lane * PR];
+    // L21 of the trace rows, x U11 = a: one thread per row, no pivots among them
+    for (int r = nu + tid; r < n; r += LU_THREADS) {
+      double* row = A + (int64_t)r * ld + kb;
+      double x[LT_NB];
+      // rows start on 32-byte boundaries (ld and kb are multiples of 4)
+#pragma unroll
+      for (int j = 0; j < LT_NB; j += 2) {
+        double2 t = make_double2(0.0, 0.0);
+        if (j + 1 < nb) t = *reinterpret_cast<const double2*>(row + j);
+        else if (j < nb) t.x = row[j];
+        x[j] = t.x;
+        x[j + 1] = t.y;
+      }
+#pragma unroll
+      for (int j = 0; j < LT_NB; ++j) {
+        if (j >= nb) break;
+        x[j] *= sh.inv[j];
+#pragma unroll
+        for (int c = j + 1; c < LT_NB; ++c) x[c] = fma(-x[j], P[j + c * PR], x[c]);
+      }
+#pragma unroll
+      for (int j = 0; j < LT_NB; j += 2) {
+        if (j + 1 < nb) *reinterpret_cast<double2*>(row + j) = make_double2(x[j], x[j + 1]);
+        else if (j < nb) row[j] = x[j];
+      }
+    }
+    // trailing columns: row interchanges (each column gathers its new top rows, then
+    // moves the displaced rows), then U12 = L11^-1 A12
+    for (int c = kb + nb + tid; c < ncol; c += LU_THREADS) {
+      double x[LT_NB];
+#pragma unroll
+      for (int j = 0; j < LT_NB; ++j) x[j] = j < nb ? A[(int64_t)(kb + sh.perm[j]) * ld + c] : 0.0;
+#pragma unroll
+      for (int j0 = 0; j0 < LT_NB; j0 += 8) {
+        double y[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+          const int r = j0 + j < nb ? sh.piv[j0 + j] : 0;
+          y[j] = (j0 + j < nb && r >= nb && sh.perm[r] != r) ? A[(int64_t)(kb + sh.perm[r]) * ld + c] : 0.0;
+        }
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+          const int r = j0 + j < nb ? sh.piv[j0 + j] : 0;
+          if (j0 + j < nb && r >= nb && sh.perm[r] != r) A[(int64_t)(kb + r) * ld + c] = y[j];
+        }
+      }
+#pragma unroll
+      for (int j = 0; j < LT_NB; ++j) {
+        if (j >= nb) break;
+#pragma unroll
+        for (int i = j + 1; i < LT_NB; ++i) x[i] = fma(-P[i + j * PR], x[j], x[i]);
+        A[(int64_t)(kb + j) * ld + c] = x[j];
+      }
+    }
+    __syncthreads();
+    if (!lt_trailing(sh, A, ld, kb, nb, kb + nb, n, nu, kb + nb, ncol, smem, tcs, bad)) break;
+    if (kb + nb < nu) bad = 0;                 // only the last panel's trace block is the Schur complement
+    __syncthreads();
+  }
+  nonfin = __syncthreads_or(nonfin);
+  bad = __syncthreads_or(bad);
+  if (tid == 0)
+    status[e] = tcs->failed ? IEDG_ELEM_TIMEOUT
+                            : (nonfin ? IEDG_ELEM_NONFINITE
+                                      : (sh.sing ? IEDG_ELEM_SINGULAR : (bad ? IEDG_ELEM_NONFINITE : IEDG_ELEM_OK)));
+  return !tcs->failed;
+}
+
+// TMEM and the completion barriers are set up once per CTA; a CTA whose wait ran out
+// factors nothing more, flags the elements it still takes from the queue, waits once
+// more (bounded) for its MMAs in flight and frees its TMEM.
+__global__ void __launch_bounds__(LU_THREADS, 2)
+k_lu64_tc(Dims dm, LuDesc lud, double* __restrict__ S, int8_t* __restrict__ status, int64_t* queue, int64_t E,
+          int* err, int wait_limit) {
+  extern __shared__ __align__(16) unsigned char smraw[];
+  unsigned char* smem = smraw + ((128u - (tc::smem_u32(smraw) & 127u)) & 127u);
+  __shared__ LtShared sh;
+  __shared__ uint32_t tmem_base;
+  __shared__ __align__(8) uint64_t mbar[2];
+  const int tid = threadIdx.x, warp = tid >> 5;
+  if (warp == 0) {
+    tc::tmem_alloc(&tmem_base, LT_TMEM_COLS);
+    tc::tmem_relinquish();
+  }
+  if (tid == 0) {
+    tc::mbar_init(&mbar[0], 1);
+    tc::mbar_init(&mbar[1], 1);
+  }
+  tc::fence_before_sync();
+  __syncthreads();
+  tc::fence_after_sync();
+  LtTc mine;
+  mine.tmem = tmem_base;
+  mine.mbar = mbar;
+  mine.phase = mine.pending = 0;
+  mine.failed = 0;
+  mine.limit = wait_limit;
+  int64_t e, it = 0;
+  for (; next_element(queue, E, it, lud.order, &e); ++it) {
+    if (!lt_element(sh, lu_elem(dm, lud, e), S, status, e, smem, &mine)) {
+      if (tid == 0) atomicOr(err, 1);
+      for (int b = 0; b < 2; ++b)      // MMAs still in flight finish before the TMEM is freed
+        if ((mine.pending >> b) & 1u) tc::mbar_wait(mbar + b, (mine.phase >> b) & 1u, kTcWaitLimit);
+      ++it;
+      break;
+    }
+  }
+  if (mine.failed)
+    for (; next_element(queue, E, it, lud.order, &e); ++it)
+      if (tid == 0) status[e] = IEDG_ELEM_TIMEOUT;
+  tc::fence_before_sync();
+  __syncthreads();
+  tc::fence_after_sync();
+  if (warp == 0) tc::tmem_dealloc(tmem_base, LT_TMEM_COLS);
 }
 
 // FP32 partial LU for the mixed path.  Same algorithm and pivot rule as k_lu, with
@@ -1151,79 +1451,6 @@ k_lu32_tc(Dims dm, LuDesc lud, float* __restrict__ S, int8_t* __restrict__ statu
   if (warp == 0) tc::tmem_dealloc(tmem_base, TC_TN);
 }
 
-// FP64 partial LU with the Schur complement on the tensor cores (schur_ozaki).  The CTA
-// holds 256 TMEM columns (two resident CTAs fit an SM's 512) and one completion barrier.
-__global__ void __launch_bounds__(LU_THREADS)
-k_lu64_oz(Dims dm, LuDesc lud, double* __restrict__ S, int8_t* __restrict__ status, int64_t* queue, int64_t E,
-          float* __restrict__ scratch, int64_t scratch_floats, int* err, int wait_limit) {
-  extern __shared__ __align__(16) unsigned char smraw[];
-  __shared__ uint32_t tmem_base;
-  __shared__ __align__(8) uint64_t mbar[2];
-  __shared__ TcState tcs;
-  const int tid = threadIdx.x, warp = tid >> 5;
-  if (warp == 0) {
-    tc::tmem_alloc(&tmem_base, OZ_TMEM_COLS);
-    tc::tmem_relinquish();
-  }
-  if (tid == 0) tc::mbar_init(&mbar[0], 1);
-  tc::fence_before_sync();
-  __syncthreads();
-  tc::fence_after_sync();
-  if (tid == 0) {
-    tcs.tmem = tmem_base;
-    tcs.mbar = mbar;
-    tcs.phase[0] = 0;
-    tcs.phase[1] = 0;
-    tcs.failed = 0;
-    tcs.limit = wait_limit;
-    tcs.pending[0] = 0;
-    tcs.pending[1] = 0;
-  }
-  __syncthreads();
-  TcState mine = tcs;
-  // this CTA's slices and scales
-  float* base = scratch + (size_t)blockIdx.x * scratch_floats;
-  OzScratch sc;
-  {
-    const size_t ntm = dm.nt + 1, num = dm.nu;
-    sc.ws = base;
-    sc.zs = sc.ws + (size_t)OZ_S * ntm * num;
-    double* dd = reinterpret_cast<double*>(sc.zs + (size_t)OZ_S * ntm * num);
-    sc.rs = dd;
-    sc.cs = dd + ntm;
-  }
-  int64_t e;
-  int64_t it = 0;
-  for (; next_element(queue, E, it, lud.order, &e); ++it) {
-    const LuElem el = lu_elem(dm, lud, e);
-    lu_element<double, 16>(el, S, status, nullptr, e, true);
-    schur_ozaki(S + el.off, el.ld, el.n, el.nu, sc, reinterpret_cast<char*>(smraw), &mine);
-    // non-finite Schur complement
-    double* A = S + el.off;
-    const int n = el.n, nu = el.nu, ncol = n + 1;
-    int bad = 0;
-    for (int idx = tid; idx < (n - nu) * (ncol - nu); idx += LU_THREADS) {
-      int r = nu + idx / (ncol - nu), c = nu + idx % (ncol - nu);
-      if (!isfinite(A[(int64_t)r * el.ld + c])) bad = 1;
-    }
-    bad = __syncthreads_or(bad);
-    if (tid == 0 && bad && status[e] == IEDG_ELEM_OK) status[e] = IEDG_ELEM_NONFINITE;
-    if (__syncthreads_or(mine.failed)) {
-      if (tid == 0) { atomicOr(err, 1); status[e] = IEDG_ELEM_TIMEOUT; }
-      tc_drain(mine);     // MMAs still in flight finish before the TMEM is freed
-      ++it;
-      break;
-    }
-  }
-  if (mine.failed)
-    for (; next_element(queue, E, it, lud.order, &e); ++it)
-      if (tid == 0) status[e] = IEDG_ELEM_TIMEOUT;
-  tc::fence_before_sync();
-  __syncthreads();
-  tc::fence_after_sync();
-  if (warp == 0) tc::tmem_dealloc(tmem_base, OZ_TMEM_COLS);
-}
-
 }  // namespace
 
 size_t lu64_smem(const Dims& dm, int nb);
@@ -1313,54 +1540,6 @@ static cudaError_t lu_t(iedg_mesh* M, T* S, int* piv, cudaStream_t st) {
 
 size_t lu64_smem(const Dims& dm, int nb) { return sizeof(double) * ((size_t)dm.n * nb + (size_t)nb * UCW); }
 
-// FP64 form with the Schur complement on the tensor cores (persistent grid only: each
-// CTA owns a slice buffer for the element it works on).  The buffers are allocated
-// when the schedule selects this form (iedg_set_schedule), never by a compute call.
-static cudaError_t lu64_oz_grid(iedg_mesh* M, size_t* smem_out, unsigned* grid, int64_t* per_cta) {
-  const Dims& dm = M->dm;
-  size_t smem = lu64_smem(dm, 16);
-  if (smem < (size_t)OZ_STAGE_BYTES) smem = OZ_STAGE_BYTES;
-  cudaError_t err = cudaFuncSetAttribute(k_lu64_oz, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (err != cudaSuccess) return err;
-  // two resident CTAs at most: each holds 256 of the SM's 512 TMEM columns
-  err = persistent_grid(k_lu64_oz, smem, M->E, grid, 2);
-  if (err != cudaSuccess) return err;
-  const int64_t ntm = dm.nt + 1;
-  *per_cta = ((2 * (int64_t)OZ_S * ntm * dm.nu + 4 * ntm) + 3) & ~(int64_t)3;
-  *smem_out = smem;
-  return cudaSuccess;
-}
-
-cudaError_t prepare_lu64_oz(iedg_mesh* M) {
-  size_t smem = 0;
-  unsigned grid = 0;
-  int64_t per = 0;
-  cudaError_t err = lu64_oz_grid(M, &smem, &grid, &per);
-  if (err != cudaSuccess) return err;
-  if (M->oz_scratch != nullptr && M->oz_grid >= grid) return cudaSuccess;
-  if (M->oz_scratch) cudaFree(M->oz_scratch);
-  M->oz_scratch = nullptr;
-  err = cudaMalloc(&M->oz_scratch, (size_t)grid * per * sizeof(float));
-  if (err != cudaSuccess) return err;
-  M->oz_grid = grid;
-  return cudaSuccess;
-}
-
-static cudaError_t lu64_oz(iedg_mesh* M, cudaStream_t st) {
-  const Dims& dm = M->dm;
-  size_t smem = 0;
-  unsigned grid = 0;
-  int64_t per = 0;
-  cudaError_t err = lu64_oz_grid(M, &smem, &grid, &per);
-  if (err != cudaSuccess) return err;
-  if (M->oz_scratch == nullptr || M->oz_grid < grid) return cudaErrorNotReady;   // set_schedule allocates
-  err = cudaMemsetAsync(M->queue, 0, sizeof(int64_t), st);
-  if (err != cudaSuccess) return err;
-  k_lu64_oz<<<grid, LU_THREADS, smem, st>>>(dm, M->lud, M->S, M->status, M->queue, M->E, M->oz_scratch, per,
-                                             M->dev_flag, tc_wait_limit(M));
-  return cudaGetLastError();
-}
-
 // FP32 partial LU with the Schur complement on the tensor cores in operand form KIND.
 template <int KIND>
 static cudaError_t lu32_tc(iedg_mesh* M, cudaStream_t st) {
@@ -1384,9 +1563,27 @@ static cudaError_t lu32_tc(iedg_mesh* M, cudaStream_t st) {
   return cudaGetLastError();
 }
 
+static cudaError_t launch_lu64_tc(iedg_mesh* M, cudaStream_t st) {
+  const size_t smem = lt_smem(M->dm);
+  cudaError_t err = cudaFuncSetAttribute(k_lu64_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (err != cudaSuccess) return err;
+  unsigned grid = (unsigned)M->E;
+  int64_t* queue = nullptr;
+  if (M->sched.lu_persistent) {
+    // two resident CTAs at most: each holds half of the SM's TMEM
+    err = persistent_grid(k_lu64_tc, smem, M->E, &grid, 2);
+    if (err == cudaSuccess) err = cudaMemsetAsync(M->queue, 0, sizeof(int64_t), st);
+    if (err != cudaSuccess) return err;
+    queue = M->queue;
+  }
+  k_lu64_tc<<<grid, LU_THREADS, smem, st>>>(M->dm, M->lud, M->S, M->status, queue, M->E, M->dev_flag,
+                                            tc_wait_limit(M));
+  return cudaGetLastError();
+}
+
 cudaError_t launch_lu(iedg_mesh* M, cudaStream_t st) {
   if (M->dm.nu > LU_MAX_NU) return cudaErrorInvalidValue;   // orders above 4 are rejected at creation
-  if (M->precision == 0 && M->sched.lu_tensor) return lu64_oz(M, st);
+  if (M->precision == 0 && (M->sched.lu_tensor || M->dm.nu >= LU64_TC_MIN_NU)) return launch_lu64_tc(M, st);
   if (M->precision == 0) {
     if (M->sched.lu_panel == 32 && lu64_smem(M->dm, 32) <= 227 * 1024) return lu_t<double, 32>(M, M->S, nullptr, st);
     return lu_t<double, 16>(M, M->S, nullptr, st);

@@ -37,8 +37,9 @@ struct Schedule {
   int lu_persistent = 1;     // batched LU as a persistent grid with an element queue
   int lu_panel = 16;         // FP64 LU panel width (16 or 32; 32 only when it fits shared memory)
   int asm_chunk = 0;         // assembly column chunk (0 = default: 8 for FP64, 16 for FP32)
-  int lu_tensor = 1;         // 0 = DFMA / FFMA updates; 1 = deferred Schur complement on tcgen05;
-                             // 2 (mixed FP32 form) = every trailing update on tcgen05 (3xTF32)
+  int lu_tensor = 0;         // FP64: 1 = digit form on tcgen05 always, 0 = by size.  Mixed: 0 = FFMA
+                             // updates; 1 = deferred Schur complement on tcgen05; 2 (FP32 form) =
+                             // every trailing update on tcgen05 (3xTF32)
   int asm_chunk_by_order[4] = {0, 0, 0, 0};   // mixed orders: chunk per order (0 = asm_chunk)
 };
 
@@ -190,8 +191,6 @@ struct iedg_mesh {
   int8_t* fb_status = nullptr;  // [slots] status of the FP64 partial LU
   int* fb_count = nullptr;      // slots in use
   int64_t* queue = nullptr;     // element counter of persistent launches
-  float* oz_scratch = nullptr;  // FP64 tensor-core Schur form: per-CTA slice buffers (freed with the handle)
-  unsigned oz_grid = 0;
   // meshes with mixed orders: the parent handle holds the trace space, the ragged
   // element matrices and the per-element sizes; one child handle per order holds the
   // element tables of that order (internal element ids are grouped by order)
@@ -256,7 +255,8 @@ bool assemble_sf_supported(const Dims& dm);
 AsmTab<double> tables64(const iedg_mesh* M);
 AsmTab<float> tables32(const iedg_mesh* M);
 cudaError_t launch_lu(iedg_mesh* M, cudaStream_t st);
-cudaError_t prepare_lu64_oz(iedg_mesh* M);   // slice buffers of the FP64 tensor-core Schur form
+// u-unknowns from which the FP64 LU takes its digit form (iedg_assemble.cu)
+constexpr int LU64_TC_MIN_NU = 64;
 cudaError_t launch_lu32_mma(iedg_mesh* M, int n_max, cudaStream_t st);   // FP32 LU, tcgen05 trailing updates
 cudaError_t launch_scatter_K(iedg_mesh* M, double* K, cudaStream_t st);
 cudaError_t launch_scatter_R_ragged(iedg_mesh* M, const RaggedSrc& src, const double* base, double* R,

@@ -12,7 +12,7 @@ constexpr int LU_THREADS = 256;
 constexpr int UCW = 64;     // trailing-update column chunk
 constexpr int LU_MAX_NU = 640;   // u-unknowns of the largest element (5 x 125 at p = 4)
 
-// Tensor-core state of a CTA (deferred Schur complement forms of the LU).
+// Tensor-core state of a CTA (FP32 forms of the LU).
 struct TcState {
   uint32_t tmem;        // TMEM base
   uint64_t* mbar;       // MMA completion barriers (one per operand stage)
