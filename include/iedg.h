@@ -231,9 +231,10 @@ int64_t iedg_element_status(iedg_mesh* mesh, int8_t* out, void* stream);
  *   rtol > 0: stop when |M^-1 (R - K dU)| <= rtol |M^-1 R| (the GMRES estimate
  *   during a cycle, recomputed at restarts).
  * Outputs iterations and the final relative preconditioned residual (may be NULL).
- * The Hessenberg matrix, its Givens rotations and the residual estimate are kept and
- * updated on the device; the host reads the estimate once per Arnoldi step (one
- * synchronisation of `stream` per step) to decide when to stop.  Workspace is
+ * The whole iteration runs on the device as one cooperative launch of at most one CTA
+ * per SM, stopping test included; the call synchronises `stream` once, to return the
+ * outcome.  A grid barrier that is not met within its bound ends the launch
+ * (IEDG_ERR_CUDA).  Workspace is
  * allocated with the mesh.  IEDG_ERR_INVALID_ARG for a singular diagonal block. */
 #define IEDG_MAX_RESTART 40
 

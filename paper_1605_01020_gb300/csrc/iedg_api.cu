@@ -445,12 +445,9 @@ static int alloc_owner(iedg_mesh* M, int64_t S_elems, int64_t piv_elems, int64_t
   }
   if (!M->dev_flag) CUDA_TRY(dalloc(M, &M->dev_flag, 1));
   CUDA_TRY(dalloc(M, &M->queue, 1));
-  CUDA_TRY(dalloc(M, &M->kry, (size_t)(IEDG_MAX_RESTART + 3) * T * m));
+  CUDA_TRY(dalloc(M, &M->kry, (size_t)(IEDG_MAX_RESTART + 2) * T * m));
   CUDA_TRY(dalloc(M, &M->dinv, (size_t)T * m * m));
-  CUDA_TRY(dalloc(M, &M->kpart, (size_t)(IEDG_MAX_RESTART + 1) * 512));
-  CUDA_TRY(dalloc(M, &M->khdev, (size_t)(IEDG_MAX_RESTART + 1)));
-  CUDA_TRY(dalloc(M, &M->kst, (size_t)(2 * (IEDG_MAX_RESTART + 1) + (IEDG_MAX_RESTART + 1) * IEDG_MAX_RESTART +
-                                       4 * IEDG_MAX_RESTART + 1 + 8)));
+  CUDA_TRY(dalloc(M, &M->kpart, (size_t)kGmresScratch));
   CUDA_TRY(cudaMemsetAsync(M->dev_flag, 0, sizeof(int), st));
   CUDA_TRY(cudaMemsetAsync(M->status, 0, E, st));
   return IEDG_OK;

@@ -213,14 +213,13 @@ struct iedg_mesh {
   double* bf = nullptr;         // BILU(0) factors [nnzb][m][m]
   int64_t* brows = nullptr;     // [T] trace nodes sorted by (colour, index)
   std::vector<int64_t> bcptr;   // colour boundaries in brows
-  double* kst = nullptr;        // trace solve: GMRES state on the device (Hessenberg, rotations, scalars)
+  int64_t* bcptr_dev = nullptr; // bcptr on the device
   int32_t* bord = nullptr;      // [nnzb] per row: entry offsets in elimination order
   int32_t* bnlow = nullptr;     // [T] entries of each row ranked before the row
   std::vector<int32_t> bcolor;  // host: colour of every trace node
-  double* kry = nullptr;        // trace solve: Krylov basis [IEDG_MAX_RESTART+1][T m] + 2 work vectors
+  double* kry = nullptr;        // trace solve: Krylov basis [IEDG_MAX_RESTART+1][T m] + 1 work vector
   double* dinv = nullptr;       // trace solve: inverted diagonal blocks [T][m][m]
-  double* kpart = nullptr;      // trace solve: dot-product partial sums
-  double* khdev = nullptr;      // trace solve: small vector of coefficients
+  double* kpart = nullptr;      // trace solve: partial sums of the dot products, result scalars, barrier
   iedg::Schedule sched;
   iedg::Fault fault;
   int* dev_flag = nullptr;      // geometry error flag
@@ -271,6 +270,9 @@ cudaError_t launch_backsub(iedg_mesh* M, const double* duhat, double* du, double
                            cudaStream_t st);
 cudaError_t launch_solve_prep(iedg_mesh* M, cudaStream_t st);
 cudaError_t launch_refine(iedg_mesh* M, cudaStream_t st);
+// doubles of iedg_mesh::kpart
+constexpr int64_t kGmresMaxCtas = 512;
+constexpr int64_t kGmresScratch = (IEDG_MAX_RESTART + 1) * kGmresMaxCtas + 8;
 // FP64 fallback of flagged elements on the mixed path (iedg_fallback.cu)
 constexpr int kFallbackSlots = 32;
 cudaError_t launch_fallback(iedg_mesh* M, cudaStream_t st);

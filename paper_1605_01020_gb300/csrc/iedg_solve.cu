@@ -2,9 +2,8 @@
 // Gram-Schmidt (two CGS passes per Arnoldi step) and left preconditioning
 // M^-1 K dU = M^-1 R, as in the paper's parallel solver (Sec. 2.2.2).  On one GPU
 // there is one subdomain; the preconditioner here is block Jacobi with the m x m
-// diagonal blocks of K (the paper notes that zero overlap gives block Jacobi).
-// The Hessenberg least-squares problem (Givens rotations) lives on the host; one
-// small device-to-host copy per Arnoldi step.
+// diagonal blocks of K (the paper notes that zero overlap gives block Jacobi), or
+// BILU(0) in multicolour order.  The whole iteration is one cooperative launch (k_gmres).
 #include <algorithm>
 #include <cmath>
 #include <cstring>
@@ -18,7 +17,6 @@ using namespace iedg;
 namespace {
 
 constexpr int SV_THREADS = 256;
-constexpr int SV_PART = 512;        // CTAs of the dot-product kernels
 
 // Dinv[t] = inverse of the diagonal block K[t][t] (Gauss-Jordan, partial pivoting).
 __global__ void k_diag_inv(int m, int64_t T, const int64_t* __restrict__ row_ptr, const int32_t* __restrict__ col,
@@ -53,111 +51,6 @@ __global__ void k_diag_inv(int m, int64_t T, const int64_t* __restrict__ row_ptr
   if (!ok) atomicOr(flag, 1);
   for (int i = 0; i < m; ++i)
     for (int j = 0; j < m; ++j) Dinv[(t * m + i) * m + j] = ok ? a[i][m + j] : (i == j);
-}
-
-// y = M^-1 (K x) (prec = true) or y = K x; one warp per block row.
-__global__ void k_spmv(int m, int64_t T, const int64_t* __restrict__ row_ptr, const int32_t* __restrict__ col,
-                       const double* __restrict__ K, const double* __restrict__ Dinv, const double* __restrict__ x,
-                       double* __restrict__ y, bool prec) {
-  const int lane = threadIdx.x & 31;
-  const int64_t t = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  if (t >= T) return;
-  double acc[5] = {0, 0, 0, 0, 0};
-  for (int64_t b = row_ptr[t] + lane; b < row_ptr[t + 1]; b += 32) {
-    const double* blk = K + b * m * m;
-    const double* xc = x + (int64_t)col[b] * m;
-    for (int i = 0; i < m; ++i) {
-      double s = 0.0;
-      for (int k = 0; k < m; ++k) s = fma(blk[i * m + k], xc[k], s);
-      acc[i] += s;
-    }
-  }
-  for (int i = 0; i < m; ++i)
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) acc[i] += __shfl_xor_sync(0xffffffffu, acc[i], o);
-  if (lane < m) {
-    double v;
-    if (prec) {
-      v = 0.0;
-      for (int k = 0; k < m; ++k) v = fma(Dinv[(t * m + lane) * m + k], acc[k], v);
-    } else {
-      v = acc[lane];
-    }
-    y[t * m + lane] = v;
-  }
-}
-
-// partial[v * SV_PART + blk] = sum over the block's slice of V[v] . w, v < nv
-__global__ void k_dots(int64_t n, int nv, const double* __restrict__ V, const double* __restrict__ w,
-                       double* __restrict__ partial) {
-  __shared__ double red[SV_THREADS / 32];
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  for (int v = 0; v < nv; ++v) {
-    const double* a = V + (int64_t)v * n;
-    double s = 0.0;
-    for (int64_t i = (int64_t)blockIdx.x * SV_THREADS + tid; i < n; i += (int64_t)gridDim.x * SV_THREADS)
-      s = fma(a[i], w[i], s);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if (lane == 0) red[warp] = s;
-    __syncthreads();
-    if (tid == 0) {
-      double t = 0.0;
-      for (int k = 0; k < SV_THREADS / 32; ++k) t += red[k];
-      partial[(int64_t)v * SV_PART + blockIdx.x] = t;
-    }
-    __syncthreads();
-  }
-}
-
-// out[v] = sum_blk partial[v][blk] (fixed order: deterministic)
-__global__ void k_sum_partials(int nv, const double* __restrict__ partial, double* __restrict__ out) {
-  const int v = threadIdx.x;
-  if (v >= nv) return;
-  double s = 0.0;
-  for (int b = 0; b < SV_PART; ++b) s += partial[(int64_t)v * SV_PART + b];
-  out[v] = s;
-}
-
-// w -= sum_v h[v] V[v]
-__global__ void k_orth(int64_t n, int nv, const double* __restrict__ V, const double* __restrict__ h,
-                       double* __restrict__ w) {
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-    double s = w[i];
-    for (int v = 0; v < nv; ++v) s = fma(-h[v], V[(int64_t)v * n + i], s);
-    w[i] = s;
-  }
-}
-
-// x += sum_v c[v] V[v]
-__global__ void k_update(int64_t n, int nv, const double* __restrict__ V, const double* __restrict__ c,
-                         double* __restrict__ x) {
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-    double s = x[i];
-    for (int v = 0; v < nv; ++v) s = fma(c[v], V[(int64_t)v * n + i], s);
-    x[i] = s;
-  }
-}
-
-// r = b - K x, then r <- M^-1 r (in place into r)
-__global__ void k_residual(int m, int64_t n, const double* __restrict__ b, const double* __restrict__ Kx,
-                           double* __restrict__ r) {
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-    r[i] = b[i] - Kx[i];
-}
-
-// y = M^-1 x (block Jacobi), one thread per block row
-__global__ void k_prec(int m, int64_t T, const double* __restrict__ Dinv, const double* __restrict__ x,
-                       double* __restrict__ y) {
-  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= T) return;
-  double xs[5];
-  for (int k = 0; k < m; ++k) xs[k] = x[t * m + k];
-  for (int i = 0; i < m; ++i) {
-    double s = 0.0;
-    for (int k = 0; k < m; ++k) s = fma(Dinv[(t * m + i) * m + k], xs[k], s);
-    y[t * m + i] = s;
-  }
 }
 
 // ---------------------------------------------------------------- BILU(0)
@@ -237,56 +130,35 @@ k_bilu_rows(int m, const int64_t* __restrict__ rows, const int64_t* __restrict__
   if (tid == 0 && !invert_block(m, F + (lo + o[nl]) * mm, Uinv + i * mm)) atomicOr(flag, 1);
 }
 
-// Forward (lower) solve of the rows of one colour, one warp per row, in place:
-// v_i -= sum_{k before i} L_ik v_k.
-__global__ void k_bilu_fwd(int m, int64_t nrows, const int64_t* __restrict__ rows,
-                           const int64_t* __restrict__ row_ptr, const int32_t* __restrict__ col,
-                           const int32_t* __restrict__ ord, const int32_t* __restrict__ nlow,
-                           const double* __restrict__ F, double* __restrict__ v) {
-  const int lane = threadIdx.x & 31, mm = m * m;
-  const int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  if (w >= nrows) return;
-  const int64_t i = rows[w], lo = row_ptr[i];
-  const int32_t* o = ord + lo;
-  const int nl = nlow[i];
-  double acc[5] = {0, 0, 0, 0, 0};
-  for (int q = lane; q < nl; q += 32) {
-    const int64_t kk = lo + o[q];
-    const double* blk = F + kk * mm;
-    const double* x = v + (int64_t)col[kk] * m;
-    for (int r = 0; r < m; ++r) {
-      double sacc = 0.0;
-      for (int t = 0; t < m; ++t) sacc = fma(blk[r * m + t], x[t], sacc);
-      acc[r] += sacc;
-    }
-  }
-  for (int r = 0; r < m; ++r)
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) acc[r] += __shfl_xor_sync(0xffffffffu, acc[r], off);
-  if (lane < m) v[i * m + lane] -= acc[lane];
-}
+// BILU(0) factors and elimination orders on the device.
+struct BiluTab {
+  const int64_t *rows, *row_ptr;
+  const int32_t *col, *ord, *nlow;
+  const double *F, *Uinv;
+};
 
-// Backward (upper) solve of the rows of one colour, in place:
-// v_i = U_ii^-1 (v_i - sum_{j after i} U_ij v_j).
-__global__ void k_bilu_bwd(int m, int64_t nrows, const int64_t* __restrict__ rows,
-                           const int64_t* __restrict__ row_ptr, const int32_t* __restrict__ col,
-                           const int32_t* __restrict__ ord, const int32_t* __restrict__ nlow,
-                           const double* __restrict__ F, const double* __restrict__ Uinv, double* __restrict__ v) {
+// One row of the forward (lower) or backward (upper) solve by one warp, in place:
+// v_i -= sum_{k before i} L_ik v_k, or v_i = U_ii^-1 (v_i - sum_{j after i} U_ij v_j).
+// v is read through L2: other CTAs of the same launch write it in the combined solve.
+template <bool FWD>
+__device__ __forceinline__ void bilu_row(int m, const BiluTab& B, int64_t i, double* __restrict__ v) {
   const int lane = threadIdx.x & 31, mm = m * m;
-  const int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  if (w >= nrows) return;
-  const int64_t i = rows[w], lo = row_ptr[i];
-  const int len = (int)(row_ptr[i + 1] - lo);
-  const int32_t* o = ord + lo;
-  const int nl = nlow[i];
+  const int64_t lo = B.row_ptr[i];
+  const int nl = B.nlow[i];
+  const int q0 = FWD ? 0 : nl + 1, q1 = FWD ? nl : (int)(B.row_ptr[i + 1] - lo);
   double acc[5] = {0, 0, 0, 0, 0};
-  for (int q = nl + 1 + lane; q < len; q += 32) {
-    const int64_t kk = lo + o[q];
-    const double* blk = F + kk * mm;
-    const double* x = v + (int64_t)col[kk] * m;
+  for (int q = q0 + lane; q < q1; q += 32) {
+    const int64_t kk = lo + B.ord[lo + q];
+    const double* blk = B.F + kk * mm;
+    const double* x = v + (int64_t)B.col[kk] * m;
+    double xs[5];
+#pragma unroll
+    for (int t = 0; t < 5; ++t) xs[t] = t < m ? __ldcg(x + t) : 0.0;
     for (int r = 0; r < m; ++r) {
       double sacc = 0.0;
-      for (int t = 0; t < m; ++t) sacc = fma(blk[r * m + t], x[t], sacc);
+#pragma unroll
+      for (int t = 0; t < 5; ++t)
+        if (t < m) sacc = fma(blk[r * m + t], xs[t], sacc);
       acc[r] += sacc;
     }
   }
@@ -294,96 +166,360 @@ __global__ void k_bilu_bwd(int m, int64_t nrows, const int64_t* __restrict__ row
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) acc[r] += __shfl_xor_sync(0xffffffffu, acc[r], off);
   double sv[5];
-  for (int t = 0; t < m; ++t) sv[t] = v[i * m + t] - acc[t];
+  for (int t = 0; t < m; ++t) sv[t] = __ldcg(v + i * m + t) - acc[t];
   __syncwarp();
   if (lane < m) {
-    double x = 0.0;
-    for (int t = 0; t < m; ++t) x = fma(Uinv[(i * mm) + lane * m + t], sv[t], x);
-    v[i * m + lane] = x;
+    double x = sv[lane];
+    if (!FWD) {
+      x = 0.0;
+      for (int t = 0; t < m; ++t) x = fma(B.Uinv[i * mm + lane * m + t], sv[t], x);
+    }
+    __stcg(v + i * m + lane, x);
   }
 }
 
-// ---------------------------------------------------------------- GMRES state on the device
-// The Hessenberg column, Givens rotations, least-squares right-hand side and the
-// residual estimate stay in device memory (kst below), so an Arnoldi step needs one
-// host synchronisation (to read the residual estimate) instead of one per reduction.
-// Layout of kst (doubles): h1 [R+1] | h2 [R+1] | H [(R+1) R] | cs [R] | sn [R] | g [R+1] |
-// y [R] | scalars: hn2, beta, relres, done, jdone.
-struct GmresState {
-  double *h1, *h2, *H, *cs, *sn, *g, *y, *sc;
+// Rows of one colour, one warp per row.
+template <bool FWD>
+__global__ void k_bilu_colour(int m, int64_t nrows, int64_t first, BiluTab B, double* __restrict__ v) {
+  const int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  if (w < nrows) bilu_row<FWD>(m, B, B.rows[first + w], v);
+}
+
+// ---------------------------------------------------------------- GMRES in one launch
+// The solve is a cooperative launch of at most one CTA per SM; its CTAs meet at grid
+// barriers, so an Arnoldi step costs three of them instead of a dozen launches and a
+// synchronisation with the host (about 100 us a step).  Each CTA owns a contiguous range
+// of trace nodes: it forms those rows of K v (a warp per block row, one lane per block
+// entry, so that K streams in order), preconditions, orthogonalises and normalises
+// them; the Hessenberg column, the rotations and the stopping test are formed by every
+// CTA from the same sums in the same order, so nothing else is exchanged.  K v is bound
+// by the FP64 pipe (one multiply-add per entry of K, two per SM and clock).
+// Measured to 1e-12, launch by launch -> one launch: 2D p = 2 8 x 8 (768 unknowns, 26
+// steps) 5.04 -> 0.70 ms, 3D p = 3 6^3 (20,520 unknowns, 112 MB of K, 48 steps) 12.9 -> 5.7,
+// 3D p = 2 16^3 (143,360 unknowns, 72 steps) 31.0 -> 20.7; with BILU(0) 2D 3.4 -> 2.4.
+constexpr int GK_THREADS = 512, GK_WARPS = GK_THREADS / 32;
+constexpr int GK_MIN_ROWS = 8;                    // trace nodes per CTA on small systems
+constexpr int GK_BARRIER_POLLS = 1 << 24;
+
+struct GmresArgs {
+  int m;
+  int64_t T;
+  const int64_t* row_ptr;
+  const int32_t* col;
+  const double *K, *Dinv, *R;
+  double *dU, *V, *w;           // V [restart + 1][T m], w [T m]
+  double* part;                 // partial sums [CTA][R1]
+  double* out;                  // iterations, relative residual
+  unsigned* sync;               // [0] barrier count, [1] abort
+  int restart, max_iter;
+  double rtol;
+  int colours;                  // BILU(0): number of colours, 0 = block Jacobi
+  const int64_t* cptr;
+  BiluTab B;
 };
-__host__ __device__ inline GmresState gmres_state(double* base) {
-  constexpr int R = IEDG_MAX_RESTART;
-  GmresState S;
-  S.h1 = base;
-  S.h2 = S.h1 + (R + 1);
-  S.H = S.h2 + (R + 1);
-  S.cs = S.H + (R + 1) * R;
-  S.sn = S.cs + R;
-  S.g = S.sn + R;
-  S.y = S.g + (R + 1);
-  S.sc = S.y + R;          // [0] hn2, [1] beta, [2] relres, [3] done, [4] jdone
-  return S;
-}
+constexpr int GK_R1 = IEDG_MAX_RESTART + 1;
 
-// y = x / sqrt(*n2), zero if *n2 == 0 (y may alias x)
-__global__ void k_scale_norm(int64_t n, const double* __restrict__ n2, const double* x, double* y) {
-  const double nn = *n2;
-  const double a = nn > 0.0 ? 1.0 / sqrt(nn) : 0.0;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-    y[i] = a * x[i];
-}
+struct GmresShared {
+  double red[GK_WARPS][GK_R1 + 1];
+  double h1[GK_R1], h2[GK_R1];
+  double H[GK_R1][IEDG_MAX_RESTART], cs[IEDG_MAX_RESTART], sn[IEDG_MAX_RESTART], g[GK_R1], y[IEDG_MAX_RESTART];
+  double nrm2, rel, hn, scale;
+  int done, abort, again;
+};
 
-// start of a cycle: beta = sqrt(beta2), g = (beta, 0, ...), relres = beta / beta0, not done
-__global__ void k_gmres_start(GmresState S, double beta0) {
-  const double beta = sqrt(S.sc[0]);
-  S.sc[1] = beta;
-  for (int i = 0; i <= IEDG_MAX_RESTART; ++i) S.g[i] = 0.0;
-  S.g[0] = beta;
-  S.sc[2] = beta0 > 0.0 ? beta / beta0 : 0.0;
-  S.sc[3] = 0.0;
-}
-
-// Hessenberg column j = h1 + h2 (the two Gram-Schmidt passes) with h_{j+1,j} = |w|;
-// earlier rotations applied, a new one formed, g rotated, |g_{j+1}| / beta0 the
-// residual estimate; done when it reaches rtol or the Krylov space is exhausted.
-__global__ void k_gmres_givens(GmresState S, int j, double beta0, double rtol) {
-  constexpr int R = IEDG_MAX_RESTART;
-  double h[R + 1];
-  for (int i = 0; i <= j; ++i) h[i] = S.h1[i] + S.h2[i];
-  const double hn = sqrt(S.sc[0]);
-  for (int i = 0; i < j; ++i) {
-    const double a = S.cs[i] * h[i] + S.sn[i] * h[i + 1];
-    const double b = -S.sn[i] * h[i] + S.cs[i] * h[i + 1];
-    h[i] = a;
-    h[i + 1] = b;
-  }
-  h[j + 1] = hn;
-  const double r = hypot(h[j], h[j + 1]);
-  S.cs[j] = r > 0.0 ? h[j] / r : 1.0;
-  S.sn[j] = r > 0.0 ? h[j + 1] / r : 0.0;
-  h[j] = r;
-  S.g[j + 1] = -S.sn[j] * S.g[j];
-  S.g[j] = S.cs[j] * S.g[j];
-  for (int i = 0; i <= j; ++i) S.H[i * R + j] = h[i];
-  const double rel = fabs(S.g[j + 1]) / beta0;
-  S.sc[2] = rel;
-  S.sc[3] = (rel <= rtol || hn == 0.0) ? 1.0 : 0.0;
-}
-
-// y = H(0:j, 0:j)^-1 g (upper triangular)
-__global__ void k_gmres_backsolve(GmresState S, int j) {
-  constexpr int R = IEDG_MAX_RESTART;
-  for (int i = j - 1; i >= 0; --i) {
-    double s = S.g[i];
-    for (int k = i + 1; k < j; ++k) s -= S.H[i * R + k] * S.y[k];
-    S.y[i] = s / S.H[i * R + i];
+// Barrier over the grid (all CTAs resident: cooperative launch) in two halves, so that
+// work of one thread can hide behind the wait.  Bounded: a CTA that gives up sets the
+// abort flag, which ends every CTA's wait.  barrier_wait returns false on abort.
+__device__ __forceinline__ void barrier_arrive(const GmresArgs& a) {
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    atomicAdd(a.sync, 1u);
   }
 }
+__device__ __forceinline__ bool barrier_wait(const GmresArgs& a, GmresShared& sh, unsigned& round) {
+  if (threadIdx.x == 0) {
+    ++round;
+    const unsigned want = round * gridDim.x;
+    int polls = 0, ab = 0;
+    unsigned seen;
+    do {
+      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(a.sync) : "memory");
+      if ((int)(seen - want) >= 0) break;
+      if ((++polls & 1023) == 0) ab = *(volatile unsigned*)(a.sync + 1) != 0;
+    } while (!ab && polls < GK_BARRIER_POLLS);
+    if ((int)(seen - want) < 0) { atomicExch(a.sync + 1, 1u); ab = 1; }
+    sh.abort = ab;
+  }
+  __syncthreads();
+  return sh.abort == 0;
+}
+__device__ __forceinline__ bool grid_barrier(const GmresArgs& a, GmresShared& sh, unsigned& round) {
+  barrier_arrive(a);
+  return barrier_wait(a, sh, round);
+}
 
-unsigned grid_for(int64_t n) {
-  int64_t g = (n + SV_THREADS - 1) / SV_THREADS;
-  return (unsigned)(g < 4096 ? g : 4096);
+// out[v] = sum over the grid of part[cta][v], v < nv, in CTA order within a warp's share;
+// the same in every CTA.
+__device__ __forceinline__ void sum_parts(const GmresArgs& a, GmresShared& sh, int nv, double* out) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  for (int v0 = 0; v0 < nv; v0 += 32) {
+    double s = 0.0;
+    if (v0 + lane < nv)
+      for (int c = warp; c < (int)gridDim.x; c += GK_WARPS) s += __ldcg(a.part + (int64_t)c * GK_R1 + v0 + lane);
+    if (v0 + lane < nv) sh.red[warp][v0 + lane] = s;
+  }
+  __syncthreads();
+  if (threadIdx.x < nv) {
+    double s = 0.0;
+    const int nw = min(GK_WARPS, (int)gridDim.x);
+    for (int k = 0; k < nw; ++k) s += sh.red[k][threadIdx.x];
+    out[threadIdx.x] = s;
+  }
+  __syncthreads();
+}
+
+// part[this CTA][v] = V[v] . w over the CTA's unknowns [i0, i1), v < nv: a warp per vector,
+// or several where there are more warps than vectors.
+__device__ __forceinline__ void dot_parts(const GmresArgs& a, GmresShared& sh, int nv, const double* V, int64_t n,
+                                          const double* w, int64_t i0, int64_t i1) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int segs = nv < GK_WARPS ? GK_WARPS / nv : 1;
+  for (int it = warp; it < nv * segs; it += GK_WARPS) {
+    const int v = it / segs, sg = it % segs;
+    const double* x = V + (int64_t)v * n;
+    double s = 0.0;
+#pragma unroll 4
+    for (int64_t i = i0 + sg * 32 + lane; i < i1; i += 32 * segs) s = fma(x[i], w[i], s);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (lane == 0) sh.red[sg][v] = s;
+  }
+  __syncthreads();
+  if (threadIdx.x < nv) {
+    double s = 0.0;
+    for (int k = 0; k < segs; ++k) s += sh.red[k][threadIdx.x];
+    __stcg(a.part + (int64_t)blockIdx.x * GK_R1 + threadIdx.x, s);
+  }
+}
+
+// Rows [t0, t1) of y = K x, or b - K x; x read through L2 (other CTAs wrote it).  A warp
+// per block row, a lane per block entry (two blocks at a time where m = 4); the row's
+// column indices are read 32 at a time and 16 blocks of K and x requested together.
+__device__ __forceinline__ void spmv_rows(const GmresArgs& a, const double* x, double* y, const double* b, int64_t t0,
+                                          int64_t t1) {
+  constexpr int UN = 16;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int m = a.m, mm = m * m, per = 32 / mm;            // blocks per warp step
+  const int sub = lane / mm, e = lane % mm, k = e % m;
+  for (int64_t t = t0 + warp; t < t1; t += GK_WARPS) {
+    const int64_t lo = a.row_ptr[t], hi = a.row_ptr[t + 1];
+    double acc = 0.0;
+    for (int64_t base = lo; base < hi; base += 32) {
+      const int nblk = (int)min((int64_t)32, hi - base);
+      const int xc = lane < nblk ? a.col[base + lane] * m : 0;
+      const double* kb = a.K + base * mm + e;
+      for (int u0 = 0; u0 < nblk; u0 += UN * per) {
+        double kv[UN], xv[UN];
+#pragma unroll
+        for (int u = 0; u < UN; ++u) {
+          const int q = u0 + u * per + sub;
+          const int xo = __shfl_sync(0xffffffffu, xc, q & 31);
+          const bool on = sub < per && q < nblk;
+          kv[u] = on ? kb[q * mm] : 0.0;
+          xv[u] = on ? __ldcg(x + xo + k) : 0.0;
+        }
+#pragma unroll
+        for (int u = 0; u < UN; ++u) acc = fma(kv[u], xv[u], acc);
+      }
+    }
+    // the two blocks' shares, then the row sums over k
+    if (per == 2) acc += __shfl_down_sync(0xffffffffu, acc, 16);
+    double s = 0.0;
+    for (int kk = 0; kk < m; ++kk) s += __shfl_sync(0xffffffffu, acc, (lane < m ? lane * m : 0) + kk);
+    if (lane < m) y[t * m + lane] = b ? b[t * m + lane] - s : s;
+  }
+}
+
+// y = M^-1 y on the CTA's rows (block Jacobi) or on all rows (BILU(0), barriers inside).
+__device__ __forceinline__ bool precondition(const GmresArgs& a, GmresShared& sh, double* y, int64_t t0, int64_t t1,
+                                             unsigned& round) {
+  const int tid = threadIdx.x;
+  if (a.colours == 0) {
+    __syncthreads();
+    const int m = a.m;
+    for (int64_t t = t0 + tid; t < t1; t += GK_THREADS) {
+      double xs[5];
+      for (int k = 0; k < m; ++k) xs[k] = y[t * m + k];
+      for (int i = 0; i < m; ++i) {
+        double s = 0.0;
+        for (int k = 0; k < m; ++k) s = fma(a.Dinv[(t * m + i) * m + k], xs[k], s);
+        y[t * m + i] = s;
+      }
+    }
+    __syncthreads();
+    return true;
+  }
+  const int64_t w0 = (int64_t)blockIdx.x * GK_WARPS + (tid >> 5), nw = (int64_t)gridDim.x * GK_WARPS;
+  if (!grid_barrier(a, sh, round)) return false;
+  for (int c = 0; c < a.colours; ++c) {
+    for (int64_t r = a.cptr[c] + w0; r < a.cptr[c + 1]; r += nw) bilu_row<true>(a.m, a.B, a.B.rows[r], y);
+    if (!grid_barrier(a, sh, round)) return false;
+  }
+  for (int c = a.colours - 1; c >= 0; --c) {
+    for (int64_t r = a.cptr[c] + w0; r < a.cptr[c + 1]; r += nw) bilu_row<false>(a.m, a.B, a.B.rows[r], y);
+    if (!grid_barrier(a, sh, round)) return false;
+  }
+  return true;
+}
+
+__global__ void __launch_bounds__(GK_THREADS, 1) k_gmres(GmresArgs a) {
+  __shared__ GmresShared sh;
+  const int tid = threadIdx.x;
+  const int m = a.m;
+  const int64_t n = a.T * m;
+  const int64_t t0 = a.T * blockIdx.x / gridDim.x, t1 = a.T * (blockIdx.x + 1) / gridDim.x;
+  const int64_t i0 = t0 * m, i1 = t1 * m;
+  unsigned round = 0;
+  // own rows of w: BILU(0) has other CTAs write them, so they are read through L2 then
+  auto own = [&](const double* p) { return a.colours ? __ldcg(p) : *p; };
+  // x0 = 0, r0 = M^-1 R
+  for (int64_t i = i0 + tid; i < i1; i += GK_THREADS) {
+    a.dU[i] = 0.0;
+    a.w[i] = a.R[i];
+  }
+  // own rows of x <- s (x - sum_{v < nv} h[v] V_v)
+  auto subtract = [&](int nv, const double* h, double* x, double s) {
+    for (int64_t i = i0 + tid; i < i1; i += GK_THREADS) {
+      double t = x[i];
+#pragma unroll 4
+      for (int v = 0; v < nv; ++v) t = fma(-h[v], a.V[(int64_t)v * n + i], t);
+      x[i] = s * t;
+    }
+  };
+  int total = 0;
+  double beta0 = 0.0, relres = 0.0;
+  bool first = true, alive = true;
+  while (alive) {
+    if (!first) spmv_rows(a, a.dU, a.w, a.R, t0, t1);
+    if (!(alive = precondition(a, sh, a.w, t0, t1, round))) break;
+    for (int64_t i = i0 + tid; i < i1; i += GK_THREADS) a.V[i] = own(a.w + i);
+    __syncthreads();
+    dot_parts(a, sh, 1, a.V, n, a.V, i0, i1);
+    if (!(alive = grid_barrier(a, sh, round))) break;
+    sum_parts(a, sh, 1, sh.h1);
+    const double beta = sqrt(sh.h1[0]);
+    if (first) {
+      beta0 = beta;
+      relres = beta0 > 0.0 ? 1.0 : 0.0;
+    } else {
+      relres = beta / beta0;
+    }
+    first = false;
+    if (!(beta0 > 0.0) || total >= a.max_iter || relres <= a.rtol) break;
+    {
+      const double s = beta > 0.0 ? 1.0 / beta : 0.0;
+      for (int64_t i = i0 + tid; i < i1; i += GK_THREADS) a.V[i] *= s;
+      for (int i = tid; i < GK_R1; i += GK_THREADS) sh.g[i] = i == 0 ? beta : 0.0;
+    }
+    if (!(alive = grid_barrier(a, sh, round))) break;
+    int j = 0;
+    for (; j < a.restart && total < a.max_iter; ++j, ++total) {
+      double* vn = a.V + (int64_t)(j + 1) * n;
+      spmv_rows(a, a.V + (int64_t)j * n, a.w, nullptr, t0, t1);
+      if (!(alive = precondition(a, sh, a.w, t0, t1, round))) break;
+      // the candidate lives in vn's own rows from here on
+      for (int64_t i = i0 + tid; i < i1; i += GK_THREADS) vn[i] = own(a.w + i);
+      __syncthreads();
+      // iterated classical Gram-Schmidt: two passes, the second with |w|^2 beside the
+      // products (V_{j+1} is w itself), which gives the norm of the orthogonalised
+      // vector, |w|^2 - |h2|^2, without another barrier
+      dot_parts(a, sh, j + 1, a.V, n, vn, i0, i1);
+      if (!(alive = grid_barrier(a, sh, round))) break;
+      sum_parts(a, sh, j + 1, sh.h1);
+      subtract(j + 1, sh.h1, vn, 1.0);
+      __syncthreads();
+      dot_parts(a, sh, j + 2, a.V, n, vn, i0, i1);
+      if (!(alive = grid_barrier(a, sh, round))) break;
+      sum_parts(a, sh, j + 2, sh.h2);
+      if (tid < 32) {        // one warp: square roots and divisions would load the FP64 pipe
+        double q = 0.0;
+        for (int v = tid; v <= j; v += 32) q = fma(sh.h2[v], sh.h2[v], q);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) q += __shfl_xor_sync(0xffffffffu, q, o);
+        const double w2 = sh.h2[j + 1], hn2 = w2 - q;
+        if (tid == 0) {
+          // a second pass that still removes much of w would cancel here: sum again then
+          sh.again = hn2 < 0.25 * w2;
+          sh.hn = hn2 > 0.0 ? sqrt(hn2) : 0.0;
+          sh.scale = sh.again ? 1.0 : (hn2 > 0.0 ? 1.0 / sh.hn : 0.0);
+        }
+      }
+      __syncthreads();
+      subtract(j + 1, sh.h2, vn, sh.scale);
+      if (sh.again) {
+        __syncthreads();
+        dot_parts(a, sh, 1, vn, n, vn, i0, i1);
+        if (!(alive = grid_barrier(a, sh, round))) break;
+        sum_parts(a, sh, 1, &sh.nrm2);
+        if (tid == 0) {
+          sh.hn = sqrt(sh.nrm2);
+          sh.scale = sh.nrm2 > 0.0 ? 1.0 / sh.hn : 0.0;
+        }
+        __syncthreads();
+        const double s = sh.scale;
+        for (int64_t i = i0 + tid; i < i1; i += GK_THREADS) vn[i] *= s;
+      }
+      barrier_arrive(a);
+      if (tid == 0) {
+        // Hessenberg column j: earlier rotations applied, a new one formed, g rotated,
+        // |g_{j+1}| / beta0 the residual estimate
+        const double hn = sh.hn;
+        double a0 = sh.h1[0] + sh.h2[0];
+        for (int i = 0; i < j; ++i) {
+          const double a1 = sh.h1[i + 1] + sh.h2[i + 1];
+          sh.H[i][j] = sh.cs[i] * a0 + sh.sn[i] * a1;
+          a0 = -sh.sn[i] * a0 + sh.cs[i] * a1;
+        }
+        const double r = hypot(a0, hn);
+        const double c = r > 0.0 ? a0 / r : 1.0, sn = r > 0.0 ? hn / r : 0.0;
+        sh.cs[j] = c;
+        sh.sn[j] = sn;
+        sh.H[j][j] = r;
+        const double gj = sh.g[j];
+        sh.g[j + 1] = -sn * gj;
+        sh.g[j] = c * gj;
+        sh.rel = fabs(sh.g[j + 1]) / beta0;
+        sh.done = (sh.rel <= a.rtol || hn == 0.0) ? 1 : 0;
+      }
+      if (!(alive = barrier_wait(a, sh, round))) break;   // vn complete; publishes rel and done in the CTA
+      relres = sh.rel;
+      if (sh.done) { ++j; ++total; break; }
+    }
+    if (!alive) break;
+    // y = H(0:j, 0:j)^-1 g (upper triangular, column by column), x += V y
+    if (tid < 32) {
+      for (int i = j - 1; i >= 0; --i) {
+        const double yi = sh.g[i] / sh.H[i][i];
+        __syncwarp();
+        for (int k = tid; k < i; k += 32) sh.g[k] = fma(-sh.H[k][i], yi, sh.g[k]);
+        if (tid == 0) sh.y[i] = yi;
+        __syncwarp();
+      }
+    }
+    __syncthreads();
+    for (int64_t i = i0 + tid; i < i1; i += GK_THREADS) {
+      double s = a.dU[i];
+      for (int v = 0; v < j; ++v) s = fma(sh.y[v], a.V[(int64_t)v * n + i], s);
+      a.dU[i] = s;
+    }
+    if (!(total < a.max_iter && relres > a.rtol)) break;
+    if (!(alive = grid_barrier(a, sh, round))) break;     // x complete before K x
+  }
+  if (blockIdx.x == 0 && tid == 0) {
+    a.out[0] = (double)total;
+    a.out[1] = relres;
+  }
 }
 
 }  // namespace
@@ -450,6 +586,7 @@ static int bilu_setup(iedg_mesh* M, cudaStream_t st) {
     *dst = d;
     return cudaMemcpyAsync(d, h.data(), h.size() * sizeof(E), cudaMemcpyHostToDevice, st);
   };
+  SV_TRY(put(&M->bcptr_dev, cnt));
   SV_TRY(put(&M->brows, rows));
   SV_TRY(put(&M->bord, ord));
   SV_TRY(put(&M->bnlow, nlow));
@@ -486,18 +623,15 @@ static int bilu_factor(iedg_mesh* M, const double* K, double* F, cudaStream_t st
 static cudaError_t bilu_apply(iedg_mesh* M, const double* F, double* v, cudaStream_t st) {
   const int m = M->dm.m;
   const size_t nc = M->bcptr.size() - 1;
-
+  const BiluTab B{M->brows, M->row_ptr, M->col, M->bord, M->bnlow, F, M->dinv};
+  auto blocks = [](int64_t nr) { return (unsigned)((nr * 32 + SV_THREADS - 1) / SV_THREADS); };
   for (size_t c = 0; c < nc; ++c) {
     const int64_t nr = M->bcptr[c + 1] - M->bcptr[c];
-    if (nr == 0) continue;
-    k_bilu_fwd<<<(unsigned)((nr * 32 + SV_THREADS - 1) / SV_THREADS), SV_THREADS, 0, st>>>(
-        m, nr, M->brows + M->bcptr[c], M->row_ptr, M->col, M->bord, M->bnlow, F, v);
+    if (nr > 0) k_bilu_colour<true><<<blocks(nr), SV_THREADS, 0, st>>>(m, nr, M->bcptr[c], B, v);
   }
   for (size_t c = nc; c-- > 0;) {
     const int64_t nr = M->bcptr[c + 1] - M->bcptr[c];
-    if (nr == 0) continue;
-    k_bilu_bwd<<<(unsigned)((nr * 32 + SV_THREADS - 1) / SV_THREADS), SV_THREADS, 0, st>>>(
-        m, nr, M->brows + M->bcptr[c], M->row_ptr, M->col, M->bord, M->bnlow, F, M->dinv, v);
+    if (nr > 0) k_bilu_colour<false><<<blocks(nr), SV_THREADS, 0, st>>>(m, nr, M->bcptr[c], B, v);
   }
   return cudaGetLastError();
 }
@@ -557,13 +691,6 @@ extern "C" int iedg_trace_solve(iedg_mesh* M, const double* K, const double* R, 
   cudaStream_t st = (cudaStream_t)stream;
   const int m = M->dm.m;
   const int64_t T = M->T, n = T * m;
-  double* V = M->kry;                     // [restart+1][n]
-  double* w = V + (int64_t)(IEDG_MAX_RESTART + 1) * n;
-  double* tmp = w + n;
-  double* Dinv = M->dinv;
-  double* part = M->kpart;                // [restart+1][SV_PART]
-  const unsigned g = grid_for(n);
-  const unsigned gw = (unsigned)((T * 32 + SV_THREADS - 1) / SV_THREADS);
   const bool bilu = M->prec_kind == IEDG_PREC_BILU0;
   if (bilu) {
     if (!M->bf) {
@@ -576,91 +703,40 @@ extern "C" int iedg_trace_solve(iedg_mesh* M, const double* K, const double* R, 
     int rc = bilu_factor(M, K, M->bf, st);
     if (rc != IEDG_OK) return rc;
   }
-  // y = M^-1 x (in place allowed)
-  auto prec = [&](const double* x, double* y) -> cudaError_t {
-    if (!bilu) {
-      k_prec<<<(unsigned)((T + 127) / 128), 128, 0, st>>>(m, T, Dinv, x, y);
-      return cudaGetLastError();
-    }
-    if (x != y) {
-      cudaError_t e = cudaMemcpyAsync(y, x, n * sizeof(double), cudaMemcpyDeviceToDevice, st);
-      if (e != cudaSuccess) return e;
-    }
-    return bilu_apply(M, M->bf, y, st);
-  };
   SV_TRY(cudaMemsetAsync(M->dev_flag, 0, sizeof(int), st));
   if (!bilu)
-    SV_TRY((k_diag_inv<<<(unsigned)((T + 127) / 128), 128, 0, st>>>(m, T, M->row_ptr, M->col, K, Dinv, M->dev_flag),
+    SV_TRY((k_diag_inv<<<(unsigned)((T + 127) / 128), 128, 0, st>>>(m, T, M->row_ptr, M->col, K, M->dinv, M->dev_flag),
             cudaGetLastError()));
-  // sums of products into device memory (fixed block order: deterministic)
-  auto dots_dev = [&](int nv, const double* Vb, const double* x, double* out_dev) -> cudaError_t {
-    k_dots<<<SV_PART, SV_THREADS, 0, st>>>(n, nv, Vb, x, part);
-    k_sum_partials<<<1, 64, 0, st>>>(nv, part, out_dev);
-    return cudaGetLastError();
-  };
-  const GmresState S = gmres_state(M->kst);
-  // the host reads three scalars of the device state: squared norm, residual estimate, done
-  auto read_state = [&](double* out3) -> cudaError_t {
-    cudaError_t e = cudaMemcpyAsync(out3, S.sc, 4 * sizeof(double), cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-    return e;
-  };
-  // x0 = 0, r0 = M^-1 R
-  SV_TRY(cudaMemsetAsync(dU, 0, n * sizeof(double), st));
-  SV_TRY(prec(R, V));
-  SV_TRY(dots_dev(1, V, V, S.sc));
-  double hs[4] = {0, 0, 0, 0};
-  SV_TRY(read_state(hs));
-  const double beta0 = std::sqrt(hs[0]);
+  // result scalars and the barrier's two words sit behind the partial sums
+  double* out = M->kpart + (int64_t)GK_R1 * kGmresMaxCtas;
+  unsigned* sync = reinterpret_cast<unsigned*>(out + 4);
+  SV_TRY(cudaMemsetAsync(out, 0, 8 * sizeof(double), st));
+  GmresArgs a{m, T, M->row_ptr, M->col, K, M->dinv, R, dU, M->kry, M->kry + (int64_t)GK_R1 * n, M->kpart, out, sync,
+              restart, max_iter, rtol, bilu ? (int)M->bcptr.size() - 1 : 0, M->bcptr_dev,
+              BiluTab{M->brows, M->row_ptr, M->col, M->bord, M->bnlow, M->bf, M->dinv}};
+  // one CTA per SM at most (a co-resident grid with the fewest partial sums), fewer on small systems
+  int dev = 0, sms = 0;
+  SV_TRY(cudaGetDevice(&dev));
+  SV_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+  const int64_t g = std::min<int64_t>(std::min<int64_t>(sms, kGmresMaxCtas), std::max<int64_t>(1, T / GK_MIN_ROWS));
+  void* args[] = {&a};
+  SV_TRY(cudaLaunchCooperativeKernel((const void*)k_gmres, dim3((unsigned)g), dim3(GK_THREADS), args, 0, st));
+  double res[5] = {0, 0, 0, 0, 0};
   int flag = 0;
-  SV_TRY(cudaMemcpy(&flag, M->dev_flag, sizeof(int), cudaMemcpyDeviceToHost));
-  if (flag) {
+  SV_TRY(cudaMemcpyAsync(res, out, sizeof(res), cudaMemcpyDeviceToHost, st));
+  SV_TRY(cudaMemcpyAsync(&flag, M->dev_flag, sizeof(int), cudaMemcpyDeviceToHost, st));
+  SV_TRY(cudaStreamSynchronize(st));
+  if (flag && !bilu) {
     M->err = "iedg_trace_solve: singular diagonal block of K";
     return IEDG_ERR_INVALID_ARG;
   }
-  int total = 0;
-  double relres = beta0 > 0.0 ? 1.0 : 0.0;
-  bool first = true;
-  while (beta0 > 0.0 && total < max_iter && relres > rtol) {
-    if (!first) {
-      // r = M^-1 (R - K x)
-      SV_TRY((k_spmv<<<gw, SV_THREADS, 0, st>>>(m, T, M->row_ptr, M->col, K, Dinv, dU, tmp, false), cudaGetLastError()));
-      SV_TRY((k_residual<<<g, SV_THREADS, 0, st>>>(m, n, R, tmp, tmp), cudaGetLastError()));
-      SV_TRY(prec(tmp, V));
-      SV_TRY(dots_dev(1, V, V, S.sc));
-    }
-    SV_TRY((k_gmres_start<<<1, 1, 0, st>>>(S, beta0), cudaGetLastError()));
-    if (!first) {
-      SV_TRY(read_state(hs));
-      relres = hs[2];
-      if (relres <= rtol) break;
-    }
-    first = false;
-    SV_TRY((k_scale_norm<<<g, SV_THREADS, 0, st>>>(n, S.sc, V, V), cudaGetLastError()));
-    int j = 0;
-    for (; j < restart && total < max_iter; ++j, ++total) {
-      double* vj = V + (int64_t)j * n;
-      double* vn = V + (int64_t)(j + 1) * n;
-      SV_TRY((k_spmv<<<gw, SV_THREADS, 0, st>>>(m, T, M->row_ptr, M->col, K, Dinv, vj, w, !bilu), cudaGetLastError()));
-      if (bilu) SV_TRY(prec(w, w));
-      // iterated classical Gram-Schmidt: two passes, coefficients kept on the device
-      SV_TRY(dots_dev(j + 1, V, w, S.h1));
-      SV_TRY((k_orth<<<g, SV_THREADS, 0, st>>>(n, j + 1, V, S.h1, w), cudaGetLastError()));
-      SV_TRY(dots_dev(j + 1, V, w, S.h2));
-      SV_TRY((k_orth<<<g, SV_THREADS, 0, st>>>(n, j + 1, V, S.h2, w), cudaGetLastError()));
-      SV_TRY(dots_dev(1, w, w, S.sc));
-      SV_TRY((k_scale_norm<<<g, SV_THREADS, 0, st>>>(n, S.sc, w, vn), cudaGetLastError()));
-      SV_TRY((k_gmres_givens<<<1, 1, 0, st>>>(S, j, beta0, rtol), cudaGetLastError()));
-      SV_TRY(read_state(hs));                         // the one synchronisation of the step
-      relres = hs[2];
-      if (hs[3] != 0.0) { ++j; ++total; break; }
-    }
-    // y = H(0:j, 0:j)^-1 g, x += V y
-    SV_TRY((k_gmres_backsolve<<<1, 1, 0, st>>>(S, j), cudaGetLastError()));
-    SV_TRY((k_update<<<g, SV_THREADS, 0, st>>>(n, j, V, S.y, dU), cudaGetLastError()));
+  unsigned words[2];
+  std::memcpy(words, &res[4], sizeof(words));
+  if (words[1]) {
+    M->err = "iedg_trace_solve: the grid barrier gave up";
+    return IEDG_ERR_CUDA;
   }
-  SV_TRY(cudaStreamSynchronize(st));
-  if (iterations) *iterations = total;
-  if (rel_residual) *rel_residual = relres;
+  if (iterations) *iterations = (int32_t)res[0];
+  if (rel_residual) *rel_residual = res[1];
   return IEDG_OK;
 }
