@@ -1087,6 +1087,8 @@ extern "C" int iedg_assemble_condensed(iedg_mesh* M, const double* u, const doub
   CUDA_TRY(TRACED("points_jacobian", launch_points(M, u, q, M->qstar, uhat, u_ref, true, nullptr, nullptr, st)));
   if (assemble_sf_supported(dm))
     CUDA_TRY(TRACED("assemble", launch_assemble_sf(M, st)));
+  else if (assemble_col_supported(M))
+    CUDA_TRY(TRACED("assemble", launch_assemble_col(M, st)));
   else
     CUDA_TRY(TRACED("assemble", launch_assemble(M, st)));
   if (M->mass_scaled) CUDA_TRY(TRACED("mass_scale", launch_mass_scale(M, st)));
