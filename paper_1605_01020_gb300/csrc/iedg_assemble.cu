@@ -19,6 +19,7 @@
 // Gt = -R_FL,e(u, q*) (exact because the fluxes are affine in q).
 #include <cuda_bf16.h>
 
+#include "iedg_digits.cuh"
 #include "iedg_internal.cuh"
 #include "iedg_lu_common.cuh"
 #include "iedg_tc.cuh"
@@ -507,15 +508,18 @@ __device__ __forceinline__ void lu_element(const LuElem& el, T* __restrict__ S, 
 // and 2 M additions of the updates (65 M multiply-adds in the DFMA form).  Two CTAs per
 // SM, so that one element's panels overlap the other's updates.
 // Measured, all elements of a mesh, DFMA form -> this one: 3D p = 3, 4096 elements
-// 505.9 -> 100.5 ms; p = 2, 2002 elements 26.5 -> 8.3 ms; p = 4, 210 elements 238.6 -> 57.9 ms;
+// 505.9 -> 95.1 ms; p = 2, 2002 elements 26.5 -> 7.7 ms; p = 4, 210 elements 238.6 -> 48.4 ms
+// (with a branch per joined entry and L21 loaded when staged: 100.5, 8.3, 57.9 ms);
 // 2D p = 3 (64 + 48 unknowns), 851 elements 1.53 -> 0.82 ms.  Below 64 u-unknowns an
 // element is at most two panels, which leaves too little to the tensor cores, and the
 // DFMA form stays: 2D p = 2 (36 + 32), 1600 elements 0.78 ms DFMA, 0.95 ms digits; 3D p = 1
-// (40 + 40), 8000 elements 4.98 and 4.92 ms.  Counters at p = 3: FP64 pipe 43 % busy, issue
-// slots 32 %, tensor pipe 8 %, 42 MB of DRAM traffic per element: latency of the panel
+// (40 + 40), 8000 elements 4.98 and 4.92 ms.  Counters at p = 3: FP64 pipe 47 % busy, issue
+// slots 35 %, tensor pipe 8 %, 42 MB of DRAM traffic per element: latency of the panel
 // steps and of the trailing block's loads, not a pipe, is what is left.
 constexpr int LT_NB = 32;                       // panel width
-constexpr int LT_S = 8;                         // digits per operand, and levels kept
+constexpr int LT_S = dig::S;                    // digits per operand, and levels kept
+using dig::exponent_of;
+using dig::scale_of;
 constexpr int LT_TC = 128, LT_TR = 16;          // columns and rows of one MMA group
 constexpr int LT_RB = 64;                       // rows of L21 staged at a time
 constexpr int LT_SLICE = LT_TC * LT_NB * 2;     // one digit of a column tile
@@ -524,8 +528,6 @@ constexpr int LT_GROUP = LT_S * LT_TR * LT_NB * 2;          // all digits of 16 
 constexpr int LT_B_BYTES = LT_RB / LT_TR * LT_GROUP;        // 32 KB
 constexpr int LT_LVL_COLS = LT_S * LT_TR;       // TMEM columns of one accumulator set
 constexpr int LT_TMEM_COLS = 2 * LT_LVL_COLS;   // two sets: epilogue of one, MMAs into the other
-constexpr int LT_BAD_EXP = 1 << 13;             // exponent of a row or column with a non-finite entry
-
 __host__ __device__ inline int lt_stride(int nu) { return nu | 1; }   // odd: conflict-free columns
 
 __host__ inline size_t lt_smem(const Dims& dm) {
@@ -533,56 +535,40 @@ __host__ inline size_t lt_smem(const Dims& dm) {
   return (panel > dig ? panel : dig) + 128;      // operand tiles start on a 128-byte boundary
 }
 
-__device__ __forceinline__ int exponent_of(double x) { return (__double2hiint(x) >> 20) & 0x7ff; }
-// biased exponent of a row's (column's) largest entry as the epilogue adds it
-__device__ __forceinline__ int scale_of(int emax) { return emax == 0x7ff ? LT_BAD_EXP : emax; }
-
 // Digits of eight values with common exponent emax >= theirs: out(s, 8 packed BF16) for
-// s = 0 (most significant) .. 7.  Entries below 2^-62 of the scale and subnormals are 0.
+// s = 0 (most significant) .. 7.
 template <class Out>
 __device__ __forceinline__ void split8(const double (&x)[8], int emax, Out out) {
-  uint32_t lo[8], hi[8];
+  uint32_t w[2][8];
 #pragma unroll
   for (int i = 0; i < 8; ++i) {
-    const long long b = __double_as_longlong(x[i]);
-    const int e = exponent_of(x[i]), sh = emax - e;
-    unsigned long long m = ((unsigned long long)b & 0xFFFFFFFFFFFFFull) | 0x10000000000000ull;
-    m = (e == 0 || sh > 62) ? 0ull : (m << 9) >> sh;
-    const unsigned long long v = (b < 0 ? 0ull - m : m) + 0x8080808080808080ull;   // digits + 128
-    lo[i] = (uint32_t)v;
-    hi[i] = (uint32_t)(v >> 32);
+    const unsigned long long v = dig::to_bytes(__double_as_longlong(x[i]), emax);
+    w[0][i] = (uint32_t)(v >> 32);
+    w[1][i] = (uint32_t)v;
   }
 #pragma unroll
   for (int s = 0; s < LT_S; ++s) {
-    uint32_t w[4];
-#pragma unroll
-    for (int p = 0; p < 4; ++p) {
-      float f[2];
-#pragma unroll
-      for (int q = 0; q < 2; ++q) {
-        const uint32_t word = s < 4 ? hi[2 * p + q] : lo[2 * p + q];
-        // byte -> float 2^23 + byte, minus 2^23 + 128: at most 8 significant bits, so
-        // the upper half of the FP32 pattern is the BF16 value
-        f[q] = __uint_as_float(__byte_perm(word, 0x4B000000u, 0x7440u | (uint32_t)(3 - (s & 3)))) - 8388736.0f;
-      }
-      w[p] = __byte_perm(__float_as_uint(f[0]), __float_as_uint(f[1]), 0x7632);
-    }
-    out(s, make_uint4(w[0], w[1], w[2], w[3]));
+    const uint32_t(&q)[8] = w[s >> 2];
+    out(s, make_uint4(dig::bf16_pair(q[0], q[1], s), dig::bf16_pair(q[2], q[3], s), dig::bf16_pair(q[4], q[5], s),
+                      dig::bf16_pair(q[6], q[7], s)));
   }
 }
 
-// One thread: all digit products of one 16-row group into the accumulator set at d.
-__device__ __forceinline__ void lt_issue(uint32_t d, uint32_t a, uint32_t b, int ksteps) {
+// One thread: all digit products of one 16-row group into the accumulator set at d; a, b:
+// descriptors of the operands' first slices (addresses in their low bits, in 16 bytes).
+__device__ __forceinline__ void lt_issue(uint32_t d, uint64_t a, uint64_t b, int ksteps) {
   for (int ks = 0; ks < ksteps; ++ks)
 #pragma unroll
     for (int s = 0; s < LT_S; ++s)
-      tc::mma_bf16(d + (uint32_t)(s * LT_TR), tc::desc_kmajor(a + s * LT_SLICE + ks * 256, 128, 512),
-                   tc::desc_kmajor(b + ks * 256, 128, 512), tc::idesc_bf16(LT_TC, LT_TR * (LT_S - s)),
-                   (ks == 0 && s == 0) ? 0u : 1u);
+      tc::mma_bf16(d + (uint32_t)(s * LT_TR), a + (uint64_t)(s * (LT_SLICE >> 4) + ks * 16), b + (uint64_t)(ks * 16),
+                   tc::idesc_bf16(LT_TC, LT_TR * (LT_S - s)), (ks == 0 && s == 0) ? 0u : 1u);
 }
 
-// minus the product sum whose level sums are t[0..7], scales ef = row + column exponent
-__device__ __forceinline__ double join_levels(const float (&t)[8], int ef) {
+// minus the product sum whose level sums are t[0..7], scales ef = row + column exponent.
+// Free of branches, so that a thread's eight entries overlap; `odd` is set where the
+// result leaves the normal range (a non-finite operand, or a product sum out of FP64's
+// exponent range), for the caller to replace it by dig::special.
+__device__ __forceinline__ double join_levels(const float (&t)[8], int ef, bool& odd) {
   uint32_t p[4];
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
@@ -593,34 +579,10 @@ __device__ __forceinline__ double join_levels(const float (&t)[8], int ef) {
   long long v = (long long)(int)p[2] * 32 + (((int)p[3] + 1024) >> 11);
   v += (long long)(int)p[1] * (1 << 21);
   v += (long long)((unsigned long long)p[0] << 37);
-  if (v == 0) return 0.0;
-  const unsigned long long mag = v < 0 ? 0ull - (unsigned long long)v : (unsigned long long)v;
-  const int lz = __clzll((long long)mag);
-  const unsigned long long mn = mag << lz;
-  const int field = ef - 1015 - lz;
-  const unsigned long long sign = v > 0 ? 0x8000000000000000ull : 0ull;
-  if ((unsigned)(field - 1) < 2045u) {
-    const unsigned long long r = (mn >> 11) + ((mn >> 10) & 1ull) + ((unsigned long long)(unsigned)(field - 1) << 52);
-    return __longlong_as_double((long long)(r | sign));
-  }
-  if (ef >= LT_BAD_EXP) return __longlong_as_double(0x7FF8000000000000ll);
-  return __longlong_as_double((long long)(sign | (field <= 0 ? 0ull : 0x7FF0000000000000ull)));
-}
-
-// the eight levels of 8 rows (TMEM columns c .. c+7 of each level) of this thread's column
-__device__ __forceinline__ void load_levels(uint32_t taddr, float (&v)[8][8]) {
-  uint32_t r[8][8];
-#pragma unroll
-  for (int l = 0; l < 8; ++l)
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-                 : "=r"(r[l][0]), "=r"(r[l][1]), "=r"(r[l][2]), "=r"(r[l][3]), "=r"(r[l][4]), "=r"(r[l][5]),
-                   "=r"(r[l][6]), "=r"(r[l][7])
-                 : "r"(taddr + (uint32_t)(l * LT_TR)));
-  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-  for (int l = 0; l < 8; ++l)
-#pragma unroll
-    for (int j = 0; j < 8; ++j) v[l][j] = __uint_as_float(r[l][j]);
+  const unsigned long long sg = (unsigned long long)(v >> 63);
+  const unsigned long long mag = ((unsigned long long)v ^ sg) - sg;
+  const int lz = __clzll((long long)(mag | 1ull));
+  return dig::from_fixed(mag, lz, ef - 1015 - lz, ~sg & 0x8000000000000000ull, odd);
 }
 
 // Tensor-core state of a CTA, the same in every thread: bit b of phase is the parity of
@@ -728,8 +690,24 @@ __device__ __forceinline__ bool lt_trailing(LtShared& sh, double* __restrict__ A
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int q = warp & 3, h = warp >> 2;
   unsigned char *da = dig, *db = dig + LT_A_BYTES;
-  const uint32_t ua = tc::smem_u32(da), ub = tc::smem_u32(db);
+  const uint64_t ua = tc::desc_kmajor(tc::smem_u32(da), 128, 512), ub = tc::desc_kmajor(tc::smem_u32(db), 128, 512);
   const int ksteps = nb > 16 ? 2 : 1;
+  // L21 rows are staged by lane = row and eight of the panel's columns; the next 64 rows
+  // are requested while the current ones are worked on
+  const int srow = 8 * warp + (lane & 7), sk8 = lane >> 3;
+  double x[8];
+  auto fetch = [&](int row) {
+#pragma unroll
+    for (int i = 0; i < 8; i += 2) {
+      const int k = 8 * sk8 + i;
+      double2 t = make_double2(0.0, 0.0);
+      if (row < n && k + 1 < nb) t = *reinterpret_cast<const double2*>(A + (int64_t)row * ld + kb + k);
+      else if (row < n && k < nb) t.x = A[(int64_t)row * ld + kb + k];
+      x[i] = t.x;
+      x[i + 1] = t.y;
+    }
+  };
+  fetch(r0 + srow);
   for (int ct = c0; ct < ncol; ct += LT_TC) {
     {
       // U12 columns ct .. ct+127: thread = column (and half of the panel's rows)
@@ -757,27 +735,17 @@ __device__ __forceinline__ bool lt_trailing(LtShared& sh, double* __restrict__ A
     int ecol = 0;                                    // set after the first barrier below
     for (int rb = r0; rb < n; rb += LT_RB) {
       {
-        // L21 rows rb .. rb+63: lane = row and eight of the panel's columns
-        const int rr = 8 * warp + (lane & 7), k8 = lane >> 3, row = rb + rr;
-        double x[8];
         int em = 0;
 #pragma unroll
-        for (int i = 0; i < 8; i += 2) {
-          const int k = 8 * k8 + i;
-          double2 t = make_double2(0.0, 0.0);
-          if (row < n && k + 1 < nb) t = *reinterpret_cast<const double2*>(A + (int64_t)row * ld + kb + k);
-          else if (row < n && k < nb) t.x = A[(int64_t)row * ld + kb + k];
-          x[i] = t.x;
-          x[i + 1] = t.y;
-          em = max(em, max(exponent_of(t.x), exponent_of(t.y)));
-        }
+        for (int i = 0; i < 8; ++i) em = max(em, exponent_of(x[i]));
         em = max(em, __shfl_xor_sync(0xffffffffu, em, 8));
         em = max(em, __shfl_xor_sync(0xffffffffu, em, 16));
-        if (k8 == 0) sh.re[rr] = scale_of(em);
+        if (sk8 == 0) sh.re[srow] = scale_of(em);
         split8(x, em, [&](int s, uint4 v) {
-          *reinterpret_cast<uint4*>(db + (rr >> 4) * LT_GROUP + s * (LT_TR * LT_NB * 2) +
-                                    tc::core_off16(rr & 15, 8 * k8)) = v;
+          *reinterpret_cast<uint4*>(db + (srow >> 4) * LT_GROUP + s * (LT_TR * LT_NB * 2) +
+                                    tc::core_off16(srow & 15, 8 * sk8)) = v;
         });
+        fetch((rb + LT_RB < n ? rb + LT_RB : r0) + srow);
       }
       tc::fence_proxy_async();
       __syncthreads();
@@ -793,7 +761,7 @@ __device__ __forceinline__ bool lt_trailing(LtShared& sh, double* __restrict__ A
         const int b = g & 1;
         if (g + 1 < ng) {        // the other accumulator set was read before the last barrier
           if (tid == 0) {
-            lt_issue(tcs->tmem + (uint32_t)((b ^ 1) * LT_LVL_COLS), ua, ub + (g + 1) * LT_GROUP, ksteps);
+            lt_issue(tcs->tmem + (uint32_t)((b ^ 1) * LT_LVL_COLS), ua, ub + (uint64_t)((g + 1) * (LT_GROUP >> 4)), ksteps);
             tc::mma_commit(tcs->mbar + (b ^ 1));
           }
           tcs->pending |= 1u << (b ^ 1);
@@ -808,11 +776,24 @@ __device__ __forceinline__ bool lt_trailing(LtShared& sh, double* __restrict__ A
         if (ok) {
           tc::fence_after_sync();
           float t[8][8];
-          load_levels(tcs->tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(b * LT_LVL_COLS + 8 * h), t);
+          dig::load_levels(tcs->tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(b * LT_LVL_COLS + 8 * h), LT_TR, t);
+          unsigned odds = 0;
+          double d[8];
 #pragma unroll
           for (int i = 0; i < 8; ++i) {
             const float lv[8] = {t[0][i], t[1][i], t[2][i], t[3][i], t[4][i], t[5][i], t[6][i], t[7][i]};
-            a[i] += join_levels(lv, ecol + sh.re[LT_TR * g + 8 * h + i]);
+            bool odd;
+            d[i] = join_levels(lv, ecol + sh.re[LT_TR * g + 8 * h + i], odd);
+            odds |= odd ? 1u << i : 0u;
+          }
+          if (odds) {
+#pragma unroll
+            for (int i = 0; i < 8; ++i)
+              if ((odds >> i) & 1u) d[i] = dig::special(d[i], ecol + sh.re[LT_TR * g + 8 * h + i]);
+          }
+#pragma unroll
+          for (int i = 0; i < 8; ++i) {
+            a[i] += d[i];
             if (col < ncol && row0 + i < n) {
               dst[(int64_t)i * ld] = a[i];
               bad |= row0 + i >= nu && col >= nu && exponent_of(a[i]) == 0x7ff;
