@@ -375,10 +375,24 @@ static int alloc_group(iedg_mesh* M, cudaStream_t st) {
   CUDA_TRY(upload(M, &M->ref.L1, R.L1, st));
   CUDA_TRY(upload(M, &M->ref.dL1, R.dL1, st));
   CUDA_TRY(upload(M, &M->ref.LQ, R.LQ, st));
+  // operands of the FP64 assembly's tensor-core form (mixed forms of mixed orders have no
+  // FP64 assembly)
+  const bool dg = assemble_dg_supported(dm) && (M->precision == IEDG_PRECISION_FP64 || M->tt.nb == nullptr);
+  std::vector<unsigned char> vdig;
+  std::vector<int> vexp;
+  if (dg) {
+    assemble_dg_table(dm, R.PhiF, R.Dxi, vdig, vexp, &M->ref.Vwindow);
+    CUDA_TRY(upload(M, &M->ref.Vdig, vdig, st));
+    CUDA_TRY(upload(M, &M->ref.Vexp, vexp, st));
+  }
   CUDA_TRY(cudaStreamSynchronize(st));
 
   const size_t d = dm.d, Np = dm.Np, Nq = dm.Nq, Nb = dm.Nb, Nfp = dm.Nfp, m = dm.m;
   Geo& G = M->geo;
+  if (dg) {
+    CUDA_TRY(dalloc(M, &G.elift, E * 2 * d * (Np + Nb)));
+    CUDA_TRY(dalloc(M, &M->pj.ecoef, E * m * m * 9));
+  }
   CUDA_TRY(dalloc(M, &G.wdet, E * Nq));
   CUDA_TRY(dalloc(M, &G.Jinv, E * Nq * d * d));
   CUDA_TRY(dalloc(M, &G.fw, E * Nfp));
@@ -467,6 +481,7 @@ static int run_geometry(iedg_mesh* M, const double* node_xyz, cudaStream_t st) {
   if (e1 != cudaSuccess) { cudaFree(X); CUDA_TRY(e1); }
   cudaError_t e2 = cudaMemcpyAsync(X, node_xyz, E * Np * d * sizeof(double), cudaMemcpyHostToDevice, st);
   if (e2 == cudaSuccess) e2 = launch_geometry(M, X, scratch, st);
+  if (e2 == cudaSuccess && G.elift) e2 = launch_lift_exp(M, st);
   if (e2 == cudaSuccess && M->precision == IEDG_PRECISION_MIXED) {
     const std::pair<const double*, float*> cv[] = {
         {G.Mass, G.Mass32}, {G.GlV, G.GlV32}, {G.HlV, G.HlV32}, {G.GlF, G.GlF32}, {G.HlF, G.HlF32},

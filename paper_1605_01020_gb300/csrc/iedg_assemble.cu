@@ -1469,7 +1469,7 @@ AsmTab<float> tables32(const iedg_mesh* M) {
 
 cudaError_t launch_assemble_list(iedg_mesh* M, double* S, const int64_t* elist, int64_t n_slots, cudaStream_t st) {
   const Dims& dm = M->dm;
-  if (assemble_sf_supported(dm)) return launch_assemble_sf_list(M, S, elist, n_slots, st);
+  if (assemble_dg_supported(dm)) return launch_assemble_dg(M, S, elist, n_slots, st);
   AsmCfg cf = asm_cfg(dm);
   int inner = 1;
   for (int r = 0; r < dm.d; ++r) inner *= dm.p - 1;

@@ -1,5 +1,6 @@
-// Element block assembly for hexahedra with sum-factorised volume terms (FP64 for
-// the FP64 path, FP32 for the mixed path).
+// Element block assembly for hexahedra: in FP32 (mixed path) with sum-factorised volume
+// terms; in FP64 the face and mass terms only, the volume terms being added on the
+// tensor cores afterwards (iedg_assemble_dg.cu).
 //
 // Same element matrix as k_assemble (iedg_assemble.cu): for equation component i
 // and unknown component k the u-rows are
@@ -31,10 +32,13 @@ template <class T, int CC>
 size_t sf_smem(const Dims& dm, bool mix) {
   const int nq1 = dm.nq1, np1 = dm.np1, d = 3;
   const int nbu = dm.Np - (np1 - 2) * (np1 - 2) * (np1 - 2);
-  size_t n = 2 * (size_t)nq1 * np1                                   // L, L'
-             + (size_t)(1 + d) * d * dm.Nq + (size_t)(2 + d) * dm.Nfp  // pair coefficients
-             + 3 * (size_t)dm.Nq * CC + 3 * (size_t)nq1 * nq1 * np1 * CC + 2 * (size_t)nq1 * np1 * np1 * CC;
-  if (!mix && sizeof(T) == 4)   // the six faces' node sums
+  size_t n = 2 * (size_t)nq1 * np1 + (size_t)(2 + d) * dm.Nfp;       // L, L', face coefficients of the pair
+  if (sizeof(T) == 4)           // volume coefficients and stages
+    n += (size_t)(1 + d) * d * dm.Nq + 3 * (size_t)dm.Nq * CC + 3 * (size_t)nq1 * nq1 * np1 * CC +
+         2 * (size_t)nq1 * np1 * np1 * CC;
+  else if (!mix)                // the six faces' stages
+    n += 6 * (size_t)(dm.Nfq + nq1 * np1) * CC;
+  if (!mix)                     // the six faces' node sums
     n += (size_t)6 * np1 * np1 * CC;
   else                          // facc, Vf, Uf; with mixed orders a wider Uf, tacc and LQ
     n += (size_t)nbu * CC + (size_t)dm.Nfq * CC + (size_t)nq1 * (mix ? 5 : np1) * CC +
@@ -67,10 +71,10 @@ __device__ __forceinline__ T face_sum(const T* fn, int a, int c) {
 // group instead of one load per multiply-add.  Face terms are contracted by two 1D
 // stages over the face's tangential directions (face point gf = g1 + nq1 g2, face
 // node tn = a1 + np1 a2, the face-normal factor of the basis being 1 on the face).
-template <class T, int NP1, int NQ1, int CC, bool MIX, bool LIST = false>
+template <class T, int NP1, int NQ1, int CC, bool MIX>
 __global__ void __launch_bounds__(SF_THREADS)
 k_assemble_sf(Dims dm, Phys ph, RefTables ref, AsmTab<T> tb, T* __restrict__ S, const double* __restrict__ rhs64,
-              TraceTab tt, const int64_t* __restrict__ elist) {
+              TraceTab tt) {
   extern __shared__ __align__(16) unsigned char smraw[];
   T* sm = reinterpret_cast<T*>(smraw);
   const int tid = threadIdx.x;
@@ -80,18 +84,10 @@ k_assemble_sf(Dims dm, Phys ph, RefTables ref, AsmTab<T> tb, T* __restrict__ S, 
   constexpr int NbU = Np - (NP1 - 2) * (NP1 - 2) * (NP1 - 2), Nfp = 6 * Nfq;
   constexpr int TS = nq1 * nq1 * np1, VS = nq1 * np1 * np1, NC = (1 + d) * d;
   constexpr int UW = MIX ? 5 : np1;              // second extent of the face stage buffer
-  // FP32 on uniform meshes: the six faces' stages run together (3 barriers per column
-  // chunk instead of 18; measured faster in FP32, slower in FP64, whose DFMA pipe is
-  // the bound there)
-  constexpr bool SIX = !MIX && sizeof(T) == 4;
-  // with an element list (FP64 fallback of the mixed path) CTA group `slot` assembles
-  // element elist[slot] into matrix slot `slot`
-  const int64_t slot = blockIdx.x / m2;
-  int64_t e = slot;
-  if constexpr (LIST) {
-    e = elist[slot];
-    if (e < 0) return;
-  }
+  // uniform meshes: the six faces' stages run together (3 barriers per column chunk
+  // instead of 18)
+  constexpr bool SIX = !MIX, VOL = sizeof(T) == 4;
+  const int64_t e = blockIdx.x / m2;
   const int pair = blockIdx.x % m2, i = pair / m, k = pair % m;
   const bool has_cq = !(i == 0 || (i <= d && k == m - 1));
   const int Nb = MIX ? tt.nb[e] : NbU;          // trace slots of this element
@@ -101,19 +97,19 @@ k_assemble_sf(Dims dm, Phys ph, RefTables ref, AsmTab<T> tb, T* __restrict__ S, 
   T* sL = sm;                                  // [nq1][np1]
   T* sdL = sL + nq1 * np1;                     // [nq1][np1]
   T* cV = sdL + nq1 * np1;                     // [NC][Nq]   cu_r (c < d), cq_lr (c = d + l d + r)
-  T* cF = cV + NC * Nq;                        // [1+d][Nfp] fuh, fq_l
+  T* cF = cV + (VOL ? NC * Nq : 0);            // [1+d][Nfp] fuh, fq_l
   T* cL = cF + (1 + d) * Nfp;                  // [Nfp]      lambda wf (diagonal pairs)
-  T* W = cL + Nfp;                             // [3][Nq][CC]
-  T* Tt = W + 3 * Nq * CC;                     // [3][TS][CC]
-  T* V = Tt + 3 * TS * CC;                     // [2][VS][CC]
+  T* W = cL + Nfp;                             // [3][Nq][CC], and the six faces' stages
+  T* Tt = W + (VOL ? 3 * Nq : (SIX ? 6 * (Nfq + nq1 * np1) : 0)) * CC;   // [3][TS][CC] (VOL)
+  T* V = Tt + (VOL ? 3 * TS * CC : 0);         // [2][VS][CC] (VOL)
   // face parts of the boundary u-rows (and trace rows): accumulated face by face in
   // facc (tacc), or with SIX the six faces' node sums fn[f][tn][c] formed together
-  T* facc = V + 2 * VS * CC;                   // [NbU][CC]
+  T* facc = V + (VOL ? 2 * VS * CC : 0);       // [NbU][CC]
   T* Vf = facc + NbU * CC;                     // [Nfq][CC]
   T* Uf = Vf + Nfq * CC;                       // [nq1 UW][CC]
   T* tacc = MIX ? Uf + nq1 * UW * CC : facc;   // [Nb][CC]   trace rows (MIX), else = facc
   T* sLQ = tacc + (MIX ? dm.Nb * CC : 0);      // [5][nq1][5] (MIX)
-  T* fn = V + 2 * VS * CC;                     // [6][Nfn][CC] (SIX)
+  T* fn = facc;                                // [6][Nfn][CC] (SIX)
   for (int idx = tid; idx < nq1 * np1; idx += SF_THREADS) { sL[idx] = (T)ref.L1[idx]; sdL[idx] = (T)ref.dL1[idx]; }
   if (MIX) {
     const T* lq = nullptr;
@@ -133,7 +129,7 @@ k_assemble_sf(Dims dm, Phys ph, RefTables ref, AsmTab<T> tb, T* __restrict__ S, 
   // The pair's point coefficients (two contiguous blocks of the point-Jacobian tables)
   // are staged by one thread with two bulk copies on the TMA engine while the others
   // fill the remaining tables; plain loads where an address is not 16-byte aligned.
-  constexpr uint32_t bytesV = NC * Nq * sizeof(T), bytesF = (1 + d) * Nfp * sizeof(T);
+  constexpr uint32_t bytesV = VOL ? NC * Nq * sizeof(T) : 0, bytesF = (1 + d) * Nfp * sizeof(T);
   static_assert(bytesV % 16 == 0 && bytesF % 16 == 0 && (2 * nq1 * np1 * sizeof(T)) % 16 == 0,
                 "bulk copies need 16-byte sizes and offsets");
   __shared__ __align__(8) uint64_t stage_bar;
@@ -143,11 +139,11 @@ k_assemble_sf(Dims dm, Phys ph, RefTables ref, AsmTab<T> tb, T* __restrict__ S, 
     if (tid == 0) {
       tc::mbar_init(&stage_bar, 1);
       tc::mbar_expect_tx(&stage_bar, bytesV + bytesF);
-      tc::bulk_g2s(cV, jv, bytesV, &stage_bar);
+      if constexpr (VOL) tc::bulk_g2s(cV, jv, bytesV, &stage_bar);
       tc::bulk_g2s(cF, jf, bytesF, &stage_bar);
     }
   } else {
-    for (int idx = tid; idx < NC * Nq; idx += SF_THREADS) cV[idx] = jv[idx];
+    for (int idx = tid; VOL && idx < NC * Nq; idx += SF_THREADS) cV[idx] = jv[idx];
     for (int idx = tid; idx < (1 + d) * Nfp; idx += SF_THREADS) cF[idx] = jf[idx];
   }
   // dfhat/du of the pair: lambda wf on the diagonal (Lax-Friedrichs) or wf S_ik (Roe-type)
@@ -161,7 +157,7 @@ k_assemble_sf(Dims dm, Phys ph, RefTables ref, AsmTab<T> tb, T* __restrict__ S, 
   const T alpha = (T)ph.alpha;
   const int64_t nn = MIX ? (int64_t)dm.nu + (int64_t)m * Nb : dm.n;
   const int64_t ld = MIX ? tt.ldv[e] : dm.ld;
-  T* Se = MIX ? S + tt.soff[e] : S + (LIST ? slot : e) * nn * ld;
+  T* Se = MIX ? S + tt.soff[e] : S + e * nn * ld;
   if (rhs64 != nullptr && pair == 0)
     for (int r = tid; r < nn; r += SF_THREADS) Se[r * ld + nn] = (T)rhs64[e * dm.n + r];
   __syncthreads();     // also publishes the barrier's initialisation
@@ -169,7 +165,7 @@ k_assemble_sf(Dims dm, Phys ph, RefTables ref, AsmTab<T> tb, T* __restrict__ S, 
   if (bulk) {
     late = !__syncthreads_and(tc::mbar_wait(&stage_bar, 0, kTcWaitLimit));
     if (late) {        // same values by plain loads (a late copy writes the same bytes)
-      for (int idx = tid; idx < NC * Nq; idx += SF_THREADS) cV[idx] = jv[idx];
+      for (int idx = tid; VOL && idx < NC * Nq; idx += SF_THREADS) cV[idx] = jv[idx];
       for (int idx = tid; idx < (1 + d) * Nfp; idx += SF_THREADS) cF[idx] = jf[idx];
       __syncthreads();
     }
@@ -182,7 +178,7 @@ k_assemble_sf(Dims dm, Phys ph, RefTables ref, AsmTab<T> tb, T* __restrict__ S, 
       // stages; the first two live in the volume buffer W, free until the volume stage
       T* Vf6 = W;                              // [6][Nfq][CC]
       T* Uf6 = W + 6 * Nfq * CC;               // [6][nq1][np1][CC]
-      static_assert(6 * (Nfq + nq1 * np1) <= 3 * Nq, "face stages must fit the volume buffer");
+      static_assert(!VOL || 6 * (Nfq + nq1 * np1) <= 3 * Nq, "face stages must fit the volume buffer");
       for (int idx = tid; idx < 6 * Nfq * CC; idx += SF_THREADS) {
         const int fp = idx / CC, c = idx % CC, col = c0 + c;
         T v = 0;
@@ -320,6 +316,7 @@ k_assemble_sf(Dims dm, Phys ph, RefTables ref, AsmTab<T> tb, T* __restrict__ S, 
       }
     }
     }
+    if constexpr (VOL) {
     // ---- volume right operands W_r[g][c] for the three reference directions.  The
     // table values of all of this thread's (g, c) entries are requested first, then
     // combined, so their latencies overlap instead of adding up.
@@ -402,13 +399,16 @@ k_assemble_sf(Dims dm, Phys ph, RefTables ref, AsmTab<T> tb, T* __restrict__ S, 
       V[(1 * VS + t) * CC + c] = s1;
     }
     __syncthreads();
+    } else {
+      __syncthreads();       // face sums of every thread
+    }
     // stage C: contract g_x and write the u-rows (volume + faces + mass)
     for (int idx = tid; idx < Np * CC; idx += SF_THREADS) {
       const int a = idx / CC, c = idx % CC, col = c0 + c;
       if (col >= ncol_all) continue;
       const int ax = a % np1, ayz = a / np1;
       T s = 0;
-      for (int gx = 0; gx < nq1; ++gx) {
+      for (int gx = 0; VOL && gx < nq1; ++gx) {
         const int t = gx + nq1 * ayz;
         s = fma(sdL[gx * np1 + ax], V[(0 * VS + t) * CC + c], s);
         s = fma(sL[gx * np1 + ax], V[(1 * VS + t) * CC + c], s);
@@ -435,17 +435,17 @@ k_assemble_sf(Dims dm, Phys ph, RefTables ref, AsmTab<T> tb, T* __restrict__ S, 
 }  // namespace
 
 template <class T, int NP1, int NQ1, int CC>
-static cudaError_t assemble_sf_t(iedg_mesh* M, T* S, const double* rhs64, const AsmTab<T>& tb, cudaStream_t st,
-                                 const int64_t* elist, int64_t n_slots) {
+static cudaError_t assemble_sf_t(iedg_mesh* M, T* S, const double* rhs64, const AsmTab<T>& tb, cudaStream_t st) {
   const Dims& dm = M->dm;
   const bool mix = M->tt.nb != nullptr;
   size_t smem = sf_smem<T, CC>(dm, mix);
-  auto kern = elist ? k_assemble_sf<T, NP1, NQ1, CC, false, true>
-                    : (mix ? k_assemble_sf<T, NP1, NQ1, CC, true> : k_assemble_sf<T, NP1, NQ1, CC, false>);
+  // FP64 runs here on meshes with mixed orders only
+  auto kern = k_assemble_sf<T, NP1, NQ1, CC, true>;
+  if constexpr (sizeof(T) == 4)
+    if (!mix) kern = k_assemble_sf<T, NP1, NQ1, CC, false>;
   cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (err != cudaSuccess) return err;
-  const int64_t E = elist ? n_slots : M->E;
-  kern<<<(unsigned)(E * dm.m * dm.m), SF_THREADS, smem, st>>>(dm, M->ph, M->ref, tb, S, rhs64, M->tt, elist);
+  kern<<<(unsigned)(M->E * dm.m * dm.m), SF_THREADS, smem, st>>>(dm, M->ph, M->ref, tb, S, rhs64, M->tt);
   return cudaGetLastError();
 }
 
@@ -453,25 +453,22 @@ static cudaError_t assemble_sf_t(iedg_mesh* M, T* S, const double* rhs64, const 
 // (more CTAs per SM) and 16 for FP32; a chunk whose shared memory does not fit
 // falls back to 8
 template <class T, int NP1, int NQ1>
-static cudaError_t assemble_sf_c(iedg_mesh* M, T* S, const double* rhs64, const AsmTab<T>& tb, cudaStream_t st,
-                                 const int64_t* elist, int64_t n_slots) {
+static cudaError_t assemble_sf_c(iedg_mesh* M, T* S, const double* rhs64, const AsmTab<T>& tb, cudaStream_t st) {
   int cc = M->sched.asm_chunk ? M->sched.asm_chunk : (sizeof(T) == 8 ? 8 : 16);
-  if (sizeof(T) == 8 && M->precision != 0) cc = 8;   // FP64 fallback of a mixed handle: the FP64 default
   const bool mix = M->tt.nb != nullptr;
   if (cc == 32 && sf_smem<T, 32>(M->dm, mix) > 227 * 1024) cc = 16;
   if (cc == 16 && sf_smem<T, 16>(M->dm, mix) > 227 * 1024) cc = 8;
-  if (cc == 32) return assemble_sf_t<T, NP1, NQ1, 32>(M, S, rhs64, tb, st, elist, n_slots);
-  if (cc == 16) return assemble_sf_t<T, NP1, NQ1, 16>(M, S, rhs64, tb, st, elist, n_slots);
-  return assemble_sf_t<T, NP1, NQ1, 8>(M, S, rhs64, tb, st, elist, n_slots);
+  if (cc == 32) return assemble_sf_t<T, NP1, NQ1, 32>(M, S, rhs64, tb, st);
+  if (cc == 16) return assemble_sf_t<T, NP1, NQ1, 16>(M, S, rhs64, tb, st);
+  return assemble_sf_t<T, NP1, NQ1, 8>(M, S, rhs64, tb, st);
 }
 
 template <class T>
-static cudaError_t assemble_sf_p(iedg_mesh* M, T* S, const double* rhs64, const AsmTab<T>& tb, cudaStream_t st,
-                                 const int64_t* elist = nullptr, int64_t n_slots = 0) {
+static cudaError_t assemble_sf_p(iedg_mesh* M, T* S, const double* rhs64, const AsmTab<T>& tb, cudaStream_t st) {
   switch (M->dm.p) {
-    case 2: return assemble_sf_c<T, 3, 4>(M, S, rhs64, tb, st, elist, n_slots);
-    case 3: return assemble_sf_c<T, 4, 5>(M, S, rhs64, tb, st, elist, n_slots);
-    default: return assemble_sf_c<T, 5, 6>(M, S, rhs64, tb, st, elist, n_slots);
+    case 2: return assemble_sf_c<T, 3, 4>(M, S, rhs64, tb, st);
+    case 3: return assemble_sf_c<T, 4, 5>(M, S, rhs64, tb, st);
+    default: return assemble_sf_c<T, 5, 6>(M, S, rhs64, tb, st);
   }
 }
 
@@ -480,12 +477,12 @@ bool assemble_sf_supported(const Dims& dm) {
 }
 
 cudaError_t launch_assemble_sf(iedg_mesh* M, cudaStream_t st) {
-  if (M->precision == 0) return assemble_sf_p<double>(M, M->S, nullptr, tables64(M), st);
-  return assemble_sf_p<float>(M, M->S32, M->rhs64, tables32(M), st);
-}
-
-cudaError_t launch_assemble_sf_list(iedg_mesh* M, double* S, const int64_t* elist, int64_t n_slots, cudaStream_t st) {
-  return assemble_sf_p<double>(M, S, M->rhs64, tables64(M), st, elist, n_slots);
+  if (M->precision != 0) return assemble_sf_p<float>(M, M->S32, M->rhs64, tables32(M), st);
+  if (M->tt.nb != nullptr) {       // mixed orders: face and mass terms here, then the volume terms
+    const cudaError_t err = assemble_sf_p<double>(M, M->S, nullptr, tables64(M), st);
+    if (err != cudaSuccess) return err;
+  }
+  return launch_assemble_dg(M, M->S, nullptr, 0, st);
 }
 
 }  // namespace iedg

@@ -68,6 +68,9 @@ struct RefTables {
   double* LQ;     // [5][nq1][5] degree-q Gauss-Lobatto Lagrange basis at the 1D Gauss points
                   //              (private face nodes of meshes with mixed orders)
   float* LQ32;
+  unsigned char* Vdig;   // digits of PhiF, Dxi in tensor-core operand order (iedg_assemble_dg.cu; null: unused)
+  int* Vexp;             // [128], [128] their lanes' scales
+  int Vwindow;           // chunks of volume points over which the level sums stay exact
   float* Phi32;   // FP32 copies for the mixed path (FP64 -> FP32 conversion is slow on GB300)
   float* Dxi32;
   float* PhiF32;
@@ -86,6 +89,7 @@ struct Geo {
   double* HlV;    // [E][d][Nq][Nb]
   double* GlF;    // [E][d][Nfp][Np]  PhiF Gl  (lifting at face points)
   double* HlF;    // [E][d][Nfp][Nb]
+  int16_t* elift; // [E][6][Np+Nb]  largest exponents of the columns of GlV, HlV; GlF, HlF (null: unused)
   // FP32 copies (mixed path only)
   float *Mass32, *GlV32, *HlV32, *GlF32, *HlF32;
 };
@@ -98,6 +102,7 @@ struct PointJac {
   double* Su;     // [E][m][m][Nfp]        : wf dfhat_i/du_k = wf S_ik (Roe-type only, else null)
   double* Jb;     // [E][m][m][2+d][Nfp]   : boundary faces only: wf dbhat/duhat, wf dbhat/du,
                   //                          wf dbhat/dq_l (null without boundary faces)
+  int16_t* ecoef; // [E][25][9] largest exponents of the pairs' coefficients (null: unused)
   float *Jv32, *Jf32, *lamw32, *Su32, *Jb32;   // FP32 copies written by the point kernel (mixed path only)
 };
 
@@ -251,6 +256,12 @@ cudaError_t launch_rq(iedg_mesh* M, const double* q, const double* qs, double* r
 cudaError_t launch_assemble(iedg_mesh* M, cudaStream_t st);
 cudaError_t launch_assemble_sf(iedg_mesh* M, cudaStream_t st);   // 3D, sum-factorised
 bool assemble_sf_supported(const Dims& dm);
+// FP64 element matrices with their contractions on the tensor cores (iedg_assemble_dg.cu)
+bool assemble_dg_supported(const Dims& dm);
+void assemble_dg_table(const Dims& dm, const std::vector<double>& PhiF, const std::vector<double>& Dxi,
+                       std::vector<unsigned char>& table, std::vector<int>& rexp, int* window);
+cudaError_t launch_lift_exp(iedg_mesh* M, cudaStream_t st);
+cudaError_t launch_assemble_dg(iedg_mesh* M, double* S, const int64_t* elist, int64_t n_slots, cudaStream_t st);
 cudaError_t launch_assemble_col(iedg_mesh* M, cudaStream_t st);  // small elements, a thread per column
 bool assemble_col_supported(const iedg_mesh* M);
 AsmTab<double> tables64(const iedg_mesh* M);
@@ -279,7 +290,6 @@ constexpr int64_t kGmresScratch = (IEDG_MAX_RESTART + 1) * kGmresMaxCtas + 8;
 constexpr int kFallbackSlots = 32;
 cudaError_t launch_fallback(iedg_mesh* M, cudaStream_t st);
 cudaError_t launch_assemble_list(iedg_mesh* M, double* S, const int64_t* elist, int64_t n_slots, cudaStream_t st);
-cudaError_t launch_assemble_sf_list(iedg_mesh* M, double* S, const int64_t* elist, int64_t n_slots, cudaStream_t st);
 cudaError_t launch_lu64_list(iedg_mesh* M, double* S, int64_t n_slots, const int64_t* active, int8_t* status,
                              cudaStream_t st);
 cudaError_t launch_zero_row_fallback(iedg_mesh* M, cudaStream_t st);
