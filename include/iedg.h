@@ -272,8 +272,9 @@ int iedg_trace_solve(iedg_mesh* mesh, const double* K, const double* R, double* 
  *                  per element.
  *   lu_panel:      panel width of the FP64 LU's DFMA form, 16 or 32 (32 falls back to 16
  *                  when the panel does not fit in shared memory).
- *   asm_chunk:     assembly column chunk, 8, 16 or 32 (0 = default: 8 for FP64, 16
- *                  for FP32; too large a chunk for shared memory falls back).
+ *   asm_chunk:     assembly column chunk on meshes with mixed orders, 8, 16 or 32 (0 =
+ *                  default: 8 for FP64, 16 for FP32; too large a chunk for shared
+ *                  memory falls back).  Uniform meshes assemble without chunks.
  *   lu_tensor:     tensor cores (tcgen05, accumulation in tensor memory) in the partial LU.
  *                  FP64 path: the trailing updates as integer products of 8-bit digits of
  *                  the FP64 operands, summed exactly and joined to FP64 (the error of an

@@ -363,6 +363,8 @@ static int alloc_group(iedg_mesh* M, cudaStream_t st) {
   const Dims& dm = M->dm;
   const int64_t E = M->E;
   HostRef R = build_reference(dm);
+  M->L1h = R.L1;
+  M->dL1h = R.dL1;
   CUDA_TRY(upload(M, &M->ref.Phi, R.Phi, st));
   CUDA_TRY(upload(M, &M->ref.Dxi, R.Dxi, st));
   CUDA_TRY(upload(M, &M->ref.Wq, R.Wq, st));
@@ -1100,10 +1102,10 @@ extern "C" int iedg_assemble_condensed(iedg_mesh* M, const double* u, const doub
   // point Jacobians at (u, q) and the right-hand sides F~ = -R_u(u, q*), G~ = -R_FL,e(u, q*)
   // written straight into the last column of the bordered element matrices
   CUDA_TRY(TRACED("points_jacobian", launch_points(M, u, q, M->qstar, uhat, u_ref, true, nullptr, nullptr, st)));
-  if (assemble_sf_supported(dm))
-    CUDA_TRY(TRACED("assemble", launch_assemble_sf(M, st)));
-  else if (assemble_col_supported(M))
+  if (assemble_col_supported(M))
     CUDA_TRY(TRACED("assemble", launch_assemble_col(M, st)));
+  else if (assemble_sf_supported(dm))
+    CUDA_TRY(TRACED("assemble", launch_assemble_sf(M, st)));
   else
     CUDA_TRY(TRACED("assemble", launch_assemble(M, st)));
   if (M->mass_scaled) CUDA_TRY(TRACED("mass_scale", launch_mass_scale(M, st)));

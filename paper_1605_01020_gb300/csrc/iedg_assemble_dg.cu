@@ -67,12 +67,6 @@ struct DgShared {
   int sexp[2][DG_COLS];     // scales (biased exponents): face, volume
 };
 
-// Pairs (i, k) of the column order: 17 whose viscous Jacobian does not vanish identically
-// (their u-columns, then their trace columns), then the 8 others' u-columns and trace
-// columns (the latter have no volume terms).
-__host__ __device__ __forceinline__ int dg_pair_cq(int q) { return q < 12 ? 5 * (1 + q / 4) + q % 4 : 20 + (q - 12); }
-__host__ __device__ __forceinline__ int dg_pair_no(int q) { return q < 5 ? q : 5 * (1 + q - 5) + 4; }
-
 struct DgArgs {
   AsmTab<double> tb;
   RefTables ref;
@@ -206,25 +200,10 @@ __global__ void __launch_bounds__(DG_THREADS, 2) k_assemble_dg(Dims dm, DgArgs a
       int nb, c0, ch1;
       if (!tile_of(id, slot, e, nb, c0, ch1)) continue;
       // this thread's column
-      int fc = c0 + c, pair = -1, col = 0;
-      bool ucol = true, cq = true;
-      const int nA = 17 * Np, nB = 17 * nb, nC = 8 * Np;
-      if (fc < nA) {
-        pair = dg_pair_cq(fc / Np);
-        col = fc % Np;
-      } else if (fc < nA + nB) {
-        pair = dg_pair_cq((fc - nA) / nb);
-        col = (fc - nA) % nb;
-        ucol = false;
-      } else if (fc < nA + nB + nC) {
-        pair = dg_pair_no((fc - nA - nB) / Np);
-        col = (fc - nA - nB) % Np;
-        cq = false;
-      } else if (fc < m2 * (Np + nb)) {
-        pair = dg_pair_no((fc - nA - nB - nC) / nb);
-        col = (fc - nA - nB - nC) % nb;
-        ucol = cq = false;
-      }
+      const HexCol hc = hex_col(c0 + c, Np, nb);
+      const int col = hc.col;
+      const bool ucol = hc.u, cq = hc.cq;
+      int pair = hc.pair;
       const bool on = pair >= 0;
       if (!on) pair = 0;
       const int pi = pair / 5, pk = pair % 5, gst = ucol ? Np : NbT;

@@ -1,6 +1,7 @@
-// Element block assembly for hexahedra: in FP32 (mixed path) with sum-factorised volume
-// terms; in FP64 the face and mass terms only, the volume terms being added on the
-// tensor cores afterwards (iedg_assemble_dg.cu).
+// Element block assembly for hexahedra on meshes with mixed orders: in FP32 (mixed path)
+// with sum-factorised volume terms; in FP64 the face and mass terms only, the volume terms
+// being added on the tensor cores afterwards (iedg_assemble_dg.cu).  Uniform meshes:
+// iedg_assemble_col.cu (FP32), iedg_assemble_dg.cu (FP64).
 //
 // Same element matrix as k_assemble (iedg_assemble.cu): for equation component i
 // and unknown component k the u-rows are
@@ -14,12 +15,11 @@
 // mass equation, and momentum equations with respect to the energy unknown) have no
 // volume trace columns and skip the lifted-gradient terms.
 //
-// Meshes with mixed orders (MIX): the element has n_b,e trace slots and its matrix sits
-// at its own offset with its own leading dimension.  The trace basis on a face shared
-// with the same order is the element basis there (trace rows = face parts of the
-// boundary u-rows restricted to those faces); a face with private nodes of degree q
-// has the degree-q Gauss-Lobatto Lagrange basis, contracted in two 1D stages like the
-// element basis.
+// The element has n_b,e trace slots and its matrix sits at its own offset with its own
+// leading dimension.  The trace basis on a face shared with the same order is the element
+// basis there (trace rows = face parts of the boundary u-rows restricted to those faces);
+// a face with private nodes of degree q has the degree-q Gauss-Lobatto Lagrange basis,
+// contracted in two 1D stages like the element basis.
 #include "iedg_internal.cuh"
 #include "iedg_tc.cuh"
 
@@ -29,39 +29,16 @@ namespace {
 constexpr int SF_THREADS = 256;
 
 template <class T, int CC>
-size_t sf_smem(const Dims& dm, bool mix) {
+size_t sf_smem(const Dims& dm) {
   const int nq1 = dm.nq1, np1 = dm.np1, d = 3;
   const int nbu = dm.Np - (np1 - 2) * (np1 - 2) * (np1 - 2);
   size_t n = 2 * (size_t)nq1 * np1 + (size_t)(2 + d) * dm.Nfp;       // L, L', face coefficients of the pair
   if (sizeof(T) == 4)           // volume coefficients and stages
     n += (size_t)(1 + d) * d * dm.Nq + 3 * (size_t)dm.Nq * CC + 3 * (size_t)nq1 * nq1 * np1 * CC +
          2 * (size_t)nq1 * np1 * np1 * CC;
-  else if (!mix)                // the six faces' stages
-    n += 6 * (size_t)(dm.Nfq + nq1 * np1) * CC;
-  if (!mix)                     // the six faces' node sums
-    n += (size_t)6 * np1 * np1 * CC;
-  else                          // facc, Vf, Uf; with mixed orders a wider Uf, tacc and LQ
-    n += (size_t)nbu * CC + (size_t)dm.Nfq * CC + (size_t)nq1 * (mix ? 5 : np1) * CC +
-         (mix ? (size_t)dm.Nb * CC + 25 * (size_t)nq1 : 0);
+  // facc, Vf, Uf, tacc and LQ
+  n += (size_t)nbu * CC + (size_t)dm.Nfq * CC + (size_t)nq1 * 5 * CC + (size_t)dm.Nb * CC + 25 * (size_t)nq1;
   return n * sizeof(T);
-}
-
-// Face part of boundary node a for column c from the six faces' node sums fn[f][tn][c]:
-// node a = (a0, a1, a2) lies on face 2r where its coordinate r is 0 and on face 2r + 1
-// where it is p; its index on that face runs over the two other coordinates in order.
-// The faces are summed in increasing order, as the face-by-face accumulation does.
-template <class T, int NP1, int CC>
-__device__ __forceinline__ T face_sum(const T* fn, int a, int c) {
-  const int c3[3] = {a % NP1, (a / NP1) % NP1, a / (NP1 * NP1)};
-  T fs = 0;
-#pragma unroll
-  for (int f = 0; f < 6; ++f) {
-    const int r = f >> 1;
-    if (c3[r] != ((f & 1) ? NP1 - 1 : 0)) continue;
-    const int tn = r == 0 ? c3[1] + NP1 * c3[2] : (r == 1 ? c3[0] + NP1 * c3[2] : c3[0] + NP1 * c3[1]);
-    fs += fn[(f * NP1 * NP1 + tn) * CC + c];
-  }
-  return fs;
 }
 
 // Element sizes are compile-time constants (NP1 = p + 1, NQ1 = p + 2), so every index
@@ -71,7 +48,7 @@ __device__ __forceinline__ T face_sum(const T* fn, int a, int c) {
 // group instead of one load per multiply-add.  Face terms are contracted by two 1D
 // stages over the face's tangential directions (face point gf = g1 + nq1 g2, face
 // node tn = a1 + np1 a2, the face-normal factor of the basis being 1 on the face).
-template <class T, int NP1, int NQ1, int CC, bool MIX>
+template <class T, int NP1, int NQ1, int CC>
 __global__ void __launch_bounds__(SF_THREADS)
 k_assemble_sf(Dims dm, Phys ph, RefTables ref, AsmTab<T> tb, T* __restrict__ S, const double* __restrict__ rhs64,
               TraceTab tt) {
@@ -83,15 +60,13 @@ k_assemble_sf(Dims dm, Phys ph, RefTables ref, AsmTab<T> tb, T* __restrict__ S, 
   constexpr int Np = NP1 * NP1 * NP1, Nq = NQ1 * NQ1 * NQ1, Nfq = NQ1 * NQ1, Nfn = NP1 * NP1;
   constexpr int NbU = Np - (NP1 - 2) * (NP1 - 2) * (NP1 - 2), Nfp = 6 * Nfq;
   constexpr int TS = nq1 * nq1 * np1, VS = nq1 * np1 * np1, NC = (1 + d) * d;
-  constexpr int UW = MIX ? 5 : np1;              // second extent of the face stage buffer
-  // uniform meshes: the six faces' stages run together (3 barriers per column chunk
-  // instead of 18)
-  constexpr bool SIX = !MIX, VOL = sizeof(T) == 4;
+  constexpr int UW = 5;                          // second extent of the face stage buffer
+  constexpr bool VOL = sizeof(T) == 4;
   const int64_t e = blockIdx.x / m2;
   const int pair = blockIdx.x % m2, i = pair / m, k = pair % m;
   const bool has_cq = !(i == 0 || (i <= d && k == m - 1));
-  const int Nb = MIX ? tt.nb[e] : NbU;          // trace slots of this element
-  const int NbT = MIX ? dm.Nb : NbU;            // slot stride of the lifting tables
+  const int Nb = tt.nb[e];         // trace slots of this element
+  const int NbT = dm.Nb;                        // slot stride of the lifting tables
   const int ncol_all = Np + Nb;
   const int ncol_vol = has_cq ? Np + Nb : Np;
   T* sL = sm;                                  // [nq1][np1]
@@ -99,26 +74,24 @@ k_assemble_sf(Dims dm, Phys ph, RefTables ref, AsmTab<T> tb, T* __restrict__ S, 
   T* cV = sdL + nq1 * np1;                     // [NC][Nq]   cu_r (c < d), cq_lr (c = d + l d + r)
   T* cF = cV + (VOL ? NC * Nq : 0);            // [1+d][Nfp] fuh, fq_l
   T* cL = cF + (1 + d) * Nfp;                  // [Nfp]      lambda wf (diagonal pairs)
-  T* W = cL + Nfp;                             // [3][Nq][CC], and the six faces' stages
-  T* Tt = W + (VOL ? 3 * Nq : (SIX ? 6 * (Nfq + nq1 * np1) : 0)) * CC;   // [3][TS][CC] (VOL)
+  T* W = cL + Nfp;                             // [3][Nq][CC] (VOL)
+  T* Tt = W + (VOL ? 3 * Nq * CC : 0);         // [3][TS][CC] (VOL)
   T* V = Tt + (VOL ? 3 * TS * CC : 0);         // [2][VS][CC] (VOL)
-  // face parts of the boundary u-rows (and trace rows): accumulated face by face in
-  // facc (tacc), or with SIX the six faces' node sums fn[f][tn][c] formed together
+  // face parts of the boundary u-rows and the trace rows, accumulated face by face
   T* facc = V + (VOL ? 2 * VS * CC : 0);       // [NbU][CC]
   T* Vf = facc + NbU * CC;                     // [Nfq][CC]
   T* Uf = Vf + Nfq * CC;                       // [nq1 UW][CC]
-  T* tacc = MIX ? Uf + nq1 * UW * CC : facc;   // [Nb][CC]   trace rows (MIX), else = facc
-  T* sLQ = tacc + (MIX ? dm.Nb * CC : 0);      // [5][nq1][5] (MIX)
-  T* fn = facc;                                // [6][Nfn][CC] (SIX)
+  T* tacc = Uf + nq1 * UW * CC;                // [Nb][CC]   trace rows
+  T* sLQ = tacc + dm.Nb * CC;                  // [5][nq1][5]
   for (int idx = tid; idx < nq1 * np1; idx += SF_THREADS) { sL[idx] = (T)ref.L1[idx]; sdL[idx] = (T)ref.dL1[idx]; }
-  if (MIX) {
+  {
     const T* lq = nullptr;
     if constexpr (sizeof(T) == 8) lq = reinterpret_cast<const T*>(ref.LQ);
     else lq = reinterpret_cast<const T*>(ref.LQ32);
     for (int idx = tid; idx < 25 * nq1; idx += SF_THREADS) sLQ[idx] = lq[idx];
   }
   const T* mutab = nullptr;                    // [nf][Nfq][NFS] of this element (MIX)
-  if (MIX) {
+  {
     if constexpr (sizeof(T) == 8) mutab = reinterpret_cast<const T*>(tt.muf);
     else mutab = reinterpret_cast<const T*>(tt.muf32);
     mutab += (size_t)e * 6 * Nfq * tt.NFS;
@@ -155,9 +128,9 @@ k_assemble_sf(Dims dm, Phys ph, RefTables ref, AsmTab<T> tb, T* __restrict__ S, 
   const T* HlF = tb.HlF + (size_t)e * d * Nfp * NbT;
   const T* Ms = tb.Mass + (size_t)e * Np * Np;
   const T alpha = (T)ph.alpha;
-  const int64_t nn = MIX ? (int64_t)dm.nu + (int64_t)m * Nb : dm.n;
-  const int64_t ld = MIX ? tt.ldv[e] : dm.ld;
-  T* Se = MIX ? S + tt.soff[e] : S + e * nn * ld;
+  const int64_t nn = (int64_t)dm.nu + (int64_t)m * Nb;
+  const int64_t ld = tt.ldv[e];
+  T* Se = S + tt.soff[e];
   if (rhs64 != nullptr && pair == 0)
     for (int r = tid; r < nn; r += SF_THREADS) Se[r * ld + nn] = (T)rhs64[e * dm.n + r];
   __syncthreads();     // also publishes the barrier's initialisation
@@ -173,53 +146,11 @@ k_assemble_sf(Dims dm, Phys ph, RefTables ref, AsmTab<T> tb, T* __restrict__ S, 
 
   for (int c0 = 0; c0 < ncol_all; c0 += CC) {
     // ---- face parts of the boundary rows for this column chunk
-    if constexpr (SIX) {
-      // all six faces per phase: right operand at the face points, then the two 1D
-      // stages; the first two live in the volume buffer W, free until the volume stage
-      T* Vf6 = W;                              // [6][Nfq][CC]
-      T* Uf6 = W + 6 * Nfq * CC;               // [6][nq1][np1][CC]
-      static_assert(!VOL || 6 * (Nfq + nq1 * np1) <= 3 * Nq, "face stages must fit the volume buffer");
-      for (int idx = tid; idx < 6 * Nfq * CC; idx += SF_THREADS) {
-        const int fp = idx / CC, c = idx % CC, col = c0 + c;
-        T v = 0;
-        if (col < Np) {
-          v = cL[fp] * tb.PhiF[(size_t)fp * Np + col];
-          if (has_cq)
-            for (int l = 0; l < d; ++l) v -= cF[(1 + l) * Nfp + fp] * GlF[((size_t)l * Nfp + fp) * Np + col];
-        } else if (col < ncol_all) {
-          const int t = col - Np;
-          v = cF[fp] * tb.PhiF[(size_t)fp * Np + ref.bnode[t]];
-          if (has_cq)
-            for (int l = 0; l < d; ++l) v += cF[(1 + l) * Nfp + fp] * HlF[((size_t)l * Nfp + fp) * NbT + t];
-        }
-        Vf6[idx] = v;
-      }
-      __syncthreads();
-      // U[f][g1][a2] = sum_g2 L[g2][a2] Vf[f][g1 + nq1 g2]
-      for (int idx = tid; idx < 6 * nq1 * np1 * CC; idx += SF_THREADS) {
-        const int c = idx % CC, t = idx / CC, f = t / (nq1 * np1), g1 = (t / np1) % nq1, a2 = t % np1;
-        T u = 0;
-        for (int g2 = 0; g2 < nq1; ++g2) u = fma(sL[g2 * np1 + a2], Vf6[(f * Nfq + g1 + nq1 * g2) * CC + c], u);
-        Uf6[idx] = u;
-      }
-      __syncthreads();
-      // node (a1, a2) of face f: sum_g1 L[g1][a1] U[f][g1][a2]
-      for (int idx = tid; idx < 6 * Nfn * CC; idx += SF_THREADS) {
-        const int c = idx % CC, t = idx / CC, f = t / Nfn, tn = t % Nfn, a1 = tn % np1, a2 = tn / np1;
-        T sacc = 0;
-        for (int g1 = 0; g1 < nq1; ++g1)
-          sacc = fma(sL[g1 * np1 + a1], Uf6[((f * nq1 + g1) * np1 + a2) * CC + c], sacc);
-        fn[idx] = sacc;
-      }
-      __syncthreads();
-    }
-    if constexpr (!SIX) {
     for (int idx = tid; idx < NbU * CC; idx += SF_THREADS) facc[idx] = (T)0;
-    if (MIX)
       for (int idx = tid; idx < Nb * CC; idx += SF_THREADS) tacc[idx] = (T)0;
     for (int f = 0; f < 6; ++f) {
-      const int fq = MIX ? tt.fdeg[e * 6 + f] : 0;
-      const int* fsf = MIX ? tt.fs + ((size_t)e * 6 + f) * tt.NFS : nullptr;
+      const int fq = tt.fdeg[e * 6 + f];
+      const int* fsf = tt.fs + ((size_t)e * 6 + f) * tt.NFS;
       __syncthreads();
       for (int idx = tid; idx < Nfq * CC; idx += SF_THREADS) {
         const int gf = idx / CC, c = idx % CC, col = c0 + c;
@@ -232,15 +163,11 @@ k_assemble_sf(Dims dm, Phys ph, RefTables ref, AsmTab<T> tb, T* __restrict__ S, 
         } else if (col < ncol_all) {
           const int t = col - Np;
           T mu = 0;
-          if (MIX) {
-            const int* fl = tt.sfl + ((size_t)e * dm.Nb + t) * 3;
+          const int* fl = tt.sfl + ((size_t)e * dm.Nb + t) * 3;
 #pragma unroll
-            for (int q = 0; q < 3; ++q) {
-              const int code = fl[q];
-              if (code >= 0 && code / tt.NFS == f) mu = mutab[((size_t)f * Nfq + gf) * tt.NFS + code % tt.NFS];
-            }
-          } else {
-            mu = tb.PhiF[(size_t)fp * Np + ref.bnode[t]];
+          for (int q = 0; q < 3; ++q) {
+            const int code = fl[q];
+            if (code >= 0 && code / tt.NFS == f) mu = mutab[((size_t)f * Nfq + gf) * tt.NFS + code % tt.NFS];
           }
           v = cF[fp] * mu;
           if (has_cq)
@@ -263,9 +190,9 @@ k_assemble_sf(Dims dm, Phys ph, RefTables ref, AsmTab<T> tb, T* __restrict__ S, 
         T s = 0;
         for (int g1 = 0; g1 < nq1; ++g1) s = fma(sL[g1 * np1 + a1], Uf[(g1 * UW + a2) * CC + c], s);
         facc[ref.slot[ref.fnode[f * Nfn + tn]] * CC + c] += s;
-        if (MIX && fq == 0) tacc[fsf[tn] * CC + c] += s;   // continuous face: same sums, trace rows
+        if (fq == 0) tacc[fsf[tn] * CC + c] += s;   // continuous face: same sums, trace rows
       }
-      if (MIX && fq > 0) {
+      if (fq > 0) {
         __syncthreads();
         if (tt.fkind && tt.fkind[e * 6 + f] != kFaceInterior) {
           // domain-boundary face: the trace rows take the boundary flux; rebuild the
@@ -314,7 +241,6 @@ k_assemble_sf(Dims dm, Phys ph, RefTables ref, AsmTab<T> tb, T* __restrict__ S, 
         }
         __syncthreads();
       }
-    }
     }
     if constexpr (VOL) {
     // ---- volume right operands W_r[g][c] for the three reference directions.  The
@@ -414,7 +340,7 @@ k_assemble_sf(Dims dm, Phys ph, RefTables ref, AsmTab<T> tb, T* __restrict__ S, 
         s = fma(sL[gx * np1 + ax], V[(1 * VS + t) * CC + c], s);
       }
       const int sl = ref.slot[a];
-      if (sl >= 0) s += SIX ? face_sum<T, NP1, CC>(fn, a, c) : facc[sl * CC + c];
+      if (sl >= 0) s += facc[sl * CC + c];
       if (i == k && col < Np) s += alpha * Ms[a * Np + col];
       const int64_t cs = col < Np ? (int64_t)k * Np + col : (int64_t)dm.nu + (int64_t)k * Nb + (col - Np);
       Se[((int64_t)i * Np + a) * ld + cs] = s;
@@ -425,7 +351,7 @@ k_assemble_sf(Dims dm, Phys ph, RefTables ref, AsmTab<T> tb, T* __restrict__ S, 
       if (col >= ncol_all) continue;
       const int64_t cs = col < Np ? (int64_t)k * Np + col : (int64_t)dm.nu + (int64_t)k * Nb + (col - Np);
       Se[((int64_t)dm.nu + (int64_t)i * Nb + sl) * ld + cs] =
-          SIX ? face_sum<T, NP1, CC>(fn, ref.bnode[sl], c) : tacc[sl * CC + c];
+          tacc[sl * CC + c];
     }
     __syncthreads();
   }
@@ -437,12 +363,8 @@ k_assemble_sf(Dims dm, Phys ph, RefTables ref, AsmTab<T> tb, T* __restrict__ S, 
 template <class T, int NP1, int NQ1, int CC>
 static cudaError_t assemble_sf_t(iedg_mesh* M, T* S, const double* rhs64, const AsmTab<T>& tb, cudaStream_t st) {
   const Dims& dm = M->dm;
-  const bool mix = M->tt.nb != nullptr;
-  size_t smem = sf_smem<T, CC>(dm, mix);
-  // FP64 runs here on meshes with mixed orders only
-  auto kern = k_assemble_sf<T, NP1, NQ1, CC, true>;
-  if constexpr (sizeof(T) == 4)
-    if (!mix) kern = k_assemble_sf<T, NP1, NQ1, CC, false>;
+  size_t smem = sf_smem<T, CC>(dm);
+  auto kern = k_assemble_sf<T, NP1, NQ1, CC>;
   cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (err != cudaSuccess) return err;
   kern<<<(unsigned)(M->E * dm.m * dm.m), SF_THREADS, smem, st>>>(dm, M->ph, M->ref, tb, S, rhs64, M->tt);
@@ -455,9 +377,8 @@ static cudaError_t assemble_sf_t(iedg_mesh* M, T* S, const double* rhs64, const 
 template <class T, int NP1, int NQ1>
 static cudaError_t assemble_sf_c(iedg_mesh* M, T* S, const double* rhs64, const AsmTab<T>& tb, cudaStream_t st) {
   int cc = M->sched.asm_chunk ? M->sched.asm_chunk : (sizeof(T) == 8 ? 8 : 16);
-  const bool mix = M->tt.nb != nullptr;
-  if (cc == 32 && sf_smem<T, 32>(M->dm, mix) > 227 * 1024) cc = 16;
-  if (cc == 16 && sf_smem<T, 16>(M->dm, mix) > 227 * 1024) cc = 8;
+  if (cc == 32 && sf_smem<T, 32>(M->dm) > 227 * 1024) cc = 16;
+  if (cc == 16 && sf_smem<T, 16>(M->dm) > 227 * 1024) cc = 8;
   if (cc == 32) return assemble_sf_t<T, NP1, NQ1, 32>(M, S, rhs64, tb, st);
   if (cc == 16) return assemble_sf_t<T, NP1, NQ1, 16>(M, S, rhs64, tb, st);
   return assemble_sf_t<T, NP1, NQ1, 8>(M, S, rhs64, tb, st);

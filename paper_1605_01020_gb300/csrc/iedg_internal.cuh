@@ -138,6 +138,36 @@ struct LuDesc {
   const int64_t* order = nullptr;
 };
 
+// Order in which the assembly kernels that work by columns take the columns of a 3D
+// element's 25 pairs (i, k): the u-columns of the 17 pairs whose viscous Jacobian does not
+// vanish identically (all but the mass equation and the momentum equations with respect
+// to the energy unknown), their trace columns, then the 8 others' u-columns and trace
+// columns (the latter have no volume terms).
+struct HexCol {
+  int pair = -1, col = 0;      // pair 5 i + k (-1: past the end); node b or trace slot t
+  bool u = true, cq = true;    // u-column, pair of the first kind
+};
+__host__ __device__ inline HexCol hex_col(int fc, int Np, int nb) {
+  HexCol h;
+  const int nA = 17 * Np, nB = 17 * nb, nC = 8 * Np;
+  int q;
+  if (fc < nA + nB) {
+    h.u = fc < nA;
+    const int f = h.u ? fc : fc - nA, w = h.u ? Np : nb;
+    q = f / w;
+    h.col = f % w;
+    h.pair = q < 12 ? 5 * (1 + q / 4) + q % 4 : 20 + (q - 12);
+  } else if (fc < 25 * (Np + nb)) {
+    h.u = fc < nA + nB + nC;
+    h.cq = false;
+    const int f = fc - nA - nB - (h.u ? 0 : nC), w = h.u ? Np : nb;
+    q = f / w;
+    h.col = f % w;
+    h.pair = q < 5 ? q : 5 * (1 + q - 5) + 4;
+  }
+  return h;
+}
+
 // Location of the per-slot values of a ragged source: value (e, s, i) at
 // base[e] + s ss[e] + i cs[e].
 struct RaggedSrc {
@@ -163,6 +193,7 @@ struct iedg_mesh {
   int64_t E = 0, T = 0, nnzb = 0;
   int64_t max_row_blocks = 0;   // longest block row of K (blocks)
   iedg::RefTables ref{};
+  std::vector<double> L1h, dL1h;   // ref.L1, ref.dL1 on the host
   iedg::Geo geo{};
   iedg::PointJac pj{};
   int64_t* etrace = nullptr;    // [E][Nb]
@@ -262,7 +293,7 @@ void assemble_dg_table(const Dims& dm, const std::vector<double>& PhiF, const st
                        std::vector<unsigned char>& table, std::vector<int>& rexp, int* window);
 cudaError_t launch_lift_exp(iedg_mesh* M, cudaStream_t st);
 cudaError_t launch_assemble_dg(iedg_mesh* M, double* S, const int64_t* elist, int64_t n_slots, cudaStream_t st);
-cudaError_t launch_assemble_col(iedg_mesh* M, cudaStream_t st);  // small elements, a thread per column
+cudaError_t launch_assemble_col(iedg_mesh* M, cudaStream_t st);  // a thread per column: small elements, FP32 hexahedra
 bool assemble_col_supported(const iedg_mesh* M);
 AsmTab<double> tables64(const iedg_mesh* M);
 AsmTab<float> tables32(const iedg_mesh* M);
