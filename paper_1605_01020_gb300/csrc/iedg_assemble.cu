@@ -17,8 +17,6 @@
 // (mu_s = phi_bnode[s] on every face), which is how they are formed here.
 // The right-hand-side column is written by the point kernel: Ft = -R_u(u, q*),
 // Gt = -R_FL,e(u, q*) (exact because the fluxes are affine in q).
-#include <cuda_bf16.h>
-
 #include "iedg_digits.cuh"
 #include "iedg_internal.cuh"
 #include "iedg_lu_common.cuh"
@@ -946,418 +944,6 @@ k_lu64_tc(Dims dm, LuDesc lud, double* __restrict__ S, int8_t* __restrict__ stat
   if (warp == 0) tc::tmem_dealloc(tmem_base, LT_TMEM_COLS);
 }
 
-// FP32 partial LU for the mixed path.  Same algorithm and pivot rule as k_lu, with
-// the panel kept column-major in shared memory (contiguous rows for the pivot search,
-// the elimination and vector loads of L21) and a 4 x 8 register tile per thread in
-// the trailing update (float4 loads: three shared loads per 32 multiply-adds), so the
-// update runs at FFMA rather than shared-memory rate, with two CTAs per SM.  The full panel (L) and the
-// pivot rows are written back for the refinement solves.
-constexpr int L32_NB = 32;
-constexpr int L32_UCW = 128;      // trailing-update column chunk
-constexpr int L32_TM = 4, L32_TN = 8;
-
-
-// The 4 x 8 tile of A at rows rr0.., columns cc + tc * 8.. (zero outside the update).
-__device__ __forceinline__ void lu32_load_tile(const float* __restrict__ A, int ld, int rr0, int r_hi, int cc, int tc,
-                                               int cw, bool cvec, float (&t)[L32_TM][L32_TN]) {
-#pragma unroll
-  for (int a = 0; a < L32_TM; ++a) {
-    const int rr = rr0 + a;
-    if (cvec && rr < r_hi) {
-      const float4* src = reinterpret_cast<const float4*>(A + (int64_t)rr * ld + cc + tc * L32_TN);
-      const float4 v0 = src[0], v1 = src[1];
-      t[a][0] = v0.x; t[a][1] = v0.y; t[a][2] = v0.z; t[a][3] = v0.w;
-      t[a][4] = v1.x; t[a][5] = v1.y; t[a][6] = v1.z; t[a][7] = v1.w;
-    } else {
-#pragma unroll
-      for (int b = 0; b < L32_TN; ++b) {
-        const int c = tc * L32_TN + b;
-        t[a][b] = (rr < r_hi && c < cw) ? A[(int64_t)rr * ld + cc + c] : 0.f;
-      }
-    }
-  }
-}
-
-// Ask L2 for the lines of the 4 x 8 tile at rows rr0.. (no registers held).
-__device__ __forceinline__ void lu32_prefetch_tile(const float* __restrict__ A, int ld, int rr0, int r_hi, int cc,
-                                                   int tc) {
-#pragma unroll
-  for (int a = 0; a < L32_TM; ++a)
-    if (rr0 + a < r_hi)
-      asm volatile("prefetch.global.L2 [%0];" ::"l"(A + (int64_t)(rr0 + a) * ld + cc + tc * L32_TN));
-}
-
-// A[r][c] -= sum_j L[r][j] U[j][c] over rows [r_lo, r_hi), cols [c_lo, c_hi): L from the
-// column-major panel P (row r at P[j n + r - kb]), U = rows kb..kb+nb of A.  4 x 8
-// register tiles, U staged in Uc by 128-column chunks; the next row block's tile is
-// requested from L2 while the current one is updated.  Columns past c_hi are written
-// back unchanged only when they are padding of the row (c_hi = n + 1).
-__device__ __forceinline__ void lu32_update_rect(float* __restrict__ A, int ld, int n, const float* __restrict__ P,
-                                                 float* __restrict__ Uc, int kb, int nb, int r_lo, int r_hi,
-                                                 int c_lo, int c_hi) {
-  const int tid = threadIdx.x;
-  const bool vec = ((nb & 3) == 0) && ((n & 3) == 0);
-  const int tc = tid % (L32_UCW / L32_TN), tr = tid / (L32_UCW / L32_TN);   // 16 x 16
-  const int vlim = (c_hi == n + 1) ? ld : c_hi;     // last column a vector access may touch
-  constexpr int RB = 16 * L32_TM;                   // rows per block of the CTA
-  for (int cc = c_lo; cc < c_hi; cc += L32_UCW) {
-    const int cw = min(L32_UCW, c_hi - cc);
-    for (int idx = tid; idx < L32_NB * L32_UCW; idx += LU_THREADS) {
-      int j = idx / L32_UCW, c = idx % L32_UCW;
-      Uc[idx] = (j < nb && c < cw) ? A[(int64_t)(kb + j) * ld + cc + c] : 0.f;
-    }
-    __syncthreads();
-    const bool cvec = ((cc & 3) == 0) && (cc + tc * L32_TN + L32_TN <= vlim);
-    for (int rb = r_lo; rb < r_hi; rb += RB) {
-      const int rr0 = rb + tr * L32_TM;
-      float acc[L32_TM][L32_TN];
-      lu32_load_tile(A, ld, rr0, r_hi, cc, tc, cw, cvec, acc);
-      if (rb + RB < r_hi) lu32_prefetch_tile(A, ld, rr0 + RB, r_hi, cc, tc);
-      if (nb == L32_NB && vec && rr0 + L32_TM <= r_hi) {
-        // full panel, whole tile: fixed trip count and no per-step bounds tests
-        const float* lp = P + (rr0 - kb);
-        const float* up = Uc + tc * L32_TN;
-#pragma unroll 2
-        for (int j = 0; j < L32_NB; ++j) {
-          const float4 l0 = *reinterpret_cast<const float4*>(lp + j * n);
-          const float4 u0 = *reinterpret_cast<const float4*>(up + j * L32_UCW);
-          const float4 u1 = *reinterpret_cast<const float4*>(up + j * L32_UCW + 4);
-          const float lv[L32_TM] = {l0.x, l0.y, l0.z, l0.w};
-          const float uv[L32_TN] = {u0.x, u0.y, u0.z, u0.w, u1.x, u1.y, u1.z, u1.w};
-#pragma unroll
-          for (int a = 0; a < L32_TM; ++a)
-#pragma unroll
-            for (int b = 0; b < L32_TN; ++b) acc[a][b] = fmaf(-lv[a], uv[b], acc[a][b]);
-        }
-      } else if (rr0 < r_hi) {
-#pragma unroll 4
-        for (int j = 0; j < nb; ++j) {
-          float lv[L32_TM], uv[L32_TN];
-          const float* lp = P + j * n + (rr0 - kb);
-          if (vec && rr0 + L32_TM <= r_hi) {
-            float4 l0 = *reinterpret_cast<const float4*>(lp);
-            lv[0] = l0.x; lv[1] = l0.y; lv[2] = l0.z; lv[3] = l0.w;
-          } else {
-#pragma unroll
-            for (int a = 0; a < L32_TM; ++a) lv[a] = (rr0 + a < r_hi) ? lp[a] : 0.f;
-          }
-          const float4 u0 = *reinterpret_cast<const float4*>(Uc + j * L32_UCW + tc * L32_TN);
-          const float4 u1 = *reinterpret_cast<const float4*>(Uc + j * L32_UCW + tc * L32_TN + 4);
-          uv[0] = u0.x; uv[1] = u0.y; uv[2] = u0.z; uv[3] = u0.w;
-          uv[4] = u1.x; uv[5] = u1.y; uv[6] = u1.z; uv[7] = u1.w;
-#pragma unroll
-          for (int a = 0; a < L32_TM; ++a)
-#pragma unroll
-            for (int b = 0; b < L32_TN; ++b) acc[a][b] = fmaf(-lv[a], uv[b], acc[a][b]);
-        }
-      }
-#pragma unroll
-      for (int a = 0; a < L32_TM; ++a) {
-        const int rr = rr0 + a;
-        if (cvec && rr < r_hi) {
-          float4* dst = reinterpret_cast<float4*>(A + (int64_t)rr * ld + cc + tc * L32_TN);
-          dst[0] = make_float4(acc[a][0], acc[a][1], acc[a][2], acc[a][3]);
-          dst[1] = make_float4(acc[a][4], acc[a][5], acc[a][6], acc[a][7]);
-        } else {
-#pragma unroll
-          for (int b = 0; b < L32_TN; ++b) {
-            int c = tc * L32_TN + b;
-            if (rr < r_hi && c < cw) A[(int64_t)rr * ld + cc + c] = acc[a][b];
-          }
-        }
-      }
-    }
-    __syncthreads();
-  }
-}
-
-// Deferred Schur complement on the tensor cores: [K | R] = [D | G] - W [Z | z] for rows
-// [nu, n) and columns [nu, n], W = A[nu:n, 0:nu] (the eliminated trace rows, L21 of
-// every panel) and Z = A[0:nu, nu:n] (U12 of every panel), so K accumulates over the
-// whole K = nu in TMEM and the trace block is read and written once.  128 x 64 output
-// tiles, K chunks of 32 in two operand stages so that one chunk is staged while the
-// tensor core works on the other; one thread issues the MMAs, completion through
-// per-stage mbarriers with bounded waits; the epilogue reads TMEM with all eight warps.
-// Operand forms (KIND): kSchurFp32 = TF32 high and low parts, three products (hi hi +
-// hi lo + lo hi, FP32 accuracy, 48 KB stages); kSchurTf32 = one product of the operands
-// rounded to TF32 (24 KB); kSchurBf16 = one product of BF16 operands (12 KB).  All
-// accumulate in FP32.
-constexpr int TC_TM = 128, TC_TN = 64, TC_KC = 32;
-constexpr int TC_STAGE_BYTES = 2 * TC_TM * TC_KC * 4 + 2 * TC_TN * TC_KC * 4;   // 48 KB, the largest form
-
-template <int KIND>
-struct SchurForm {
-  static constexpr int EB = KIND == kSchurBf16 ? 2 : 4;          // bytes per operand value
-  static constexpr int PARTS = KIND == kSchurFp32 ? 2 : 1;       // hi (+ lo)
-  static constexpr int A_BYTES = TC_TM * TC_KC * EB, B_BYTES = TC_TN * TC_KC * EB;
-  static constexpr int SBO = TC_KC * EB / 16 * 128;               // 8-row group stride
-  __device__ static uint32_t off(int row, int k) { return EB == 4 ? tc::core_off32(row, k) : tc::core_off16(row, k); }
-  // value v at (row, k) of the A (b = false) or B operand tile
-  __device__ static void put(char* stage, bool b, int row, int k, float v) {
-    char* base = stage + (b ? PARTS * A_BYTES : 0);
-    const uint32_t o = off(row, k);
-    if constexpr (KIND == kSchurFp32) {
-      float hi, lo;
-      tc::split_tf32(v, hi, lo);
-      *reinterpret_cast<float*>(base + o) = hi;
-      *reinterpret_cast<float*>(base + (b ? B_BYTES : A_BYTES) + o) = lo;
-    } else if constexpr (KIND == kSchurTf32) {
-      *reinterpret_cast<float*>(base + o) = tc::round_tf32(v);
-    } else {
-      *reinterpret_cast<__nv_bfloat16*>(base + o) = __float2bfloat16_rn(v);
-    }
-  }
-};
-
-template <int KIND>
-__device__ __forceinline__ void schur_stage(const float* __restrict__ A, int ld, int n, int nu, int ncol, int rt,
-                                            int ct, int kc, char* stage) {
-  using F = SchurForm<KIND>;
-  const int tid = threadIdx.x;
-  // A operand: W rows rt .. rt+127, K columns kc .. kc+31 (k fastest: coalesced rows)
-  for (int idx = tid; idx < TC_TM * TC_KC; idx += LU_THREADS) {
-    const int mm = idx >> 5, k = idx & 31;
-    const int r = rt + mm, c = kc + k;
-    F::put(stage, false, mm, k, (r < n && c < nu) ? A[(int64_t)r * ld + c] : 0.f);
-  }
-  // B operand (N x K, K-major): Z rows kc .. kc+31, columns ct .. ct+63 (column fastest)
-  for (int idx = tid; idx < TC_TN * TC_KC; idx += LU_THREADS) {
-    const int k = idx >> 6, nn = idx & 63;
-    const int r = kc + k, c = ct + nn;
-    F::put(stage, true, nn, k, (r < nu && c < ncol) ? A[(int64_t)r * ld + c] : 0.f);
-  }
-}
-
-template <int KIND>
-__device__ __forceinline__ void schur_issue(uint32_t tmem, const char* stage, bool first) {
-  using F = SchurForm<KIND>;
-  const uint32_t aH = tc::smem_u32(stage), aL = aH + F::A_BYTES;
-  const uint32_t bH = aH + F::PARTS * F::A_BYTES, bL = bH + F::B_BYTES;
-  // one instruction covers 32 bytes of K (8 TF32 or 16 BF16 values): two core matrices
-#pragma unroll
-  for (int st = 0; st < TC_KC * F::EB / 32; ++st) {
-    const uint32_t ko = st * 256, acc = (first && st == 0) ? 0u : 1u;
-    if constexpr (KIND == kSchurBf16) {
-      constexpr uint32_t IDESC = tc::idesc_bf16(TC_TM, TC_TN);
-      tc::mma_bf16(tmem, tc::desc_kmajor(aH + ko, 128, F::SBO), tc::desc_kmajor(bH + ko, 128, F::SBO), IDESC, acc);
-    } else {
-      constexpr uint32_t IDESC = tc::idesc_tf32(TC_TM, TC_TN);
-      tc::mma_tf32(tmem, tc::desc_kmajor(aH + ko, 128, F::SBO), tc::desc_kmajor(bH + ko, 128, F::SBO), IDESC, acc);
-      if constexpr (KIND == kSchurFp32) {
-        tc::mma_tf32(tmem, tc::desc_kmajor(aH + ko, 128, F::SBO), tc::desc_kmajor(bL + ko, 128, F::SBO), IDESC, 1);
-        tc::mma_tf32(tmem, tc::desc_kmajor(aL + ko, 128, F::SBO), tc::desc_kmajor(bH + ko, 128, F::SBO), IDESC, 1);
-      }
-    }
-  }
-}
-
-// Bounded wait on stage b's barrier by every thread; the outcome is made uniform.
-// (A wait that ran out leaves the phase where it was, so the drain can wait for it.)
-__device__ __forceinline__ bool schur_wait(TcState* tcs, int b) {
-  const bool ok = __syncthreads_and(tc::mbar_wait(tcs->mbar + b, tcs->phase[b], tcs->limit));
-  if (ok) { tcs->phase[b] ^= 1u; tcs->pending[b] = 0; }
-  else tcs->failed = 1;
-  return ok;
-}
-
-template <int KIND>
-__device__ void schur_tc(float* __restrict__ A, int ld, int n, int nu, char* smem, TcState* tcs) {
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int ncol = n + 1;
-  const int nk = (nu + TC_KC - 1) / TC_KC;
-  const int q = warp & 3, h = warp >> 2;
-  for (int rt = nu; rt < n && !tcs->failed; rt += TC_TM) {
-    for (int ct = nu; ct < ncol && !tcs->failed; ct += TC_TN) {
-      schur_stage<KIND>(A, ld, n, nu, ncol, rt, ct, 0, smem);
-      tc::fence_proxy_async();
-      __syncthreads();
-      tc::fence_after_sync();
-      for (int c = 0; c < nk; ++c) {
-        const int b = c & 1;
-        if (tid == 0) {
-          schur_issue<KIND>(tcs->tmem, smem + b * TC_STAGE_BYTES, c == 0);
-          tc::mma_commit(tcs->mbar + b);
-        }
-        tcs->pending[b] = 1;
-        if (c + 1 < nk) {
-          // the other stage was last read by the MMAs of chunk c - 1
-          if (c >= 1 && !schur_wait(tcs, b ^ 1)) break;
-          schur_stage<KIND>(A, ld, n, nu, ncol, rt, ct, (c + 1) * TC_KC, smem + (b ^ 1) * TC_STAGE_BYTES);
-          tc::fence_proxy_async();
-          __syncthreads();
-          tc::fence_after_sync();
-        }
-      }
-      if (tcs->failed) break;
-      // the two commits not waited for yet: chunks nk - 2 and nk - 1
-      if (nk >= 2 && !schur_wait(tcs, (nk - 2) & 1)) break;
-      if (!schur_wait(tcs, (nk - 1) & 1)) break;
-      tc::fence_after_sync();
-      // epilogue: warp (q, h) owns rows 32 q .. 32 q + 31 and columns 32 h .. 32 h + 31
-      const int row = rt + 32 * q + lane;
-#pragma unroll 1
-      for (int c8 = 0; c8 < 4; ++c8) {
-        const int c0 = 32 * h + 8 * c8;
-        float pv8[8];
-        tc::tmem_ld8(tcs->tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)c0, pv8);
-        if (row >= n || ct + c0 >= ncol) continue;
-        float* dst = A + (int64_t)row * ld + ct + c0;
-#pragma unroll
-        for (int j = 0; j < 8; ++j)
-          if (ct + c0 + j < ncol) dst[j] -= pv8[j];
-      }
-      tc::fence_before_sync();
-      __syncthreads();
-    }
-  }
-}
-
-template <bool TC, int KIND = kSchurFp32>
-__device__ __forceinline__ void lu32_element(const LuElem& el, float* __restrict__ S, int8_t* __restrict__ status,
-                                             int* __restrict__ pivots, const int64_t e, TcState* tcs) {
-  extern __shared__ __align__(16) unsigned char smraw[];
-  float* P = reinterpret_cast<float*>(smraw);          // [NB][n] column-major panel
-  float* Uc = P + (size_t)L32_NB * el.n;                // [NB][UCW]
-  __shared__ int piv[L32_NB];
-  __shared__ int perm[LU_MAX_NU];   // net row permutation of the current panel's interchanges
-  __shared__ float rv[LU_THREADS / 32];
-  __shared__ int ri[LU_THREADS / 32];
-  __shared__ int sing;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int n = el.n, nu = el.nu, ld = el.ld, ncol = n + 1;
-  float* A = S + el.off;
-  int nonfin = 0;                       // a pivot candidate was NaN or infinite
-  if (tid == 0) sing = 0;
-  for (int kb = 0; kb < nu; kb += L32_NB) {
-    const int nb = min(L32_NB, nu - kb), rows = n - kb, prow = nu - kb;
-    for (int idx = tid; idx < rows * L32_NB; idx += LU_THREADS) {
-      int r = idx / L32_NB, j = idx % L32_NB;
-      P[j * n + r] = j < nb ? A[(int64_t)(kb + r) * ld + kb + j] : 0.f;
-    }
-    for (int r = tid; r < prow; r += LU_THREADS) perm[r] = r;
-    __syncthreads();
-    for (int j = 0; j < nb; ++j) {
-      const float* Pj = P + j * n;
-      float best = -1.f;
-      int bi = j;
-      for (int r = j + tid; r < prow; r += LU_THREADS) {
-        float v = fabsf(Pj[r]);
-        nonfin |= !(v <= 3.402823466e38f);
-        if (v > best) { best = v; bi = r; }
-      }
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        float ov = __shfl_xor_sync(0xffffffffu, best, o);
-        int oi = __shfl_xor_sync(0xffffffffu, bi, o);
-        if (ov > best || (ov == best && oi < bi)) { best = ov; bi = oi; }
-      }
-      if (lane == 0) { rv[warp] = best; ri[warp] = bi; }
-      __syncthreads();
-      // every thread combines the warps' candidates (same order, same result)
-      float bv = rv[0];
-      int pr = ri[0];
-      for (int w = 1; w < LU_THREADS / 32; ++w)
-        if (rv[w] > bv || (rv[w] == bv && ri[w] < pr)) { bv = rv[w]; pr = ri[w]; }
-      if (!(bv > 0.f)) pr = j;
-      if (tid == 0) {
-        if (!(bv > 0.f)) sing = 1;
-        piv[j] = pr;
-        pivots[el.poff + kb + j] = kb + pr;
-        if (pr != j) { const int t = perm[j]; perm[j] = perm[pr]; perm[pr] = t; }
-      }
-      if (pr != j && tid < L32_NB) {
-        float t = P[tid * n + j];
-        P[tid * n + j] = P[tid * n + pr];
-        P[tid * n + pr] = t;
-      }
-      __syncthreads();
-      const float pv = Pj[j];
-      const float inv = pv != 0.f ? 1.f / pv : 0.f;
-      for (int r = j + 1 + tid; r < rows; r += LU_THREADS) {
-        float l = Pj[r] * inv;
-        P[j * n + r] = l;
-        for (int c = j + 1; c < nb; ++c) P[c * n + r] = fmaf(-l, P[c * n + j], P[c * n + r]);
-      }
-      __syncthreads();
-    }
-    // full panel back (U11, L11, L21): needed by the refinement solves
-    for (int idx = tid; idx < rows * nb; idx += LU_THREADS) {
-      int r = idx / nb, j = idx % nb;
-      A[(int64_t)(kb + r) * ld + kb + j] = P[j * n + r];
-    }
-    // trailing columns: row interchanges, then U12 = L11^-1 A12.  The panel's
-    // interchanges, applied in order, leave row r holding the original row perm[r]; the
-    // rows below the panel that change are among the pivot rows piv[j] >= nb, and they
-    // receive original rows above nb.  Each column gathers its new top rows first
-    // (independent loads), then moves the displaced rows, then stores the top rows.
-    for (int c = kb + nb + tid; c < ncol; c += LU_THREADS) {
-      float x[L32_NB];
-#pragma unroll
-      for (int j = 0; j < L32_NB; ++j) {
-        if (j >= nb) break;
-        x[j] = A[(int64_t)(kb + perm[j]) * ld + c];
-      }
-      // displaced rows take original top rows (unchanged until the stores below), in
-      // groups of 8 loads before their stores
-#pragma unroll
-      for (int j0 = 0; j0 < L32_NB; j0 += 8) {
-        float y[8];
-#pragma unroll
-        for (int j = 0; j < 8; ++j) {
-          const int r = j0 + j < nb ? piv[j0 + j] : 0;
-          y[j] = (j0 + j < nb && r >= nb && perm[r] != r) ? A[(int64_t)(kb + perm[r]) * ld + c] : 0.f;
-        }
-#pragma unroll
-        for (int j = 0; j < 8; ++j) {
-          const int r = j0 + j < nb ? piv[j0 + j] : 0;
-          if (j0 + j < nb && r >= nb && perm[r] != r) A[(int64_t)(kb + r) * ld + c] = y[j];
-        }
-      }
-#pragma unroll
-      for (int j = 0; j < L32_NB; ++j) {
-        if (j >= nb) break;
-        float s = x[j];
-#pragma unroll
-        for (int jj = 0; jj < L32_NB; ++jj) {
-          if (jj >= j) break;
-          s = fmaf(-P[jj * n + j], x[jj], s);
-        }
-        x[j] = s;
-        A[(int64_t)(kb + j) * ld + c] = s;
-      }
-    }
-    __syncthreads();
-    const int r0 = kb + nb;
-    if constexpr (TC) {
-      // deferred Schur complement: the u-columns of every row and the trace columns of
-      // the u-rows are updated now (the next panels and U12 need them); the trace block
-      // of the trace rows receives all panels at once on the tensor cores below
-      lu32_update_rect(A, ld, n, P, Uc, kb, nb, r0, n, r0, nu);
-      lu32_update_rect(A, ld, n, P, Uc, kb, nb, r0, nu, nu, ncol);
-    } else {
-      // A22 -= L21 U12, rows [kb+nb, n), cols [kb+nb, n]
-      lu32_update_rect(A, ld, n, P, Uc, kb, nb, r0, n, r0, ncol);
-    }
-  }
-  if constexpr (TC) {
-    __syncthreads();
-    schur_tc<KIND>(A, ld, n, nu, reinterpret_cast<char*>(smraw), tcs);     // the panel buffer is free now
-  }
-  __syncthreads();
-  int bad = 0;
-  for (int idx = tid; idx < (n - nu) * (ncol - nu); idx += LU_THREADS) {
-    int r = nu + idx / (ncol - nu), c = nu + idx % (ncol - nu);
-    if (!isfinite(A[(int64_t)r * ld + c])) bad = 1;
-  }
-  bad = __syncthreads_or(bad);
-  nonfin = __syncthreads_or(nonfin);
-  if (tid == 0) {
-    if (TC && tcs->failed) status[e] = IEDG_ELEM_TIMEOUT;
-    else status[e] = nonfin ? IEDG_ELEM_NONFINITE
-                            : (sing ? IEDG_ELEM_SINGULAR : (bad ? IEDG_ELEM_NONFINITE : IEDG_ELEM_OK));
-  }
-}
-
 template <class T, int NB>
 __global__ void __launch_bounds__(LU_THREADS)
 k_lu(Dims dm, LuDesc lud, T* __restrict__ S, int8_t* __restrict__ status, int* __restrict__ pivots, int64_t* queue,
@@ -1365,71 +951,6 @@ k_lu(Dims dm, LuDesc lud, T* __restrict__ S, int8_t* __restrict__ status, int* _
   int64_t e;
   for (int64_t it = 0; next_element(queue, E, it, lud.order, &e); ++it)
     if (active == nullptr || active[e] >= 0) lu_element<T, NB>(lu_elem(dm, lud, e), S, status, pivots, e);
-}
-
-__global__ void __launch_bounds__(LU_THREADS, 2)
-k_lu32(Dims dm, LuDesc lud, float* __restrict__ S, int8_t* __restrict__ status, int* __restrict__ pivots,
-       int64_t* queue, int64_t E) {
-  int64_t e;
-  for (int64_t it = 0; next_element(queue, E, it, lud.order, &e); ++it)
-    lu32_element<false>(lu_elem(dm, lud, e), S, status, pivots, e, nullptr);
-}
-
-// Tensor-core form: TMEM (128 columns) and the completion barrier are set up once per
-// CTA; a CTA whose completion wait ran out stops taking elements, waits once more
-// (bounded) for its MMAs, and frees its TMEM.
-template <int KIND>
-__global__ void __launch_bounds__(LU_THREADS, 2)
-k_lu32_tc(Dims dm, LuDesc lud, float* __restrict__ S, int8_t* __restrict__ status, int* __restrict__ pivots,
-          int64_t* queue, int64_t E, int* err, int wait_limit) {
-  __shared__ uint32_t tmem_base;
-  __shared__ __align__(8) uint64_t mbar[2];
-  __shared__ TcState tcs;
-  const int tid = threadIdx.x, warp = tid >> 5;
-  if (warp == 0) {
-    tc::tmem_alloc(&tmem_base, TC_TN);
-    tc::tmem_relinquish();
-  }
-  if (tid == 0) {
-    tc::mbar_init(&mbar[0], 1);
-    tc::mbar_init(&mbar[1], 1);
-  }
-  tc::fence_before_sync();
-  __syncthreads();
-  tc::fence_after_sync();
-  if (tid == 0) {
-    tcs.tmem = tmem_base;
-    tcs.mbar = mbar;
-    tcs.phase[0] = 0;
-    tcs.phase[1] = 0;
-    tcs.failed = 0;
-    tcs.limit = wait_limit;
-    tcs.pending[0] = 0;
-    tcs.pending[1] = 0;
-  }
-  __syncthreads();
-  // each thread keeps its own copy of the phases; the shared copy is only the start
-  TcState mine = tcs;
-  int64_t e;
-  int64_t it = 0;
-  for (; next_element(queue, E, it, lud.order, &e); ++it) {
-    lu32_element<true, KIND>(lu_elem(dm, lud, e), S, status, pivots, e, &mine);
-    if (__syncthreads_or(mine.failed)) {
-      if (tid == 0) atomicOr(err, 1);
-      tc_drain(mine);     // MMAs still in flight finish before the TMEM is freed
-      ++it;
-      break;
-    }
-  }
-  // after a failed wait this CTA factors nothing more: the elements it still takes from
-  // the queue are flagged, so no element is left unfactored with an OK status
-  if (mine.failed)
-    for (; next_element(queue, E, it, lud.order, &e); ++it)
-      if (tid == 0) status[e] = IEDG_ELEM_TIMEOUT;
-  tc::fence_before_sync();
-  __syncthreads();
-  tc::fence_after_sync();
-  if (warp == 0) tc::tmem_dealloc(tmem_base, TC_TN);
 }
 
 }  // namespace
@@ -1521,29 +1042,6 @@ static cudaError_t lu_t(iedg_mesh* M, T* S, int* piv, cudaStream_t st) {
 
 size_t lu64_smem(const Dims& dm, int nb) { return sizeof(double) * ((size_t)dm.n * nb + (size_t)nb * UCW); }
 
-// FP32 partial LU with the Schur complement on the tensor cores in operand form KIND.
-template <int KIND>
-static cudaError_t lu32_tc(iedg_mesh* M, cudaStream_t st) {
-  const Dims& dm = M->dm;
-  // panel + U chunk during the factorisation; the two operand stages of the Schur GEMM
-  // reuse the same buffer afterwards
-  size_t smem = sizeof(float) * ((size_t)L32_NB * dm.n + (size_t)L32_NB * L32_UCW);
-  if (smem < 2 * (size_t)TC_STAGE_BYTES) smem = 2 * (size_t)TC_STAGE_BYTES;
-  cudaError_t err = cudaFuncSetAttribute(k_lu32_tc<KIND>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (err != cudaSuccess) return err;
-  unsigned grid = (unsigned)M->E;
-  int64_t* queue = nullptr;
-  if (M->sched.lu_persistent) {
-    err = persistent_grid(k_lu32_tc<KIND>, smem, M->E, &grid);
-    if (err == cudaSuccess) err = cudaMemsetAsync(M->queue, 0, sizeof(int64_t), st);
-    if (err != cudaSuccess) return err;
-    queue = M->queue;
-  }
-  k_lu32_tc<KIND><<<grid, LU_THREADS, smem, st>>>(dm, M->lud, M->S32, M->status, M->piv, queue, M->E, M->dev_flag,
-                                                   tc_wait_limit(M));
-  return cudaGetLastError();
-}
-
 static cudaError_t launch_lu64_tc(iedg_mesh* M, cudaStream_t st) {
   const size_t smem = lt_smem(M->dm);
   cudaError_t err = cudaFuncSetAttribute(k_lu64_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -1569,24 +1067,8 @@ cudaError_t launch_lu(iedg_mesh* M, cudaStream_t st) {
     if (M->sched.lu_panel == 32 && lu64_smem(M->dm, 32) <= 227 * 1024) return lu_t<double, 32>(M, M->S, nullptr, st);
     return lu_t<double, 16>(M, M->S, nullptr, st);
   }
-  if (M->schur_in == kSchurTf32) return lu32_tc<kSchurTf32>(M, st);
-  if (M->schur_in == kSchurBf16) return lu32_tc<kSchurBf16>(M, st);
-  if (M->sched.lu_tensor == 2) return launch_lu32_mma(M, M->dm.n, st);
-  if (M->sched.lu_tensor) return lu32_tc<kSchurFp32>(M, st);
-  const Dims& dm = M->dm;
-  size_t smem = sizeof(float) * ((size_t)L32_NB * dm.n + (size_t)L32_NB * L32_UCW);
-  cudaError_t err = cudaFuncSetAttribute(k_lu32, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (err != cudaSuccess) return err;
-  if (M->sched.lu_persistent) {
-    unsigned grid = 0;
-    err = persistent_grid(k_lu32, smem, M->E, &grid);
-    if (err == cudaSuccess) err = cudaMemsetAsync(M->queue, 0, sizeof(int64_t), st);
-    if (err != cudaSuccess) return err;
-    k_lu32<<<grid, LU_THREADS, smem, st>>>(dm, M->lud, M->S32, M->status, M->piv, M->queue, M->E);
-  } else {
-    k_lu32<<<(unsigned)M->E, LU_THREADS, smem, st>>>(dm, M->lud, M->S32, M->status, M->piv, nullptr, M->E);
-  }
-  return cudaGetLastError();
+  if (M->schur_in == kSchurFp32 && M->sched.lu_tensor == 2) return launch_lu32_mma(M, M->dm.n, st);
+  return launch_lu32(M, st);
 }
 
 }  // namespace iedg

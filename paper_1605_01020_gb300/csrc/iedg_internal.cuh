@@ -300,6 +300,7 @@ AsmTab<float> tables32(const iedg_mesh* M);
 cudaError_t launch_lu(iedg_mesh* M, cudaStream_t st);
 // u-unknowns from which the FP64 LU takes its digit form (iedg_assemble.cu)
 constexpr int LU64_TC_MIN_NU = 64;
+cudaError_t launch_lu32(iedg_mesh* M, cudaStream_t st);   // FP32 LU, FFMA updates or deferred tensor-core Schur complement
 cudaError_t launch_lu32_mma(iedg_mesh* M, int n_max, cudaStream_t st);   // FP32 LU, tcgen05 trailing updates
 cudaError_t launch_scatter_K(iedg_mesh* M, double* K, cudaStream_t st);
 cudaError_t launch_scatter_R_ragged(iedg_mesh* M, const RaggedSrc& src, const double* base, double* R,
