@@ -189,14 +189,16 @@ __global__ void k_bilu_colour(int m, int64_t nrows, int64_t first, BiluTab B, do
 // The solve is a cooperative launch of at most one CTA per SM; its CTAs meet at grid
 // barriers, so an Arnoldi step costs three of them instead of a dozen launches and a
 // synchronisation with the host (about 100 us a step).  Each CTA owns a contiguous range
-// of trace nodes: it forms those rows of K v (a warp per block row, one lane per block
-// entry, so that K streams in order), preconditions, orthogonalises and normalises
+// of trace nodes: it forms those rows of K v (one lane per block entry, so that K
+// streams in order), preconditions, orthogonalises and normalises
 // them; the Hessenberg column, the rotations and the stopping test are formed by every
 // CTA from the same sums in the same order, so nothing else is exchanged.  K v is bound
 // by the FP64 pipe (one multiply-add per entry of K, two per SM and clock).
-// Measured to 1e-12, launch by launch -> one launch: 2D p = 2 8 x 8 (768 unknowns, 26
-// steps) 5.04 -> 0.70 ms, 3D p = 3 6^3 (20,520 unknowns, 112 MB of K, 48 steps) 12.9 -> 5.7,
-// 3D p = 2 16^3 (143,360 unknowns, 72 steps) 31.0 -> 20.7; with BILU(0) 2D 3.4 -> 2.4.
+// Measured to 1e-12, launch by launch -> one launch (in brackets: a warp per block row, its
+// longest row the critical path of every step): 2D p = 2 8 x 8 (768 unknowns, 26 steps)
+// 5.04 -> 0.73 ms [0.70], 3D p = 3 6^3 (20,520 unknowns, 112 MB of K, 48 steps) 12.9 -> 3.3
+// [5.7], 3D p = 2 16^3 (143,360 unknowns, 72 steps) 31.0 -> 14.3 [20.7]; with BILU(0) 2D
+// 3.4 -> 2.5.
 constexpr int GK_THREADS = 512, GK_WARPS = GK_THREADS / 32;
 constexpr int GK_MIN_ROWS = 8;                    // trace nodes per CTA on small systems
 constexpr int GK_BARRIER_POLLS = 1 << 24;
@@ -223,6 +225,8 @@ struct GmresShared {
   double red[GK_WARPS][GK_R1 + 1];
   double h1[GK_R1], h2[GK_R1];
   double H[GK_R1][IEDG_MAX_RESTART], cs[IEDG_MAX_RESTART], sn[IEDG_MAX_RESTART], g[GK_R1], y[IEDG_MAX_RESTART];
+  double psum[GK_WARPS][2][5];            // K x: the warps' shares of rows they do not hold alone
+  int prow[GK_WARPS][2];
   double nrm2, rel, hn, scale;
   int done, abort, again;
 };
@@ -266,6 +270,7 @@ __device__ __forceinline__ void sum_parts(const GmresArgs& a, GmresShared& sh, i
   for (int v0 = 0; v0 < nv; v0 += 32) {
     double s = 0.0;
     if (v0 + lane < nv)
+#pragma unroll 10
       for (int c = warp; c < (int)gridDim.x; c += GK_WARPS) s += __ldcg(a.part + (int64_t)c * GK_R1 + v0 + lane);
     if (v0 + lane < nv) sh.red[warp][v0 + lane] = s;
   }
@@ -303,59 +308,118 @@ __device__ __forceinline__ void dot_parts(const GmresArgs& a, GmresShared& sh, i
   }
 }
 
-// Rows [t0, t1) of y = K x, or b - K x; x read through L2 (other CTAs wrote it).  A warp
-// per block row, a lane per block entry (two blocks at a time where m = 4); the row's
-// column indices are read 32 at a time and 16 blocks of K and x requested together.
-__device__ __forceinline__ void spmv_rows(const GmresArgs& a, const double* x, double* y, const double* b, int64_t t0,
-                                          int64_t t1) {
-  constexpr int UN = 16;
+// Rows [t0, t1) of y = K x, or b - K x; x read through L2 (other CTAs wrote it).  The CTA's
+// blocks of K, consecutive in memory, are split evenly over its warps (a block row's
+// length varies with the elements at its node); rows that cross warps are summed in warp
+// order at the end.  A lane per block entry (two blocks at a time where M = 4; the spare
+// lanes repeat others), the column indices read 32 at a time, GK_UN blocks of K and x
+// requested together.  Ends with the CTA's threads in step.
+constexpr int GK_UN = 16;
+template <int M>
+__device__ __forceinline__ void spmv_rows_m(const GmresArgs& a, GmresShared& sh, const double* __restrict__ x,
+                                            double* __restrict__ y, const double* __restrict__ b, int64_t t0, int64_t t1) {
+  constexpr int MM = M * M, PER = 32 / MM;                 // blocks per warp step
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int m = a.m, mm = m * m, per = 32 / mm;            // blocks per warp step
-  const int sub = lane / mm, e = lane % mm, k = e % m;
-  for (int64_t t = t0 + warp; t < t1; t += GK_WARPS) {
-    const int64_t lo = a.row_ptr[t], hi = a.row_ptr[t + 1];
+  const int sub = PER > 1 ? (lane / MM) % PER : 0, e = lane % MM, k = e % M;
+  if (lane < 2) sh.prow[warp][lane] = -1;
+  __syncwarp();
+  const int64_t q0 = a.row_ptr[t0], nq = a.row_ptr[t1] - q0;
+  int64_t q = q0 + nq * warp / GK_WARPS;
+  const int64_t qb = q0 + nq * (warp + 1) / GK_WARPS, qa = q;
+  int64_t t = t0;
+  if (q < qb) {                                            // row of block q
+    int64_t lo = t0, hi = t1;                              // last row that starts at or before q
+    while (hi - lo > 1) {
+      const int64_t mid = (lo + hi) >> 1;
+      if (a.row_ptr[mid] <= q) lo = mid;
+      else hi = mid;
+    }
+    t = lo;
+  }
+  for (; q < qb; ++t) {
+    const int64_t rend = a.row_ptr[t + 1], end = min(rend, qb);
     double acc = 0.0;
-    for (int64_t base = lo; base < hi; base += 32) {
-      const int nblk = (int)min((int64_t)32, hi - base);
-      const int xc = lane < nblk ? a.col[base + lane] * m : 0;
-      const double* kb = a.K + base * mm + e;
-      for (int u0 = 0; u0 < nblk; u0 += UN * per) {
-        double kv[UN], xv[UN];
+    for (int64_t base = q; base < end; base += 32) {
+      const int nblk = (int)min((int64_t)32, end - base);
+      const int xc = lane < nblk ? a.col[base + lane] * M : 0;
+      const double* kb = a.K + base * MM + sub * MM + e;
+      const double* xk = x + k;
+      int u0 = 0;
+      for (; u0 + GK_UN * PER <= nblk; u0 += GK_UN * PER) {
+        double kv[GK_UN], xv[GK_UN];
 #pragma unroll
-        for (int u = 0; u < UN; ++u) {
-          const int q = u0 + u * per + sub;
-          const int xo = __shfl_sync(0xffffffffu, xc, q & 31);
-          const bool on = sub < per && q < nblk;
-          kv[u] = on ? kb[q * mm] : 0.0;
-          xv[u] = on ? __ldcg(x + xo + k) : 0.0;
+        for (int u = 0; u < GK_UN; ++u) {
+          kv[u] = kb[(u0 + u * PER) * MM];
+          xv[u] = __ldcg(xk + __shfl_sync(0xffffffffu, xc, u0 + u * PER + sub));
         }
 #pragma unroll
-        for (int u = 0; u < UN; ++u) acc = fma(kv[u], xv[u], acc);
+        for (int u = 0; u < GK_UN; ++u) acc = fma(kv[u], xv[u], acc);
+      }
+      for (; u0 < nblk; u0 += 4 * PER) {
+        double kv[4], xv[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const int p = u0 + u * PER + sub;
+          const int xo = __shfl_sync(0xffffffffu, xc, p & 31);
+          const bool on = p < nblk;
+          kv[u] = on ? kb[(u0 + u * PER) * MM] : 0.0;
+          xv[u] = on ? __ldcg(xk + xo) : 0.0;
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) acc = fma(kv[u], xv[u], acc);
       }
     }
-    // the two blocks' shares, then the row sums over k
-    if (per == 2) acc += __shfl_down_sync(0xffffffffu, acc, 16);
+    if (PER == 2) acc += __shfl_down_sync(0xffffffffu, acc, 16);
     double s = 0.0;
-    for (int kk = 0; kk < m; ++kk) s += __shfl_sync(0xffffffffu, acc, (lane < m ? lane * m : 0) + kk);
-    if (lane < m) y[t * m + lane] = b ? b[t * m + lane] - s : s;
+#pragma unroll
+    for (int kk = 0; kk < M; ++kk) s += __shfl_sync(0xffffffffu, acc, (lane < M ? lane * M : 0) + kk);
+    if (q == a.row_ptr[t] && end == rend) {
+      if (lane < M) y[t * M + lane] = b ? b[t * M + lane] - s : s;
+    } else {
+      const int slot = q == qa ? 0 : 1;
+      if (lane < M) sh.psum[warp][slot][lane] = s;
+      if (lane == 0) sh.prow[warp][slot] = (int)(t - t0);
+    }
+    q = end;
   }
+  __syncthreads();
+  if (threadIdx.x < M) {                                   // rows shared by warps, in warp order
+    int cur = -1;
+    double v = 0.0;
+    for (int w = 0; w < 2 * GK_WARPS; ++w) {
+      const int r = sh.prow[w >> 1][w & 1];
+      if (r < 0) continue;
+      if (r != cur) {
+        if (cur >= 0) y[(t0 + cur) * M + threadIdx.x] = b ? b[(t0 + cur) * M + threadIdx.x] - v : v;
+        cur = r;
+        v = 0.0;
+      }
+      v += sh.psum[w >> 1][w & 1][threadIdx.x];
+    }
+    if (cur >= 0) y[(t0 + cur) * M + threadIdx.x] = b ? b[(t0 + cur) * M + threadIdx.x] - v : v;
+  }
+  __syncthreads();
+}
+__device__ __forceinline__ void spmv_rows(const GmresArgs& a, GmresShared& sh, const double* x, double* y,
+                                          const double* b, int64_t t0, int64_t t1) {
+  if (a.m == 5) spmv_rows_m<5>(a, sh, x, y, b, t0, t1);
+  else spmv_rows_m<4>(a, sh, x, y, b, t0, t1);
 }
 
-// y = M^-1 y on the CTA's rows (block Jacobi) or on all rows (BILU(0), barriers inside).
-__device__ __forceinline__ bool precondition(const GmresArgs& a, GmresShared& sh, double* y, int64_t t0, int64_t t1,
-                                             unsigned& round) {
-  const int tid = threadIdx.x;
+// z = M^-1 y on the CTA's rows: block Jacobi, or BILU(0) in place on all rows of y (other
+// CTAs work on this one's rows: barriers inside, y read through L2) and then copied.
+__device__ __forceinline__ bool precondition(const GmresArgs& a, GmresShared& sh, double* y, double* z, int64_t t0,
+                                             int64_t t1, unsigned& round) {
+  const int tid = threadIdx.x, m = a.m;
+  const int64_t i0 = t0 * m, i1 = t1 * m;
   if (a.colours == 0) {
-    __syncthreads();
-    const int m = a.m;
-    for (int64_t t = t0 + tid; t < t1; t += GK_THREADS) {
-      double xs[5];
-      for (int k = 0; k < m; ++k) xs[k] = y[t * m + k];
-      for (int i = 0; i < m; ++i) {
-        double s = 0.0;
-        for (int k = 0; k < m; ++k) s = fma(a.Dinv[(t * m + i) * m + k], xs[k], s);
-        y[t * m + i] = s;
-      }
+    for (int64_t i = i0 + tid; i < i1; i += GK_THREADS) {
+      const int64_t t = i / m;
+      double s = 0.0;
+#pragma unroll
+      for (int k = 0; k < 5; ++k)
+        if (k < m) s = fma(a.Dinv[i * m + k], y[t * m + k], s);
+      z[i] = s;
     }
     __syncthreads();
     return true;
@@ -370,7 +434,21 @@ __device__ __forceinline__ bool precondition(const GmresArgs& a, GmresShared& sh
     for (int64_t r = a.cptr[c] + w0; r < a.cptr[c + 1]; r += nw) bilu_row<false>(a.m, a.B, a.B.rows[r], y);
     if (!grid_barrier(a, sh, round)) return false;
   }
+  for (int64_t i = i0 + tid; i < i1; i += GK_THREADS) z[i] = __ldcg(y + i);
+  __syncthreads();
   return true;
+}
+
+// First trace node of CTA b: the rows are split by blocks of K.
+__device__ __forceinline__ int64_t first_row(const GmresArgs& a, int b) {
+  const int64_t want = a.row_ptr[a.T] * b / (int)gridDim.x;
+  int64_t lo = 0, hi = a.T;
+  while (lo < hi) {
+    const int64_t mid = (lo + hi) >> 1;
+    if (a.row_ptr[mid] < want) lo = mid + 1;
+    else hi = mid;
+  }
+  return lo;
 }
 
 __global__ void __launch_bounds__(GK_THREADS, 1) k_gmres(GmresArgs a) {
@@ -378,21 +456,20 @@ __global__ void __launch_bounds__(GK_THREADS, 1) k_gmres(GmresArgs a) {
   const int tid = threadIdx.x;
   const int m = a.m;
   const int64_t n = a.T * m;
-  const int64_t t0 = a.T * blockIdx.x / gridDim.x, t1 = a.T * (blockIdx.x + 1) / gridDim.x;
+  const int64_t t0 = first_row(a, blockIdx.x), t1 = blockIdx.x + 1 == gridDim.x ? a.T : first_row(a, blockIdx.x + 1);
   const int64_t i0 = t0 * m, i1 = t1 * m;
   unsigned round = 0;
-  // own rows of w: BILU(0) has other CTAs write them, so they are read through L2 then
-  auto own = [&](const double* p) { return a.colours ? __ldcg(p) : *p; };
   // x0 = 0, r0 = M^-1 R
   for (int64_t i = i0 + tid; i < i1; i += GK_THREADS) {
     a.dU[i] = 0.0;
     a.w[i] = a.R[i];
   }
+  __syncthreads();
   // own rows of x <- s (x - sum_{v < nv} h[v] V_v)
   auto subtract = [&](int nv, const double* h, double* x, double s) {
     for (int64_t i = i0 + tid; i < i1; i += GK_THREADS) {
       double t = x[i];
-#pragma unroll 4
+#pragma unroll 8
       for (int v = 0; v < nv; ++v) t = fma(-h[v], a.V[(int64_t)v * n + i], t);
       x[i] = s * t;
     }
@@ -401,10 +478,8 @@ __global__ void __launch_bounds__(GK_THREADS, 1) k_gmres(GmresArgs a) {
   double beta0 = 0.0, relres = 0.0;
   bool first = true, alive = true;
   while (alive) {
-    if (!first) spmv_rows(a, a.dU, a.w, a.R, t0, t1);
-    if (!(alive = precondition(a, sh, a.w, t0, t1, round))) break;
-    for (int64_t i = i0 + tid; i < i1; i += GK_THREADS) a.V[i] = own(a.w + i);
-    __syncthreads();
+    if (!first) spmv_rows(a, sh, a.dU, a.w, a.R, t0, t1);
+    if (!(alive = precondition(a, sh, a.w, a.V, t0, t1, round))) break;
     dot_parts(a, sh, 1, a.V, n, a.V, i0, i1);
     if (!(alive = grid_barrier(a, sh, round))) break;
     sum_parts(a, sh, 1, sh.h1);
@@ -423,14 +498,44 @@ __global__ void __launch_bounds__(GK_THREADS, 1) k_gmres(GmresArgs a) {
       for (int i = tid; i < GK_R1; i += GK_THREADS) sh.g[i] = i == 0 ? beta : 0.0;
     }
     if (!(alive = grid_barrier(a, sh, round))) break;
+    // Hessenberg column c: earlier rotations applied, a new one formed, g rotated,
+    // |g_{c+1}| / beta0 the residual estimate
+    auto givens = [&](int c) {
+      const double hn = sh.hn;
+      double a0 = sh.h1[0] + sh.h2[0];
+      for (int i = 0; i < c; ++i) {
+        const double a1 = sh.h1[i + 1] + sh.h2[i + 1];
+        sh.H[i][c] = sh.cs[i] * a0 + sh.sn[i] * a1;
+        a0 = -sh.sn[i] * a0 + sh.cs[i] * a1;
+      }
+      const double r = hypot(a0, hn);
+      const double cc = r > 0.0 ? a0 / r : 1.0, sn = r > 0.0 ? hn / r : 0.0;
+      sh.cs[c] = cc;
+      sh.sn[c] = sn;
+      sh.H[c][c] = r;
+      const double gc = sh.g[c];
+      sh.g[c + 1] = -sn * gc;
+      sh.g[c] = cc * gc;
+      sh.rel = fabs(sh.g[c + 1]) / beta0;
+      sh.done = (sh.rel <= a.rtol || hn == 0.0) ? 1 : 0;
+    };
     int j = 0;
-    for (; j < a.restart && total < a.max_iter; ++j, ++total) {
+    for (;;) {
+      // one thread closes step j - 1 while the others start on K v_j: the stopping test
+      // costs at most a product that is not used
+      const bool more = j < a.restart && total < a.max_iter;
+      if (j > 0 && tid >= GK_THREADS - 32) {
+        if (tid == GK_THREADS - 32) givens(j - 1);
+        __syncwarp();
+      }
+      if (more) spmv_rows(a, sh, a.V + (int64_t)j * n, a.w, nullptr, t0, t1);
+      else __syncthreads();
+      if (j > 0) {
+        relres = sh.rel;
+        if (sh.done || !more) break;
+      }
       double* vn = a.V + (int64_t)(j + 1) * n;
-      spmv_rows(a, a.V + (int64_t)j * n, a.w, nullptr, t0, t1);
-      if (!(alive = precondition(a, sh, a.w, t0, t1, round))) break;
-      // the candidate lives in vn's own rows from here on
-      for (int64_t i = i0 + tid; i < i1; i += GK_THREADS) vn[i] = own(a.w + i);
-      __syncthreads();
+      if (!(alive = precondition(a, sh, a.w, vn, t0, t1, round))) break;
       // iterated classical Gram-Schmidt: two passes, the second with |w|^2 beside the
       // products (V_{j+1} is w itself), which gives the norm of the orthogonalised
       // vector, |w|^2 - |h2|^2, without another barrier
@@ -451,8 +556,9 @@ __global__ void __launch_bounds__(GK_THREADS, 1) k_gmres(GmresArgs a) {
         if (tid == 0) {
           // a second pass that still removes much of w would cancel here: sum again then
           sh.again = hn2 < 0.25 * w2;
-          sh.hn = hn2 > 0.0 ? sqrt(hn2) : 0.0;
-          sh.scale = sh.again ? 1.0 : (hn2 > 0.0 ? 1.0 / sh.hn : 0.0);
+          const double r = hn2 > 0.0 ? 1.0 / sqrt(hn2) : 0.0;
+          sh.hn = hn2 * r;
+          sh.scale = sh.again ? 1.0 : r;
         }
       }
       __syncthreads();
@@ -470,31 +576,9 @@ __global__ void __launch_bounds__(GK_THREADS, 1) k_gmres(GmresArgs a) {
         const double s = sh.scale;
         for (int64_t i = i0 + tid; i < i1; i += GK_THREADS) vn[i] *= s;
       }
-      barrier_arrive(a);
-      if (tid == 0) {
-        // Hessenberg column j: earlier rotations applied, a new one formed, g rotated,
-        // |g_{j+1}| / beta0 the residual estimate
-        const double hn = sh.hn;
-        double a0 = sh.h1[0] + sh.h2[0];
-        for (int i = 0; i < j; ++i) {
-          const double a1 = sh.h1[i + 1] + sh.h2[i + 1];
-          sh.H[i][j] = sh.cs[i] * a0 + sh.sn[i] * a1;
-          a0 = -sh.sn[i] * a0 + sh.cs[i] * a1;
-        }
-        const double r = hypot(a0, hn);
-        const double c = r > 0.0 ? a0 / r : 1.0, sn = r > 0.0 ? hn / r : 0.0;
-        sh.cs[j] = c;
-        sh.sn[j] = sn;
-        sh.H[j][j] = r;
-        const double gj = sh.g[j];
-        sh.g[j + 1] = -sn * gj;
-        sh.g[j] = c * gj;
-        sh.rel = fabs(sh.g[j + 1]) / beta0;
-        sh.done = (sh.rel <= a.rtol || hn == 0.0) ? 1 : 0;
-      }
-      if (!(alive = barrier_wait(a, sh, round))) break;   // vn complete; publishes rel and done in the CTA
-      relres = sh.rel;
-      if (sh.done) { ++j; ++total; break; }
+      if (!(alive = grid_barrier(a, sh, round))) break;   // v_{j+1} complete
+      ++j;
+      ++total;
     }
     if (!alive) break;
     // y = H(0:j, 0:j)^-1 g (upper triangular, column by column), x += V y
