@@ -273,6 +273,24 @@ struct iedg_mesh {
 
 namespace iedg {
 
+#ifdef __CUDACC__
+// Face part of the u-row of boundary node a, component i, from the face projections
+// fb[i][f][tn] (3D): node a lies on face 2r where its coordinate r is 0 and on face
+// 2r + 1 where it is p, at index tn over its two other coordinates in order.
+__device__ __forceinline__ double face_part(const Dims& dm, const double* fb, int i, int a) {
+  const int np1 = dm.np1, Nfn1 = np1 * np1;
+  const int c3[3] = {a % np1, (a / np1) % np1, a / (np1 * np1)};
+  double s = 0.0;
+  for (int f = 0; f < 6; ++f) {
+    const int r = f >> 1;
+    if (c3[r] != ((f & 1) ? np1 - 1 : 0)) continue;
+    const int tn = r == 0 ? c3[1] + np1 * c3[2] : (r == 1 ? c3[0] + np1 * c3[2] : c3[0] + np1 * c3[1]);
+    s += fb[((size_t)i * 6 + f) * Nfn1 + tn];
+  }
+  return s;
+}
+#endif
+
 inline int idiv_up(int a, int b) { return (a + b - 1) / b; }
 
 // kernels (launchers)
