@@ -378,88 +378,328 @@ __device__ __forceinline__ void flux_jacobians(const double* u, const double (*q
   }
 }
 
-// ------------------------------------------------------------------ point kernel
-// One CTA per element.  jac = false: residual at (u, q).  jac = true: Jacobians at
-// (u, q) into PointJac, right-hand sides -R_u(u, q*), -Rhat(u, q*) into the last
-// column of the bordered element matrix.
-// JAC is a compile-time choice so that the residual form carries none of the Jacobian
-// code's registers and local arrays (it runs at a higher occupancy).
-// Bound by the FP64 pipe (two FMAs a clock and SM).  Two thirds of its work were multiplications
-// with zero tangents and dense projections: in the passes over q everything that depends on u
-// alone is a double, and the 3D projections go one direction at a time, as in the refinement's
-// operator.  Jacobian form at 3D p = 3, 4,096 elements 11.9 -> 8.8 ms, residual form 4.7 -> 2.8 ms.
-template <int D, int STAB, bool JAC>
-__global__ void k_points(Dims dm, Phys ph, RefTables ref, Geo G, PointJac PJ,
-                         const int64_t* __restrict__ etrace, const double* __restrict__ U,
-                         const double* __restrict__ Q, const double* __restrict__ QS,
-                         const double* __restrict__ UH, const double* __restrict__ UREF,
-                         double* __restrict__ RU, double* __restrict__ RHAT, double* __restrict__ RHS,
-                         int64_t rhs_es, int64_t rhs_rs, TraceTab tt, int nodal) {
-  constexpr int M = D + 2;
-  constexpr bool jac = JAC;
-  extern __shared__ double sm[];
-  const int64_t e = blockIdx.x;
-  const int tid = threadIdx.x, nth = blockDim.x;
-  const int Np = dm.Np, Nq = dm.Nq, Nb = dm.Nb, Nfp = dm.Nfp, Nfq = dm.Nfq, Nfn = dm.Nfn;
-  double* su = sm;                         // [Np][M]
-  double* sq = su + Np * M;                // [Np][M][D]
-  double* sqs = JAC ? sq + Np * M * D : sq; // [Np][M][D]  (q* for the right-hand side; residual form: q)
-  double* sur = sq + 2 * Np * M * D;       // [Np][M]
-  double* suh = sur + Np * M;              // [Nb][M]
-  double* fvol = su + nodal;               // [M][D][Nq]
-  double* mvol = fvol + M * D * Nq;        // [M][Nq]
-  double* fsur = mvol + M * Nq;            // [M][Nfp]
-  double* ftr = fsur + M * Nfp;            // [M][Nfp]  flux of the trace rows (bhat on boundary faces)
-  const bool has_ref = UREF != nullptr && ph.alpha != 0.0;
-  for (int i = tid; i < Np * M; i += nth) {
-    su[i] = U[e * Np * M + i];
-    sur[i] = has_ref ? UREF[e * Np * M + i] : 0.0;
-  }
-  for (int i = tid; i < Np * M * D; i += nth) {
-    sq[i] = Q[e * Np * M * D + i];
-    if (JAC) sqs[i] = QS[e * Np * M * D + i];
-  }
-  const int nbe = tt.nb ? tt.nb[e] : Nb;         // trace slots of this element
-  for (int i = tid; i < nbe * M; i += nth) {
-    int s = i / M, k = i % M;
-    suh[i] = UH[etrace[e * Nb + s] * M + k];
+// ------------------------------------------------------------------ point kernels
+// One CTA per element each.  k_point_res: the residual at (u, q), or at (u, q*) with the
+// opposite sign into the right-hand sides of the bordered element matrices.  k_point_jac:
+// the Jacobians at (u, q) into PointJac.  Two kernels, so that neither carries the other's
+// gradient at the points, shared arrays and registers.
+// Bound by the FP64 pipe (two FMAs a clock and SM).  What cut its work: in the passes over q
+// everything that depends on u alone is a double; in 3D the projections, and the interpolation
+// where its rounding is free, go one direction at a time.  A warp takes 32 volume points or 32
+// face points, whichever comes next in one list, so that in small elements the two run side by
+// side.  3D p = 3, 4,096 elements: residual 4.7 -> 1.3 ms, Jacobians with their right-hand
+// sides 11.9 -> 7.2 ms (mixed forms 8.4); 2D p = 2, 64 elements: residual 28 -> 20 us.
+
+// One-direction-at-a-time interpolation of F nodal fields to the volume points (3D):
+// field(a, f) at the nodes -> S1 (x) -> S2 (y); the z sums are left to the point's thread.
+// Fields are fastest, their stride FS odd: conflict-free both over f and over the points.
+template <class Field>
+__device__ __forceinline__ void interpolate_xy(const Dims& dm, const RefTables& ref, int F, int FS, double* S1,
+                                               double* S2, Field field) {
+  const int np1 = dm.np1, nq1 = dm.nq1;
+  for (int idx = threadIdx.x; idx < F * nq1 * np1 * np1; idx += blockDim.x) {
+    const int f = idx % F, t = idx / F, gx = t % nq1, ayz = t / nq1;
+    double s = 0.0;
+    for (int ax = 0; ax < np1; ++ax) s = fma(ref.L1[gx * np1 + ax], field(ax + np1 * ayz, f), s);
+    S1[t * FS + f] = s;
   }
   __syncthreads();
-  const size_t jvs = (size_t)(1 + D) * D * Nq;    // stride of one (i,k) pair in Jv
-  const size_t jfs = (size_t)(1 + D) * Nfp;
-  // ---- volume points
-  for (int g = tid; g < Nq; g += nth) {
-    double u[M], q[M][D], qr[M][D], du[M];
+  for (int idx = threadIdx.x; idx < F * nq1 * nq1 * np1; idx += blockDim.x) {
+    const int f = idx % F, t = idx / F, gx = t % nq1, gy = (t / nq1) % nq1, az = t / (nq1 * nq1);
+    double s = 0.0;
+    for (int ay = 0; ay < np1; ++ay)
+      s = fma(ref.L1[gy * np1 + ay], S1[(gx + nq1 * (ay + np1 * az)) * FS + f], s);
+    S2[t * FS + f] = s;
+  }
+  __syncthreads();
+}
+
+// u, q at volume point g: from S2, or (null) by the dense sum over the nodes
+template <int D>
+__device__ __forceinline__ void volume_state(const Dims& dm, const RefTables& ref, int g, const double* su,
+                                             const double* sq, const double* S2, int FS, double* u,
+                                             double (*q)[D]) {
+  constexpr int M = D + 2;
 #pragma unroll
-    for (int i = 0; i < M; ++i) {
-      u[i] = 0; du[i] = 0;
+  for (int i = 0; i < M; ++i) {
+    u[i] = 0;
 #pragma unroll
-      for (int j = 0; j < D; ++j) { q[i][j] = 0; qr[i][j] = 0; }
-    }
-    const double* phi = ref.Phi + (size_t)g * Np;
-    for (int a = 0; a < Np; ++a) {
-      double ph_a = phi[a];
+    for (int j = 0; j < D; ++j) q[i][j] = 0;
+  }
+  if (D == 3 && S2) {
+    const int np1 = dm.np1, nq2 = dm.nq1 * dm.nq1, gxy = g % nq2, gz = g / nq2;
+    for (int az = 0; az < np1; ++az) {
+      const double l = ref.L1[gz * np1 + az];
+      const double* src = S2 + (size_t)(gxy + nq2 * az) * FS;
 #pragma unroll
       for (int i = 0; i < M; ++i) {
-        u[i] += ph_a * su[a * M + i];
-        if (has_ref) du[i] += ph_a * (su[a * M + i] - sur[a * M + i]);
+        u[i] = fma(l, src[i], u[i]);
 #pragma unroll
-        for (int j = 0; j < D; ++j) {
-          if (JAC) q[i][j] += ph_a * sq[(a * M + i) * D + j];
-          qr[i][j] += ph_a * sqs[(a * M + i) * D + j];
-        }
+        for (int j = 0; j < D; ++j) q[i][j] = fma(l, src[M + i * D + j], q[i][j]);
       }
     }
+    return;
+  }
+  const double* phi = ref.Phi + (size_t)g * dm.Np;
+  for (int a = 0; a < dm.Np; ++a) {
+    const double ph_a = phi[a];
+#pragma unroll
+    for (int i = 0; i < M; ++i) {
+      u[i] += ph_a * su[a * M + i];
+#pragma unroll
+      for (int j = 0; j < D; ++j) q[i][j] += ph_a * sq[(a * M + i) * D + j];
+    }
+  }
+}
+
+// u, q and the trace state uh at face point fp
+template <int D>
+__device__ __forceinline__ void face_state(const Dims& dm, const RefTables& ref, const TraceTab& tt, int64_t e,
+                                           int fp, const double* su, const double* sq, const double* suh,
+                                           double* u, double (*q)[D], double* uh) {
+  constexpr int M = D + 2;
+  const int f = fp / dm.Nfq;
+#pragma unroll
+  for (int i = 0; i < M; ++i) {
+    u[i] = 0; uh[i] = 0;
+#pragma unroll
+    for (int j = 0; j < D; ++j) q[i][j] = 0;
+  }
+  const double* phi = ref.PhiF + (size_t)fp * dm.Np;
+  for (int t = 0; t < dm.Nfn; ++t) {
+    const int a = ref.fnode[f * dm.Nfn + t];
+    const double ph_a = phi[a];
+#pragma unroll
+    for (int i = 0; i < M; ++i) {
+      u[i] += ph_a * su[a * M + i];
+      if (!tt.nfs) uh[i] += ph_a * suh[ref.slot[a] * M + i];
+#pragma unroll
+      for (int j = 0; j < D; ++j) q[i][j] += ph_a * sq[(a * M + i) * D + j];
+    }
+  }
+  if (tt.nfs) {
+    // trace basis of this face from the element's table
+    const int cnt = tt.nfs[e * dm.nf + f];
+    const int* fsf = tt.fs + ((size_t)e * dm.nf + f) * tt.NFS;
+    const double* mu = tt.muf + (((size_t)e * dm.nf + f) * dm.Nfq + (fp - f * dm.Nfq)) * tt.NFS;
+    for (int j = 0; j < cnt; ++j)
+#pragma unroll
+      for (int i = 0; i < M; ++i) uh[i] += mu[j] * suh[fsf[j] * M + i];
+  }
+}
+
+// nodal u, q and the trace nodes of element e into shared memory
+__device__ __forceinline__ void load_nodal(const Dims& dm, const TraceTab& tt, const int64_t* etrace, int64_t e,
+                                           const double* U, const double* Q, const double* UH, double* su,
+                                           double* sq, double* suh) {
+  const int m = dm.m, nu = dm.Np * m, nq = nu * dm.d;
+  const int nbe = tt.nb ? tt.nb[e] : dm.Nb;
+  for (int i = threadIdx.x; i < nbe * m; i += blockDim.x) suh[i] = UH[etrace[e * dm.Nb + i / m] * m + i % m];
+  for (int i = threadIdx.x; i < nu; i += blockDim.x) su[i] = U[e * nu + i];
+  for (int i = threadIdx.x; i < nq; i += blockDim.x) sq[i] = Q[e * nq + i];
+}
+
+template <int D, int STAB>
+__global__ void k_point_jac(Dims dm, Phys ph, RefTables ref, Geo G, PointJac PJ,
+                            const int64_t* __restrict__ etrace, const double* __restrict__ U,
+                            const double* __restrict__ Q, const double* __restrict__ UH, TraceTab tt, int FS) {
+  constexpr int M = D + 2;
+  extern __shared__ double sm[];
+  const int64_t e = blockIdx.x;
+  const int Np = dm.Np, Nq = dm.Nq, Nfp = dm.Nfp, Nfq = dm.Nfq;
+  double* su = sm;                         // [Np][M]
+  double* sq = su + Np * M;                // [Np][M][D]
+  double* suh = sq + Np * M * D;           // [Nb][M]
+  double* S2 = FS ? suh + dm.Nb * M : nullptr;
+  load_nodal(dm, tt, etrace, e, U, Q, UH, su, sq, suh);
+  __syncthreads();
+  if (D == 3 && FS)
+    interpolate_xy(dm, ref, M * (1 + D), FS, S2 + dm.nq1 * dm.nq1 * dm.np1 * FS, S2,
+                   [&](int a, int f) { return f < M ? su[a * M + f] : sq[a * M * D + f - M]; });
+  const size_t jvs = (size_t)(1 + D) * D * Nq;    // stride of one (i,k) pair in Jv
+  const size_t jfs = (size_t)(1 + D) * Nfp;
+  const int lane = threadIdx.x & 31, nvw = (Nq + 31) / 32, nw = nvw + (Nfp + 31) / 32;
+  for (int w32 = threadIdx.x >> 5; w32 < nw; w32 += blockDim.x >> 5) {
+  // ---- volume points
+  const int g = w32 * 32 + lane, fp = g - nvw * 32;
+  if (w32 < nvw && g < Nq) {
+    double u[M], q[M][D];
+    volume_state<D>(dm, ref, g, su, sq, S2, FS, u, q);
     const double w = G.wdet[e * Nq + g];
     double Ji[D][D];
 #pragma unroll
     for (int r = 0; r < D; ++r)
 #pragma unroll
       for (int j = 0; j < D; ++j) Ji[r][j] = G.Jinv[((e * Nq + g) * D + r) * D + j];
-    double F[M][D];
-    ns_flux<D, double, double>(u, qr, ph, F);
+    double* jv = PJ.Jv + (size_t)e * M * M * jvs;
+    float* jv32 = PJ.Jv32 ? PJ.Jv32 + (size_t)e * M * M * jvs : nullptr;
+    // entry c of pair (i, k): -w sum_j Ji[r][j] dF_ij/d(unknown), c = r for u, D + l D + r for q_l
+    auto put = [&](int c0, const Dual<M> (*Fd)[D]) {
 #pragma unroll
-    for (int i = 0; i < M; ++i) {
+      for (int i = 0; i < M; ++i)
+#pragma unroll
+        for (int k = 0; k < M; ++k) {
+          double* o = jv + (size_t)(i * M + k) * jvs;
+#pragma unroll
+          for (int r = 0; r < D; ++r) {
+            double s = 0;
+#pragma unroll
+            for (int j = 0; j < D; ++j) s += Ji[r][j] * Fd[i][j].t[k];
+            o[(size_t)(c0 + r) * Nq + g] = -w * s;
+            if (jv32) jv32[(size_t)(i * M + k) * jvs + (size_t)(c0 + r) * Nq + g] = (float)(-w * s);
+          }
+        }
+    };
+    flux_jacobians<D>(u, q, ph, [&](const Dual<M> (*Fd)[D]) { put(0, Fd); },
+                      [&](int l, const Dual<M> (*Fd)[D]) { put(D + l * D, Fd); });
+  }
+  // ---- face points
+  if (w32 >= nvw && fp < Nfp) {
+    double u[M], uh[M], q[M][D];
+    face_state<D>(dm, ref, tt, e, fp, su, sq, suh, u, q, uh);
+    const double wf = G.fw[e * Nfp + fp];
+    double n[D];
+#pragma unroll
+    for (int j = 0; j < D; ++j) n[j] = G.fn[(e * Nfp + fp) * D + j];
+    double lam = 0.0;
+    if constexpr (STAB == 0) lam = lf_lambda<D, double>(uh, n, ph);
+    Dual<M> ud[M];
+#pragma unroll
+    for (int k = 0; k < M; ++k) { ud[k] = mkconst<M>(uh[k]); ud[k].t[k] = 1.0; }
+    // d/duhat of the stabilisation term: LF  dlambda/duhat (u - uh) - lambda I;
+    // Roe  d/duhat [ |A_n(uh)| (u - uh) ] by duals (includes - |A_n|)
+    Dual<M> lamd = mkconst<M>(0.0);
+    Dual<M> gd[M];
+    if constexpr (STAB == 1) {
+      Dual<M> dd[M];
+#pragma unroll
+      for (int i = 0; i < M; ++i) dd[i] = mkconst<M>(u[i]) - ud[i];
+      roe_apply<D, Dual<M>>(ud, dd, n, ph, gd);
+      // dfhat/du = S: its columns S e_k
+#pragma unroll 1
+      for (int k = 0; k < M; ++k) {
+        double ek[M], sk[M];
+#pragma unroll
+        for (int i = 0; i < M; ++i) ek[i] = (i == k) ? 1.0 : 0.0;
+        roe_apply<D, double>(uh, ek, n, ph, sk);
+#pragma unroll
+        for (int i = 0; i < M; ++i) {
+          const size_t o = ((size_t)(e * M + i) * M + k) * Nfp + fp;
+          PJ.Su[o] = wf * sk[i];
+          if (PJ.Su32) PJ.Su32[o] = (float)(wf * sk[i]);
+        }
+      }
+    } else {
+      lamd = lf_lambda<D, Dual<M>>(ud, n, ph);
+    }
+    double* jf = PJ.Jf + (size_t)e * M * M * jfs;
+    float* jf32 = PJ.Jf32 ? PJ.Jf32 + (size_t)e * M * M * jfs : nullptr;
+    // entry 0 of pair (i, k): the stabilisation's derivative + dfhat/du n; entry 1 + l:
+    // dfhat/dq_l n
+    flux_jacobians<D>(
+        uh, q, ph,
+        [&](const Dual<M> (*Fd)[D]) {
+#pragma unroll
+          for (int i = 0; i < M; ++i)
+#pragma unroll
+            for (int k = 0; k < M; ++k) {
+              double s = STAB == 1 ? gd[i].t[k] : lamd.t[k] * (u[i] - uh[i]) - (i == k ? lam : 0.0);
+#pragma unroll
+              for (int j = 0; j < D; ++j) s += Fd[i][j].t[k] * n[j];
+              jf[(size_t)(i * M + k) * jfs + fp] = wf * s;
+              if (jf32) jf32[(size_t)(i * M + k) * jfs + fp] = (float)(wf * s);
+            }
+        },
+        [&](int l, const Dual<M> (*Fd)[D]) {
+#pragma unroll
+          for (int i = 0; i < M; ++i)
+#pragma unroll
+            for (int k = 0; k < M; ++k) {
+              double t = 0;
+#pragma unroll
+              for (int j = 0; j < D; ++j) t += Fd[i][j].t[k] * n[j];
+              jf[(size_t)(i * M + k) * jfs + (size_t)(1 + l) * Nfp + fp] = wf * t;
+              if (jf32) jf32[(size_t)(i * M + k) * jfs + (size_t)(1 + l) * Nfp + fp] = (float)(wf * t);
+            }
+        });
+    PJ.lamw[e * Nfp + fp] = wf * lam;
+    if (PJ.lamw32) PJ.lamw32[e * Nfp + fp] = (float)(wf * lam);
+    const int fk = tt.fkind ? tt.fkind[e * dm.nf + fp / Nfq] : kFaceInterior;
+    if (fk != kFaceInterior) {
+      double bval[M];
+      boundary_point<D, STAB>(fk, uh, u, n, wf, ph, 0.0, true, PJ, e, fp, Nfp, bval);
+    }
+  }
+  }
+}
+
+template <int D, int STAB>
+__global__ void k_point_res(Dims dm, Phys ph, RefTables ref, Geo G, PointJac PJ,
+                            const int64_t* __restrict__ etrace, const double* __restrict__ U,
+                            const double* __restrict__ Q, const double* __restrict__ UH,
+                            const double* __restrict__ UREF, double* __restrict__ RU, double* __restrict__ RHAT,
+                            double* __restrict__ RHS, int64_t rhs_es, int64_t rhs_rs, TraceTab tt, int FS,
+                            int work) {
+  constexpr int M = D + 2;
+  const bool jac = RHS != nullptr;
+  extern __shared__ double sm[];
+  const int64_t e = blockIdx.x;
+  const int tid = threadIdx.x, nth = blockDim.x;
+  const int Np = dm.Np, Nq = dm.Nq, Nb = dm.Nb, Nfp = dm.Nfp, Nfq = dm.Nfq;
+  const bool has_ref = UREF != nullptr && ph.alpha != 0.0;
+  double* su = sm;                         // [Np][M]
+  double* sq = su + Np * M;                // [Np][M][D]
+  double* suh = sq + Np * M * D;           // [Nb][M]
+  double* sdu = suh + Nb * M;              // [Np][M]  u - u_ref (only with a reference state)
+  double* S2 = sdu + (has_ref ? Np * M : 0);   // 3D: fields after two directions
+  double* fvol = su + work;                // [M][D][Nq]  (S1 before)
+  double* fsur = fvol + M * D * Nq;        // [M][Nfp]
+  double* mvol = fsur + M * Nfp;           // [M][Nq]   (only with a reference state)
+  double* ftr = mvol + (has_ref ? M * Nq : 0); // [M][Nfp]  flux of the trace rows (bhat on boundary faces; mixed orders)
+  load_nodal(dm, tt, etrace, e, U, Q, UH, su, sq, suh);
+  if (has_ref)
+    for (int i = tid; i < Np * M; i += nth) sdu[i] = U[e * Np * M + i] - UREF[e * Np * M + i];
+  const int nbe = tt.nb ? tt.nb[e] : Nb;         // trace slots of this element
+  __syncthreads();
+  if constexpr (D == 3)
+    interpolate_xy(dm, ref, M * (has_ref ? 2 + D : 1 + D), FS, fvol, S2, [&](int a, int f) {
+      return f < M ? su[a * M + f] : (f < M * (1 + D) ? sq[a * M * D + f - M] : sdu[a * M + f - M * (1 + D)]);
+    });
+  const int lane = tid & 31, nvw = (Nq + 31) / 32, nw = nvw + (Nfp + 31) / 32;
+  for (int w32 = tid >> 5; w32 < nw; w32 += nth >> 5) {
+  // ---- volume points
+  const int g = w32 * 32 + lane, fp = g - nvw * 32;
+  if (w32 < nvw && g < Nq) {
+    double u[M], q[M][D];
+    volume_state<D>(dm, ref, g, su, sq, D == 3 ? S2 : nullptr, FS, u, q);
+    const double w = G.wdet[e * Nq + g];
+    if (has_ref) {
+      double du[M];
+#pragma unroll
+      for (int i = 0; i < M; ++i) du[i] = 0;
+      if constexpr (D == 3) {
+        const int np1 = dm.np1, nq2 = dm.nq1 * dm.nq1, gxy = g % nq2, gz = g / nq2;
+        for (int az = 0; az < np1; ++az)
+#pragma unroll
+          for (int i = 0; i < M; ++i)
+            du[i] = fma(ref.L1[gz * np1 + az], S2[(size_t)(gxy + nq2 * az) * FS + M * (1 + D) + i], du[i]);
+      } else {
+        for (int a = 0; a < Np; ++a)
+#pragma unroll
+          for (int i = 0; i < M; ++i) du[i] += ref.Phi[(size_t)g * Np + a] * sdu[a * M + i];
+      }
+#pragma unroll
+      for (int i = 0; i < M; ++i) mvol[i * Nq + g] = ph.alpha * w * du[i];
+    }
+    double Ji[D][D];
+#pragma unroll
+    for (int r = 0; r < D; ++r)
+#pragma unroll
+      for (int j = 0; j < D; ++j) Ji[r][j] = G.Jinv[((e * Nq + g) * D + r) * D + j];
+    double F[M][D];
+    ns_flux<D, double, double>(u, q, ph, F);
+#pragma unroll
+    for (int i = 0; i < M; ++i)
 #pragma unroll
       for (int r = 0; r < D; ++r) {
         double s = 0;
@@ -467,166 +707,50 @@ __global__ void k_points(Dims dm, Phys ph, RefTables ref, Geo G, PointJac PJ,
         for (int j = 0; j < D; ++j) s += Ji[r][j] * F[i][j];
         fvol[(i * D + r) * Nq + g] = -w * s;
       }
-      mvol[i * Nq + g] = has_ref ? ph.alpha * w * du[i] : 0.0;
-    }
-    if constexpr (JAC) {
-      double* jv = PJ.Jv + (size_t)e * M * M * jvs;
-      float* jv32 = PJ.Jv32 ? PJ.Jv32 + (size_t)e * M * M * jvs : nullptr;
-      // entry c of pair (i, k): -w sum_j Ji[r][j] dF_ij/d(unknown), c = r for u, D + l D + r for q_l
-      auto put = [&](int c0, const Dual<M> (*Fd)[D]) {
-#pragma unroll
-        for (int i = 0; i < M; ++i)
-#pragma unroll
-          for (int k = 0; k < M; ++k) {
-            double* o = jv + (size_t)(i * M + k) * jvs;
-#pragma unroll
-            for (int r = 0; r < D; ++r) {
-              double s = 0;
-#pragma unroll
-              for (int j = 0; j < D; ++j) s += Ji[r][j] * Fd[i][j].t[k];
-              o[(size_t)(c0 + r) * Nq + g] = -w * s;
-              if (jv32) jv32[(size_t)(i * M + k) * jvs + (size_t)(c0 + r) * Nq + g] = (float)(-w * s);
-            }
-          }
-      };
-      flux_jacobians<D>(u, q, ph, [&](const Dual<M> (*Fd)[D]) { put(0, Fd); },
-                        [&](int l, const Dual<M> (*Fd)[D]) { put(D + l * D, Fd); });
-    }
   }
   // ---- face points
-  for (int fp = tid; fp < Nfp; fp += nth) {
-    const int f = fp / Nfq;
-    double u[M], uh[M], q[M][D], qr[M][D];
-#pragma unroll
-    for (int i = 0; i < M; ++i) {
-      u[i] = 0; uh[i] = 0;
-#pragma unroll
-      for (int j = 0; j < D; ++j) { q[i][j] = 0; qr[i][j] = 0; }
-    }
-    const double* phi = ref.PhiF + (size_t)fp * Np;
-    for (int t = 0; t < Nfn; ++t) {
-      int a = ref.fnode[f * Nfn + t];
-      double ph_a = phi[a];
-#pragma unroll
-      for (int i = 0; i < M; ++i) {
-        u[i] += ph_a * su[a * M + i];
-        if (!tt.nfs) uh[i] += ph_a * suh[ref.slot[a] * M + i];
-#pragma unroll
-        for (int j = 0; j < D; ++j) {
-          if (JAC) q[i][j] += ph_a * sq[(a * M + i) * D + j];
-          qr[i][j] += ph_a * sqs[(a * M + i) * D + j];
-        }
-      }
-    }
-    if (tt.nfs) {
-      // trace basis of this face from the element's table
-      const int cnt = tt.nfs[e * dm.nf + f];
-      const int* fsf = tt.fs + ((size_t)e * dm.nf + f) * tt.NFS;
-      const double* mu = tt.muf + (((size_t)e * dm.nf + f) * Nfq + (fp - f * Nfq)) * tt.NFS;
-      for (int j = 0; j < cnt; ++j)
-#pragma unroll
-        for (int i = 0; i < M; ++i) uh[i] += mu[j] * suh[fsf[j] * M + i];
-    }
+  if (w32 >= nvw && fp < Nfp) {
+    double u[M], uh[M], q[M][D];
+    face_state<D>(dm, ref, tt, e, fp, su, sq, suh, u, q, uh);
     const double wf = G.fw[e * Nfp + fp];
     double n[D];
 #pragma unroll
     for (int j = 0; j < D; ++j) n[j] = G.fn[(e * Nfp + fp) * D + j];
     double F[M][D];
-    ns_flux<D, double, double>(uh, qr, ph, F);
+    ns_flux<D, double, double>(uh, q, ph, F);
     // stabilisation S (u - uh): lambda I (Lax-Friedrichs) or |A_n(uh)| (Roe-type)
-    double sdu[M];
+    double stab[M];
     double lam = 0.0;
     if constexpr (STAB == 1) {
       double dd[M];
 #pragma unroll
       for (int i = 0; i < M; ++i) dd[i] = u[i] - uh[i];
-      roe_apply<D, double>(uh, dd, n, ph, sdu);
+      roe_apply<D, double>(uh, dd, n, ph, stab);
     } else {
       lam = lf_lambda<D, double>(uh, n, ph);
 #pragma unroll
-      for (int i = 0; i < M; ++i) sdu[i] = lam * (u[i] - uh[i]);
+      for (int i = 0; i < M; ++i) stab[i] = lam * (u[i] - uh[i]);
     }
 #pragma unroll
     for (int i = 0; i < M; ++i) {
-      double s = sdu[i];
+      double s = stab[i];
 #pragma unroll
       for (int j = 0; j < D; ++j) s += F[i][j] * n[j];
       fsur[i * Nfp + fp] = wf * s;
     }
-    if (jac) {
-      Dual<M> ud[M];
-#pragma unroll
-      for (int k = 0; k < M; ++k) { ud[k] = mkconst<M>(uh[k]); ud[k].t[k] = 1.0; }
-      // d/duhat of the stabilisation term: LF  dlambda/duhat (u - uh) - lambda I;
-      // Roe  d/duhat [ |A_n(uh)| (u - uh) ] by duals (includes - |A_n|)
-      Dual<M> lamd = mkconst<M>(0.0);
-      Dual<M> gd[M];
-      if constexpr (STAB == 1) {
-        Dual<M> dd[M];
-#pragma unroll
-        for (int i = 0; i < M; ++i) dd[i] = mkconst<M>(u[i]) - ud[i];
-        roe_apply<D, Dual<M>>(ud, dd, n, ph, gd);
-        // dfhat/du = S: its columns S e_k
-#pragma unroll 1
-        for (int k = 0; k < M; ++k) {
-          double ek[M], sk[M];
-#pragma unroll
-          for (int i = 0; i < M; ++i) ek[i] = (i == k) ? 1.0 : 0.0;
-          roe_apply<D, double>(uh, ek, n, ph, sk);
-#pragma unroll
-          for (int i = 0; i < M; ++i) {
-            const size_t o = ((size_t)(e * M + i) * M + k) * Nfp + fp;
-            PJ.Su[o] = wf * sk[i];
-            if (PJ.Su32) PJ.Su32[o] = (float)(wf * sk[i]);
-          }
-        }
-      } else {
-        lamd = lf_lambda<D, Dual<M>>(ud, n, ph);
-      }
-      double* jf = PJ.Jf + (size_t)e * M * M * jfs;
-      float* jf32 = PJ.Jf32 ? PJ.Jf32 + (size_t)e * M * M * jfs : nullptr;
-      // entry 0 of pair (i, k): the stabilisation's derivative + dfhat/du n; entry 1 + l:
-      // dfhat/dq_l n
-      flux_jacobians<D>(
-          uh, q, ph,
-          [&](const Dual<M> (*Fd)[D]) {
-#pragma unroll
-            for (int i = 0; i < M; ++i)
-#pragma unroll
-              for (int k = 0; k < M; ++k) {
-                double s = STAB == 1 ? gd[i].t[k] : lamd.t[k] * (u[i] - uh[i]) - (i == k ? lam : 0.0);
-#pragma unroll
-                for (int j = 0; j < D; ++j) s += Fd[i][j].t[k] * n[j];
-                jf[(size_t)(i * M + k) * jfs + fp] = wf * s;
-                if (jf32) jf32[(size_t)(i * M + k) * jfs + fp] = (float)(wf * s);
-              }
-          },
-          [&](int l, const Dual<M> (*Fd)[D]) {
-#pragma unroll
-            for (int i = 0; i < M; ++i)
-#pragma unroll
-              for (int k = 0; k < M; ++k) {
-                double t = 0;
-#pragma unroll
-                for (int j = 0; j < D; ++j) t += Fd[i][j].t[k] * n[j];
-                jf[(size_t)(i * M + k) * jfs + (size_t)(1 + l) * Nfp + fp] = wf * t;
-                if (jf32) jf32[(size_t)(i * M + k) * jfs + (size_t)(1 + l) * Nfp + fp] = (float)(wf * t);
-              }
-          });
-      PJ.lamw[e * Nfp + fp] = wf * lam;
-      if (PJ.lamw32) PJ.lamw32[e * Nfp + fp] = (float)(wf * lam);
-    }
+    if (!tt.nfs) continue;                 // uniform order: the trace rows take fsur
     // trace rows: fhat on interior faces, the boundary flux on domain-boundary faces
-    const int fk = tt.fkind ? tt.fkind[e * dm.nf + f] : kFaceInterior;
+    const int fk = tt.fkind ? tt.fkind[e * dm.nf + fp / Nfq] : kFaceInterior;
     if (fk != kFaceInterior) {
       double bval[M];
-      boundary_point<D, STAB>(fk, uh, u, n, wf, ph, fsur[(M - 1) * Nfp + fp] / wf, jac, PJ, e, fp, Nfp, bval);
+      boundary_point<D, STAB>(fk, uh, u, n, wf, ph, fsur[(M - 1) * Nfp + fp] / wf, false, PJ, e, fp, Nfp, bval);
 #pragma unroll
       for (int i = 0; i < M; ++i) ftr[i * Nfp + fp] = bval[i];
     } else {
 #pragma unroll
       for (int i = 0; i < M; ++i) ftr[i * Nfp + fp] = fsur[i * Nfp + fp];
     }
+  }
   }
   __syncthreads();
   // ---- projections onto the test functions
@@ -706,7 +830,7 @@ __global__ void k_points(Dims dm, Phys ph, RefTables ref, Geo G, PointJac PJ,
       else if (RU) RU[(e * Np + a) * M + i] = s;
     }
     if (!tt.nfs) {                         // uniform order: a trace row is its node's face part
-      for (int si = tid; si < nbe * M; si += nth) {
+      for (int si = nth - 1 - tid; si < nbe * M; si += nth) {
         const int s = si / M, i = si % M;
         const double t = face_part(dm, fb, i, ref.bnode[s]);
         if (jac) rhs_e[((int64_t)dm.nu + (int64_t)i * nbe + s) * rrs] = sgn * t;
@@ -719,7 +843,7 @@ __global__ void k_points(Dims dm, Phys ph, RefTables ref, Geo G, PointJac PJ,
     const int a = ai / M, i = ai % M;
     double s = 0;
     for (int g = 0; g < Nq; ++g) {
-      double t = ref.Phi[(size_t)g * Np + a] * mvol[i * Nq + g];
+      double t = has_ref ? ref.Phi[(size_t)g * Np + a] * mvol[i * Nq + g] : 0.0;
 #pragma unroll
       for (int r = 0; r < D; ++r) t += ref.Dxi[((size_t)r * Nq + g) * Np + a] * fvol[(i * D + r) * Nq + g];
       s += t;
@@ -730,7 +854,7 @@ __global__ void k_points(Dims dm, Phys ph, RefTables ref, Geo G, PointJac PJ,
     else if (RU) RU[(e * Np + a) * M + i] = s;
   }
   }
-  for (int si = tid; si < nbe * M; si += nth) {
+  for (int si = nth - 1 - tid; si < nbe * M; si += nth) {
     const int s = si / M, i = si % M;
     double t = 0;
     if (tt.nfs) {
@@ -805,31 +929,46 @@ cudaError_t launch_points(iedg_mesh* M, const double* u, const double* q, const 
                           const double* uhat, const double* u_ref, bool jacobians, double* r_u,
                           double* rhat, cudaStream_t st) {
   const Dims& dm = M->dm;
-  // nodal arrays, later (3D) the projection stages; fluxes at the points
-  size_t nodal = (size_t)dm.Np * dm.m * (2 + 2 * dm.d) + dm.Nb * dm.m;
-  const size_t points = (size_t)dm.m * dm.d * dm.Nq + dm.m * dm.Nq + 2 * dm.m * dm.Nfp;
-  if (dm.d == 3) {
-    const size_t np1 = dm.np1, nq1 = dm.nq1,
-                 stages = dm.m * (3 * nq1 * nq1 * np1 + 2 * nq1 * np1 * np1 + 6 * nq1 * np1 + 6 * np1 * np1);
-    nodal = nodal > stages ? nodal : stages;
-  }
-  const size_t smem = sizeof(double) * (nodal + points);
   const int threads = 128;
+  const size_t nodal = (size_t)dm.Np * dm.m * (1 + dm.d) + (size_t)dm.Nb * dm.m;
+  const size_t np1 = dm.np1, nq1 = dm.nq1;
+  cudaError_t err;
+  if (jacobians) {
+    // mixed forms: K depends on the FP32 roundings of these Jacobians, so u and q at the
+    // points keep the order of the dense sum; FP64 forms in 3D sum one direction at a time
+    const int FS = dm.d == 3 && M->precision == 0 ? (dm.m * (1 + dm.d)) | 1 : 0;
+    const size_t smem = sizeof(double) * (nodal + FS * (nq1 * nq1 * np1 + nq1 * np1 * np1));
+    auto kern = dm.d == 2 ? (M->ph.stab == 1 ? k_point_jac<2, 1> : k_point_jac<2, 0>)
+                          : (M->ph.stab == 1 ? k_point_jac<3, 1> : k_point_jac<3, 0>);
+    err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (err != cudaSuccess) return err;
+    kern<<<(unsigned)M->E, threads, smem, st>>>(dm, M->ph, M->ref, M->geo, M->pj, M->etrace, u, q, uhat, M->tt, FS);
+    err = cudaGetLastError();
+    if (err != cudaSuccess) return err;
+  }
+  const bool has_ref = u_ref && M->ph.alpha != 0.0;
+  const int FS = dm.d == 3 ? (dm.m * (1 + dm.d + (has_ref ? 1 : 0))) | 1 : 0;
+  // nodal arrays and S2, later (3D) the projection stages; S1, later the fluxes at the points
+  size_t work = nodal + (has_ref ? (size_t)dm.Np * dm.m : 0) + FS * nq1 * nq1 * np1;
+  size_t points = (size_t)dm.m * dm.d * dm.Nq + (has_ref ? dm.m * dm.Nq : 0) +
+                  (size_t)(M->tt.nfs ? 2 : 1) * dm.m * dm.Nfp;
+  if (dm.d == 3) {
+    const size_t stages = dm.m * (3 * nq1 * nq1 * np1 + 2 * nq1 * np1 * np1 + 6 * nq1 * np1 + 6 * np1 * np1);
+    work = work > stages ? work : stages;
+    points = points > FS * nq1 * np1 * np1 ? points : FS * nq1 * np1 * np1;
+  }
+  const size_t smem = sizeof(double) * (work + points);
   // right-hand sides: column n of the FP64 bordered matrix, or the FP64 rhs array
   // (ragged FP64 matrices: the kernel adds the element's offset and n_e to S itself)
-  double* rhs = M->precision == 0 ? (M->tt.soff ? M->S : M->S + dm.n) : M->rhs64;
+  double* rhs = !jacobians ? nullptr : (M->precision == 0 ? (M->tt.soff ? M->S : M->S + dm.n) : M->rhs64);
   int64_t es = M->precision == 0 ? (int64_t)dm.n * dm.ld : dm.n;
   int64_t rs = M->precision == 0 ? dm.ld : 1;
-  auto pick = [&](auto j) {
-    constexpr bool J = decltype(j)::value;
-    return dm.d == 2 ? (M->ph.stab == 1 ? k_points<2, 1, J> : k_points<2, 0, J>)
-                     : (M->ph.stab == 1 ? k_points<3, 1, J> : k_points<3, 0, J>);
-  };
-  auto kern = jacobians ? pick(std::true_type{}) : pick(std::false_type{});
-  cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  auto kern = dm.d == 2 ? (M->ph.stab == 1 ? k_point_res<2, 1> : k_point_res<2, 0>)
+                        : (M->ph.stab == 1 ? k_point_res<3, 1> : k_point_res<3, 0>);
+  err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (err != cudaSuccess) return err;
-  kern<<<(unsigned)M->E, threads, smem, st>>>(dm, M->ph, M->ref, M->geo, M->pj, M->etrace, u, q, qs, uhat, u_ref,
-                                              r_u, rhat, rhs, es, rs, M->tt, (int)nodal);
+  kern<<<(unsigned)M->E, threads, smem, st>>>(dm, M->ph, M->ref, M->geo, M->pj, M->etrace, u, jacobians ? qs : q,
+                                              uhat, u_ref, r_u, rhat, rhs, es, rs, M->tt, FS, (int)work);
   return cudaGetLastError();
 }
 

@@ -14,7 +14,7 @@ pytestmark = pytest.mark.gpu
 @pytest.mark.parametrize("p,extra,ref", [(1, 1, True), (1, 3, False), (2, 1, False), (2, 3, True), (3, 3, True),
                                          (4, 1, True), (4, 3, False)])
 def test_residual_with_other_quadrature_rules(p, extra, ref):
-    mesh = W.structured_mesh(3, (2, 1, 1), p, mapping=W.stretched_mapping(5, ratio=3.0))
+    mesh = W.structured_mesh(3, 2, p, mapping=W.stretched_mapping(5, ratio=3.0))
     st = W.make_state(mesh, W.taylor_green_field(0.2), 3, noise=0.01, uref_shift=0.01)
     prm = dict(gamma=1.4, Pr=0.72, Re=200.0, Minf=0.2, alpha=W.dirk_alpha())
     uref = st.u_ref if ref else None
