@@ -519,7 +519,8 @@ __global__ void k_point_jac(Dims dm, Phys ph, RefTables ref, Geo G, PointJac PJ,
   const size_t jvs = (size_t)(1 + D) * D * Nq;    // stride of one (i,k) pair in Jv
   const size_t jfs = (size_t)(1 + D) * Nfp;
   const int lane = threadIdx.x & 31, nvw = (Nq + 31) / 32, nw = nvw + (Nfp + 31) / 32;
-  for (int w32 = threadIdx.x >> 5; w32 < nw; w32 += blockDim.x >> 5) {
+  const int wpb = blockDim.x >> 5;                // blockIdx.y: a share of the list
+  for (int w32 = blockIdx.y * wpb + (threadIdx.x >> 5); w32 < nw; w32 += gridDim.y * wpb) {
   // ---- volume points
   const int g = w32 * 32 + lane, fp = g - nvw * 32;
   if (w32 < nvw && g < Nq) {
@@ -875,7 +876,13 @@ __global__ void k_point_res(Dims dm, Phys ph, RefTables ref, Geo G, PointJac PJ,
   }
 }
 
+constexpr int64_t kSpread = 8 * 152;   // blocks of 128 threads that keep every SM evenly busy
+
 // q*[e][c][k][l] = sum_t H_l[c][t] uhat_k(t) - sum_b G_l[c][b] u_k(b)
+// One output a thread, an element's outputs over several blocks: a thread's chain of loads and
+// FMAs is as long as a row, and with one block per element a mesh of few large elements left
+// most of the chip idle behind it.  3D p = 4, 210 elements 0.48 -> 0.17 ms;
+// 175 elements of orders 2..4 0.80 -> 0.13 ms; 4,096 at p = 3 0.79 -> 0.77 (FP64 pipe).
 __global__ void k_lift(Dims dm, Geo G, const int64_t* __restrict__ etrace, const double* __restrict__ U,
                        const double* __restrict__ UH, double* __restrict__ QS, TraceTab tt) {
   extern __shared__ double sm[];
@@ -888,7 +895,8 @@ __global__ void k_lift(Dims dm, Geo G, const int64_t* __restrict__ etrace, const
   const int nbe = tt.nb ? tt.nb[e] : Nb;
   for (int i = tid; i < nbe * m; i += nth) suh[i] = UH[etrace[e * Nb + i / m] * m + i % m];
   __syncthreads();
-  for (int idx = tid; idx < Np * m * d; idx += nth) {
+  const int idx = blockIdx.y * nth + tid;
+  if (idx < Np * m * d) {
     int c = idx / (m * d), k = (idx / d) % m, l = idx % d;
     const double* gl = G.Gl + (((size_t)e * d + l) * Np + c) * Np;
     const double* hl = G.Hl + (((size_t)e * d + l) * Np + c) * Nb;
@@ -899,7 +907,8 @@ __global__ void k_lift(Dims dm, Geo G, const int64_t* __restrict__ etrace, const
   }
 }
 
-// R_q = M (q - q*), optionally rhoq = q - q*
+// R_q = M (q - q*), optionally rhoq = q - q*; small meshes over several blocks per element
+// (3D p = 4, 210 elements, both forms together 0.21 -> 0.12 ms).
 __global__ void k_rq(Dims dm, Geo G, const double* __restrict__ Q, const double* __restrict__ QS,
                      double* __restrict__ RQ, double* __restrict__ RHOQ) {
   extern __shared__ double sm[];
@@ -910,12 +919,12 @@ __global__ void k_rq(Dims dm, Geo G, const double* __restrict__ Q, const double*
   for (int i = tid; i < Np * w; i += nth) {
     double v = Q[e * Np * w + i] - QS[e * Np * w + i];
     dq[i] = v;
-    if (RHOQ) RHOQ[e * Np * w + i] = v;
+    if (RHOQ && blockIdx.y == 0) RHOQ[e * Np * w + i] = v;
   }
   __syncthreads();
   if (!RQ) return;
   const double* Ms = G.Mass + (size_t)e * Np * Np;
-  for (int idx = tid; idx < Np * w; idx += nth) {
+  for (int idx = blockIdx.y * nth + tid; idx < Np * w; idx += nth * gridDim.y) {
     int a = idx / w, c = idx % w;
     double s = 0;
     for (int b = 0; b < Np; ++b) s += Ms[a * Np + b] * dq[b * w + c];
@@ -942,7 +951,14 @@ cudaError_t launch_points(iedg_mesh* M, const double* u, const double* q, const 
                           : (M->ph.stab == 1 ? k_point_jac<3, 1> : k_point_jac<3, 0>);
     err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (err != cudaSuccess) return err;
-    kern<<<(unsigned)M->E, threads, smem, st>>>(dm, M->ph, M->ref, M->geo, M->pj, M->etrace, u, q, uhat, M->tt, FS);
+    // An element's warps over several blocks where the elements alone are too few to fill the
+    // chip evenly (below kSpread blocks): each block repeats the nodal loads (and, in FP64, the
+    // interpolation), which large meshes need not pay.  3D p = 4, 210 elements 1.0 -> 0.84 ms
+    // (FP32 1.34 -> 1.10); 175 elements of orders 2..4 1.9 -> 1.2 ms.
+    const int items = (dm.Nq + 31) / 32 + (dm.Nfp + 31) / 32, most = (items + threads / 32 - 1) / (threads / 32);
+    const int64_t want = (kSpread + M->E - 1) / M->E;
+    const dim3 grid((unsigned)M->E, (unsigned)(want < most ? want : most));
+    kern<<<grid, threads, smem, st>>>(dm, M->ph, M->ref, M->geo, M->pj, M->etrace, u, q, uhat, M->tt, FS);
     err = cudaGetLastError();
     if (err != cudaSuccess) return err;
   }
@@ -975,7 +991,8 @@ cudaError_t launch_points(iedg_mesh* M, const double* u, const double* q, const 
 cudaError_t launch_lift(iedg_mesh* M, const double* u, const double* uhat, double* qstar, cudaStream_t st) {
   const Dims& dm = M->dm;
   size_t smem = sizeof(double) * (size_t)(dm.Np + dm.Nb) * dm.m;
-  k_lift<<<(unsigned)M->E, 128, smem, st>>>(dm, M->geo, M->etrace, u, uhat, qstar, M->tt);
+  const dim3 grid((unsigned)M->E, (unsigned)idiv_up(dm.Np * dm.m * dm.d, 128));
+  k_lift<<<grid, 128, smem, st>>>(dm, M->geo, M->etrace, u, uhat, qstar, M->tt);
   return cudaGetLastError();
 }
 
@@ -983,7 +1000,9 @@ cudaError_t launch_rq(iedg_mesh* M, const double* q, const double* qs, double* r
                       cudaStream_t st) {
   const Dims& dm = M->dm;
   size_t smem = sizeof(double) * (size_t)dm.Np * dm.m * dm.d;
-  k_rq<<<(unsigned)M->E, 128, smem, st>>>(dm, M->geo, q, qs, r_q, rhoq);
+  const int64_t want = (kSpread + M->E - 1) / M->E, most = idiv_up(dm.Np * dm.m * dm.d, 128);
+  const dim3 grid((unsigned)M->E, r_q ? (unsigned)(want < most ? want : most) : 1u);
+  k_rq<<<grid, 128, smem, st>>>(dm, M->geo, q, qs, r_q, rhoq);
   return cudaGetLastError();
 }
 
