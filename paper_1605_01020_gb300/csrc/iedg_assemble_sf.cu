@@ -90,7 +90,7 @@ k_assemble_sf(Dims dm, Phys ph, RefTables ref, AsmTab<T> tb, T* __restrict__ S, 
     else lq = reinterpret_cast<const T*>(ref.LQ32);
     for (int idx = tid; idx < 25 * nq1; idx += SF_THREADS) sLQ[idx] = lq[idx];
   }
-  const T* mutab = nullptr;                    // [nf][Nfq][NFS] of this element (MIX)
+  const T* mutab = nullptr;                    // [nf][Nfq][NFS] of this element
   {
     if constexpr (sizeof(T) == 8) mutab = reinterpret_cast<const T*>(tt.muf);
     else mutab = reinterpret_cast<const T*>(tt.muf32);
