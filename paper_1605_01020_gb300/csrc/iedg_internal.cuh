@@ -333,9 +333,9 @@ cudaError_t launch_backsub(iedg_mesh* M, const double* duhat, double* du, double
                            cudaStream_t st);
 cudaError_t launch_solve_prep(iedg_mesh* M, cudaStream_t st);
 cudaError_t launch_refine(iedg_mesh* M, cudaStream_t st);
-// doubles of iedg_mesh::kpart
+// doubles of iedg_mesh::kpart: two halves of partial sums, result scalars, barrier
 constexpr int64_t kGmresMaxCtas = 512;
-constexpr int64_t kGmresScratch = (IEDG_MAX_RESTART + 1) * kGmresMaxCtas + 8;
+constexpr int64_t kGmresScratch = 2 * (IEDG_MAX_RESTART + 1) * kGmresMaxCtas + 8;
 // FP64 fallback of flagged elements on the mixed path (iedg_fallback.cu)
 constexpr int kFallbackSlots = 32;
 cudaError_t launch_fallback(iedg_mesh* M, cudaStream_t st);

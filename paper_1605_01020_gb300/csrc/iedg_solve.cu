@@ -210,7 +210,7 @@ struct GmresArgs {
   const int32_t* col;
   const double *K, *Dinv, *R;
   double *dU, *V, *w;           // V [restart + 1][T m], w [T m]
-  double* part;                 // partial sums [CTA][R1]
+  double* part;                 // partial sums [2][CTA][R1], the halves in turn (dot_parts)
   double* out;                  // iterations, relative residual
   unsigned* sync;               // [0] barrier count, [1] abort
   int restart, max_iter;
@@ -263,15 +263,27 @@ __device__ __forceinline__ bool grid_barrier(const GmresArgs& a, GmresShared& sh
   return barrier_wait(a, sh, round);
 }
 
+// Sums over the grid go through a.part: every CTA writes its own row (dot_parts), meets
+// the others at a grid barrier and reads all rows (sum_parts).  Successive sums alternate
+// between two halves (`turn`, the same in every thread of every CTA).  A row is written again
+// two sums later, so there is always the barrier of the sum in between: a CTA arrives there
+// only after it has read all rows of the earlier sum, and no CTA writes before all have
+// arrived.  (With one half, a CTA that leaves the barrier first could overwrite its row with
+// the next sum's while another has yet to read it.)
+__device__ __forceinline__ double* part_rows(const GmresArgs& a, unsigned turn) {
+  return a.part + (int64_t)(turn & 1u) * kGmresMaxCtas * GK_R1;
+}
+
 // out[v] = sum over the grid of part[cta][v], v < nv, in CTA order within a warp's share;
-// the same in every CTA.
-__device__ __forceinline__ void sum_parts(const GmresArgs& a, GmresShared& sh, int nv, double* out) {
+// the same in every CTA.  Ends the sum: the next one takes the other half.
+__device__ __forceinline__ void sum_parts(const GmresArgs& a, GmresShared& sh, int nv, double* out, unsigned& turn) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const double* part = part_rows(a, turn++);
   for (int v0 = 0; v0 < nv; v0 += 32) {
     double s = 0.0;
     if (v0 + lane < nv)
 #pragma unroll 10
-      for (int c = warp; c < (int)gridDim.x; c += GK_WARPS) s += __ldcg(a.part + (int64_t)c * GK_R1 + v0 + lane);
+      for (int c = warp; c < (int)gridDim.x; c += GK_WARPS) s += __ldcg(part + (int64_t)c * GK_R1 + v0 + lane);
     if (v0 + lane < nv) sh.red[warp][v0 + lane] = s;
   }
   __syncthreads();
@@ -287,7 +299,7 @@ __device__ __forceinline__ void sum_parts(const GmresArgs& a, GmresShared& sh, i
 // part[this CTA][v] = V[v] . w over the CTA's unknowns [i0, i1), v < nv: a warp per vector,
 // or several where there are more warps than vectors.
 __device__ __forceinline__ void dot_parts(const GmresArgs& a, GmresShared& sh, int nv, const double* V, int64_t n,
-                                          const double* w, int64_t i0, int64_t i1) {
+                                          const double* w, int64_t i0, int64_t i1, unsigned turn) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int segs = nv < GK_WARPS ? GK_WARPS / nv : 1;
   for (int it = warp; it < nv * segs; it += GK_WARPS) {
@@ -304,7 +316,7 @@ __device__ __forceinline__ void dot_parts(const GmresArgs& a, GmresShared& sh, i
   if (threadIdx.x < nv) {
     double s = 0.0;
     for (int k = 0; k < segs; ++k) s += sh.red[k][threadIdx.x];
-    __stcg(a.part + (int64_t)blockIdx.x * GK_R1 + threadIdx.x, s);
+    __stcg(part_rows(a, turn) + (int64_t)blockIdx.x * GK_R1 + threadIdx.x, s);
   }
 }
 
@@ -458,7 +470,7 @@ __global__ void __launch_bounds__(GK_THREADS, 1) k_gmres(GmresArgs a) {
   const int64_t n = a.T * m;
   const int64_t t0 = first_row(a, blockIdx.x), t1 = blockIdx.x + 1 == gridDim.x ? a.T : first_row(a, blockIdx.x + 1);
   const int64_t i0 = t0 * m, i1 = t1 * m;
-  unsigned round = 0;
+  unsigned round = 0, turn = 0;
   // x0 = 0, r0 = M^-1 R
   for (int64_t i = i0 + tid; i < i1; i += GK_THREADS) {
     a.dU[i] = 0.0;
@@ -480,9 +492,9 @@ __global__ void __launch_bounds__(GK_THREADS, 1) k_gmres(GmresArgs a) {
   while (alive) {
     if (!first) spmv_rows(a, sh, a.dU, a.w, a.R, t0, t1);
     if (!(alive = precondition(a, sh, a.w, a.V, t0, t1, round))) break;
-    dot_parts(a, sh, 1, a.V, n, a.V, i0, i1);
+    dot_parts(a, sh, 1, a.V, n, a.V, i0, i1, turn);
     if (!(alive = grid_barrier(a, sh, round))) break;
-    sum_parts(a, sh, 1, sh.h1);
+    sum_parts(a, sh, 1, sh.h1, turn);
     const double beta = sqrt(sh.h1[0]);
     if (first) {
       beta0 = beta;
@@ -539,14 +551,14 @@ __global__ void __launch_bounds__(GK_THREADS, 1) k_gmres(GmresArgs a) {
       // iterated classical Gram-Schmidt: two passes, the second with |w|^2 beside the
       // products (V_{j+1} is w itself), which gives the norm of the orthogonalised
       // vector, |w|^2 - |h2|^2, without another barrier
-      dot_parts(a, sh, j + 1, a.V, n, vn, i0, i1);
+      dot_parts(a, sh, j + 1, a.V, n, vn, i0, i1, turn);
       if (!(alive = grid_barrier(a, sh, round))) break;
-      sum_parts(a, sh, j + 1, sh.h1);
+      sum_parts(a, sh, j + 1, sh.h1, turn);
       subtract(j + 1, sh.h1, vn, 1.0);
       __syncthreads();
-      dot_parts(a, sh, j + 2, a.V, n, vn, i0, i1);
+      dot_parts(a, sh, j + 2, a.V, n, vn, i0, i1, turn);
       if (!(alive = grid_barrier(a, sh, round))) break;
-      sum_parts(a, sh, j + 2, sh.h2);
+      sum_parts(a, sh, j + 2, sh.h2, turn);
       if (tid < 32) {        // one warp: square roots and divisions would load the FP64 pipe
         double q = 0.0;
         for (int v = tid; v <= j; v += 32) q = fma(sh.h2[v], sh.h2[v], q);
@@ -565,9 +577,9 @@ __global__ void __launch_bounds__(GK_THREADS, 1) k_gmres(GmresArgs a) {
       subtract(j + 1, sh.h2, vn, sh.scale);
       if (sh.again) {
         __syncthreads();
-        dot_parts(a, sh, 1, vn, n, vn, i0, i1);
+        dot_parts(a, sh, 1, vn, n, vn, i0, i1, turn);
         if (!(alive = grid_barrier(a, sh, round))) break;
-        sum_parts(a, sh, 1, &sh.nrm2);
+        sum_parts(a, sh, 1, &sh.nrm2, turn);
         if (tid == 0) {
           sh.hn = sqrt(sh.nrm2);
           sh.scale = sh.nrm2 > 0.0 ? 1.0 / sh.hn : 0.0;
@@ -792,7 +804,7 @@ extern "C" int iedg_trace_solve(iedg_mesh* M, const double* K, const double* R, 
     SV_TRY((k_diag_inv<<<(unsigned)((T + 127) / 128), 128, 0, st>>>(m, T, M->row_ptr, M->col, K, M->dinv, M->dev_flag),
             cudaGetLastError()));
   // result scalars and the barrier's two words sit behind the partial sums
-  double* out = M->kpart + (int64_t)GK_R1 * kGmresMaxCtas;
+  double* out = M->kpart + 2 * (int64_t)GK_R1 * kGmresMaxCtas;
   unsigned* sync = reinterpret_cast<unsigned*>(out + 4);
   SV_TRY(cudaMemsetAsync(out, 0, 8 * sizeof(double), st));
   GmresArgs a{m, T, M->row_ptr, M->col, K, M->dinv, R, dU, M->kry, M->kry + (int64_t)GK_R1 * n, M->kpart, out, sync,
