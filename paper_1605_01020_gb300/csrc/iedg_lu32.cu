@@ -171,12 +171,12 @@ __device__ __forceinline__ void lu32_update(float* __restrict__ A, int ld, float
       float acc[8][8];
       const int ca = cc + 4 * tc, cb = ca + 64;
       if (rb + RT < r_hi) {
-        // 16 threads cover a row's four lines of the tile, eight rows each
-        const float* pf = A + (int64_t)(rb + RT + 8 * tr + (tc >> 1)) * ld + cc + 64 * (tc & 1);
-        if (rb + RT + 8 * tr + (tc >> 1) < r_hi) {
-          asm volatile("prefetch.global.L2 [%0];" ::"l"(pf));
-          asm volatile("prefetch.global.L2 [%0];" ::"l"(pf + 32));
-        }
+        // 16 threads cover a row's four lines of the tile, eight rows each; the tile's columns
+        // past the last one are in no row of this element (past the last row: in no matrix)
+        const int pr = rb + RT + 8 * tr + (tc >> 1), pc = cc + 64 * (tc & 1);
+        const float* pf = A + (int64_t)pr * ld + pc;
+        if (pr < r_hi && pc < c_hi) asm volatile("prefetch.global.L2 [%0];" ::"l"(pf));
+        if (pr < r_hi && pc + 32 < c_hi) asm volatile("prefetch.global.L2 [%0];" ::"l"(pf + 32));
       }
       const bool va = aligned && ca + 4 <= vlim, vb = aligned && cb + 4 <= vlim;
 #pragma unroll
