@@ -319,7 +319,10 @@ int iedg_set_schedule(iedg_mesh* mesh, const iedg_schedule* in);
  *                  MMAs in flight drain at the default limit and its TMEM is freed);
  *                  that element and every element the CTA still takes from the queue
  *                  come back IEDG_ELEM_TIMEOUT.
- * The settings stay until changed; {-1, 0, -1, 0} restores normal operation.
+ *   asm_wait_limit: the same for the waits of the FP64 assembly on the tensor cores (3D,
+ *                  degree 2..4): a wait that gives up leaves NaN in the matrices of that
+ *                  CTA's elements, which come back IEDG_ELEM_NONFINITE.
+ * The settings stay until changed; {-1, 0, -1, 0, 0} restores normal operation.
  * IEDG_ERR_INVALID_ARG for values out of range, IEDG_ERR_UNSUPPORTED for zero_row_elem
  * on meshes with mixed orders. */
 typedef struct {
@@ -327,7 +330,7 @@ typedef struct {
   int32_t zero_row;
   int32_t refine_iters;
   int32_t tc_wait_limit;
-  int32_t reserved;
+  int32_t asm_wait_limit;
 } iedg_fault_injection;
 int iedg_set_fault_injection(iedg_mesh* mesh, const iedg_fault_injection* f);
 

@@ -23,7 +23,8 @@
 //     tables' own digits when they are laid out; then the levels are joined in 96-bit
 //     integers, rounded once to FP64 and added to the element matrix.
 // Warps: 8 form and convert W and read the accumulators, one issues the MMAs, one the
-// copies; two CTAs per SM, so that one's conversion and results overlap the other's FP64.
+// copies; they meet at mbarriers, all waits bounded.  Two CTAs per SM, so that one's
+// conversion and results overlap the other's FP64.
 // Meshes with mixed orders have trace bases of their own: there the face terms come from
 // k_assemble_sf first and this kernel adds the volume terms.
 // Measured, all elements, sum-factorised on the FP64 pipe -> this kernel: 3D p = 3, 4096
@@ -58,7 +59,8 @@ __host__ __device__ constexpr int dg_face_chunks(int Nfp) { return (Nfp + 3 * DG
 __host__ __device__ constexpr int dg_vol_chunks(int Nq) { return (Nq + DG_GP - 1) / DG_GP; }
 
 struct DgShared {
-  uint64_t full[DG_RING], empty[DG_RING], bempty, dfull;
+  // table stage filled / read, right operands staged / read, accumulators complete / read, end
+  uint64_t full[DG_RING], empty[DG_RING], bfull, bempty, dfull, dread, drain;
   uint32_t tmem;
   int failed;
   int scol[DG_COLS];        // column of the bordered matrix, -1 = none
@@ -78,6 +80,7 @@ struct DgArgs {
   TraceTab tt;
   const int64_t* elist;           // list form: element of each slot
   int64_t n_el;
+  int wait_limit;                 // polls of a wait before it gives up
 };
 
 template <int NP1, bool MIX>
@@ -97,8 +100,11 @@ __global__ void __launch_bounds__(DG_THREADS, 2) k_assemble_dg(Dims dm, DgArgs a
   }
   if (tid == 0) {
     for (int i = 0; i < DG_RING; ++i) { tc::mbar_init(&sh.full[i], 1); tc::mbar_init(&sh.empty[i], 1); }
+    tc::mbar_init(&sh.bfull, DG_BUILD / 32);
     tc::mbar_init(&sh.bempty, 1);
     tc::mbar_init(&sh.dfull, 1);
+    tc::mbar_init(&sh.dread, DG_BUILD / 32);
+    tc::mbar_init(&sh.drain, 1);
     sh.failed = 0;
   }
   tc::fence_before_sync();
@@ -106,9 +112,12 @@ __global__ void __launch_bounds__(DG_THREADS, 2) k_assemble_dg(Dims dm, DgArgs a
   tc::fence_after_sync();
   const uint32_t tmem = sh.tmem;
   volatile int* failed = &sh.failed;
-  // bounded; once a wait has run out the others poll only once
+  // All roles meet at mbarriers and every wait on them is bounded.  Once one has run out the
+  // others poll only once: the copies and the MMAs stop (no stage is overwritten), what is in
+  // flight is waited for, and the build warps go through the tiles that are left writing NaN.
+  // Arrivals then no longer match the waits, which costs nothing: nobody waits for them.
   auto wait = [&](uint64_t* bar, uint32_t parity) {
-    if (!tc::mbar_wait(bar, parity & 1u, *failed ? 1 : kTcWaitLimit)) *failed = 1;
+    if (!tc::mbar_wait(bar, parity & 1u, *failed ? 1 : a.wait_limit)) *failed = 1;
   };
   // element, trace slots, first column and chunk range of tile `id`; false: nothing to do
   const int ch0 = MIX ? NFC : 0;
@@ -131,13 +140,14 @@ __global__ void __launch_bounds__(DG_THREADS, 2) k_assemble_dg(Dims dm, DgArgs a
     // ---- copies of the tables
     if (lane == 0) {
       uint32_t q = 0;
-      for (int64_t id = blockIdx.x; id < total; id += gridDim.x) {
+      for (int64_t id = blockIdx.x; id < total && !*failed; id += gridDim.x) {
         int64_t slot, e;
         int nb, c0, ch1;
         if (!tile_of(id, slot, e, nb, c0, ch1)) continue;
         for (int s = 3 * ch0; s < 3 * ch1; ++s, ++q) {
           const uint32_t st = q % DG_RING;
           if (q >= DG_RING) wait(&sh.empty[st], q / DG_RING - 1);
+          if (*failed) break;
           tc::mbar_expect_tx(&sh.full[st], DG_STEP_A);
           tc::bulk_g2s(ring + st * DG_STEP_A, a.ref.Vdig + (size_t)s * DG_STEP_A, DG_STEP_A, &sh.full[st]);
         }
@@ -148,23 +158,23 @@ __global__ void __launch_bounds__(DG_THREADS, 2) k_assemble_dg(Dims dm, DgArgs a
     }
   } else if (warp == 8) {
     // ---- MMAs
-    const uint64_t da0 = tc::desc_kmajor(tc::smem_u32(ring), 128, 256);
-    const uint64_t db0 = tc::desc_kmajor(tc::smem_u32(bbuf), 128, 256);
-    uint32_t q = 0, nwin = 0;
-    bool start = true;
-    for (int64_t id = blockIdx.x; id < total; id += gridDim.x) {
-      int64_t slot, e;
-      int nb, c0, ch1;
-      if (!tile_of(id, slot, e, nb, c0, ch1)) continue;
-      for (int ch = ch0; ch < ch1; ++ch) {
-        if (start && nwin > 0) asm volatile("bar.sync 2, 288;" ::: "memory");   // accumulators read
-        asm volatile("bar.sync 1, 288;" ::: "memory");                           // W of this chunk staged
-        tc::fence_after_sync();
-        const bool end = window_end(ch, ch1);
-        if (lane == 0) {
-          for (int r = 0; r < 3; ++r) {
-            const uint32_t st = (q + r) % DG_RING;
-            wait(&sh.full[st], (q + r) / DG_RING);
+    if (lane == 0) {
+      const uint64_t da0 = tc::desc_kmajor(tc::smem_u32(ring), 128, 256);
+      const uint64_t db0 = tc::desc_kmajor(tc::smem_u32(bbuf), 128, 256);
+      uint32_t q = 0, nch = 0, nwin = 0;
+      bool start = true;
+      for (int64_t id = blockIdx.x; id < total && !*failed; id += gridDim.x) {
+        int64_t slot, e;
+        int nb, c0, ch1;
+        if (!tile_of(id, slot, e, nb, c0, ch1)) continue;
+        for (int ch = ch0; ch < ch1; ++ch, ++nch) {
+          if (start && nwin > 0) wait(&sh.dread, nwin - 1);   // accumulators read
+          wait(&sh.bfull, nch);                               // W of this chunk staged
+          const bool end = window_end(ch, ch1);
+          for (int r = 0; r < 3 && !*failed; ++r, ++q) {
+            const uint32_t st = q % DG_RING;
+            wait(&sh.full[st], q / DG_RING);
+            if (*failed) break;
             tc::fence_after_sync();
 #pragma unroll
             for (int s = 0; s < dig::S; ++s)
@@ -173,21 +183,19 @@ __global__ void __launch_bounds__(DG_THREADS, 2) k_assemble_dg(Dims dm, DgArgs a
                            (start && r == 0 && s == 0) ? 0u : 1u);
             tc::mma_commit(&sh.empty[st]);
           }
+          if (*failed) break;
           tc::mma_commit(&sh.bempty);
           if (end) tc::mma_commit(&sh.dfull);
+          nwin += end;
+          start = end;
         }
-        __syncwarp();
-        q += 3;
-        nwin += end;
-        start = end;
+      }
+      if (q > 0) {       // no MMA in flight when the TMEM is freed
+        tc::mma_commit(&sh.drain);
+        tc::mbar_wait(&sh.drain, 0, kTcWaitLimit);
       }
     }
-    if (nwin > 0) {
-      asm volatile("bar.sync 2, 288;" ::: "memory");
-      // no MMA in flight when the TMEM is freed (done already unless a wait gave up)
-      if (lane == 0) tc::mbar_wait(&sh.dfull, (nwin - 1) & 1u, kTcWaitLimit);
-      __syncwarp();
-    }
+    __syncwarp();
   } else {
     // ---- right operands and results
     const int c = lane, gq = warp;                 // column of the tile, values 2 gq, 2 gq + 1 of every step
@@ -300,19 +308,22 @@ __global__ void __launch_bounds__(DG_THREADS, 2) k_assemble_dg(Dims dm, DgArgs a
         if (ch + 1 >= NFC && ch + 1 < ch1) fetch(ch + 1 - NFC);
         if (nch > 0) wait(&sh.bempty, nch - 1);                 // the MMAs have read the previous chunk
         const int em = face ? emF : emV;
+        if (!*failed) {
 #pragma unroll
-        for (int r = 0; r < 3; ++r) {
-          const unsigned long long v0 = dig::to_bytes(__double_as_longlong(w[r][0]), em);
-          const unsigned long long v1 = dig::to_bytes(__double_as_longlong(w[r][1]), em);
-          unsigned char* base = bbuf + r * DG_STEP_B + dg_off(c, 2 * gq);
+          for (int r = 0; r < 3; ++r) {
+            const unsigned long long v0 = dig::to_bytes(__double_as_longlong(w[r][0]), em);
+            const unsigned long long v1 = dig::to_bytes(__double_as_longlong(w[r][1]), em);
+            unsigned char* base = bbuf + r * DG_STEP_B + dg_off(c, 2 * gq);
 #pragma unroll
-          for (int s = 0; s < dig::S; ++s)
-            *reinterpret_cast<uint32_t*>(base + s * (DG_COLS * DG_GP * 2)) =
-                s < 4 ? dig::bf16_pair((uint32_t)(v0 >> 32), (uint32_t)(v1 >> 32), s)
-                      : dig::bf16_pair((uint32_t)v0, (uint32_t)v1, s);
+            for (int s = 0; s < dig::S; ++s)
+              *reinterpret_cast<uint32_t*>(base + s * (DG_COLS * DG_GP * 2)) =
+                  s < 4 ? dig::bf16_pair((uint32_t)(v0 >> 32), (uint32_t)(v1 >> 32), s)
+                        : dig::bf16_pair((uint32_t)v0, (uint32_t)v1, s);
+          }
         }
         tc::fence_proxy_async();
-        asm volatile("bar.arrive 1, 288;" ::: "memory");
+        __syncwarp();
+        if (lane == 0) tc::mbar_arrive(&sh.bfull);
         if (window_end(ch, ch1)) {
           wait(&sh.dfull, nwin++);
           tc::fence_after_sync();
@@ -363,7 +374,8 @@ __global__ void __launch_bounds__(DG_THREADS, 2) k_assemble_dg(Dims dm, DgArgs a
             }
           }
           tc::fence_before_sync();
-          asm volatile("bar.arrive 2, 288;" ::: "memory");
+          __syncwarp();
+          if (lane == 0) tc::mbar_arrive(&sh.dread);
         }
       }
     }
@@ -498,7 +510,8 @@ cudaError_t launch_assemble_dg(iedg_mesh* M, double* S, const int64_t* elist, in
   k_coef_exp<<<(unsigned)((nw * 32 + 255) / 256), 256, 0, st>>>(dm.Nq, dm.Nfp, tb, M->pj.ecoef, nw, elist);
   cudaError_t err = cudaGetLastError();
   if (err != cudaSuccess) return err;
-  const DgArgs a{tb, M->ref, M->pj.ecoef, M->geo.elift, elist ? M->rhs64 : nullptr, S, M->ph.alpha, M->tt, elist, n_el};
+  const DgArgs a{tb, M->ref, M->pj.ecoef, M->geo.elift, elist ? M->rhs64 : nullptr, S, M->ph.alpha, M->tt, elist, n_el,
+                 asm_wait_limit(M)};
   if (dm.p == 2) return dg_launch<3>(M, a, st);
   if (dm.p == 3) return dg_launch<4>(M, a, st);
   return dg_launch<5>(M, a, st);

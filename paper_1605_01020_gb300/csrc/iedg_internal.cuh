@@ -49,6 +49,7 @@ struct Fault {
   int zero_row = 0;
   int refine_iters = -1;        // correction steps of the refinement (-1 = kRefineMaxIter)
   int tc_wait_limit = 0;        // polls of a tensor-core completion wait (0 = kTcWaitLimit, -1 = none)
+  int asm_wait_limit = 0;       // the same for the waits of the FP64 digit assembly
 };
 constexpr int kTcWaitLimit = 1 << 26;
 
@@ -354,6 +355,10 @@ cudaError_t launch_backsub_mixed(iedg_mesh* M, const double* duhat, double* du, 
 inline int refine_iters(const iedg_mesh* M) { return M->fault.refine_iters >= 0 ? M->fault.refine_iters : 8; }
 inline int tc_wait_limit(const iedg_mesh* M) {
   return M->fault.tc_wait_limit > 0 ? M->fault.tc_wait_limit : (M->fault.tc_wait_limit < 0 ? 0 : kTcWaitLimit);
+}
+
+inline int asm_wait_limit(const iedg_mesh* M) {
+  return M->fault.asm_wait_limit > 0 ? M->fault.asm_wait_limit : (M->fault.asm_wait_limit < 0 ? 0 : kTcWaitLimit);
 }
 
 // refinement controls of the mixed path

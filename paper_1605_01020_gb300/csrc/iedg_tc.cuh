@@ -111,6 +111,11 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* mbar, uint32_t parity, int m
   return done != 0;
 }
 
+// The calling thread's arrival on mbar; its earlier writes are visible to who waits for the phase.
+__device__ __forceinline__ void mbar_arrive(uint64_t* mbar) {
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(mbar)) : "memory");
+}
+
 // The calling thread's arrival on mbar, announcing `bytes` of asynchronous copies that
 // complete on it.
 __device__ __forceinline__ void mbar_expect_tx(uint64_t* mbar, uint32_t bytes) {
