@@ -400,6 +400,7 @@ def run_ours(args, wl, rank, world, local_rank):
     # the FP64 handle and the step buffers are released before the other legs (the
     # largest workload, p=4 24^3, does not fit twice in HBM); K, R, du, dq stay for the
     # error of the mixed form
+    lu_tensor = mesh.get_schedule()["lu_tensor"]
     mesh.close()
     del q, rq, ru, rfl, du_in, uh_in, duh_in, hu, huh, hduh, hK, hR, hdu, hdq
     torch.cuda.empty_cache()
@@ -462,7 +463,7 @@ def run_ours(args, wl, rank, world, local_rank):
         if name == "assemble" and d == 3:
             roof["note"] = ("frac above 1: dense count of the definition (actual: the sum-factorised form's) over the "
                             "DFMA peak; the kernel contracts by exact digit products on the BF16 tensor cores")
-        if name == "lu_schur" and m * Np >= 64:
+        if name == "lu_schur" and lu_tensor:
             # FP64 updates as exact products of 8 x 8-bit digits on the BF16 tensor cores, the
             # 36 digit pairs of levels 0..7: above the DFMA peak without less precision
             bf16 = 36 * flops[name] / t_launch / 1e12

@@ -278,14 +278,15 @@ int iedg_trace_solve(iedg_mesh* mesh, const double* K, const double* R, double* 
  *   lu_tensor:     tensor cores (tcgen05, accumulation in tensor memory) in the partial LU.
  *                  FP64 path: the trailing updates as integer products of 8-bit digits of
  *                  the FP64 operands, summed exactly and joined to FP64 (the error of an
- *                  update is below that of the DFMA form).  1 = always; 0 = on elements
- *                  of at least 64 u-unknowns, where it is the faster form, DFMA updates
- *                  below.  Mixed path: 1 = the Schur complement K = D - W Z, TF32 operands
+ *                  update is below that of the DFMA form).  1 = that form; 0 = DFMA
+ *                  updates, at every size.  Mixed path: 1 = the Schur complement K = D - W Z, TF32 operands
  *                  split in high and low parts, three products ("3xTF32"); 2 (mixed FP32
  *                  form only) = every trailing update of the FP32 LU (3xTF32, 128 x 64
  *                  tiles accumulated in TMEM and subtracted from the trailing block by
- *                  reductions in L2); 0 = FFMA updates.  Default 0, except 2
- *                  for mixed FP32 handles of meshes with mixed orders.  Handles created with
+ *                  reductions in L2); 0 = FFMA updates.  Default: FP64 1 where the
+ *                  (largest) element has at least 64 u-unknowns, from where it is the
+ *                  faster form, 0 below; mixed 0, except 2 for FP32 handles of meshes
+ *                  with mixed orders.  Handles created with
  *                  IEDG_PRECISION_MIXED_TF32 or _MIXED_BF16 always take the tensor-core
  *                  form in their own operand precision (the schedule never changes
  *                  what is computed, only how).

@@ -536,16 +536,22 @@ static int create_impl(const iedg_mesh_desc* D, cudaStream_t st, iedg_mesh* M) {
   return IEDG_OK;
 }
 
-// Storage precision (FP64 or FP32 element matrices), the Schur GEMM's operands on the
-// mixed path and the default LU form, the fastest measured on GB300: FP64 DFMA; FP32
-// with FFMA updates on uniform meshes, with every trailing update on the tensor cores
-// on meshes of mixed orders (the order-4 elements' long panels favour it).
-static void set_precision(iedg_mesh* M, int precision, bool mixed_orders) {
+// Storage precision (FP64 or FP32 element matrices) and the Schur GEMM's operands on the
+// mixed path.
+static void set_precision(iedg_mesh* M, int precision) {
   M->precision = precision == IEDG_PRECISION_FP64 ? 0 : 1;
   M->schur_in = precision == IEDG_PRECISION_MIXED_TF32   ? kSchurTf32
                 : precision == IEDG_PRECISION_MIXED_BF16 ? kSchurBf16
                                                          : kSchurFp32;
-  M->sched.lu_tensor = M->precision == 0 ? 0 : (M->schur_in != kSchurFp32 ? 1 : (mixed_orders ? 2 : 0));
+}
+
+// The default LU form, the fastest measured on GB300: FP64 in digit form from
+// LU64_TC_MIN_NU u-unknowns (of the largest element), DFMA below; FP32 with FFMA updates
+// on uniform meshes, with every trailing update on the tensor cores on meshes of mixed
+// orders (the order-4 elements' long panels favour it).  Needs the sizes M->dm.
+static void default_lu_form(iedg_mesh* M, bool mixed_orders) {
+  M->sched.lu_tensor = M->precision == 0 ? (M->dm.nu >= LU64_TC_MIN_NU ? 1 : 0)
+                                         : (M->schur_in != kSchurFp32 ? 1 : (mixed_orders ? 2 : 0));
 }
 
 static int check_desc(const iedg_mesh_desc* D, bool mixed) {
@@ -589,7 +595,8 @@ extern "C" int iedg_create_mesh(const iedg_mesh_desc* D, void* stream, iedg_mesh
   M = new iedg_mesh();
   M->dm = make_dims(D->dim, D->order, D->quad_extra);
   M->ph = Phys{D->gamma, D->Pr, D->Re, D->alpha, D->stab, {0, 0, 0, 0, 0}};
-  set_precision(M, D->precision, false);
+  set_precision(M, D->precision);
+  default_lu_form(M, false);
   M->mass_scaled = (D->flags & IEDG_FLAG_MASS_SCALING) != 0;
   M->E = D->n_elem;
   M->T = D->n_trace;
@@ -715,6 +722,7 @@ static int create_mixed_impl(const iedg_mesh_desc* D, const int32_t* ord, const 
   pd.nu = *std::max_element(in_nu.begin(), in_nu.end());
   pd.ld = *std::max_element(in_ld.begin(), in_ld.end());
   M->dm = pd;
+  default_lu_form(M, true);
   // pattern and gather lists (user element order)
   {
     std::vector<const int64_t*> lists(E);
@@ -919,7 +927,7 @@ extern "C" int iedg_create_mesh_bc(const iedg_mesh_desc* D, const int32_t* elem_
   M->ph = Phys{D->gamma, D->Pr, D->Re, D->alpha, D->stab, {0, 0, 0, 0, 0}};
   if (u_far)
     for (int i = 0; i < m; ++i) M->ph.ub[i] = u_far[i];
-  set_precision(M, D->precision, true);
+  set_precision(M, D->precision);
   M->E = D->n_elem;
   M->T = D->n_trace;
   rc = create_mixed_impl(D, elem_order, face_degree, face_kind, (cudaStream_t)stream, M);

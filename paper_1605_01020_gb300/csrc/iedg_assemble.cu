@@ -1062,7 +1062,7 @@ static cudaError_t launch_lu64_tc(iedg_mesh* M, cudaStream_t st) {
 
 cudaError_t launch_lu(iedg_mesh* M, cudaStream_t st) {
   if (M->dm.nu > LU_MAX_NU) return cudaErrorInvalidValue;   // orders above 4 are rejected at creation
-  if (M->precision == 0 && (M->sched.lu_tensor || M->dm.nu >= LU64_TC_MIN_NU)) return launch_lu64_tc(M, st);
+  if (M->precision == 0 && M->sched.lu_tensor) return launch_lu64_tc(M, st);
   if (M->precision == 0) {
     if (M->sched.lu_panel == 32 && lu64_smem(M->dm, 32) <= 227 * 1024) return lu_t<double, 32>(M, M->S, nullptr, st);
     return lu_t<double, 16>(M, M->S, nullptr, st);

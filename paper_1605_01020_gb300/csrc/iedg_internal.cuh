@@ -37,7 +37,7 @@ struct Schedule {
   int lu_persistent = 1;     // batched LU as a persistent grid with an element queue
   int lu_panel = 16;         // FP64 LU panel width (16 or 32; 32 only when it fits shared memory)
   int asm_chunk = 0;         // assembly column chunk (0 = default: 8 for FP64, 16 for FP32)
-  int lu_tensor = 0;         // FP64: 1 = digit form on tcgen05 always, 0 = by size.  Mixed: 0 = FFMA
+  int lu_tensor = 0;         // FP64: 1 = digit form on tcgen05, 0 = DFMA updates.  Mixed: 0 = FFMA
                              // updates; 1 = deferred Schur complement on tcgen05; 2 (FP32 form) =
                              // every trailing update on tcgen05 (3xTF32)
   int asm_chunk_by_order[4] = {0, 0, 0, 0};   // mixed orders: chunk per order (0 = asm_chunk)
@@ -317,7 +317,7 @@ bool assemble_col_supported(const iedg_mesh* M);
 AsmTab<double> tables64(const iedg_mesh* M);
 AsmTab<float> tables32(const iedg_mesh* M);
 cudaError_t launch_lu(iedg_mesh* M, cudaStream_t st);
-// u-unknowns from which the FP64 LU takes its digit form (iedg_assemble.cu)
+// u-unknowns from which handles default to the FP64 LU's digit form (iedg_assemble.cu)
 constexpr int LU64_TC_MIN_NU = 64;
 cudaError_t launch_lu32(iedg_mesh* M, cudaStream_t st);   // FP32 LU, FFMA updates or deferred tensor-core Schur complement
 cudaError_t launch_lu32_mma(iedg_mesh* M, int n_max, cudaStream_t st);   // FP32 LU, tcgen05 trailing updates
