@@ -277,9 +277,12 @@ int iedg_trace_solve(iedg_mesh* mesh, const double* K, const double* R, double* 
  *                  memory falls back).  Uniform meshes assemble without chunks.
  *   lu_tensor:     tensor cores (tcgen05, accumulation in tensor memory) in the partial LU.
  *                  FP64 path: the trailing updates as integer products of 8-bit digits of
- *                  the FP64 operands, summed exactly and joined to FP64 (the error of an
- *                  update is below that of the DFMA form).  1 = that form; 0 = DFMA
- *                  updates, at every size.  Mixed path: 1 = the Schur complement K = D - W Z, TF32 operands
+ *                  the FP64 operands, summed exactly and joined to FP64.  The error of an
+ *                  update is then relative to (largest entry of its row) x (largest of
+ *                  its column), about 2^-60 after a scaling that evens out the panel's
+ *                  rows, where the DFMA form's is relative to the entry's own terms;
+ *                  entries far below that product are formed by DFMA.  1 = that form;
+ *                  0 = DFMA updates, at every size.  Mixed path: 1 = the Schur complement K = D - W Z, TF32 operands
  *                  split in high and low parts, three products ("3xTF32"); 2 (mixed FP32
  *                  form only) = every trailing update of the FP32 LU (3xTF32, 128 x 64
  *                  tiles accumulated in TMEM and subtracted from the trailing block by

@@ -481,49 +481,68 @@ __device__ __forceinline__ void lu_element(const LuElem& el, T* __restrict__ S, 
 // two FP64 multiply-adds per SM and clock against 4096 BF16 ones on the tensor cores,
 // so the bulk of the arithmetic, A22 -= L21 U12 (rows x 32 times 32 x columns), goes
 // there in integers:
-//   * each row of L21 and each column of U12 is scaled by the power of two of its
-//     largest entry and rounded to a 63-bit integer X, |X| < 2^62, written in balanced
-//     base 256: X = sum_s d_s 256^(8-s), s = 1..8, |d_s| <= 128, exact in BF16;
-//   * digit products of equal weight, s + t = l, l = 2..9, share one FP32 accumulator in
-//     TMEM.  A level's sum is an integer of at most 8 32 2^14 = 2^22, so the tensor core
-//     adds exactly (the splitting of Ozaki, Ogita, Oishi and Rump, "Error-free
-//     transformations of matrix multiplication", 2012, with K short enough that no
-//     level has to be flushed).  Levels past 9 (below 2^-60 of the largest product)
-//     are dropped;
-//   * the levels are joined in a 64-bit integer, normalised to an FP64 number with
-//     integer instructions, and subtracted: one FP64 addition per entry and panel
-//     where the DFMA form spends 32 multiply-adds.
-// The error of an update is 2^-57 of the largest product of its row and column plus the
-// rounding of one FP64 subtraction; the DFMA form rounds 32 times.
+//   * the panel's unknowns are scaled by powers of two, u_kj 2^-s_k and l_ik 2^s_k, so that
+//     every row k of U12 has its largest entry near 1 (pivot rows of different equations
+//     differ by powers of the Mach number); then each row of L21 and each column of U12 is
+//     scaled by a power of two (by its largest entry) to integers |X| < 2^61 and cut into
+//     eight balanced base-256 digits (iedg_digits.cuh), s = 0 the leading one, |d_0| <= 32;
+//   * digit products of equal weight, s + t = l <= 8, share one FP32 accumulator in TMEM,
+//     level 0 that of level 1 (256 d_0 is another slice of the row operand).  All sums are
+//     integers below 2^24 (levels 0 and 1: 32 (32^2 256 + 2 32 128) < 2^23.1; the others
+//     below 2^22), so the tensor core adds exactly (the splitting of Ozaki, Ogita, Oishi and
+//     Rump, "Error-free transformations of matrix multiplication", 2012, with K short enough
+//     that no level has to be flushed);
+//   * the levels are joined in 96-bit integers, rounded once to FP64 and subtracted: one
+//     FP64 addition per entry and panel where the DFMA form spends 32 multiply-adds.
+// Accuracy.  The error of an update is absolute in its row and column: about 2^-60 times
+// (largest |l_ik 2^s_k|) (largest |u_kj 2^-s_k|) over k, from rounding the operands and the
+// levels past 8, at most 2^-54; then one FP64 rounding.  The DFMA form's is relative to the
+// entry's own terms, 32 roundings of 2^-53.  So the digit form is the more accurate one for
+// entries within about 2^-6 of that product, and the less accurate one far below it; entries
+// whose old value and update are both below 2^-28 of it are formed by DFMA (0.4 % of them in
+// the fourth line below, 1 % in the fifth, whose state has a direction at rest; that costs
+// 3 % of the kernel, at 2^-20 it cost 9 %).
+// Errors of K against 80-bit elimination, numpy model of both forms, DFMA | digits: largest
+// entry, worst of the 25 component blocks, median entry:
+//   p = 2, Re 2.5e5, M 0.2, cubes          2.2e-15 3.7e-13 4.6e-15 | 3.0e-16 2.7e-13 3.2e-15
+//   p = 2, Re 1, M 0.02, cells 1 : 50      1.7e-15 1.5e-11 3.0e-14 | 2.1e-15 3.2e-12 2.0e-14
+//   p = 2, Re 1, M 0.01, cells 1 : 1e4     7.5e-13 4.3e-07 1.7e-11 | 2.5e-13 3.9e-08 8.8e-12
+//   p = 2, Re 1e-3, M 1e-4, cells 1 : 1000 1.3e-13 5.9e-07 1.0e-10 | 6.1e-14 3.4e-07 5.4e-11
+//   p = 3, Re 2.5e5, M 0.2, cubes          3.6e-15 2.4e-13 2.2e-14 | 7.3e-16 1.7e-13 1.0e-14
+//   p = 3, Re 10, M 0.05, cells 1 : 200    7.6e-15 1.9e-10 1.1e-13 | 5.6e-15 5.5e-11 5.3e-14
+// (without s_k, level 8 and the rounding of the operands the second line's digits were
+// 5.1e-15 1.8e-11 2.0e-13, the fourth's 100 to 300 times DFMA's).
 //
 // Roles: the 128 TMEM lanes are columns of A22 (the MMA's A operand is U12^T), so a
 // warp's accesses of A22 are rows of 32 consecutive columns; the B operand stacks the
-// digits t of 16 rows of L21, so that digit s of U12 meets all digits t <= 9 - s in one
-// instruction whose columns land on the levels s + 1 .. 9 in order.
+// digits t of 16 rows of L21, so that digit s of U12 meets all digits t <= 8 - s in one
+// instruction whose columns land on the levels s .. 8 in order.
 //
 // Panel factorisation, the trace rows of L21 and U12 = L11^-1 A12 stay on the FP64 pipe,
 // which bounds the kernel: per element of 320 + 280 unknowns 2.3 M multiply-adds there
 // and 2 M additions of the updates (65 M multiply-adds in the DFMA form).  Two CTAs per
 // SM, so that one element's panels overlap the other's updates.
 // Measured, all elements of a mesh, DFMA form -> this one: 3D p = 3, 4096 elements
-// 505.9 -> 95.1 ms; p = 2, 2002 elements 26.5 -> 7.7 ms; p = 4, 210 elements 238.6 -> 48.4 ms
-// (with a branch per joined entry and L21 loaded when staged: 100.5, 8.3, 57.9 ms);
-// 2D p = 3 (64 + 48 unknowns), 851 elements 1.53 -> 0.82 ms.  Below 64 u-unknowns an
+// 505.9 -> 102.1 ms; p = 2, 2002 elements 26.5 -> 7.9 ms; p = 4, 210 elements 238.6 -> 52.7 ms
+// (without s_k, level 8, rounded operands and DFMA entries 96.0, 7.7, 48.4 ms);
+// 2D p = 3 (64 + 48 unknowns), 851 elements 1.53 -> 0.84 ms.  Below 64 u-unknowns an
 // element is at most two panels, which leaves too little to the tensor cores, and the
-// DFMA form stays: 2D p = 2 (36 + 32), 1600 elements 0.78 ms DFMA, 0.95 ms digits; 3D p = 1
-// (40 + 40), 8000 elements 4.98 and 4.92 ms.  Counters at p = 3: FP64 pipe 47 % busy, issue
+// DFMA form stays: 2D p = 2 (36 + 32), 1600 elements 0.79 ms DFMA, 0.98 ms digits; 3D p = 1
+// (40 + 40), 8000 elements 4.98 and 5.10 ms.  Counters at p = 3: FP64 pipe 47 % busy, issue
 // slots 35 %, tensor pipe 8 %, 42 MB of DRAM traffic per element: latency of the panel
 // steps and of the trailing block's loads, not a pipe, is what is left.
 constexpr int LT_NB = 32;                       // panel width
 constexpr int LT_S = dig::S;                    // digits per operand, and levels kept
 using dig::exponent_of;
-using dig::scale_of;
+constexpr int LT_ZERO = -4096;                  // exponent of a row or column of zeros
 constexpr int LT_TC = 128, LT_TR = 16;          // columns and rows of one MMA group
 constexpr int LT_RB = 64;                       // rows of L21 staged at a time
 constexpr int LT_SLICE = LT_TC * LT_NB * 2;     // one digit of a column tile
 constexpr int LT_A_BYTES = LT_S * LT_SLICE;     // 64 KB
-constexpr int LT_GROUP = LT_S * LT_TR * LT_NB * 2;          // all digits of 16 rows
-constexpr int LT_B_BYTES = LT_RB / LT_TR * LT_GROUP;        // 32 KB
+constexpr int LT_BSLICE = LT_TR * LT_NB * 2;    // one digit of 16 rows
+constexpr int LT_GROUP = (LT_S + 1) * LT_BSLICE;            // their digits 0..7, then 256 d_0
+constexpr int LT_B_BYTES = LT_RB / LT_TR * LT_GROUP;        // 36 KB
+constexpr int LT_LOW = 28;                      // entries below 2^-LT_LOW of row x column take DFMA
 constexpr int LT_LVL_COLS = LT_S * LT_TR;       // TMEM columns of one accumulator set
 constexpr int LT_TMEM_COLS = 2 * LT_LVL_COLS;   // two sets: epilogue of one, MMAs into the other
 __host__ __device__ inline int lt_stride(int nu) { return nu | 1; }   // odd: conflict-free columns
@@ -533,14 +552,28 @@ __host__ inline size_t lt_smem(const Dims& dm) {
   return (panel > dig ? panel : dig) + 128;      // operand tiles start on a 128-byte boundary
 }
 
-// Digits of eight values with common exponent emax >= theirs: out(s, 8 packed BF16) for
-// s = 0 (most significant) .. 7.
-template <class Out>
-__device__ __forceinline__ void split8(const double (&x)[8], int emax, Out out) {
+// sign s_k of eight of the panel's unknowns, from the largest exponents of their rows of U12.
+__device__ __forceinline__ void load_shifts(const int* sk, int sign, int (&shift)[8]) {
+  const int4 a = reinterpret_cast<const int4*>(sk)[0], b = reinterpret_cast<const int4*>(sk)[1];
+  const int e[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+#pragma unroll
+  for (int i = 0; i < 8; ++i) shift[i] = sign * (e[i] - 1023);
+}
+
+// Exponent with which a value that is scaled by 2^shift enters its row's or column's largest.
+__device__ __forceinline__ int scaled_exp(double x, int shift) {
+  const int e = exponent_of(x);
+  return e == 0 ? LT_ZERO : (e == 0x7ff ? dig::BAD_EXP : e + shift);
+}
+
+// Digits of eight values scaled by 2^shift[i], emax the largest exponent then, |X| < 2^61:
+// out(s, 8 packed BF16) for s = 0 (most significant) .. 7 and, TOP, 256 d_0 as s = 8.
+template <bool TOP, class Out>
+__device__ __forceinline__ void split8(const double (&x)[8], const int (&shift)[8], int emax, Out out) {
   uint32_t w[2][8];
 #pragma unroll
   for (int i = 0; i < 8; ++i) {
-    const unsigned long long v = dig::to_bytes(__double_as_longlong(x[i]), emax);
+    const unsigned long long v = dig::to_bytes(__double_as_longlong(x[i]), emax + 1 - shift[i]);
     w[0][i] = (uint32_t)(v >> 32);
     w[1][i] = (uint32_t)v;
   }
@@ -550,37 +583,63 @@ __device__ __forceinline__ void split8(const double (&x)[8], int emax, Out out) 
     out(s, make_uint4(dig::bf16_pair(q[0], q[1], s), dig::bf16_pair(q[2], q[3], s), dig::bf16_pair(q[4], q[5], s),
                       dig::bf16_pair(q[6], q[7], s)));
   }
-}
-
-// One thread: all digit products of one 16-row group into the accumulator set at d; a, b:
-// descriptors of the operands' first slices (addresses in their low bits, in 16 bytes).
-__device__ __forceinline__ void lt_issue(uint32_t d, uint64_t a, uint64_t b, int ksteps) {
-  for (int ks = 0; ks < ksteps; ++ks)
-#pragma unroll
-    for (int s = 0; s < LT_S; ++s)
-      tc::mma_bf16(d + (uint32_t)(s * LT_TR), a + (uint64_t)(s * (LT_SLICE >> 4) + ks * 16), b + (uint64_t)(ks * 16),
-                   tc::idesc_bf16(LT_TC, LT_TR * (LT_S - s)), (ks == 0 && s == 0) ? 0u : 1u);
-}
-
-// minus the product sum whose level sums are t[0..7], scales ef = row + column exponent.
-// Free of branches, so that a thread's eight entries overlap; `odd` is set where the
-// result leaves the normal range (a non-finite operand, or a product sum out of FP64's
-// exponent range), for the caller to replace it by dig::special.
-__device__ __forceinline__ double join_levels(const float (&t)[8], int ef, bool& odd) {
-  uint32_t p[4];
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    // integer-valued |t| <= 2^22 -> bits 0x4B400000 + t; two neighbouring levels per word
-    const uint32_t a = __float_as_uint(t[2 * i] + 12582912.0f), b = __float_as_uint(t[2 * i + 1] + 12582912.0f);
-    p[i] = (a << 8) + b - 0x8B400000u;
+  if constexpr (TOP) {
+    const uint32_t(&q)[8] = w[0];
+    out(LT_S, make_uint4(dig::bf16_pair(q[0], q[1], 0, 256.0f), dig::bf16_pair(q[2], q[3], 0, 256.0f),
+                         dig::bf16_pair(q[4], q[5], 0, 256.0f), dig::bf16_pair(q[6], q[7], 0, 256.0f)));
   }
-  long long v = (long long)(int)p[2] * 32 + (((int)p[3] + 1024) >> 11);
-  v += (long long)(int)p[1] * (1 << 21);
-  v += (long long)((unsigned long long)p[0] << 37);
-  const unsigned long long sg = (unsigned long long)(v >> 63);
-  const unsigned long long mag = ((unsigned long long)v ^ sg) - sg;
-  const int lz = __clzll((long long)(mag | 1ull));
-  return dig::from_fixed(mag, lz, ef - 1015 - lz, ~sg & 0x8000000000000000ull, odd);
+}
+
+// One thread: all digit products of one 16-row group into the accumulator set at d (levels
+// 0 and 1, then 2 .. 8); a, b: descriptors of the operands' first slices (addresses in their
+// low bits, in 16 bytes).
+__device__ __forceinline__ void lt_issue(uint32_t d, uint64_t a, uint64_t b, int ksteps) {
+  auto mma = [&](int acc0, int s, int t, int nt, int ks, uint32_t add) {
+    tc::mma_bf16(d + (uint32_t)(acc0 * LT_TR), a + (uint64_t)(s * (LT_SLICE >> 4) + ks * 16),
+                 b + (uint64_t)(t * (LT_BSLICE >> 4) + ks * 16), tc::idesc_bf16(LT_TC, LT_TR * nt), add);
+  };
+  for (int ks = 0; ks < ksteps; ++ks) {
+    mma(0, 1, 0, 8, ks, ks == 0 ? 0u : 1u);      // s = 1, t = 0..7: every accumulator
+    mma(0, 0, 8, 1, ks, 1u);                     // s = 0, t = 0 by 256
+    mma(0, 0, 1, 7, ks, 1u);                     // s = 0, t = 1..7
+#pragma unroll
+    for (int s = 2; s < LT_S; ++s) mma(s - 1, s, 0, 9 - s, ks, 1u);
+  }
+}
+
+// minus the product sum whose accumulators are t[0..7] (256 level 0 + level 1, levels
+// 2 .. 8), scales ef = row + column exponent.  Free of branches, so that a thread's eight
+// entries overlap; `odd` is set where it cannot say: outside FP64's normal range, or below
+// 2^32 units of the last level (2^-42 of row x column) and not zero.
+__device__ __forceinline__ double join_levels(const float (&t)[8], int ef, bool& odd) {
+  // integer-valued |t| <= 2^22 -> bits 0x4B400000 + t
+  uint32_t b[8];
+#pragma unroll
+  for (int i = 1; i < 8; ++i) b[i] = __float_as_uint(t[i] + 12582912.0f);
+  const int h = (int)((b[1] << 8) + b[2] - 0x8B400000u);        // 256 t1 + t2
+  const int m = (int)((b[4] << 8) + b[5] - 0x8B400000u), n = (int)((b[6] << 8) + b[7] - 0x8B400000u);
+  const long long L = (long long)m * 65536 + n;
+  const long long H = (long long)__float2int_rn(t[0]) * (1 << 24) + (long long)h * 256 + (int)(b[3] - 0x4B400000u) + (L >> 32);
+  // |H 2^32 + low word of L| (up to its last bit) in three words, normalised to two
+  const uint32_t sg = (uint32_t)(int)(H >> 63);
+  const uint32_t w2 = (uint32_t)((unsigned long long)H >> 32) ^ sg, w1 = (uint32_t)H ^ sg, w0 = (uint32_t)L ^ sg;
+  const bool top = w2 != 0;
+  const uint32_t x = top ? w2 : w1, y = top ? w1 : w0, z = top ? w0 : 0u;
+  const int lz = __clz((int)x);
+  const uint32_t hi = __funnelshift_l(y, x, lz), lo = __funnelshift_l(z, y, lz);
+  const int field = ef - (top ? 1001 : 1033) - lz;              // biased exponent - 1
+  const unsigned long long r = (((unsigned long long)hi << 21) | (lo >> 11)) + ((lo >> 10) & 1u) +
+                               ((unsigned long long)(unsigned)field << 52);
+  odd = x != 0 ? (unsigned)field >= 2045u : w0 != 0;
+  return __longlong_as_double(x != 0 ? (long long)(r | ((unsigned long long)(~sg & 0x80000000u) << 32)) : 0ll);
+}
+
+// One entry of A22 by DFMA, in the DFMA form's order: l, u point to its row of L21 and its
+// column of U12.
+__device__ __forceinline__ double lt_entry(const double* l, const double* u, int ld, int nb, double a) {
+#pragma unroll 4
+  for (int k = 0; k < nb; ++k) a = fma(-l[k], u[(int64_t)k * ld], a);
+  return a;
 }
 
 // Tensor-core state of a CTA, the same in every thread: bit b of phase is the parity of
@@ -605,8 +664,10 @@ struct LtShared {
   long long rv[LU_THREADS / 32];
   int ri[LU_THREADS / 32];
   int sing;
+  alignas(16) int sk[LT_NB];         // largest exponents of the rows of U12: s_k = sk - 1023
   int ce[2][LT_TC];                  // column exponents, two halves of the panel's rows
   int re[LT_RB];                     // row exponents of the staged rows
+  uint32_t cm[2][LT_TC], rm[LT_RB];  // which of the panel's 32 values are not zero
 };
 
 // Panel columns kb .. kb+nb-1 over the u-rows, P column-major (column j at P + j PR).
@@ -711,36 +772,51 @@ __device__ __forceinline__ bool lt_trailing(LtShared& sh, double* __restrict__ A
       // U12 columns ct .. ct+127: thread = column (and half of the panel's rows)
       const int c = tid & (LT_TC - 1), kh = tid >> 7, col = ct + c;
       double x[2][8];
-      int em = 0;
+      int em = LT_ZERO, shift[2][8];
+      uint32_t nz = 0;
+#pragma unroll
+      for (int u = 0; u < 2; ++u) load_shifts(sh.sk + 16 * kh + 8 * u, -1, shift[u]);
 #pragma unroll
       for (int u = 0; u < 2; ++u)
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
           const int k = 16 * kh + 8 * u + i;
           x[u][i] = (k < nb && col < ncol) ? A[(int64_t)(kb + k) * ld + col] : 0.0;
-          em = max(em, exponent_of(x[u][i]));
+          const int e = scaled_exp(x[u][i], shift[u][i]);
+          em = max(em, e);
+          nz |= e != LT_ZERO ? 1u << (8 * u + i) : 0u;
         }
       sh.ce[kh][c] = em;
+      sh.cm[kh][c] = nz << (16 * kh);
       __syncthreads();
       em = max(em, sh.ce[kh ^ 1][c]);
 #pragma unroll
       for (int u = 0; u < 2; ++u)
-        split8(x[u], em, [&](int s, uint4 v) {
+        split8<false>(x[u], shift[u], em, [&](int s, uint4 v) {
           *reinterpret_cast<uint4*>(da + s * LT_SLICE + tc::core_off16(c, 16 * kh + 8 * u)) = v;
         });
     }
     const int c = 32 * q + lane, col = ct + c;
     int ecol = 0;                                    // set after the first barrier below
+    uint32_t cmask = 0;
     for (int rb = r0; rb < n; rb += LT_RB) {
       {
-        int em = 0;
+        int em = LT_ZERO, shift[8];
+        uint32_t nz = 0;
+        load_shifts(sh.sk + 8 * sk8, 1, shift);
 #pragma unroll
-        for (int i = 0; i < 8; ++i) em = max(em, exponent_of(x[i]));
+        for (int i = 0; i < 8; ++i) {
+          const int e = scaled_exp(x[i], shift[i]);
+          em = max(em, e);
+          nz |= e != LT_ZERO ? 1u << (8 * sk8 + i) : 0u;
+        }
         em = max(em, __shfl_xor_sync(0xffffffffu, em, 8));
         em = max(em, __shfl_xor_sync(0xffffffffu, em, 16));
-        if (sk8 == 0) sh.re[srow] = scale_of(em);
-        split8(x, em, [&](int s, uint4 v) {
-          *reinterpret_cast<uint4*>(db + (srow >> 4) * LT_GROUP + s * (LT_TR * LT_NB * 2) +
+        nz |= __shfl_xor_sync(0xffffffffu, nz, 8);
+        nz |= __shfl_xor_sync(0xffffffffu, nz, 16);
+        if (sk8 == 0) { sh.re[srow] = em; sh.rm[srow] = nz; }
+        split8<true>(x, shift, em, [&](int s, uint4 v) {
+          *reinterpret_cast<uint4*>(db + (srow >> 4) * LT_GROUP + s * LT_BSLICE +
                                     tc::core_off16(srow & 15, 8 * sk8)) = v;
         });
         fetch((rb + LT_RB < n ? rb + LT_RB : r0) + srow);
@@ -748,7 +824,10 @@ __device__ __forceinline__ bool lt_trailing(LtShared& sh, double* __restrict__ A
       tc::fence_proxy_async();
       __syncthreads();
       tc::fence_after_sync();
-      if (rb == r0) ecol = scale_of(max(sh.ce[0][c], sh.ce[1][c]));
+      if (rb == r0) {
+        ecol = max(sh.ce[0][c], sh.ce[1][c]);
+        cmask = sh.cm[0][c] | sh.cm[1][c];
+      }
       const int ng = (min(LT_RB, n - rb) + LT_TR - 1) / LT_TR;
       if (tid == 0) {
         lt_issue(tcs->tmem, ua, ub, ksteps);
@@ -775,27 +854,33 @@ __device__ __forceinline__ bool lt_trailing(LtShared& sh, double* __restrict__ A
           tc::fence_after_sync();
           float t[8][8];
           dig::load_levels(tcs->tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(b * LT_LVL_COLS + 8 * h), LT_TR, t);
-          unsigned odds = 0;
+          // entries for DFMA: those join_levels cannot say, with non-finite operands, or far below
+          // row x column
+          unsigned redo = 0;
           double d[8];
 #pragma unroll
           for (int i = 0; i < 8; ++i) {
             const float lv[8] = {t[0][i], t[1][i], t[2][i], t[3][i], t[4][i], t[5][i], t[6][i], t[7][i]};
+            const int lr = LT_TR * g + 8 * h + i, ef = ecol + sh.re[lr];
             bool odd;
-            d[i] = join_levels(lv, ecol + sh.re[LT_TR * g + 8 * h + i], odd);
-            odds |= odd ? 1u << i : 0u;
-          }
-          if (odds) {
-#pragma unroll
-            for (int i = 0; i < 8; ++i)
-              if ((odds >> i) & 1u) d[i] = dig::special(d[i], ecol + sh.re[LT_TR * g + 8 * h + i]);
+            d[i] = join_levels(lv, ef, odd);
+            const int eo = max(exponent_of(a[i]), exponent_of(d[i]));
+            if (odd || eo <= ef - 1022 - LT_LOW) redo |= 1u << i;
+            d[i] += a[i];
           }
 #pragma unroll
-          for (int i = 0; i < 8; ++i) {
-            a[i] += d[i];
-            if (col < ncol && row0 + i < n) {
-              dst[(int64_t)i * ld] = a[i];
-              bad |= row0 + i >= nu && col >= nu && exponent_of(a[i]) == 0x7ff;
+          for (int i = 0; i < 8; ++i)
+            if (col < ncol && row0 + i < n && !((redo >> i) & 1u)) {
+              dst[(int64_t)i * ld] = d[i];
+              bad |= row0 + i >= nu && col >= nu && exponent_of(d[i]) == 0x7ff;
             }
+          for (; redo; redo &= redo - 1) {
+            const int row = row0 + __ffs(redo) - 1, lr = row - rb;
+            // products that all vanish leave the entry as it is, unless an operand is not finite
+            if (col >= ncol || row >= n || ((cmask & sh.rm[lr]) == 0 && ecol + sh.re[lr] < dig::BAD_EXP)) continue;
+            double* v = A + (int64_t)row * ld + col;
+            *v = lt_entry(A + (int64_t)row * ld + kb, A + (int64_t)kb * ld + col, ld, nb, *v);
+            bad |= row >= nu && col >= nu && exponent_of(*v) == 0x7ff;
           }
         }
         tc::fence_before_sync();
@@ -823,6 +908,7 @@ __device__ __forceinline__ bool lt_element(LtShared& sh, const LuElem& el, doubl
     for (int r = warp; r < prow; r += LU_THREADS / 32)
       P[r + lane * PR] = lane < nb ? A[(int64_t)(kb + r) * ld + kb + lane] : 0.0;
     for (int r = tid; r < prow; r += LU_THREADS) sh.perm[r] = r;
+    if (tid < LT_NB) sh.sk[tid] = 0;
     __syncthreads();
     lt_panel(sh, P, PR, prow, nb, nonfin);
     // [L11 \ U11], L21 of the u-rows back
@@ -855,23 +941,25 @@ __device__ __forceinline__ bool lt_element(LtShared& sh, const LuElem& el, doubl
       }
     }
     // trailing columns: row interchanges (each column gathers its new top rows, then
-    // moves the displaced rows), then U12 = L11^-1 A12
-    for (int c = kb + nb + tid; c < ncol; c += LU_THREADS) {
+    // moves the displaced rows), then U12 = L11^-1 A12 and the largest exponents of its rows
+    for (int c0 = kb + nb + 32 * warp; c0 < ncol; c0 += LU_THREADS) {
+      const int c = c0 + lane;
+      const bool in = c < ncol;
       double x[LT_NB];
 #pragma unroll
-      for (int j = 0; j < LT_NB; ++j) x[j] = j < nb ? A[(int64_t)(kb + sh.perm[j]) * ld + c] : 0.0;
+      for (int j = 0; j < LT_NB; ++j) x[j] = (in && j < nb) ? A[(int64_t)(kb + sh.perm[j]) * ld + c] : 0.0;
 #pragma unroll
       for (int j0 = 0; j0 < LT_NB; j0 += 8) {
         double y[8];
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
           const int r = j0 + j < nb ? sh.piv[j0 + j] : 0;
-          y[j] = (j0 + j < nb && r >= nb && sh.perm[r] != r) ? A[(int64_t)(kb + sh.perm[r]) * ld + c] : 0.0;
+          y[j] = (in && j0 + j < nb && r >= nb && sh.perm[r] != r) ? A[(int64_t)(kb + sh.perm[r]) * ld + c] : 0.0;
         }
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
           const int r = j0 + j < nb ? sh.piv[j0 + j] : 0;
-          if (j0 + j < nb && r >= nb && sh.perm[r] != r) A[(int64_t)(kb + r) * ld + c] = y[j];
+          if (in && j0 + j < nb && r >= nb && sh.perm[r] != r) A[(int64_t)(kb + r) * ld + c] = y[j];
         }
       }
 #pragma unroll
@@ -879,8 +967,15 @@ __device__ __forceinline__ bool lt_element(LtShared& sh, const LuElem& el, doubl
         if (j >= nb) break;
 #pragma unroll
         for (int i = j + 1; i < LT_NB; ++i) x[i] = fma(-P[i + j * PR], x[j], x[i]);
-        A[(int64_t)(kb + j) * ld + c] = x[j];
+        if (in) A[(int64_t)(kb + j) * ld + c] = x[j];
       }
+      int top = 0;                           // lane j keeps row j's
+#pragma unroll
+      for (int j = 0; j < LT_NB; ++j) {
+        const int e = __reduce_max_sync(0xffffffffu, exponent_of(x[j]));
+        top = lane == j ? e : top;
+      }
+      if (lane < nb) atomicMax(&sh.sk[lane], top);
     }
     __syncthreads();
     if (!lt_trailing(sh, A, ld, kb, nb, kb + nb, n, nu, kb + nb, ncol, smem, tcs, bad)) break;

@@ -2,9 +2,10 @@
 // partial LU; csrc/iedg_assemble_dg.cu, the volume terms of the assembly).
 //
 // With emax the biased exponent of (a bound on) a row's or column's largest entry, an
-// entry x becomes the integer X = x 2^(61 - (emax - 1023)), |X| < 2^62, in balanced base
-// 256: X = sum_s d_s 256^(7 - s), s = 0..7, -128 <= d_s <= 127 and |d_0| <= 64.  Digits are
-// exact in BF16 and their products' sums exact in FP32 below 2^24.
+// entry x becomes the integer X nearest to x 2^(61 - (emax - 1023)), |X| < 2^62, in balanced
+// base 256: X = sum_s d_s 256^(7 - s), s = 0..7, -128 <= d_s <= 127 and |d_0| <= 64.  Digits
+// are exact in BF16 and their products' sums exact in FP32 below 2^24.  X is in error by up to
+// 2^-62 of the largest entry: entries far below it keep fewer bits than FP64 holds.
 #pragma once
 #include <cstdint>
 #include <cuda_runtime.h>
@@ -18,11 +19,11 @@ constexpr int BAD_EXP = 1 << 13;         // exponent of a row or column with a n
 __host__ __device__ __forceinline__ int exponent_bits(long long b) { return (int)((b >> 52) & 0x7ff); }
 
 // The digits of x, each with 128 added, most significant in the top byte.  Entries below
-// 2^-62 of the scale and subnormals become 0.
+// 2^-63 of the scale and subnormals become 0.
 __host__ __device__ __forceinline__ unsigned long long to_bytes(long long b, int emax) {
   const int e = exponent_bits(b), sh = emax - e;
   unsigned long long m = ((unsigned long long)b & 0xFFFFFFFFFFFFFull) | 0x10000000000000ull;
-  m = (e == 0 || sh > 62 || sh < 0) ? 0ull : (m << 9) >> sh;
+  m = (e == 0 || sh > 62 || sh < 0) ? 0ull : (((m << 10) >> sh) + 1) >> 1;
   return (b < 0 ? 0ull - m : m) + 0x8080808080808080ull;
 }
 
@@ -33,11 +34,11 @@ __device__ __forceinline__ int scale_of(int emax) { return emax >= 0x7ff ? BAD_E
 
 // Two values' digits s as packed BF16; w: the word of to_bytes that holds digit s (the upper
 // one for s < 4).  byte -> float 2^23 + byte, minus 2^23 + 128: at most 8 significant
-// bits, so the upper half of the FP32 pattern is the BF16 value.
-__device__ __forceinline__ uint32_t bf16_pair(uint32_t w0, uint32_t w1, int s) {
+// bits, so the upper half of the FP32 pattern is the BF16 value; `scale`: a power of two.
+__device__ __forceinline__ uint32_t bf16_pair(uint32_t w0, uint32_t w1, int s, float scale = 1.0f) {
   const uint32_t sel = 0x7440u | (uint32_t)(3 - (s & 3));
-  const float f0 = __uint_as_float(__byte_perm(w0, 0x4B000000u, sel)) - 8388736.0f;
-  const float f1 = __uint_as_float(__byte_perm(w1, 0x4B000000u, sel)) - 8388736.0f;
+  const float f0 = (__uint_as_float(__byte_perm(w0, 0x4B000000u, sel)) - 8388736.0f) * scale;
+  const float f1 = (__uint_as_float(__byte_perm(w1, 0x4B000000u, sel)) - 8388736.0f) * scale;
   return __byte_perm(__float_as_uint(f0), __float_as_uint(f1), 0x7632);
 }
 
