@@ -394,6 +394,8 @@ static int alloc_group(iedg_mesh* M, cudaStream_t st) {
   if (dg) {
     CUDA_TRY(dalloc(M, &G.elift, E * 2 * d * (Np + Nb)));
     CUDA_TRY(dalloc(M, &M->pj.ecoef, E * m * m * 9));
+    const size_t slots = M->precision == IEDG_PRECISION_FP64 ? (size_t)E : (size_t)kFallbackSlots;
+    CUDA_TRY(dalloc(M, &M->pj.ew, slots * m * m * 2 * (Np + Nb)));
   }
   CUDA_TRY(dalloc(M, &G.wdet, E * Nq));
   CUDA_TRY(dalloc(M, &G.Jinv, E * Nq * d * d));

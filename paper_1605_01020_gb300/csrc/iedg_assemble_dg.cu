@@ -16,9 +16,8 @@
 //   * the B operand is W (V) for 32 columns of the element, which may belong to several
 //     pairs: the digits t are stacked, so that digit s of the table meets all digits t <=
 //     7 - s in one instruction (see k_lu64_tc);
-//   * a column's scale is a bound on its largest |W| from the exponents of its factors
-//     (largest exponents per pair, and per column of Gl, Hl), so W is converted as it is
-//     formed; the bound costs a few of the 62 digit bits;
+//   * a column's scale is the exponent of its largest |W| (|V|), which k_w_exp finds in FP32
+//     beforehand, so W is converted as it is formed;
 //   * FP32 level sums stay exact (below 2^24) over a window of chunks, checked for the
 //     tables' own digits when they are laid out; then the levels are joined in 96-bit
 //     integers, rounded once to FP64 and added to the element matrix.
@@ -27,13 +26,22 @@
 // conversion and results overlap the other's FP64.
 // Meshes with mixed orders have trace bases of their own: there the face terms come from
 // k_assemble_sf first and this kernel adds the volume terms.
-// Measured, all elements, sum-factorised on the FP64 pipe -> this kernel: 3D p = 3, 4096
-// elements 135.4 -> 95.8 ms; p = 2, 2002 elements 14.0 -> 12.4 ms; p = 4, 210 elements 32.8 ->
-// 17.2 ms; orders 2, 3, 4 mixed, 324 elements 25.6 -> 16.8 ms.  Counters at p = 3: FP64 pipe
-// 50 % busy, tensor pipe 26 %, 7.9 TB/s from L2, two thirds of it the tables.
+// Accuracy.  An entry's error is about 2^-58 of (largest table value of its row) (largest |W| of
+// its column), then one FP64 rounding; FP64 sums round every term.  Errors of the element
+// matrix and, through an exact elimination, of K against 80-bit arithmetic (numpy model, FP64
+// sums | this kernel, median entry): p = 3, Re 2.5e5, cubes 1.4e-16 7.4e-16 | 1.0e-16 3.3e-16;
+// p = 3, Re 1e4, cells 1 : 50 1.6e-16 1.2e-15 | 1.2e-16 3.9e-16; p = 3, Re 0.1, M 0.01, cells
+// 1 : 1000 1.8e-16 1.8e-12 | 1.1e-16 1.1e-12 (with the bound from separate maxima as scale
+// 4.5e-15 1.4e-14, 9.3e-15 2.5e-14, 4.8e-15 2.4e-11).
+// Measured, all elements, sum-factorised on the FP64 pipe -> this form (k_coef_exp, k_w_exp,
+// k_assemble_dg): 3D p = 3, 4096 elements 135.4 -> 101.2 ms; p = 2, 2002 elements 14.0 ->
+// 13.4 ms; p = 4, 210 elements 32.8 -> 19.2 ms; orders 2, 3, 4 mixed, 324 elements 25.6 ->
+// 17.6 ms.  Counters at p = 3: FP64 pipe 50 % busy, tensor pipe 26 %, 7.9 TB/s from L2, two
+// thirds of it the tables.
 #include <algorithm>
 #include <cstdlib>
 #include <cstring>
+#include <type_traits>
 
 #include "iedg_digits.cuh"
 #include "iedg_internal.cuh"
@@ -74,6 +82,7 @@ struct DgArgs {
   RefTables ref;
   const int16_t* ecoef;           // [E][25][9] largest exponents of cu, cq_l; fuh, fq_l; S_ik (lambda)
   const int16_t* elift;           // [E][6][Np + Nb] largest exponents of the columns of Gl, Hl: volume, face
+  int16_t* ew;                    // [slot][25][2][Np + Nb] exponents of the columns of V, W (k_w_exp)
   const double* rhs64;            // mixed handles: FP64 right-hand sides
   double* S;
   double alpha;
@@ -117,7 +126,9 @@ __global__ void __launch_bounds__(DG_THREADS, 2) k_assemble_dg(Dims dm, DgArgs a
   // flight is waited for, and the build warps go through the tiles that are left writing NaN.
   // Arrivals then no longer match the waits, which costs nothing: nobody waits for them.
   auto wait = [&](uint64_t* bar, uint32_t parity) {
-    if (!tc::mbar_wait(bar, parity & 1u, *failed ? 1 : a.wait_limit)) *failed = 1;
+    const bool ok = tc::mbar_wait(bar, parity & 1u, *failed ? 1 : a.wait_limit);
+    if (!ok) *failed = 1;
+    return ok;
   };
   // element, trace slots, first column and chunk range of tile `id`; false: nothing to do
   const int ch0 = MIX ? NFC : 0;
@@ -224,23 +235,11 @@ __global__ void __launch_bounds__(DG_THREADS, 2) k_assemble_dg(Dims dm, DgArgs a
       const double* jfu = !ucol ? jf : (a.tb.Su ? a.tb.Su + ep * Nfp : a.tb.lamw + (size_t)e * Nfp);
       const bool fu = on && (!ucol || a.tb.Su != nullptr || pi == pk);
       const int bcol = ucol ? col : (MIX ? 0 : a.ref.bnode[col]);
-      // scales: |W| <= 4 max of the terms; a term's exponent is at most ea + eb + 1, that of
-      // a basis value (below 2) 1023; one more for the terms' rounding
-      int emV = 0, emF = 0;
+      int emF = 0, emV = 0;
       if (on) {
-        const int16_t* ec = a.ecoef + ep * 9;
-        const int16_t* eg = a.elift + (size_t)e * 6 * (Np + NbT) + (ucol ? col : Np + col);
-        auto term = [](int ea, int eb) { return ea == 0x7ff ? 3 * 0x7ff : ea + eb - 1022; };
-        if (ucol) emV = term(ec[0], 1023);
-        if (fu) emF = term(ec[ucol ? 8 : 4], 1023);
-        if (cq)
-#pragma unroll
-          for (int l = 0; l < 3; ++l) {
-            emV = max(emV, term(ec[1 + l], eg[l * (Np + NbT)]));
-            emF = max(emF, term(ec[5 + l], eg[(3 + l) * (Np + NbT)]));
-          }
-        emV += 3;
-        emF += 3;
+        const int16_t* ew = a.ew + ((size_t)slot * m2 + pair) * 2 * (Np + NbT) + (ucol ? col : Np + col);
+        emF = ew[0];
+        emV = ew[Np + NbT];
       }
       asm volatile("bar.sync 3, 256;" ::: "memory");          // the last tile's results are written
       if (gq == 0) {
@@ -306,13 +305,12 @@ __global__ void __launch_bounds__(DG_THREADS, 2) k_assemble_dg(Dims dm, DgArgs a
           }
         }
         if (ch + 1 >= NFC && ch + 1 < ch1) fetch(ch + 1 - NFC);
-        if (nch > 0) wait(&sh.bempty, nch - 1);                 // the MMAs have read the previous chunk
         const int em = face ? emF : emV;
-        if (!*failed) {
+        if (nch == 0 || wait(&sh.bempty, nch - 1)) {            // the MMAs have read the previous chunk
 #pragma unroll
           for (int r = 0; r < 3; ++r) {
-            const unsigned long long v0 = dig::to_bytes(__double_as_longlong(w[r][0]), em);
-            const unsigned long long v1 = dig::to_bytes(__double_as_longlong(w[r][1]), em);
+            const unsigned long long v0 = dig::to_bytes<false>(__double_as_longlong(w[r][0]), em);
+            const unsigned long long v1 = dig::to_bytes<false>(__double_as_longlong(w[r][1]), em);
             unsigned char* base = bbuf + r * DG_STEP_B + dg_off(c, 2 * gq);
 #pragma unroll
             for (int s = 0; s < dig::S; ++s)
@@ -325,10 +323,10 @@ __global__ void __launch_bounds__(DG_THREADS, 2) k_assemble_dg(Dims dm, DgArgs a
         __syncwarp();
         if (lane == 0) tc::mbar_arrive(&sh.bfull);
         if (window_end(ch, ch1)) {
-          wait(&sh.dfull, nwin++);
+          bool bad = !wait(&sh.dfull, nwin++);
           tc::fence_after_sync();
           if (32 * qt < Np) {
-            const bool bad = *failed != 0;
+            bad |= *failed != 0;
             const int rexp = face ? rexpF : rexpV;
             const bool init = !MIX && ch < NFC;
 #pragma unroll 1
@@ -428,6 +426,144 @@ __global__ void k_lift_exp(int Np, int Nb, int Nq, int Nfp, Geo G, int16_t* __re
   out[idx] = (int16_t)mx;
 }
 
+// x 2^(1023 - e) in FP32 from the upper word h of x, e >= 127: the lower mantissa bits are cut
+// off (relative error 2^-20), values below FP32's range become 0.
+__device__ __forceinline__ float norm32(int h, int e) {
+  const int m = max((h & 0x7fffffff) - ((e - 127) << 20), 0);
+  return __int_as_float((m << 3) | (h & (int)0x80000000));
+}
+
+// The exponents of the columns of V and W: em with |W| < 2^(em - 1022) for all points and
+// directions, as low as possible (a bound from the factors' separate maxima was 6 bits too
+// high on most columns and up to 15 on some, bits that the digits then lacked).  The sums
+// are formed in FP32 in one scale per element: their error is below 2^-15 of the largest term
+// a pair and column can have, and that, twice, is added to the largest one.  Pairs and columns
+// too small for FP32 beside the element's others keep the bound from the maxima.
+// A block takes an element, a warp 32 columns (lane = column) and a share of the points, with
+// all pairs' maxima in registers; the coefficients go through shared memory 32 points at a
+// time.  3D p = 3, 4096 elements 2.7 ms, p = 2, 2002 elements
+// 0.5 ms, p = 4, 210 elements 0.5 ms (a warp per pair with the operators in shared memory: 6.4 ms
+// at p = 3).
+constexpr int WE_PTS = 32, WE_WARPS = 16;
+template <int NP1, bool MIX>
+__global__ void __launch_bounds__(32 * WE_WARPS, 2) k_w_exp(Dims dm, DgArgs a, int groups) {
+  constexpr int NQ1 = NP1 + 1, Np = NP1 * NP1 * NP1, Nq = NQ1 * NQ1 * NQ1, Nfp = 6 * NQ1 * NQ1, m2 = 25;
+  constexpr int NbU = Np - (NP1 - 2) * (NP1 - 2) * (NP1 - 2);
+  __shared__ __align__(16) float sc[WE_PTS][m2][12];      // coefficients of a chunk of points
+  extern __shared__ int smx[];                            // [25][columns] largest sums (bits of FP32)
+  __shared__ int sref[3];                                 // largest exponents: basis value's coefficient, lifted, their coefficients
+  const int tid = threadIdx.x, nth = blockDim.x, lane = tid & 31, warp = tid >> 5;
+  const int64_t slot = blockIdx.x, e = a.elist ? a.elist[slot] : slot;
+  if (e < 0) return;
+  const int NbT = MIX ? dm.Nb : NbU, nb = MIX ? a.tt.nb[e] : NbU, w = Np + NbT, ncol = Np + nb, C = 32 * groups;
+  const int c = 32 * (warp % groups) + lane, share = warp / groups, shares = nth / C;
+  const bool on = c < ncol, ucol = c < Np;
+  const int col = ucol ? c : c - Np, bcol = ucol ? col : (MIX || !on ? 0 : a.ref.bnode[col]);
+  const int gst = ucol ? Np : NbT;
+  const int16_t* ec = a.ecoef + (size_t)e * m2 * 9;
+  auto hi = [](const double* p) { return reinterpret_cast<const int*>(p)[1]; };
+  auto has_cq = [](int pair) { return !(pair < 5 || (pair < 20 && pair % 5 == 4)); };
+  auto points = [&](auto at_faces) {
+    constexpr bool face = decltype(at_faces)::value;
+    constexpr int n = face ? Nfp : Nq;
+    const int16_t* eg = a.elift + ((size_t)e * 6 + 3 * face) * w;
+    // the element's scale
+    __syncthreads();
+    if (tid < 3) sref[tid] = 0;
+    for (int i = tid; i < m2 * C; i += nth) smx[i] = 0;
+    __syncthreads();
+    for (int i = tid; i < m2 * 9; i += nth) {
+      const int seg = i % 9, x = ec[i];
+      if (x != 0x7ff && (face ? seg >= 4 : seg < 4)) atomicMax(&sref[seg == 0 || seg == 4 || seg == 8 ? 0 : 2], x);
+    }
+    for (int i = tid; i < 3 * ncol; i += nth) atomicMax(&sref[1], (int)eg[(i / ncol) * w + i % ncol]);
+    __syncthreads();
+    const int scale = max(sref[0] + 1023, sref[2] + sref[1]);            // of a product, 2^(scale - 2046)
+    const int e_bas = min(scale - 1023, 127 + 2047), e_lift = sref[1], e_coef = min(scale - e_lift, 127 + 2047);
+    const bool fits = e_bas >= 127 && e_coef >= 127 && e_lift >= 127;
+    const double* G = face ? (ucol ? a.tb.GlF + (size_t)e * 3 * Nfp * Np + col : a.tb.HlF + (size_t)e * 3 * Nfp * NbT + col)
+                           : (ucol ? a.tb.GlV + (size_t)e * 3 * Nq * Np + col : a.tb.HlV + (size_t)e * 3 * Nq * NbT + col);
+    const double* B = (face ? a.tb.PhiF : a.tb.Phi) + bcol;
+    const bool basis = on && (face || ucol);
+    float mx[m2];
+#pragma unroll
+    for (int p = 0; p < m2; ++p) mx[p] = 0.f;
+    for (int g0 = 0; fits && g0 < n; g0 += WE_PTS) {
+      const int cnt = min(WE_PTS, n - g0);
+      __syncthreads();
+      // volume: cu_0..2, cq_00 .. cq_22 (l slow); faces: fq_0..2, fuh, S_ik or lambda
+      constexpr int per = face ? 5 : 12;
+      for (int i = tid; i < per * m2 * WE_PTS; i += nth) {
+        const int q = i % WE_PTS, k = (i / WE_PTS) % per, pair = i / (WE_PTS * per), g = g0 + q;
+        if (q >= cnt) continue;
+        const size_t ep = (size_t)e * m2 + pair;
+        const double* src;
+        if (!face) src = a.tb.Jv + (ep * 12 + k) * Nq + g;
+        else if (k < 4) src = a.tb.Jf + (ep * 4 + (k + 1) % 4) * Nfp + g;
+        else src = a.tb.Su ? a.tb.Su + ep * Nfp + g : a.tb.lamw + (size_t)e * Nfp + g;
+        const bool none = face && k == 4 && a.tb.Su == nullptr && pair % 6 != 0;       // lambda delta_ik
+        sc[q][pair][k] = none ? 0.f : norm32(hi(src), (face ? k >= 3 : k < 3) ? e_bas : e_coef);
+      }
+      __syncthreads();
+      for (int q = share; q < cnt; q += shares) {
+        const int g = g0 + q;
+        float x[3];
+#pragma unroll
+        for (int l = 0; l < 3; ++l) {
+          const float v = on ? norm32(hi(G + ((size_t)l * n + g) * gst), e_lift) : 0.f;
+          x[l] = ucol ? -v : v;
+        }
+        const float b = basis ? norm32(hi(B + (size_t)g * Np), 1023) : 0.f;
+#pragma unroll
+        for (int p = 0; p < m2; ++p) {
+          const float4 k0 = *reinterpret_cast<const float4*>(sc[q][p]);
+          if constexpr (face) {
+            float v = (ucol ? sc[q][p][4] : k0.w) * b;
+            if (has_cq(p)) v = fmaf(k0.z, x[2], fmaf(k0.y, x[1], fmaf(k0.x, x[0], v)));
+            mx[p] = fmaxf(mx[p], fabsf(v));
+          } else {
+            float v0 = k0.x * b, v1 = k0.y * b, v2 = k0.z * b;
+            if (has_cq(p)) {
+              const float4 k1 = *reinterpret_cast<const float4*>(sc[q][p] + 4), k2 = *reinterpret_cast<const float4*>(sc[q][p] + 8);
+              v0 = fmaf(k2.y, x[2], fmaf(k1.z, x[1], fmaf(k0.w, x[0], v0)));
+              v1 = fmaf(k2.z, x[2], fmaf(k1.w, x[1], fmaf(k1.x, x[0], v1)));
+              v2 = fmaf(k2.w, x[2], fmaf(k2.x, x[1], fmaf(k1.y, x[0], v2)));
+            }
+            mx[p] = fmaxf(fmaxf(mx[p], fabsf(v0)), fmaxf(fabsf(v1), fabsf(v2)));
+          }
+        }
+      }
+    }
+#pragma unroll
+    for (int p = 0; p < m2; ++p) atomicMax(&smx[p * C + c], __float_as_int(mx[p]));
+    __syncthreads();
+    for (int i = tid; i < m2 * ncol; i += nth) {
+      const int p = i / ncol, cc = i % ncol;
+      const bool uc = cc < Np;
+      // exponents of the pair's and column's terms; the largest real term is below 2^(top - 2044)
+      const int eb = (face && uc) ? (a.tb.Su || p % 6 == 0 ? ec[p * 9 + 8] : 0) : (face || uc ? ec[p * 9 + (face ? 4 : 0)] : 0);
+      int top = eb ? eb + 1023 : 0;
+      bool bad = eb == 0x7ff;
+      if (has_cq(p))
+        for (int l = 0; l < 3; ++l) {
+          const int el = ec[p * 9 + (face ? 5 : 1) + l], gl = eg[l * w + cc];
+          if (el && gl) top = max(top, el + gl);
+          bad |= el == 0x7ff;
+        }
+      int em = 0;
+      if (top) {
+        const int d = top - scale;
+        em = top - 1019;
+        if (fits && d > -90)
+          em = min(em, scale - 1150 + (__float_as_int(__int_as_float(smx[p * C + cc]) + __int_as_float((127 + d - 14) << 23)) >> 23));
+      }
+      a.ew[(((size_t)slot * m2 + p) * 2 + (face ? 0 : 1)) * w + cc] = (int16_t)(bad ? 3 * 0x7ff : max(em, 0));
+    }
+  };
+  if constexpr (!MIX) points(std::true_type{});
+  points(std::false_type{});
+}
+
 template <int NP1>
 cudaError_t dg_launch(iedg_mesh* M, const DgArgs& a, cudaStream_t st) {
   const Dims& dm = M->dm;
@@ -439,6 +575,15 @@ cudaError_t dg_launch(iedg_mesh* M, const DgArgs& a, cudaStream_t st) {
   int dev = 0, sms = 0;
   if (err == cudaSuccess) err = cudaGetDevice(&dev);
   if (err == cudaSuccess) err = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (err != cudaSuccess) return err;
+  const int groups = idiv_up(dm.Np + dm.Nb, 32);       // of columns; as many warps as fit share the points
+  if (groups > WE_WARPS) return cudaErrorInvalidValue;
+  const size_t wsmem = sizeof(int) * 25 * 32 * (size_t)groups;
+  auto wexp = mix ? k_w_exp<NP1, true> : k_w_exp<NP1, false>;
+  err = cudaFuncSetAttribute(wexp, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)wsmem);
+  if (err != cudaSuccess) return err;
+  wexp<<<(unsigned)a.n_el, 32 * groups * (WE_WARPS / groups), wsmem, st>>>(dm, a, groups);
+  err = cudaGetLastError();
   if (err != cudaSuccess) return err;
   const int tiles = idiv_up(25 * (dm.Np + dm.Nb), DG_COLS);
   const int64_t n = a.n_el * tiles, g = 2 * (int64_t)sms;
@@ -510,7 +655,7 @@ cudaError_t launch_assemble_dg(iedg_mesh* M, double* S, const int64_t* elist, in
   k_coef_exp<<<(unsigned)((nw * 32 + 255) / 256), 256, 0, st>>>(dm.Nq, dm.Nfp, tb, M->pj.ecoef, nw, elist);
   cudaError_t err = cudaGetLastError();
   if (err != cudaSuccess) return err;
-  const DgArgs a{tb, M->ref, M->pj.ecoef, M->geo.elift, elist ? M->rhs64 : nullptr, S, M->ph.alpha, M->tt, elist, n_el,
+  const DgArgs a{tb, M->ref, M->pj.ecoef, M->geo.elift, M->pj.ew, elist ? M->rhs64 : nullptr, S, M->ph.alpha, M->tt, elist, n_el,
                  asm_wait_limit(M)};
   if (dm.p == 2) return dg_launch<3>(M, a, st);
   if (dm.p == 3) return dg_launch<4>(M, a, st);

@@ -2,10 +2,11 @@
 // partial LU; csrc/iedg_assemble_dg.cu, the volume terms of the assembly).
 //
 // With emax the biased exponent of (a bound on) a row's or column's largest entry, an
-// entry x becomes the integer X nearest to x 2^(61 - (emax - 1023)), |X| < 2^62, in balanced
+// entry x becomes the integer X next to x 2^(61 - (emax - 1023)), |X| < 2^62, in balanced
 // base 256: X = sum_s d_s 256^(7 - s), s = 0..7, -128 <= d_s <= 127 and |d_0| <= 64.  Digits
 // are exact in BF16 and their products' sums exact in FP32 below 2^24.  X is in error by up to
-// 2^-62 of the largest entry: entries far below it keep fewer bits than FP64 holds.
+// 2^-62 (rounded; 2^-61 cut off) of the largest entry, or of a bound on it: entries far below
+// it keep fewer bits than FP64 holds.
 #pragma once
 #include <cstdint>
 #include <cuda_runtime.h>
@@ -19,11 +20,12 @@ constexpr int BAD_EXP = 1 << 13;         // exponent of a row or column with a n
 __host__ __device__ __forceinline__ int exponent_bits(long long b) { return (int)((b >> 52) & 0x7ff); }
 
 // The digits of x, each with 128 added, most significant in the top byte.  Entries below
-// 2^-63 of the scale and subnormals become 0.
+// 2^-62 of the scale and subnormals become 0.  NEAREST: rounded, not cut off (towards zero).
+template <bool NEAREST = true>
 __host__ __device__ __forceinline__ unsigned long long to_bytes(long long b, int emax) {
   const int e = exponent_bits(b), sh = emax - e;
   unsigned long long m = ((unsigned long long)b & 0xFFFFFFFFFFFFFull) | 0x10000000000000ull;
-  m = (e == 0 || sh > 62 || sh < 0) ? 0ull : (((m << 10) >> sh) + 1) >> 1;
+  m = (e == 0 || sh > 62 || sh < 0) ? 0ull : (NEAREST ? (((m << 10) >> sh) + 1) >> 1 : (m << 9) >> sh);
   return (b < 0 ? 0ull - m : m) + 0x8080808080808080ull;
 }
 

@@ -104,6 +104,8 @@ struct PointJac {
   double* Jb;     // [E][m][m][2+d][Nfp]   : boundary faces only: wf dbhat/duhat, wf dbhat/du,
                   //                          wf dbhat/dq_l (null without boundary faces)
   int16_t* ecoef; // [E][25][9] largest exponents of the pairs' coefficients (null: unused)
+  int16_t* ew;    // [E][25][2][Np+Nb] exponents of the columns of V, W (null: unused; mixed forms:
+                  //                   [kFallbackSlots][25][2][Np+Nb])
   float *Jv32, *Jf32, *lamw32, *Su32, *Jb32;   // FP32 copies written by the point kernel (mixed path only)
 };
 
