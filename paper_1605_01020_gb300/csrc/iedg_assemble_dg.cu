@@ -34,9 +34,9 @@
 // 1 : 1000 1.8e-16 1.8e-12 | 1.1e-16 1.1e-12 (with the bound from separate maxima as scale
 // 4.5e-15 1.4e-14, 9.3e-15 2.5e-14, 4.8e-15 2.4e-11).
 // Measured, all elements, sum-factorised on the FP64 pipe -> this form (k_coef_exp, k_w_exp,
-// k_assemble_dg): 3D p = 3, 4096 elements 135.4 -> 101.2 ms; p = 2, 2002 elements 14.0 ->
-// 13.4 ms; p = 4, 210 elements 32.8 -> 19.2 ms; orders 2, 3, 4 mixed, 324 elements 25.6 ->
-// 17.6 ms.  Counters at p = 3: FP64 pipe 50 % busy, tensor pipe 26 %, 7.9 TB/s from L2, two
+// k_assemble_dg): 3D p = 3, 4096 elements 135.4 -> 100.6 ms; p = 2, 2002 elements 14.0 ->
+// 13.1 ms; p = 4, 210 elements 32.8 -> 18.8 ms; orders 2, 3, 4 mixed, 324 elements 25.6 ->
+// 17.4 ms.  Counters at p = 3: FP64 pipe 50 % busy, tensor pipe 26 %, 7.9 TB/s from L2, two
 // thirds of it the tables.
 #include <algorithm>
 #include <cstdlib>
@@ -126,7 +126,9 @@ __global__ void __launch_bounds__(DG_THREADS, 2) k_assemble_dg(Dims dm, DgArgs a
   // flight is waited for, and the build warps go through the tiles that are left writing NaN.
   // Arrivals then no longer match the waits, which costs nothing: nobody waits for them.
   auto wait = [&](uint64_t* bar, uint32_t parity) {
-    const bool ok = tc::mbar_wait(bar, parity & 1u, *failed ? 1 : a.wait_limit);
+    // (the flag is read only when the first poll, the usual case, did not do)
+    bool ok = a.wait_limit > 0 && tc::mbar_wait(bar, parity & 1u, 1);
+    if (!ok) ok = tc::mbar_wait(bar, parity & 1u, *failed ? 1 : a.wait_limit);
     if (!ok) *failed = 1;
     return ok;
   };
@@ -157,8 +159,7 @@ __global__ void __launch_bounds__(DG_THREADS, 2) k_assemble_dg(Dims dm, DgArgs a
         if (!tile_of(id, slot, e, nb, c0, ch1)) continue;
         for (int s = 3 * ch0; s < 3 * ch1; ++s, ++q) {
           const uint32_t st = q % DG_RING;
-          if (q >= DG_RING) wait(&sh.empty[st], q / DG_RING - 1);
-          if (*failed) break;
+          if (q >= DG_RING && !wait(&sh.empty[st], q / DG_RING - 1)) break;
           tc::mbar_expect_tx(&sh.full[st], DG_STEP_A);
           tc::bulk_g2s(ring + st * DG_STEP_A, a.ref.Vdig + (size_t)s * DG_STEP_A, DG_STEP_A, &sh.full[st]);
         }
@@ -179,13 +180,13 @@ __global__ void __launch_bounds__(DG_THREADS, 2) k_assemble_dg(Dims dm, DgArgs a
         int nb, c0, ch1;
         if (!tile_of(id, slot, e, nb, c0, ch1)) continue;
         for (int ch = ch0; ch < ch1; ++ch, ++nch) {
-          if (start && nwin > 0) wait(&sh.dread, nwin - 1);   // accumulators read
-          wait(&sh.bfull, nch);                               // W of this chunk staged
+          bool ok = !start || nwin == 0 || wait(&sh.dread, nwin - 1);   // accumulators read
+          ok = ok && wait(&sh.bfull, nch) && !*failed;                  // W of this chunk staged
           const bool end = window_end(ch, ch1);
-          for (int r = 0; r < 3 && !*failed; ++r, ++q) {
+          for (int r = 0; r < 3; ++r, ++q) {
             const uint32_t st = q % DG_RING;
-            wait(&sh.full[st], q / DG_RING);
-            if (*failed) break;
+            ok = ok && wait(&sh.full[st], q / DG_RING);
+            if (!ok) break;
             tc::fence_after_sync();
 #pragma unroll
             for (int s = 0; s < dig::S; ++s)
@@ -194,7 +195,7 @@ __global__ void __launch_bounds__(DG_THREADS, 2) k_assemble_dg(Dims dm, DgArgs a
                            (start && r == 0 && s == 0) ? 0u : 1u);
             tc::mma_commit(&sh.empty[st]);
           }
-          if (*failed) break;
+          if (!ok) break;
           tc::mma_commit(&sh.bempty);
           if (end) tc::mma_commit(&sh.dfull);
           nwin += end;
