@@ -2,10 +2,10 @@
 
 For one mesh (fixed dimension, order, quadrature and precision) it times
 iedg_assemble_condensed under every candidate iedg_schedule (persistent or
-one-CTA-per-element LU, FP64 LU panel width, assembly column chunk) with CUDA
-events, keeps the fastest, and caches the choice in a JSON file keyed by the GPU
-name and the mesh class, so later runs on the same kind of GPU skip the sweep.
-Results do not depend on the schedule (beyond summation order in the LU).
+one-CTA-per-element LU, the LU's form, FP64 DFMA panel width, assembly column chunk on
+meshes with mixed orders) with CUDA events, keeps the fastest, and caches the choice in
+a JSON file keyed by the GPU name and the mesh class, so later runs on the same kind of
+GPU skip the sweep.  Results do not depend on the schedule (beyond rounding in the LU).
 """
 import itertools
 import json
@@ -14,32 +14,33 @@ import os
 DEFAULT_CACHE = os.path.join(os.path.expanduser("~"), ".cache", "iedg", "schedules.json")
 
 
+# what the schedule's values select; choices cached under another number are not used
+SCHEDULE_VERSION = 2
+
+
 def mesh_key(mesh, precision, gpu_name):
     extra = getattr(mesh, "orders_key", "")
-    return f"{gpu_name}|d{mesh.d}|p{mesh.order}|Np{mesh.Np}|prec{precision}{extra}"
+    return f"{gpu_name}|d{mesh.d}|p{mesh.order}|Np{mesh.Np}|prec{precision}{extra}|schedule{SCHEDULE_VERSION}"
 
 
 def candidates(precision, order):
-    """Candidate schedules: persistent LU on/off x FP64 panel 16/32 x assembly chunk,
-    and the tensor-core forms (FP64: the digit form, which 0 also takes on elements of
-    64 u-unknowns or more; on the mixed path the FP32 LU with every trailing update in 3xTF32, or only its
-    deferred Schur complement; handles with TF32 or BF16 Schur operands always take
-    the tensor-core form).
-    order 0 (mixed orders): the FP64 panel stays 16 (the largest elements' panel of
-    32 does not fit in shared memory)."""
-    panels = [16, 32] if (precision == 0 and 1 <= order <= 3) else [16]
-    chunks = [8, 16] if precision == 0 else [16, 32]
+    """Candidate schedules, one for each choice of kernels: persistent LU on/off, and
+      FP64: the DFMA form with panels of 16 and 32 (order 4 and mixed orders: 16 only, the
+        wider panel does not fit in shared memory), and the digit form on the tensor cores
+        (persistent);
+      mixed FP32: every trailing update on the tensor cores in 3xTF32 (lu_tensor 2), only the
+        deferred Schur complement (1), FFMA updates (0); handles with TF32 or BF16 Schur
+        operands always take the deferred form (1).
+    The assembly's column chunk exists on meshes with mixed orders (order 0) only."""
+    chunks = ([8, 16] if precision == 0 else [16, 32]) if order == 0 else [0]
     if precision == 0:
-        # the form chosen by size, then the tensor-core form (persistent, panel 16 only)
-        out = [dict(lu_persistent=a, lu_panel=b, asm_chunk=c, lu_tensor=0)
-               for a, b, c in itertools.product([1, 0], panels, chunks)]
-        return out + [dict(lu_persistent=1, lu_panel=16, asm_chunk=c, lu_tensor=1) for c in chunks]
-    # TF32 / BF16 Schur operands: the tensor-core form is what the precision means.
-    # FP32 form: every trailing update on the tensor cores (2), the deferred Schur
-    # complement on the tensor cores (1), or FFMA updates (0)
-    tensor = [2, 1, 0] if precision == 1 else [1]
-    return [dict(lu_persistent=a, lu_panel=b, asm_chunk=c, lu_tensor=t)
-            for a, b, c, t in itertools.product([1, 0], panels, chunks, tensor)]
+        panels = [16, 32] if 1 <= order <= 3 else [16]
+        lu = [dict(lu_persistent=a, lu_panel=b, lu_tensor=0) for a, b in itertools.product([1, 0], panels)]
+        lu.append(dict(lu_persistent=1, lu_panel=16, lu_tensor=1))
+    else:
+        tensor = [2, 1, 0] if precision == 1 else [1]
+        lu = [dict(lu_persistent=a, lu_panel=16, lu_tensor=t) for a, t in itertools.product([1, 0], tensor)]
+    return [dict(x, asm_chunk=c) for x, c in itertools.product(lu, chunks)]
 
 
 def time_assemble(mesh, u, q, uh, K, R, reps, warm=True):
