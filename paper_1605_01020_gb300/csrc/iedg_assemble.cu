@@ -500,8 +500,8 @@ __device__ __forceinline__ void lu_element(const LuElem& el, T* __restrict__ S, 
 // entry's own terms, 32 roundings of 2^-53.  So the digit form is the more accurate one for
 // entries within about 2^-6 of that product, and the less accurate one far below it; entries
 // whose old value and update are both below 2^-28 of it are formed by DFMA (0.4 % of them in
-// the fourth line below, 1 % in the fifth, whose state has a direction at rest; that costs
-// 3 % of the kernel, at 2^-20 it cost 9 %).
+// the fourth line below, 1 % in the fifth, whose state has a direction at rest; 3 % of the
+// kernel's time, 10 % with a line at 2^-20).
 // Errors of K against 80-bit elimination, numpy model of both forms, DFMA | digits: largest
 // entry, worst of the 25 component blocks, median entry:
 //   p = 2, Re 2.5e5, M 0.2, cubes          2.2e-15 3.7e-13 4.6e-15 | 3.0e-16 2.7e-13 3.2e-15
@@ -511,7 +511,7 @@ __device__ __forceinline__ void lu_element(const LuElem& el, T* __restrict__ S, 
 //   p = 3, Re 2.5e5, M 0.2, cubes          3.6e-15 2.4e-13 2.2e-14 | 7.3e-16 1.7e-13 1.0e-14
 //   p = 3, Re 10, M 0.05, cells 1 : 200    7.6e-15 1.9e-10 1.1e-13 | 5.6e-15 5.5e-11 5.3e-14
 // (without s_k, level 8 and the rounding of the operands the second line's digits were
-// 5.1e-15 1.8e-11 2.0e-13, the fourth's 100 to 300 times DFMA's).
+// 5.1e-15 1.8e-11 2.0e-13, the fourth's hundreds of times DFMA's).
 //
 // Roles: the 128 TMEM lanes are columns of A22 (the MMA's A operand is U12^T), so a
 // warp's accesses of A22 are rows of 32 consecutive columns; the B operand stacks the
@@ -528,8 +528,7 @@ __device__ __forceinline__ void lu_element(const LuElem& el, T* __restrict__ S, 
 // 2D p = 3 (64 + 48 unknowns), 851 elements 1.53 -> 0.84 ms.  Below 64 u-unknowns an
 // element is at most two panels, which leaves too little to the tensor cores, and the
 // DFMA form stays: 2D p = 2 (36 + 32), 1600 elements 0.79 ms DFMA, 0.98 ms digits; 3D p = 1
-// (40 + 40), 8000 elements 4.98 and 5.10 ms.  Counters at p = 3: FP64 pipe 47 % busy, issue
-// slots 35 %, tensor pipe 8 %, 42 MB of DRAM traffic per element: latency of the panel
+// (40 + 40), 8000 elements 4.98 and 5.10 ms.  Latency of the panel
 // steps and of the trailing block's loads, not a pipe, is what is left.
 constexpr int LT_NB = 32;                       // panel width
 constexpr int LT_S = dig::S;                    // digits per operand, and levels kept
