@@ -876,7 +876,14 @@ __global__ void k_point_res(Dims dm, Phys ph, RefTables ref, Geo G, PointJac PJ,
   }
 }
 
-constexpr int64_t kSpread = 8 * 152;   // blocks of 128 threads that keep every SM evenly busy
+// Blocks of 128 threads that keep every SM of the current device evenly busy (8 per SM).
+cudaError_t spread_blocks(int64_t* blocks) {
+  int dev = 0, sms = 0;
+  cudaError_t err = cudaGetDevice(&dev);
+  if (err == cudaSuccess) err = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  *blocks = 8 * (int64_t)sms;
+  return err;
+}
 
 // q*[e][c][k][l] = sum_t H_l[c][t] uhat_k(t) - sum_b G_l[c][b] u_k(b)
 // One output a thread, an element's outputs over several blocks: a thread's chain of loads and
@@ -952,11 +959,14 @@ cudaError_t launch_points(iedg_mesh* M, const double* u, const double* q, const 
     err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (err != cudaSuccess) return err;
     // An element's warps over several blocks where the elements alone are too few to fill the
-    // chip evenly (below kSpread blocks): each block repeats the nodal loads (and, in FP64, the
+    // chip evenly (below spread_blocks): each block repeats the nodal loads (and, in FP64, the
     // interpolation), which large meshes need not pay.  3D p = 4, 210 elements 1.0 -> 0.84 ms
     // (FP32 1.34 -> 1.10); 175 elements of orders 2..4 1.9 -> 1.2 ms.
     const int items = (dm.Nq + 31) / 32 + (dm.Nfp + 31) / 32, most = (items + threads / 32 - 1) / (threads / 32);
-    const int64_t want = (kSpread + M->E - 1) / M->E;
+    int64_t spread = 0;
+    err = spread_blocks(&spread);
+    if (err != cudaSuccess) return err;
+    const int64_t want = (spread + M->E - 1) / M->E;
     const dim3 grid((unsigned)M->E, (unsigned)(want < most ? want : most));
     kern<<<grid, threads, smem, st>>>(dm, M->ph, M->ref, M->geo, M->pj, M->etrace, u, q, uhat, M->tt, FS);
     err = cudaGetLastError();
@@ -1000,7 +1010,10 @@ cudaError_t launch_rq(iedg_mesh* M, const double* q, const double* qs, double* r
                       cudaStream_t st) {
   const Dims& dm = M->dm;
   size_t smem = sizeof(double) * (size_t)dm.Np * dm.m * dm.d;
-  const int64_t want = (kSpread + M->E - 1) / M->E, most = idiv_up(dm.Np * dm.m * dm.d, 128);
+  int64_t spread = 0;
+  const cudaError_t err = spread_blocks(&spread);
+  if (err != cudaSuccess) return err;
+  const int64_t want = (spread + M->E - 1) / M->E, most = idiv_up(dm.Np * dm.m * dm.d, 128);
   const dim3 grid((unsigned)M->E, r_q ? (unsigned)(want < most ? want : most) : 1u);
   k_rq<<<grid, 128, smem, st>>>(dm, M->geo, q, qs, r_q, rhoq);
   return cudaGetLastError();
