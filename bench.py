@@ -99,6 +99,40 @@ def traffic_record(kernel, precision, dims):
     return None
 
 
+def short(x):
+    """x with every float at seven significant digits: the line stays within the few
+    kilobytes that its readers keep of a program's output."""
+    if isinstance(x, float):
+        return float(f"{x:.7g}")
+    if isinstance(x, dict):
+        return {k: short(v) for k, v in x.items()}
+    return [short(v) for v in x] if isinstance(x, (list, tuple)) else x
+
+
+def kernel_table(prof):
+    """Launches, milliseconds and share of the device time per kernel name."""
+    tot = sum(v[1] for v in prof.values())
+    return {k: {"launches": v[0], "ms": float(f"{v[1]:.4g}"), "share": round(v[1] / tot, 4) if tot else None}
+            for k, v in prof.items()}
+
+
+def slim(line, low):
+    """The printed line: the legs beside the FP64 one keep their rates, errors and schedules,
+    and milliseconds per kernel where the form is not a variant of another leg's."""
+    ms = lambda r: {**r, "kernels": {k: v["ms"] for k, v in r["kernels"].items()}} if r and "kernels" in r else r
+    out = {**line, "mixed": ms(line["mixed"])}
+    if line["mixed_orders"]:
+        out["mixed_orders"] = {k: ms(v) if isinstance(v, dict) else v for k, v in line["mixed_orders"].items()}
+    keep = ("value", "ms_per_step", "speedup_vs_fp64", "err_vs_fp64", "schedule", "element_status_nonzero", "gpu_launches")
+    out.update({k: {q: r[q] for q in keep if q in r} for k, r in low.items()})
+    return out
+
+
+def print_timings(leg, timings):
+    """The autotuner's table goes to stderr, beside the one line of stdout."""
+    print(json.dumps({"autotune_ms": leg, **short(timings)}), file=sys.stderr, flush=True)
+
+
 def workload_name(wl):
     return f"{wl.name} ({wl.mesh.n_elem} elements), FP64: residual + condensed trace Jacobian + back-substitution"
 
@@ -300,11 +334,12 @@ def run_ours(args, wl, rank, world, local_rank):
     u = torch.as_tensor(st.u, dtype=f64, device=dev)
     uh = torch.as_tensor(st.uhat, dtype=f64, device=dev)
     duh = torch.as_tensor(st.duhat, dtype=f64, device=dev)
-    schedule, timings64 = None, {}
+    schedule = None
     if not args.no_autotune:
         from paper_1605_01020_gb300 import autotune
         qt = torch.as_tensor(st.q, dtype=f64, device=dev)
         schedule, timings64 = autotune.autotune(mesh, u, qt, uh, 0, reps=1)
+        print_timings("fp64", timings64)
         del qt
     q = torch.empty(E, Np, m, d, dtype=f64, device=dev)
     rq = torch.empty_like(q)
@@ -433,7 +468,6 @@ def run_ours(args, wl, rank, world, local_rank):
     # roofline of the dominant kernel (largest summed device time)
     top = max(prof.items(), key=lambda kv: kv[1][1])
     name, (launches, kms) = top
-    tot_ms = sum(v[1] for v in prof.values())
     props = torch.cuda.get_device_properties(dev)
     sm_max = clocks["sm_max_mhz"] or 2070.0
     up = unit_peaks()
@@ -489,21 +523,20 @@ def run_ours(args, wl, rank, world, local_rank):
             "vs_baseline": None, "dtype": "f64", "data": "synthetic",
             "config": {"workload": workload_name(wl), "elements": E, "order": wl.mesh.p, "precision": "fp64",
                        "l2": "flushed between steps (512 MB write); per-step workspace 12 GB >> L2",
-                       "per_rank_elements": E, "schedule": schedule, "autotune_ms": timings64},
+                       "per_rank_elements": E, "schedule": schedule},
             "roofline": roof, "cpu_baseline": cpu,
             "e2e": {"value": value_e2e, "unit": "elements/s", "h2d_bytes_per_step": h2d,
                     "d2h_bytes_per_step": d2h,
                     "overlap": "results copied to pinned host memory on a second stream during the next step"},
             "clocks": clocks, "gpu_launches": sum(v[0] for v in prof.values()),
-            "kernels": {k: {"launches": v[0], "ms": v[1], "share": v[1] / tot_ms if tot_ms else None}
-                        for k, v in prof.items()},
+            "kernels": kernel_table(prof),
             "element_status_nonzero": int((status != 0).sum()),
             "mixed": mixed,
-            **low,
             "mixed_orders": mixed_orders,
             "extras": extras,
             "peaks": {"source": src, **{k: v for k, v in peaks.items() if isinstance(v, (int, float))}}}
-    print(json.dumps(line), flush=True)
+    print(json.dumps({"detail": short({**line, **low})}), file=sys.stderr, flush=True)
+    print(json.dumps(short(slim(line, low))), flush=True)
 
 
 MIXED_FORMS = {1: "FP32 element matrix + partial LU, FP64 refinement",
@@ -525,7 +558,7 @@ def run_mixed(args, wl, mesh64, dev, step_outputs, inputs, flush, barrier, preci
     mesh = iedg.mesh_from_workload(wl, precision=precision, flags=flags)
     E, Np, m, d, T = mesh.E, mesh.Np, mesh.m, mesh.d, mesh.T
     f64 = torch.float64
-    schedule, timings = None, {}
+    schedule = None
     if args.mixed_lu_tensor is not None and precision == 1:
         mesh.set_schedule(lu_tensor=args.mixed_lu_tensor)
         schedule = mesh.get_schedule()
@@ -533,6 +566,7 @@ def run_mixed(args, wl, mesh64, dev, step_outputs, inputs, flush, barrier, preci
         from paper_1605_01020_gb300 import autotune
         qt = torch.as_tensor(wl.state.q, dtype=f64, device=dev)
         schedule, timings = autotune.autotune(mesh, u, qt, uh, precision, reps=1)
+        print_timings(f"precision {precision} flags {flags}", timings)
         del qt
     q = torch.empty(E, Np, m, d, dtype=f64, device=dev)
     rq, ru, rfl = torch.empty_like(q), torch.empty(E, Np, m, dtype=f64, device=dev), torch.empty(T, m, dtype=f64, device=dev)
@@ -589,11 +623,11 @@ def run_mixed(args, wl, mesh64, dev, step_outputs, inputs, flush, barrier, preci
     out = {"ms_total": e0.elapsed_time(e1),
            "precision": MIXED_FORMS[precision] + ("; element systems scaled by the mass matrix's inverse Cholesky "
                                                   "factor before the factorisation" if flags else ""),
-           "schedule": schedule, "autotune_ms": timings, "roofline": roof,
+           "schedule": schedule, "roofline": roof,
            "err_vs_fp64": {"K": err(K, K64), "R": err(R, R64), "du": err(du, du64), "dq": err(dq, dq64)},
            "element_status_nonzero": int((status != 0).sum()),
            "gpu_launches": sum(v[0] for v in prof.values()),
-           "kernels": {k: {"launches": v[0], "ms": v[1], "share": v[1] / tot if tot else None} for k, v in prof.items()}}
+           "kernels": kernel_table(prof)}
     mesh.close()
     return out
 
@@ -627,10 +661,11 @@ def run_mixed_orders(args, dev, flush):
         mesh = iedg.MixedOrderMesh(msh.node_xyz, msh.elem_trace, msh.n_trace, msh.orders, msh.face_degree,
                                    gamma=prm["gamma"], Pr=prm["Pr"], Re=prm["Re"], Minf=prm["Minf"],
                                    alpha=prm["alpha"], precision=precision)
-        schedule, timings = None, {}
+        schedule = None
         if not args.no_autotune:
             from paper_1605_01020_gb300 import autotune
             schedule, timings = autotune.autotune(mesh, u, qin, uh, precision, reps=1)
+            print_timings(f"mixed orders precision {precision}", timings)
         q = torch.empty(mesh._qshape, dtype=f64, device=dev)
         rq, dq = torch.empty_like(q), torch.empty_like(q)
         ru, du = torch.empty(mesh._ushape, dtype=f64, device=dev), torch.empty(mesh._ushape, dtype=f64, device=dev)
@@ -674,15 +709,13 @@ def run_mixed_orders(args, dev, flush):
             torch.cuda.synchronize()
             ms += e0.elapsed_time(e1)
         status = mesh.element_status()
-        tot = sum(v[1] for v in prof.values())
         lu = prof.get("lu_schur", (1, float("nan")))
-        r = {"schedule": schedule, "autotune_ms": timings, "value": E * args.steps / (ms / 1e3),
+        r = {"schedule": schedule, "value": E * args.steps / (ms / 1e3),
              "unit": "elements/s", "ms_per_step": ms / args.steps, "timing": "CUDA graph replay of one step",
              "gpu_launches_per_step": launches_per_step,
              "element_status_nonzero": int((status != 0).sum()),
              "lu_schur_ms": lu[1] / lu[0], "lu_schur_tflops": lu_flops / (lu[1] / lu[0] / 1e3) / 1e12,
-             "kernels": {k: {"launches": v[0], "ms": v[1], "share": v[1] / tot if tot else None}
-                         for k, v in prof.items()}}
+             "kernels": kernel_table(prof)}
         outs[precision] = [t.clone() for t in (K, R, du, dq)]
         res["fp64" if precision == 0 else "mixed"] = r
         del g
