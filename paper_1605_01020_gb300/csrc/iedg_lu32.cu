@@ -167,17 +167,10 @@ __device__ __forceinline__ void lu32_update(float* __restrict__ A, int ld, float
         Ls[(j + 2) * LS + r] = v.z;
         Ls[(j + 3) * LS + r] = v.w;
       }
-      // this thread's 8 rows x (4 + 4) columns; the next row block's lines are asked of L2
+      // this thread's 8 rows x (4 + 4) columns (an L2 prefetch of the next row block's lines, kept
+      // inside the matrix, made it slower: p = 3 31.8 -> 32.9 ms, p = 4 16.6 -> 18.4)
       float acc[8][8];
       const int ca = cc + 4 * tc, cb = ca + 64;
-      if (rb + RT < r_hi) {
-        // 16 threads cover a row's four lines of the tile, eight rows each; the tile's columns
-        // past the last one are in no row of this element (past the last row: in no matrix)
-        const int pr = rb + RT + 8 * tr + (tc >> 1), pc = cc + 64 * (tc & 1);
-        const float* pf = A + (int64_t)pr * ld + pc;
-        if (pr < r_hi && pc < c_hi) asm volatile("prefetch.global.L2 [%0];" ::"l"(pf));
-        if (pr < r_hi && pc + 32 < c_hi) asm volatile("prefetch.global.L2 [%0];" ::"l"(pf + 32));
-      }
       const bool va = aligned && ca + 4 <= vlim, vb = aligned && cb + 4 <= vlim;
 #pragma unroll
       for (int i = 0; i < 8; ++i) {
