@@ -49,6 +49,7 @@ class Problem:
         self.fmu = ref.fphi[:, :, ref.bnodes] if fmu is None else np.asarray(fmu)   # [nf, Nfq, Nb]
         self.Nb = self.fmu.shape[2]
         self.source = source
+        self._blocks = {}          # element_blocks: the last few elements' blocks by their inputs
 
     # ------------------------------------------------------------------ points
     def points(self, els, u, q, uhat):
@@ -129,7 +130,21 @@ class Problem:
     # ------------------------------------------------------------ Newton blocks
     def element_blocks(self, e, u, q, uhat, u_ref=None):
         """Dense Newton blocks of element e in the ordering of the module docstring.
-        Returns dict with A_qq, A_qu, B_q, A_uq, A_uu, B_u, C_q, C_u, D, F_q, F_u, G."""
+        Returns dict with A_qq, A_qu, B_q, A_uq, A_uu, B_u, C_q, C_u, D, F_q, F_u, G.
+        Condensation and back-substitution of an element ask for the same blocks; those of
+        the last eight sets of inputs (compared by value) are kept, read-only."""
+        key = (e, *(None if x is None else np.asarray(x).tobytes()
+                    for x in (u[e], q[e], uhat[self.elem_trace[e]], None if u_ref is None else u_ref[e])))
+        if key not in self._blocks:
+            while len(self._blocks) >= 8:
+                self._blocks.pop(next(iter(self._blocks)))
+            blk = self._element_blocks(e, u, q, uhat, u_ref)
+            for x in blk.values():
+                x.flags.writeable = False
+            self._blocks[key] = blk
+        return dict(self._blocks[key])
+
+    def _element_blocks(self, e, u, q, uhat, u_ref):
         ref, geo, prm, d, m = self.ref, self.geo, self.prm, self.d, self.m
         Np, Nb = ref.Np, self.Nb
         els = np.array([e])
