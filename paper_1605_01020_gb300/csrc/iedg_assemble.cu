@@ -528,8 +528,8 @@ __device__ __forceinline__ void lu_element(const LuElem& el, T* __restrict__ S, 
 // 2D p = 3 (64 + 48 unknowns), 851 elements 1.53 -> 0.84 ms.  Below 64 u-unknowns an
 // element is at most two panels, which leaves too little to the tensor cores, and the
 // DFMA form stays: 2D p = 2 (36 + 32), 1600 elements 0.79 ms DFMA, 0.98 ms digits; 3D p = 1
-// (40 + 40), 8000 elements 4.98 and 5.10 ms.  Latency of the panel
-// steps and of the trailing block's loads, not a pipe, is what is left.
+// (40 + 40), 8000 elements 4.98 and 5.10 ms.  Latency of the panel steps and of the
+// trailing block's loads, not a pipe, is what is left.
 constexpr int LT_NB = 32;                       // panel width
 constexpr int LT_S = dig::S;                    // digits per operand, and levels kept
 using dig::exponent_of;
@@ -876,7 +876,7 @@ __device__ __forceinline__ bool lt_trailing(LtShared& sh, double* __restrict__ A
           for (; redo; redo &= redo - 1) {
             const int row = row0 + __ffs(redo) - 1, lr = row - rb;
             // products that all vanish leave the entry as it is, unless an operand is not finite
-            if (col >= ncol || row >= n || ((cmask & sh.rm[lr]) == 0 && ecol + sh.re[lr] < dig::BAD_EXP)) continue;
+            if (col >= ncol || row >= n || ((cmask & sh.rm[lr]) == 0 && max(ecol, sh.re[lr]) < dig::BAD_EXP)) continue;
             double* v = A + (int64_t)row * ld + col;
             *v = lt_entry(A + (int64_t)row * ld + kb, A + (int64_t)kb * ld + col, ld, nb, *v);
             bad |= row >= nu && col >= nu && exponent_of(*v) == 0x7ff;
