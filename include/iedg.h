@@ -276,20 +276,21 @@ int iedg_trace_solve(iedg_mesh* mesh, const double* K, const double* R, double* 
  *                  default: 8 for FP64, 16 for FP32; too large a chunk for shared
  *                  memory falls back).  Uniform meshes assemble without chunks.
  *   lu_tensor:     tensor cores (tcgen05, accumulation in tensor memory) in the partial LU.
- *                  FP64 path: the trailing updates as integer products of 8-bit digits of
- *                  the FP64 operands, summed exactly and joined to FP64.  The error of an
- *                  update is then relative to (largest entry of its row) x (largest of
- *                  its column), about 2^-60 after a scaling that evens out the panel's
- *                  rows, where the DFMA form's is relative to the entry's own terms;
- *                  entries far below that product are formed by DFMA.  1 = that form;
- *                  0 = DFMA updates, at every size.  Mixed path: 1 = the Schur complement K = D - W Z, TF32 operands
- *                  split in high and low parts, three products ("3xTF32"); 2 (mixed FP32
- *                  form only) = every trailing update of the FP32 LU (3xTF32, 128 x 64
- *                  tiles accumulated in TMEM and subtracted from the trailing block by
- *                  reductions in L2); 0 = FFMA updates.  Default: FP64 1 where the
- *                  (largest) element has at least 64 u-unknowns, from where it is the
- *                  faster form, 0 below; mixed 0, except 2 for FP32 handles of meshes
- *                  with mixed orders.  Handles created with
+ *                  FP64 path: 1 = the trailing updates as integer products of 8-bit digits
+ *                  of the FP64 operands, summed exactly and joined to FP64; 0 = DFMA
+ *                  updates.  The error of an update by digits is relative to (largest
+ *                  entry of its row) x (largest of its column), about 2^-60 after a
+ *                  scaling that evens out the panel's rows, where the DFMA form's is
+ *                  relative to the entry's own terms; entries far below that product are
+ *                  formed by DFMA.
+ *                  Mixed path: 1 = the Schur complement K = D - W Z, TF32 operands split
+ *                  in high and low parts, three products ("3xTF32"); 2 (mixed FP32 form
+ *                  only) = every trailing update of the FP32 LU (3xTF32, 128 x 64 tiles
+ *                  accumulated in TMEM and subtracted from the trailing block by
+ *                  reductions in L2); 0 = FFMA updates.
+ *                  Default: FP64 1 where the (largest) element has at least 64
+ *                  u-unknowns, from where it is the faster form, 0 below; mixed 0, except
+ *                  2 for FP32 handles of meshes with mixed orders.  Handles created with
  *                  IEDG_PRECISION_MIXED_TF32 or _MIXED_BF16 always take the tensor-core
  *                  form in their own operand precision (the schedule never changes
  *                  what is computed, only how).
@@ -323,10 +324,10 @@ int iedg_set_schedule(iedg_mesh* mesh, const iedg_schedule* in);
  *                  MMAs in flight drain at the default limit and its TMEM is freed);
  *                  that element and every element the CTA still takes from the queue
  *                  come back IEDG_ELEM_TIMEOUT.
- *   asm_wait_limit: the same for the waits of the FP64 assembly on the tensor cores (3D,
- *                  degree 2..4): a wait that gives up leaves NaN in the matrices of that
- *                  CTA's elements, which come back IEDG_ELEM_NONFINITE.
- * The settings stay until changed; {-1, 0, -1, 0, 0} restores normal operation.
+ *                  On FP64 handles it also holds for the assembly's waits (3D, degree
+ *                  2..4): one that gives up leaves NaN in the matrices of that CTA's
+ *                  elements, which a DFMA LU then reports as IEDG_ELEM_NONFINITE.
+ * The settings stay until changed; {-1, 0, -1, 0} restores normal operation.
  * IEDG_ERR_INVALID_ARG for values out of range, IEDG_ERR_UNSUPPORTED for zero_row_elem
  * on meshes with mixed orders. */
 typedef struct {
@@ -334,7 +335,7 @@ typedef struct {
   int32_t zero_row;
   int32_t refine_iters;
   int32_t tc_wait_limit;
-  int32_t asm_wait_limit;
+  int32_t reserved;
 } iedg_fault_injection;
 int iedg_set_fault_injection(iedg_mesh* mesh, const iedg_fault_injection* f);
 

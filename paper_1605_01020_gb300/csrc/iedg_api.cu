@@ -1204,7 +1204,7 @@ extern "C" int iedg_profile_reset(iedg_mesh* M) {
 extern "C" int iedg_set_fault_injection(iedg_mesh* M, const iedg_fault_injection* f) {
   if (!M || !f) return fail(M, IEDG_ERR_INVALID_ARG, "null argument");
   if (f->zero_row_elem < -1 || f->zero_row_elem >= M->E || f->refine_iters < -1 || f->refine_iters > 16 ||
-      f->tc_wait_limit < -1 || f->asm_wait_limit < -1 || (f->zero_row_elem >= 0 && (f->zero_row < 0 || f->zero_row >= M->dm.nu)))
+      f->tc_wait_limit < -1 || (f->zero_row_elem >= 0 && (f->zero_row < 0 || f->zero_row >= M->dm.nu)))
     return fail(M, IEDG_ERR_INVALID_ARG, "fault injection values out of range");
   if (f->zero_row_elem >= 0 && M->mixed_orders)
     return fail(M, IEDG_ERR_UNSUPPORTED, "zero-row injection is only available on uniform meshes");
@@ -1212,7 +1212,6 @@ extern "C" int iedg_set_fault_injection(iedg_mesh* M, const iedg_fault_injection
   M->fault.zero_row = f->zero_row;
   M->fault.refine_iters = f->refine_iters;
   M->fault.tc_wait_limit = f->tc_wait_limit;
-  M->fault.asm_wait_limit = f->asm_wait_limit;
   for (iedg_mesh* C : M->groups) C->fault = M->fault;
   return IEDG_OK;
 }

@@ -49,7 +49,6 @@ struct Fault {
   int zero_row = 0;
   int refine_iters = -1;        // correction steps of the refinement (-1 = kRefineMaxIter)
   int tc_wait_limit = 0;        // polls of a tensor-core completion wait (0 = kTcWaitLimit, -1 = none)
-  int asm_wait_limit = 0;       // the same for the waits of the FP64 digit assembly
 };
 constexpr int kTcWaitLimit = 1 << 26;
 
@@ -359,9 +358,8 @@ inline int tc_wait_limit(const iedg_mesh* M) {
   return M->fault.tc_wait_limit > 0 ? M->fault.tc_wait_limit : (M->fault.tc_wait_limit < 0 ? 0 : kTcWaitLimit);
 }
 
-inline int asm_wait_limit(const iedg_mesh* M) {
-  return M->fault.asm_wait_limit > 0 ? M->fault.asm_wait_limit : (M->fault.asm_wait_limit < 0 ? 0 : kTcWaitLimit);
-}
+// the FP64 digit assembly's waits; as the fallback of the mixed forms it keeps the usual limit
+inline int asm_wait_limit(const iedg_mesh* M) { return M->precision == 0 ? tc_wait_limit(M) : kTcWaitLimit; }
 
 // refinement controls of the mixed path
 constexpr int kRefineMaxIter = 8;

@@ -52,7 +52,7 @@ class Schedule(ctypes.Structure):
 
 class FaultInjection(ctypes.Structure):
     _fields_ = [("zero_row_elem", ctypes.c_int64), ("zero_row", ctypes.c_int32), ("refine_iters", ctypes.c_int32),
-                ("tc_wait_limit", ctypes.c_int32), ("asm_wait_limit", ctypes.c_int32)]
+                ("tc_wait_limit", ctypes.c_int32), ("reserved", ctypes.c_int32)]
 
 
 _lib = None
@@ -320,12 +320,10 @@ class Mesh:
         sc = Schedule(cur["lu_persistent"], cur["lu_panel"], cur["asm_chunk"], cur["lu_tensor"], by)
         self._check(load().iedg_set_schedule(self._h, ctypes.byref(sc)))
 
-    def set_fault_injection(self, zero_row_elem=-1, zero_row=0, refine_iters=-1, tc_wait_limit=0,
-                            asm_wait_limit=0):
+    def set_fault_injection(self, zero_row_elem=-1, zero_row=0, refine_iters=-1, tc_wait_limit=0):
         """Host-side fault injection for tests (iedg_set_fault_injection); the defaults
         restore normal operation."""
-        f = FaultInjection(int(zero_row_elem), int(zero_row), int(refine_iters), int(tc_wait_limit),
-                           int(asm_wait_limit))
+        f = FaultInjection(int(zero_row_elem), int(zero_row), int(refine_iters), int(tc_wait_limit), 0)
         self._check(load().iedg_set_fault_injection(self._h, ctypes.byref(f)))
 
     # ------------------------------------------------------------------ tracing
